@@ -18,11 +18,13 @@ extern "C" {
  * (one thread per output, one launch per phase), 2 = fast kernels (tensor-core projection,
  * persistent recurrent kernel); 2 fails with QLSTM_ERR_DIM at run time if a shape is unsupported.
  * recurrent_impl 2 always runs layer after layer (projection launch + persistent kernel per layer), where 0 takes the
- * whole-stack kernel at small batches (up to 4 rows; up to 8 for stacks of two or more layers; up to 16 for four or more); 3 = like 2 but with the tensor-core matmuls even at batch <= 4, where 2 uses dp4a
+ * wavefront kernel for stacks of three or more layers beyond 4 rows and for dimensions that are no multiples of 16, and
+ * the whole-stack kernel at small batches; 3 = like 2 but with the tensor-core matmuls even at batch <= 4, where 2 uses dp4a
  * mat-vecs; 4 = like 2 but with the dp4a mat-vecs up to batch 16 (the crossover is a measured default, not a limit);
  * 5 = the whole-stack kernel or QLSTM_ERR_DIM (batch > 16, or a dimension that is not a multiple of 16), with its
  * schedule chosen from the call's length; 6 = the same with the wavefront schedule (one group of blocks per layer)
- * forced, 7 = with the sequential schedule (every layer on all blocks) forced. */
+ * forced, 7 = with the sequential schedule (every layer on all blocks) forced; 8 = the wavefront kernel (every layer at
+ * once on its own group of SMs, tensor-core products, up to 256 rows, any dimensions) or QLSTM_ERR_DIM. */
 int qlstm_set_impl(qlstm_t *q, int projection_impl, int recurrent_impl);
 
 /* Failure-path check: with missing_arrivals > 0 every grid barrier of the persistent recurrent kernel (and every

@@ -88,6 +88,18 @@ int launch_stack_small(StackSmall *s, const int8_t *x, int T, int B, int8_t *h, 
 void stack_small_debug_timeout(StackSmall *s, unsigned missing_arrivals, unsigned long long limit_ns);
 int stack_small_groups(const StackSmall *s, int *blocks_per_layer);     // layers, and the blocks each layer's group has
 
+// ---- wavefront kernel (wave_sm100.cu): all layers and steps in one cooperative launch, tensor-core products, batches up to
+// 256 rows, any dimensions.
+struct WaveStack;
+int wave_create(const std::vector<const LayerParams *> &layers, int max_T, int max_B, int sm_count, WaveStack **out);
+void wave_destroy(WaveStack *s);
+bool wave_supported(const WaveStack *s, int T, int B);
+bool wave_preferred(const WaveStack *s, int T, int B);             // supported and, by measurement, the faster path
+// tables: memoised nonlinearities where they pay.  The launch clears the status word itself.
+int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *h, int16_t *c, int8_t *y, int *status, bool tables, cudaStream_t st,
+                int *launches);
+void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns);
+
 int debug_ring_plan(int stages, int n_own, int contig, int per, int n_total, int *out);
 int debug_projection_plan(long long rows_hint, long long rows, int N, int K, int sm_count, int max_smem, int *out5);
 

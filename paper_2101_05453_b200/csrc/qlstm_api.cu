@@ -39,6 +39,8 @@ struct qlstm {
     SimpleScratch scratch = {};
     FastScratch fscratch = {};
     StackSmall *stack = nullptr;    // whole-stack kernel for small batches, or null
+    WaveStack *wave = nullptr;      // wavefront kernel, or null
+    bool tables = true;             // memoised nonlinearities (a test turns them off)
     int *status = nullptr;          // device status word of the persistent kernel
     unsigned long long *phase_ns = nullptr;   // device phase timers of the persistent kernel (profiling)
     // staging for qlstm_run_host
@@ -155,6 +157,12 @@ int build_layer(const qlstm_layer_t &l, LayerHost &L)
             if (peep && g != 2) P[n] = l.P[g][u];
         }
     }
+    auto largest = [](const auto &v) {
+        int64_t m = 0;
+        for (auto x : v) { const int64_t a = x < 0 ? -(int64_t)x : (int64_t)x; if (a > m) m = a; }
+        return m;
+    };
+    p.max_bx = largest(bx); p.max_bh = largest(bh); p.max_bln = largest(bln); p.max_L = largest(Lw);
     cudaError_t e;
     if ((e = dev_upload(L, W, &p.W)) != cudaSuccess) return QLSTM_ERR_NOMEM;
     if ((e = dev_upload(L, R, &p.R)) != cudaSuccess) return QLSTM_ERR_NOMEM;
@@ -174,6 +182,7 @@ int build_layer(const qlstm_layer_t &l, LayerHost &L)
             if (f > INT32_MAX || f < INT32_MIN) return QLSTM_ERR_RANGE;
             bp[o] = (int32_t)f;
         }
+        p.max_bp = largest(bp);
         if ((e = dev_upload(L, Wp, &p.Wproj)) != cudaSuccess) return QLSTM_ERR_NOMEM;
         if ((e = dev_upload(L, bp, &p.bp)) != cudaSuccess) return QLSTM_ERR_NOMEM;
     }
@@ -313,6 +322,7 @@ int qlstm_create(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B
         std::vector<const LayerParams *> lp;
         for (auto &L : q->layers) lp.push_back(&L.p);
         int src = stack_small_create(lp, max_T, max_B, q->sm_count, &q->stack);
+        if (src == QLSTM_OK) src = wave_create(lp, max_T, max_B, q->sm_count, &q->wave);
         if (src != QLSTM_OK) { ok = false; rc = src; }
     }
     if (!ok) { qlstm_destroy(q); return rc; }
@@ -331,6 +341,7 @@ void qlstm_destroy(qlstm_t *q)
     }
     fast_scratch_destroy(q->fscratch);
     stack_small_destroy(q->stack);
+    wave_destroy(q->wave);
     cudaFree(q->X); cudaFree(q->seq[0]); cudaFree(q->seq[1]);
     cudaFree(q->scratch.pre); cudaFree(q->scratch.po); cudaFree(q->scratch.stats); cudaFree(q->scratch.m);
     cudaFree(q->status);
@@ -367,6 +378,16 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
     if (trace && cudaMemsetAsync(trace, 0, qlstm_trace_bytes(q, T, B), st) != cudaSuccess) return QLSTM_ERR_CUDA;
     const int nl = (int)q->layers.size();
     // small batches: the whole stack in one launch (layers as a wavefront, input projection inside the step)
+    if (!trace && (q->impl_rec == 0 || q->impl_rec == 8) && q->impl_proj != 1) {
+        if (q->impl_rec == 0 ? wave_preferred(q->wave, T, B) : wave_supported(q->wave, T, B)) {
+            SpanGuard g(q, st, 1);
+            int launches = 0;
+            const int rc = launch_wave(q->wave, x_dev, T, B, h_dev, c_dev, y_dev, q->status, q->tables, st, &launches);
+            g.done(launches);
+            return rc;
+        }
+        if (q->impl_rec == 8) return QLSTM_ERR_DIM;
+    }
     if (!trace && (q->impl_rec == 0 || q->impl_rec >= 5) && q->impl_proj != 1) {
         if (q->impl_rec == 0 ? stack_small_preferred(q->stack, T, B) : stack_small_supported(q->stack, T, B)) {
             SpanGuard g(q, st, 1);
@@ -477,7 +498,7 @@ int qlstm_last_status(qlstm_t *q)
 
 int qlstm_set_impl(qlstm_t *q, int projection_impl, int recurrent_impl)
 {
-    if (!q || projection_impl < 0 || projection_impl > 2 || recurrent_impl < 0 || recurrent_impl > 7) return QLSTM_ERR_ARG;
+    if (!q || projection_impl < 0 || projection_impl > 2 || recurrent_impl < 0 || recurrent_impl > 8) return QLSTM_ERR_ARG;
     q->impl_proj = projection_impl;
     q->impl_rec = recurrent_impl;
     return QLSTM_OK;
@@ -492,6 +513,7 @@ int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long 
         L.fast.dbg_spin_limit_ns = missing_arrivals > 0 ? limit_ns : 0;
     }
     stack_small_debug_timeout(q->stack, (unsigned)missing_arrivals, limit_ns);
+    wave_debug_timeout(q->wave, (unsigned)missing_arrivals, limit_ns);
     return QLSTM_OK;
 }
 
@@ -499,6 +521,7 @@ int qlstm_debug_activation_tables(qlstm_t *q, int enable)
 {
     if (!q || enable < 0 || enable > 2) return QLSTM_ERR_ARG;
     int n = 0;
+    q->tables = enable == 1;
     for (auto &L : q->layers) {
         L.fast.dbg_no_tables = enable == 0;
         L.fast.dbg_general_kernel = enable == 2;

@@ -31,6 +31,7 @@ struct LayerParams {
     const int32_t *bln;                // [N]  layer-norm bias
     Scale eff_x[4], eff_h[4], eff_c[4], eff_ln[4];   // indexed by gi
     Scale eff_m, eff_proj;
+    int64_t max_bx, max_bh, max_bp, max_bln, max_L;  // largest magnitudes of the vectors above
 };
 
 // Views into one trace record (see include/qlstm.h); all null when tracing is off.

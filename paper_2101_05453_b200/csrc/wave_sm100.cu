@@ -1,0 +1,1288 @@
+// Wavefront kernel: every layer and every time step of a stack in ONE cooperative launch, all matrix products on the
+// tensor cores, batches up to 256 rows.
+//
+// A stack run layer after layer is a chain of T x L layer-steps, each of which crosses the whole machine three or four
+// times (statistics, hidden state, output) and gives an SM only a few dozen cells to work on in between: at eight
+// 2048-cell layers and 64 rows a layer-step took 20.6 us for 2 us of arithmetic.  Here the SMs are split into one group
+// per layer (and, for shallow stacks, per range of batch rows), layer l + 1 works on a step while layer l works on a
+// later one, and the exchanges involve the 18 or so blocks of a group.  The input term W x_t of Section 3.2.4 is part of
+// the step, so no activation makes a round trip through memory beyond the layers' int8 outputs.
+//
+// A block owns a range of cells (all their gate rows) and a range of projection rows.  Its weights do not fit in shared
+// memory (656 KB for an eighteenth of a 2048-cell layer): they lie in global memory in the order and in the
+// shared-memory image in which the block's MMAs read them, and stream through a ring of contiguous bulk copies that runs
+// ahead of the dependency chain.  The batch is the M side of the MMAs: a tensor-memory lane is a batch row.
+//
+//   X(t+1)  W x_{t+1}  -> rescale -> int16                                          needs the layer below at t + 1
+//   H(t)    R h^{t-1}  -> + bias, rescale, + X(t) (+ peephole) -> gate sums, sums for the layer norm's statistics
+//           [layer norm: the group adds its sums up in L2]
+//   B(t)    layer norm, sigmoid / tanh, cell update, hidden state m (= h without a projection)
+//   P(t)    W_proj m   -> h^t
+//
+// The rows are worked on in units of at most 128.  One unit: X(t+1) is computed while the block would otherwise wait for
+// the statistics and for m.  Two units: each one's exchanges pass while the block works on the other.
+//
+// Warp roles: 0 copies activations, 1 copies weights, 2 issues MMAs, 4..19 epilogues and elementwise work.  All four
+// walk the same table of operations, so that no role needs to tell another what comes next.
+//
+// Every wait is bounded; on expiry the block sets the abort word, all blocks see it at their next wait and leave, and the
+// host reports QLSTM_ERR_TIMEOUT.
+#include <algorithm>
+#include <cstring>
+#include <utility>
+#include <vector>
+
+#include "../../include/qlstm.h"
+#include "act_table.cuh"
+#include "fast_kernels.h"
+#include "sm100_ptx.cuh"
+
+namespace ql {
+
+namespace {
+
+constexpr int WV_THREADS = 640;
+constexpr int WV_EPI_WARP0 = 4;
+constexpr int WV_EPI = WV_THREADS - 32 * WV_EPI_WARP0;         // 512 epilogue threads
+constexpr int WV_MAX_LAYERS = 16;
+constexpr int WV_A_SLOT = 128 * 128;                           // one k-block of 128 activation rows
+constexpr int WV_MAX_SLOTS = 8;
+constexpr int WV_MAX_OPS = 96;
+constexpr int WV_ACC_COLS = 256;                               // columns of each of the two accumulators
+constexpr unsigned long long WV_WAIT_LIMIT_NS = 2000000000ull;
+
+// counters of one (layer, unit), each on a line of its own
+enum { WC_STATS = 0, WC_STATS2 = 1, WC_M = 2, WC_H = 3, WC_PER_UNIT = 4, WC_WORDS = 32 };
+
+enum { OP_X = 0, OP_H = 1, OP_P = 2, OP_S = 3, OP_B = 4, OP_F = 5 };
+struct WaveOp { uint8_t kind, u, tile, pad; };
+
+struct WaveLayer {
+    int I, C, O;
+    uint32_t flags;
+    int m_bits, zp_m, zp_h;
+    int cta0, n;                   // first block of row group 0, blocks per (layer, row group)
+    int ppc;                       // cell pairs per block
+    int nt, ppt, npad;             // gate tiles: count, pairs per tile, MMA columns
+    int opc, ntp, opt, npadp;      // outputs per block; projection tiles: count, outputs per tile, MMA columns
+    int kb_i, kb_h, kb_c;          // 128-byte k-blocks of the three products
+    int k32_i, k32_h, k32_c;       // K steps of 32
+    const int8_t *img_w, *img_r, *img_p;
+    const int32_t *bx, *bh, *bln, *bp;
+    const int16_t *P, *L;
+    int x_left[4], h_left[4];      // left shift before the rescale of the input / recurrent term (0 for scales below 1)
+    FastScale f_x[4], f_h[4], f_c[4], f_ln[4], f_m, f_proj;      // by gate slot
+    float ln_limit;                // layer-norm quotients below this keep q' L + b inside an int32
+    DivMagic div_c;
+    int8_t *in_img;                // [T][units][kb_i][ra][128] input activations
+    int8_t *out_img;               // [T + 1][units][kb_h][ra][128]: slot t + 1 holds h^t
+    int8_t *m_img;                 // [units][kb_c][ra][128]
+    long long *totals;             // [2][units][ra][4][2] layer-norm sums of the group
+    unsigned *cnt;                 // [units][WC_PER_UNIT][WC_WORDS]
+    int below;                     // blocks of the layer below, 0: none
+    long long h_off, c_off;        // of this layer in the caller's state, in units of one batch row
+    const uint8_t *tab;
+    ActTabLayout tab_lay;
+};
+
+struct WaveCall {
+    int T, B, n_layers, rg, units; // row groups; units of a row group
+    int nu, ra;                    // units in all, rows of an activation image's k-block
+    int nrep;                      // copies of a unit's rows in the 128 lanes
+    int early;                     // one unit: X(t + 1) before B(t) and P(t)
+    int tab;                       // memoised nonlinearities (resident in shared memory)
+    int na, nb, b_slot;            // ring depths, bytes of a weight slot
+    int gx_s;                      // gate buffers in shared memory
+    int nbuf;                      // gate buffers per unit: [gate sums | X ...]
+    int max_ppc, max_opc, max_tab;
+    int8_t *h; int16_t *c; int8_t *y;
+    uint4 *gbuf;                   // [blocks][units][nbuf][max_ppc][max rows] gate buffers in global memory
+    uint32_t *cbuf;                // [blocks][units][max_ppc][max rows] cell states
+    unsigned *abort_word;
+    int *status;
+    unsigned long long limit_ns;
+    unsigned missing;
+    WaveLayer layer[WV_MAX_LAYERS];
+};
+
+struct WaveCtl {
+    uint64_t a_full[WV_MAX_SLOTS], a_empty[WV_MAX_SLOTS], b_full[WV_MAX_SLOTS], b_empty[WV_MAX_SLOTS];
+    uint64_t t_full[2], t_empty[2], tab_full;
+    uint32_t tmem_base;
+    int abort_flag;
+    int exit_at;                   // meeting point of the epilogue threads at which they all leave
+    int n_ops, n_pro;              // operations of a step; of the prologue (X of step 0)
+    WaveOp ops[WV_MAX_OPS];
+};
+
+// ---- waits ---------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ bool wv_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
+{
+    // each attempt parks the thread for up to 20 us; 100 000 attempts bound the wait to about 2 s
+    for (uint32_t i = 0; i < 100000u; ++i) {
+        if (ptx::mbar_try_wait_parked(bar, parity, 20000u)) return *abort_flag == 0;
+        if (*abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+__device__ __forceinline__ unsigned wv_ld_acquire(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long wv_timer()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)::"memory");
+    return t;
+}
+__device__ __forceinline__ void wv_fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
+// one thread: until *cnt has reached target (bounded); false once an abort is seen
+__device__ __forceinline__ bool wv_wait_count(const WaveCall &k, const unsigned *cnt, unsigned target, volatile int *abort_flag)
+{
+    target += k.missing;
+    if (wv_ld_acquire(cnt) >= target) return *abort_flag == 0;
+    const unsigned long long t0 = wv_timer();
+    unsigned spins = 0;
+    while (wv_ld_acquire(cnt) < target) {
+        if ((++spins & 31u) == 0u) {
+            if (*abort_flag) return false;
+            if (wv_ld_acquire(k.abort_word) != 0u) { *abort_flag = 1; return false; }
+            if (wv_timer() - t0 > k.limit_ns) { atomicExch(k.abort_word, 1u); *abort_flag = 1; return false; }
+        }
+    }
+    return *abort_flag == 0;
+}
+__device__ __forceinline__ void wv_epi_sync() { asm volatile("barrier.sync 1, 512;" ::: "memory"); }
+
+// ---- fixed-point pieces ----------------------------------------------------------------------------------------------
+__device__ __forceinline__ int32_t wv_lo(uint32_t w) { return (int32_t)(w << 16) >> 16; }
+__device__ __forceinline__ int32_t wv_hi(uint32_t w) { return (int32_t)w >> 16; }
+
+// byte offset of element (row, col) in a unit's activation image (see tile_off in recurrent_sm100.cu; k-blocks of ra rows)
+__device__ __forceinline__ uint32_t wv_img_off(int row, int col, int ra)
+{
+    return (uint32_t)((col >> 7) * (ra * 128) + (row << 7) + (((((col >> 4) & 7) ^ (row & 7)) << 4) | (col & 15)));
+}
+
+// What a block keeps in shared memory besides the rings.  Columns of a pair of cells: slot-major, [slot][cell of the pair].
+struct WaveSmem {
+    int32_t *bx, *bh, *bln;        // [ppc][8]
+    int16_t *L, *P;                // [ppc][8]
+    int32_t *bp;                   // [opc]
+    uint32_t *st;                  // [4 slots][3][128] layer-norm sums of the block: sum, low 20 bits and rest of the squares
+    int4 *ln;                      // [4 slots][128] mean, sigma, 1024 / sigma, estimate's offset
+    uint8_t *tab;
+};
+
+// Who a block is, and the buffers of its rows.
+struct WaveRole {
+    int li, rank, rgi;
+    int pairs, u0;                 // own cell pairs, first cell
+    int o_lo, outs;                // own projection outputs
+    int row0[2], rows[2];          // units: first batch row, rows
+    int gu[2];                     // unit numbers among all units
+    uint4 *g[2];                   // gate buffers of the units: nbuf x [pairs][rows]
+    uint32_t *c[2];                // cell states [pairs][rows]
+    int n_rows_max;
+};
+
+// X and H epilogue of one tile for one thread = one batch row: pairs part, part + nparts, ... of the tile, two at a time.
+// Per column:  X = sat16(rescale(acc + bx, eff_x));  H = sat16(rescale(acc + bh, eff_h)); gate = sat16(X + H [+ peephole])
+// (the sums acc + b fit 32 bits: checked on the host).
+template <int G, bool LN, bool PEEP, bool IS_H>
+__device__ __forceinline__ void wv_gate_tile(const WaveLayer &L, const WaveSmem &s, uint32_t taddr, int pair0, int np, int part, int nparts,
+                                             int row, int rows, bool valid, const uint4 *xbuf, uint4 *gbuf, const uint32_t *cbuf)
+{
+    constexpr int SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
+    int32_t sum[4] = {0, 0, 0, 0};
+    long long sq[4] = {0, 0, 0, 0};
+    auto one = [&](const uint32_t (&r)[8], int p, const uint4 &x4) {
+        const int pr = pair0 + p;
+        const int32_t *bias = (IS_H ? s.bh : s.bx) + pr * 8;
+        const int4 b0 = *reinterpret_cast<const int4 *>(bias), b1 = *reinterpret_cast<const int4 *>(bias + 4);
+        const int32_t bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        const uint32_t xw[4] = {x4.x, x4.y, x4.z, x4.w};
+        uint32_t w[4] = {0, 0, 0, 0};
+        int32_t c_old[2] = {0, 0};
+        uint32_t pw[4] = {0, 0, 0, 0};
+        if (IS_H && PEEP) {
+            const uint32_t cw = cbuf[pr * rows + row];
+            c_old[0] = wv_lo(cw); c_old[1] = wv_hi(cw);
+            const uint4 p4 = *reinterpret_cast<const uint4 *>(s.P + pr * 8);
+            pw[0] = p4.x; pw[1] = p4.y; pw[2] = p4.z; pw[3] = p4.w;
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            int32_t v[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                int32_t acc = (int32_t)r[2 * g + k] + bb[2 * g + k];
+                acc <<= IS_H ? L.h_left[g] : L.x_left[g];
+                v[k] = fast_rescale(acc, IS_H ? L.f_h[g] : L.f_x[g]);
+                if (IS_H && !(PEEP && g == SO)) {
+                    v[k] = sat16(v[k]) + (k ? wv_hi(xw[g]) : wv_lo(xw[g]));
+                    if (PEEP && g != SZ) {
+                        const int32_t P = k ? wv_hi(pw[g]) : wv_lo(pw[g]);
+                        v[k] += sat16(fast_rescale(P * c_old[k], L.f_c[g]));
+                    }
+                }
+            }
+            w[g] = ptx::pack_sat_s16(v[0], v[1]);          // (output gate with a peephole: H alone, the rest once c^t exists)
+            if (IS_H && LN && !(PEEP && g == SO)) {
+                const int32_t a = wv_lo(w[g]), b = wv_hi(w[g]);
+                sum[g] = __dp2a_lo((int)w[g], 0x0101, sum[g]);
+                sq[g] += (long long)a * a;
+                sq[g] += (long long)b * b;
+            }
+        }
+        gbuf[pr * rows + row] = make_uint4(w[0], w[1], w[2], w[3]);
+    };
+    // four gates: two pairs nparts apart, eight columns each; three gates: two adjacent pairs, twelve columns in pieces of
+    // four (np is then even)
+#pragma unroll 1
+    for (int p = (G == 4 ? part : 2 * part); p < np; p += 2 * nparts) {
+        const int pb = G == 4 ? p + nparts : p + 1;
+        const bool two = G == 3 || pb < np;                // warp-uniform
+        uint32_t acc[2][8];
+        __syncwarp();
+        if (G == 4) {
+            ptx::tmem_ld_32x8(taddr + (uint32_t)(p * 8), acc[0]);
+            if (two) ptx::tmem_ld_32x8(taddr + (uint32_t)(pb * 8), acc[1]);
+        } else {
+            uint32_t q[3][4];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) ptx::tmem_ld_32x4(taddr + (uint32_t)(p * 6 + 4 * i), q[i]);
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 12; ++i) acc[i / 6][i % 6] = q[i >> 2][i & 3];
+            acc[0][6] = acc[0][7] = acc[1][6] = acc[1][7] = 0;
+        }
+        uint4 xa = make_uint4(0, 0, 0, 0), xb = xa;
+        if (IS_H && valid) {
+            xa = xbuf[(pair0 + p) * rows + row];
+            if (two) xb = xbuf[(pair0 + pb) * rows + row];
+        }
+        if (G == 4) ptx::tmem_ld_wait();
+        if (valid) {
+            one(acc[0], p, xa);
+            if (two) one(acc[1], pb, xb);
+        }
+    }
+    if (IS_H && LN && valid) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            if (PEEP && g == SO) continue;
+            uint32_t *st = s.st + (g * 3) * 128 + row;
+            atomicAdd(st, (uint32_t)sum[g]);
+            atomicAdd(st + 128, (uint32_t)((unsigned long long)sq[g] & 0xfffffu));
+            atomicAdd(st + 256, (uint32_t)((unsigned long long)sq[g] >> 20));
+        }
+    }
+}
+
+// Projection epilogue of one tile for one thread = one batch row, four outputs at a time.
+__device__ __forceinline__ void wv_proj_tile(const WaveCall &k, const WaveLayer &L, const WaveSmem &s, const WaveRole &r, uint32_t taddr,
+                                             int o_first, int no, int part, int nparts, int row, bool valid, int8_t *out_unit, int b, int t,
+                                             bool last_layer)
+{
+    const int nq = (no + 3) >> 2;
+#pragma unroll 1
+    for (int q = part; q < nq; q += nparts) {
+        uint32_t a[4];
+        __syncwarp();
+        ptx::tmem_ld_32x4(taddr + (uint32_t)(q * 4), a);
+        ptx::tmem_ld_wait();
+        const int col = r.o_lo + o_first + q * 4;
+        if (!valid || col >= L.O) continue;
+        const int4 b4 = *reinterpret_cast<const int4 *>(s.bp + o_first + q * 4);
+        const int32_t bb[4] = {b4.x, b4.y, b4.z, b4.w};
+        uint32_t w = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int32_t v = sat8(fast_rescale((int32_t)a[j] + bb[j], L.f_proj) + L.zp_h);
+            w |= (uint32_t)(v & 0xff) << (8 * j);
+        }
+        *reinterpret_cast<uint32_t *>(out_unit + wv_img_off(row, col, k.ra)) = w;
+        const bool fin = t == k.T - 1;
+        if (last_layer || fin) {
+            int8_t *dst[2] = {last_layer ? k.y + ((size_t)t * k.B + b) * L.O + col : nullptr,
+                              fin ? k.h + L.h_off * k.B + (size_t)b * L.O + col : nullptr};
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                if (!dst[d]) continue;
+                if (((uintptr_t)dst[d] & 3) == 0 && col + 4 <= L.O) *reinterpret_cast<uint32_t *>(dst[d]) = w;
+                else
+                    for (int j = 0; j < 4; ++j)
+                        if (col + j < L.O) dst[d][j] = (int8_t)(w >> (8 * j));
+            }
+        }
+    }
+}
+
+// ---- elementwise phase -----------------------------------------------------------------------------------------------
+
+struct WvLnRow { int32_t mean; uint32_t sigma; float inv1024, off; };      // see ln_quotient_core in qmath.cuh
+
+__device__ __forceinline__ int4 wv_make_ln(long long sum, long long sq, const DivMagic &div)
+{
+    const LnRow r = make_ln_row(ln_stats_fast(sum, sq, div));
+    // sigma = 0: the quotient is 0; a divisor that no remainder reaches keeps the correction step from adding to it
+    const uint32_t sg = r.sigma ? r.sigma : 0xffffffffu;
+    const float off = (float)(r.sigma >> 1) * r.inv_sigma - 0.05f;
+    return make_int4(r.mean, (int)sg, __float_as_int(1024.0f * r.inv_sigma), __float_as_int(off));
+}
+
+// exact value for quotients beyond the fast range (a tiny sigma against a large deviation), out of line
+__device__ __noinline__ int32_t wv_ln_slow(int32_t q, int4 row, int32_t Lw, int32_t b)
+{
+    const int32_t d = 1024 * q - row.x;
+    const uint32_t ad = (uint32_t)(d < 0 ? -d : d), sg = (uint32_t)row.y;
+    const uint64_t quo = sg == 0xffffffffu ? 0u : ((uint64_t)ad * 1024u + (sg >> 1)) / sg;
+    const int64_t qp = d < 0 ? -(int64_t)quo : (int64_t)quo;
+    return sat32_halves(qp * (int64_t)Lw + (int64_t)b);
+}
+
+// sat32(q' L + b) with q' = round(2^10 (2^10 q - mean) / sigma): fp32 estimate biased low by 0.05 (its error is below 0.02
+// for quotients under 2^16: four roundings of 2^-24 and 2^-25), one exact remainder test.  slow: the quotient is beyond
+// `limit` and the value is not usable.
+__device__ __forceinline__ int32_t wv_ln_fast(int32_t q, const int4 &row, int32_t Lw, int32_t b, float limit, bool &slow)
+{
+    const int32_t d = 1024 * q - row.x;
+    const uint32_t ad = (uint32_t)(d < 0 ? -d : d);
+    const float est = __fmaf_rn((float)ad, __int_as_float(row.z), __int_as_float(row.w));
+    slow = slow || !(est < limit);
+    uint32_t qe = __float2uint_rz(est);
+    const uint32_t sg = (uint32_t)row.y, half = sg == 0xffffffffu ? 0u : sg >> 1;
+    const uint32_t rem = (ad << 10) + half - qe * sg;
+    qe += rem >= sg ? 1u : 0u;
+    const int32_t qp = d < 0 ? -(int32_t)qe : (int32_t)qe;
+    return qp * Lw + b;
+}
+
+// The gate values of a pair after layer norm (slots in `mask`), in place.
+template <int G>
+__device__ __forceinline__ void wv_ln_pair(const WaveLayer &L, const WaveSmem &s, const int4 (&row)[4], int pr, unsigned mask, int32_t (&a)[4][2])
+{
+    const uint4 lw = *reinterpret_cast<const uint4 *>(s.L + pr * 8);
+    const uint32_t lws[4] = {lw.x, lw.y, lw.z, lw.w};
+    const int4 b0 = *reinterpret_cast<const int4 *>(s.bln + pr * 8), b1 = *reinterpret_cast<const int4 *>(s.bln + pr * 8 + 4);
+    const int32_t bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+    int32_t v[4][2];
+    bool slow = false;
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if ((mask >> g) & 1u) v[g][k] = wv_ln_fast(a[g][k], row[g], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k], L.ln_limit, slow);
+    if (slow) {
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if ((mask >> g) & 1u) v[g][k] = wv_ln_slow(a[g][k], row[g], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k]);
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if ((mask >> g) & 1u) a[g][k] = sat16(fast_rescale(v[g][k], L.f_ln[g]));
+}
+
+template <bool TAB>
+__device__ __forceinline__ int32_t wv_sigmoid(const ActTabs &at, int32_t x)
+{
+    if constexpr (TAB) return tab_sigmoid(at, x);
+    else return sigmoid_q_fast(x, 3);
+}
+template <bool TAB>
+__device__ __forceinline__ int32_t wv_tanh(const ActTabs &at, int32_t x)
+{
+    if constexpr (TAB) return tab_tanh_gate(at, x);
+    else return tanh_q_fast(x, 3);
+}
+template <bool TAB>
+__device__ __forceinline__ int32_t wv_hidden(const WaveLayer &L, const ActTabs &at, int32_t o, int32_t c_new)
+{
+    int32_t tc;
+    if constexpr (TAB) tc = tab_tanh_cell(at, c_new);
+    else tc = tanh_q_fast(c_new, L.m_bits);
+    return sat8(fast_rescale(o * tc, L.f_m) + L.zp_m);                     // Section 3.2.7
+}
+
+// m of a pair of cells (h of a layer without a projection) to where the next product and the caller read it
+__device__ __forceinline__ void wv_store_m(const WaveCall &k, const WaveLayer &L, int8_t *img_unit, int row, int u, int b, int t, int32_t m0, int32_t m1,
+                                           bool last_layer)
+{
+    if (u >= L.C) return;
+    const uint16_t w = (uint16_t)((m0 & 0xff) | ((m1 & 0xff) << 8));
+    *reinterpret_cast<uint16_t *>(img_unit + wv_img_off(row, u, k.ra)) = w;
+    if (L.flags & F_PROJECTION) return;
+    const bool both = u + 1 < L.C, fin = t == k.T - 1;
+    if (last_layer) {
+        int8_t *y = k.y + ((size_t)t * k.B + b) * L.O + u;
+        if (both && ((uintptr_t)y & 1) == 0) *reinterpret_cast<uint16_t *>(y) = w;
+        else { y[0] = (int8_t)m0; if (both) y[1] = (int8_t)m1; }
+    }
+    if (fin) {
+        int8_t *h = k.h + L.h_off * k.B + (size_t)b * L.O + u;
+        h[0] = (int8_t)m0;
+        if (both) h[1] = (int8_t)m1;
+    }
+}
+
+__device__ __forceinline__ void wv_store_c(const WaveCall &k, const WaveLayer &L, int u, int b, int32_t c0, int32_t c1)
+{
+    int16_t *c = k.c + L.c_off * k.B + (size_t)b * L.C + u;
+    if (u < L.C) c[0] = (int16_t)c0;
+    if (u + 1 < L.C) c[1] = (int16_t)c1;
+}
+
+// sums of a unit's rows (gate slots in `mask`) from shared memory into the group's totals; clears the block's own
+template <int G>
+__device__ __forceinline__ void wv_push_stats(const WaveSmem &s, long long *totals, int rows, unsigned mask, int tid)
+{
+    for (int i = tid; i < rows * G; i += WV_EPI) {
+        const int g = i / rows, row = i - g * rows;
+        if (!((mask >> g) & 1u)) continue;
+        uint32_t *st = s.st + (g * 3) * 128 + row;
+        const long long sum = (long long)(int32_t)st[0];
+        const unsigned long long sq = ((unsigned long long)st[256] << 20) + st[128];
+        st[0] = st[128] = st[256] = 0u;
+        unsigned long long *dst = reinterpret_cast<unsigned long long *>(totals + (size_t)(row * 4 + g) * 2);
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"((unsigned long long)sum) : "memory");
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst + 1), "l"(sq) : "memory");
+    }
+}
+// layer-norm constants of a unit's rows from the group's totals
+template <int G>
+__device__ __forceinline__ void wv_pull_stats(const WaveLayer &L, const WaveSmem &s, const long long *totals, int rows, unsigned mask, int tid)
+{
+    for (int i = tid; i < rows * G; i += WV_EPI) {
+        const int g = i / rows, row = i - g * rows;
+        if (!((mask >> g) & 1u)) continue;
+        const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(totals + (size_t)(row * 4 + g) * 2));
+        s.ln[g * 128 + row] = wv_make_ln(v.x, v.y, L.div_c);
+    }
+}
+// The epilogue threads meet at named barriers, so they have to agree on where to leave after an abort: one thread looks at
+// the abort flag before the barrier of a meeting point and writes the point's number down; everybody leaves at the first
+// point that is not before it.
+struct WvPoint { volatile int *abort_flag, *exit_at; int n; };
+
+__device__ __forceinline__ bool wv_point(WvPoint &pt, int tid)
+{
+    if (tid == 0 && *pt.abort_flag) { if (*pt.exit_at > pt.n) *pt.exit_at = pt.n; }
+    wv_epi_sync();
+    const bool stay = *pt.exit_at > pt.n;
+    ++pt.n;
+    return stay;
+}
+// all epilogue threads: publish their writes and add one arrival; false: leave
+__device__ __forceinline__ bool wv_publish(unsigned *cnt, bool operands, WvPoint &pt, int tid)
+{
+    if (operands) wv_fence_async_global();
+    const bool stay = wv_point(pt, tid);
+    if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+    return stay;
+}
+// all epilogue threads: wait for the group; false: leave
+__device__ __forceinline__ bool wv_meet(const WaveCall &k, const unsigned *cnt, unsigned target, WvPoint &pt, int tid)
+{
+    if (tid == 0) wv_wait_count(k, cnt, target, pt.abort_flag);
+    return wv_point(pt, tid);
+}
+
+// Everything between the gate sums and m for one unit.  Tasks are (pair, row) with the row fastest, so that the gate
+// buffers are read as contiguous runs; a thread keeps one row, whose layer-norm constants stay in registers.
+template <int G, bool LN, bool PEEP, bool TAB>
+__device__ __forceinline__ bool wv_elementwise(const WaveCall &k, const WaveLayer &L, const WaveSmem &s, const WaveRole &r, const ActTabs &at, int u,
+                                               int t, bool last_layer, WvPoint &pt, int tid)
+{
+    constexpr int SI = 0, SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
+    constexpr unsigned ALL = (1u << G) - 1u;
+    const int rows = r.rows[u], gu = r.gu[u];
+    unsigned *cnt = L.cnt + (size_t)gu * WC_PER_UNIT * WC_WORDS;
+    long long *tot = L.totals ? L.totals + ((size_t)(t & 1) * k.nu + gu) * k.ra * 8 : nullptr;
+    if (LN) {
+        if (!wv_meet(k, cnt + WC_STATS * WC_WORDS, (unsigned)(t + 1) * L.n, pt, tid)) return false;
+        wv_pull_stats<G>(L, s, tot, rows, PEEP ? ALL & ~(1u << SO) : ALL, tid);
+        // the other set of totals was read by everyone before this step's sums were complete: cleared for the next step,
+        // each block a share
+        long long *next = L.totals + ((size_t)((t + 1) & 1) * k.nu + gu) * k.ra * 8;
+        for (int i = r.rank * WV_EPI + tid; i < rows * 8; i += L.n * WV_EPI) next[i] = 0;
+        wv_epi_sync();
+    }
+    const int per = rows < WV_EPI ? WV_EPI / rows : 1;          // pairs in flight: threads beyond per * rows have no task
+    const int row = tid % rows, p0 = tid / rows;
+    const int b = r.row0[u] + row;
+    uint4 *g_s = r.g[u];
+    const uint4 *x_s = g_s + (size_t)(k.units == 1 ? 1 + (t & 1) : 1) * r.pairs * rows;    // peephole: X(t) is kept beside the sums
+    uint32_t *c_s = r.c[u];
+    int8_t *img = (L.flags & F_PROJECTION) ? L.m_img + (size_t)gu * L.kb_c * k.ra * 128
+                                           : L.out_img + ((size_t)(t + 1) * k.nu + gu) * L.kb_h * k.ra * 128;
+    const bool fin = t == k.T - 1;
+    int4 lr[4] = {};
+    if (LN && p0 < per) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) lr[g] = s.ln[g * 128 + row];
+    }
+    if (p0 < per) {
+#pragma unroll 1
+        for (int pr = p0; pr < r.pairs; pr += per) {
+            const uint4 g4 = g_s[pr * rows + row];
+            const uint32_t cw = c_s[pr * rows + row];
+            const uint32_t gw[4] = {g4.x, g4.y, g4.z, g4.w};
+            int32_t a[4][2];
+#pragma unroll
+            for (int g = 0; g < G; ++g) { a[g][0] = wv_lo(gw[g]); a[g][1] = wv_hi(gw[g]); }
+            if (LN) wv_ln_pair<G>(L, s, lr, pr, PEEP ? ALL & ~(1u << SO) : ALL, a);
+            const int32_t c_old[2] = {wv_lo(cw), wv_hi(cw)};
+            int32_t c_new[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int32_t f = wv_sigmoid<TAB>(at, a[SF][q]), z = wv_tanh<TAB>(at, a[SZ][q]);
+                int32_t i;
+                if (G == 4) i = wv_sigmoid<TAB>(at, a[SI][q]);
+                else { i = 32768 - f; if (i > 32767) i = 32767; }          // coupled input gate, Section 3.2.9
+                c_new[q] = cell_update_fast(i, z, f, c_old[q], L.m_bits);
+            }
+            c_s[pr * rows + row] = ((uint32_t)c_new[0] & 0xffffu) | ((uint32_t)c_new[1] << 16);
+            const int uc = r.u0 + 2 * pr;
+            if (fin) wv_store_c(k, L, uc, b, c_new[0], c_new[1]);
+            int32_t ao[2] = {a[SO][0], a[SO][1]};
+            if (PEEP) {
+                const uint4 x4 = x_s[pr * rows + row];
+                const uint32_t xo = G == 4 ? x4.w : x4.z;
+                const int32_t X[2] = {wv_lo(xo), wv_hi(xo)};
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int32_t P = s.P[pr * 8 + 2 * SO + q];
+                    ao[q] = sat16(X[q] + a[SO][q] + sat16(fast_rescale(P * c_new[q], L.f_c[SO])));     // Eq. 5: o sees c^t
+                }
+                if (LN) {
+                    // waits for the row's statistics
+                    const uint32_t w = ((uint32_t)ao[0] & 0xffffu) | ((uint32_t)ao[1] << 16);
+                    reinterpret_cast<uint32_t *>(&g_s[pr * rows + row])[SO] = w;
+                    uint32_t *st = s.st + (SO * 3) * 128 + row;
+                    const unsigned long long sq = (unsigned long long)((long long)ao[0] * ao[0] + (long long)ao[1] * ao[1]);
+                    atomicAdd(st, (uint32_t)(ao[0] + ao[1]));
+                    atomicAdd(st + 128, (uint32_t)(sq & 0xfffffu));
+                    atomicAdd(st + 256, (uint32_t)(sq >> 20));
+                    continue;
+                }
+            }
+            const int32_t m0 = wv_hidden<TAB>(L, at, wv_sigmoid<TAB>(at, ao[0]), c_new[0]);
+            const int32_t m1 = wv_hidden<TAB>(L, at, wv_sigmoid<TAB>(at, ao[1]), c_new[1]);
+            wv_store_m(k, L, img, row, uc, b, t, m0, m1, last_layer);
+        }
+    }
+    if (LN && PEEP) {
+        wv_epi_sync();
+        wv_push_stats<G>(s, tot, rows, 1u << SO, tid);
+        if (!wv_publish(cnt + WC_STATS2 * WC_WORDS, false, pt, tid)) return false;
+        if (!wv_meet(k, cnt + WC_STATS2 * WC_WORDS, (unsigned)(t + 1) * L.n, pt, tid)) return false;
+        wv_pull_stats<G>(L, s, tot, rows, 1u << SO, tid);
+        wv_epi_sync();
+        if (p0 < per) {
+            lr[SO] = s.ln[SO * 128 + row];
+#pragma unroll 1
+            for (int pr = p0; pr < r.pairs; pr += per) {
+                const uint32_t gw = reinterpret_cast<const uint32_t *>(&g_s[pr * rows + row])[SO];
+                const uint32_t cw = c_s[pr * rows + row];
+                int32_t a[4][2] = {};
+                a[SO][0] = wv_lo(gw); a[SO][1] = wv_hi(gw);
+                wv_ln_pair<G>(L, s, lr, pr, 1u << SO, a);
+                const int32_t m0 = wv_hidden<TAB>(L, at, wv_sigmoid<TAB>(at, a[SO][0]), wv_lo(cw));
+                const int32_t m1 = wv_hidden<TAB>(L, at, wv_sigmoid<TAB>(at, a[SO][1]), wv_hi(cw));
+                wv_store_m(k, L, img, row, r.u0 + 2 * pr, b, t, m0, m1, last_layer);
+            }
+        }
+    }
+    return wv_publish(cnt + ((L.flags & F_PROJECTION) ? WC_M : WC_H) * WC_WORDS, true, pt, tid);
+}
+
+// ---- the table of operations -------------------------------------------------------------------------------------------
+
+// first the prologue (X of step 0), then the operations of a step, in the order all roles follow
+__device__ void wv_build_ops(const WaveCall &k, const WaveLayer &L, const WaveRole &r, WaveCtl *ctl)
+{
+    int n = 0;
+    auto add = [&](int kind, int u, int tile) { ctl->ops[n].kind = (uint8_t)kind; ctl->ops[n].u = (uint8_t)u; ctl->ops[n].tile = (uint8_t)tile; ++n; };
+    const bool proj = (L.flags & F_PROJECTION) != 0;
+    const int nt = (r.pairs + L.ppt - 1) / L.ppt, ntp = proj ? (r.outs + L.opt - 1) / L.opt : 0;
+    auto gates = [&](int kind, int u, int from, int to) { for (int i = from; i < to; ++i) add(kind, u, i); };
+    auto project = [&](int u) {
+        if (!proj) return;
+        for (int i = 0; i < ntp; ++i) add(OP_P, u, i);
+        add(OP_F, u, 0);
+    };
+    int nu = 0;
+    while (nu < k.units && r.rows[nu] > 0) ++nu;
+    for (int u = 0; u < nu; ++u) gates(OP_X, u, 0, nt);
+    ctl->n_pro = n;
+    if (nu == 1) {
+        gates(OP_H, 0, 0, nt);
+        add(OP_S, 0, 0);
+        if (k.early) gates(OP_X, 0, 0, (nt + 1) / 2);
+        add(OP_B, 0, 0);
+        if (k.early) gates(OP_X, 0, (nt + 1) / 2, nt);
+        project(0);
+        if (!k.early) gates(OP_X, 0, 0, nt);
+    } else if (nu == 2) {
+        for (int u = 0; u < 2; ++u) { gates(OP_H, u, 0, nt); add(OP_S, u, 0); }
+        for (int u = 0; u < 2; ++u) add(OP_B, u, 0);
+        for (int u = 0; u < 2; ++u) { project(u); gates(OP_X, u, 0, nt); }
+    }
+    ctl->n_ops = n - ctl->n_pro;
+}
+
+// calls f(op, t) for every operation in order (X with the step it belongs to); stops when f returns false
+template <class F>
+__device__ __forceinline__ bool wv_walk(const WaveCtl *ctl, int T, F f)
+{
+    for (int i = 0; i < ctl->n_pro; ++i)
+        if (!f(ctl->ops[i], 0)) return false;
+    for (int t = 0; t < T; ++t)
+        for (int i = 0; i < ctl->n_ops; ++i) {
+            const WaveOp op = ctl->ops[ctl->n_pro + i];
+            if (op.kind == OP_X && t + 1 == T) continue;
+            if (!f(op, op.kind == OP_X ? t + 1 : t)) return false;
+        }
+    return true;
+}
+
+__host__ __device__ inline size_t wv_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// shared memory of a block: [A slots][B slots][control][constants][statistics][tables][gate buffers, cell states]
+struct WvLayout { size_t b_ring, ctl, consts, st, ln, tab, gates, total; };
+__host__ __device__ inline WvLayout wv_layout(int na, int nb, int b_slot, int max_ppc, int max_opc, int max_tab, size_t gates_bytes)
+{
+    WvLayout l;
+    l.b_ring = (size_t)na * WV_A_SLOT;
+    l.ctl = l.b_ring + (size_t)nb * b_slot;
+    l.consts = l.ctl + wv_up(sizeof(WaveCtl), 16);
+    l.st = l.consts + (size_t)max_ppc * 8 * (3 * 4 + 2 * 2) + wv_up((size_t)max_opc * 4, 16);
+    l.ln = l.st + 12 * 128 * 4;
+    l.tab = l.ln + 4 * 128 * 16;
+    l.gates = l.tab + wv_up((size_t)max_tab, 16);
+    l.total = l.gates + gates_bytes + 1024;        // 1024: alignment of the rings
+    return l;
+}
+
+template <int G, bool LN, bool PEEP, bool TAB>
+__global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_constant__ WaveCall k)
+{
+    extern __shared__ uint8_t wv_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)wv_raw + 1023) & ~(uintptr_t)1023);
+    const WvLayout lay = wv_layout(k.na, k.nb, k.b_slot, k.max_ppc, k.max_opc, k.max_tab, 0);
+    uint8_t *a_ring = smem, *b_ring = smem + lay.b_ring;
+    WaveCtl *ctl = reinterpret_cast<WaveCtl *>(smem + lay.ctl);
+    WaveSmem s;
+    {
+        uint8_t *p = smem + lay.consts;
+        s.bx = (int32_t *)p;  p += (size_t)k.max_ppc * 32;
+        s.bh = (int32_t *)p;  p += (size_t)k.max_ppc * 32;
+        s.bln = (int32_t *)p; p += (size_t)k.max_ppc * 32;
+        s.L = (int16_t *)p;   p += (size_t)k.max_ppc * 16;
+        s.P = (int16_t *)p;   p += (size_t)k.max_ppc * 16;
+        s.bp = (int32_t *)p;
+        s.st = (uint32_t *)(smem + lay.st);
+        s.ln = (int4 *)(smem + lay.ln);
+        s.tab = smem + lay.tab;
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = blockIdx.x;
+    volatile int *abort_flag = &ctl->abort_flag;
+
+    WaveRole r;
+    r.li = -1;
+    for (int l = 0; l < k.n_layers; ++l)
+        if (cta >= k.layer[l].cta0 && cta < k.layer[l].cta0 + k.layer[l].n * k.rg) r.li = l;
+    if (r.li < 0) return;                                      // spare block: takes no part in any counter
+    const WaveLayer &L = k.layer[r.li];
+    const bool proj = (L.flags & F_PROJECTION) != 0, last_layer = r.li == k.n_layers - 1;
+    r.rgi = (cta - L.cta0) / L.n;
+    r.rank = cta - L.cta0 - r.rgi * L.n;
+    r.u0 = r.rank * L.ppc * 2;
+    r.pairs = L.C > r.u0 ? (L.C - r.u0 + 1) / 2 : 0;
+    if (r.pairs > L.ppc) r.pairs = L.ppc;
+    if (G == 3) r.pairs = (r.pairs + 1) & ~1;
+    r.o_lo = r.rank * L.opc;
+    r.outs = proj ? (L.O - r.o_lo < L.opc ? L.O - r.o_lo : L.opc) : 0;
+    if (r.outs < 0) r.outs = 0;
+    r.n_rows_max = (k.B + k.nu - 1) / k.nu;
+    for (int u = 0; u < 2; ++u) {
+        r.gu[u] = u < k.units ? r.rgi * k.units + u : 0;
+        r.row0[u] = (int)((long long)r.gu[u] * k.B / k.nu);
+        r.rows[u] = u < k.units ? (int)((long long)(r.gu[u] + 1) * k.B / k.nu) - r.row0[u] : 0;
+        const size_t per_unit = (size_t)k.nbuf * k.max_ppc * r.n_rows_max;
+        if (k.gx_s) {
+            r.g[u] = reinterpret_cast<uint4 *>(smem + lay.gates) + u * per_unit;
+            r.c[u] = reinterpret_cast<uint32_t *>(smem + lay.gates + (size_t)k.units * per_unit * 16) + (size_t)u * k.max_ppc * r.n_rows_max;
+        } else {
+            r.g[u] = k.gbuf + ((size_t)cta * k.units + u) * per_unit;
+            r.c[u] = k.cbuf + ((size_t)cta * k.units + u) * k.max_ppc * r.n_rows_max;
+        }
+    }
+    if (r.rows[0] == 0) return;                                // fewer rows than row groups: this group is idle
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < WV_MAX_SLOTS; ++i) {
+            ptx::mbar_init(&ctl->a_full[i], 1); ptx::mbar_init(&ctl->a_empty[i], 1);
+            ptx::mbar_init(&ctl->b_full[i], 1); ptx::mbar_init(&ctl->b_empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) { ptx::mbar_init(&ctl->t_full[i], 1); ptx::mbar_init(&ctl->t_empty[i], WV_EPI / 32); }
+        ptx::mbar_init(&ctl->tab_full, 1);
+        ctl->abort_flag = 0;
+        ctl->exit_at = 0x7fffffff;
+        ptx::fence_barrier_init();
+        wv_build_ops(k, L, r, ctl);
+        if (TAB) {
+            ptx::mbar_arrive_expect_tx(&ctl->tab_full, L.tab_lay.bytes);
+            ptx::bulk_load_1d(s.tab, L.tab, L.tab_lay.bytes, &ctl->tab_full);
+        }
+    }
+    if (warp == 2) {
+        ptx::tmem_alloc(&ctl->tmem_base, 512);
+        ptx::tmem_relinquish();
+    }
+    // constants of the block's columns, slot-major within a pair of cells
+    for (int i = threadIdx.x; i < r.pairs * 8; i += WV_THREADS) {
+        const int pr = i >> 3, g = (i >> 1) & 3, u = r.u0 + 2 * pr + (i & 1);
+        const bool in = g < G && u < L.C;
+        const int n = u * G + g;
+        s.bx[i] = in ? L.bx[n] : 0;
+        s.bh[i] = in ? L.bh[n] : 0;
+        s.bln[i] = in && LN ? L.bln[n] : 0;
+        s.L[i] = in && LN ? L.L[n] : (int16_t)0;
+        s.P[i] = in && PEEP ? L.P[n] : (int16_t)0;
+    }
+    for (int i = threadIdx.x; i < r.outs; i += WV_THREADS) s.bp[i] = L.bp[r.o_lo + i];
+    for (int i = threadIdx.x; i < 12 * 128; i += WV_THREADS) s.st[i] = 0u;
+    for (int u = 0; u < 2; ++u)
+        for (int i = threadIdx.x; i < r.pairs * r.rows[u]; i += WV_THREADS) {
+            const int pr = i / r.rows[u], b = r.row0[u] + i - pr * r.rows[u], c = r.u0 + 2 * pr;
+            const int16_t *src = k.c + L.c_off * k.B + (size_t)b * L.C + c;
+            const uint32_t lo = c < L.C ? (uint16_t)src[0] : 0u, hi = c + 1 < L.C ? (uint16_t)src[1] : 0u;
+            r.c[u][i] = lo | (hi << 16);
+        }
+    ptx::tc_fence_before();
+    ptx::cta_sync();
+    ptx::tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    unsigned *cnt0 = L.cnt;
+    auto gate_tile_pairs = [&](int tile) { const int left = r.pairs - tile * L.ppt; return left < L.ppt ? left : L.ppt; };
+
+    if (warp == 0) {
+        // ---------------- activations ----------------
+        int slot = 0; uint32_t phase = 0;
+        const uint32_t kb_bytes = (uint32_t)k.ra * 128u;
+        const bool copier = lane < k.nrep;
+        wv_walk(ctl, k.T, [&](const WaveOp &op, int t) -> bool {
+            if (op.kind > OP_P) return true;
+            const int gu = r.gu[op.u];
+            const int8_t *src;
+            const unsigned *cnt = nullptr;
+            unsigned target = 0;
+            int nkb;
+            if (op.kind == OP_X) {
+                nkb = L.kb_i;
+                src = L.in_img + ((size_t)(t + (L.below ? 1 : 0)) * k.nu + gu) * nkb * kb_bytes;      // (slot 0 of a layer's outputs is h^-1)
+                if (L.below) { cnt = k.layer[r.li - 1].cnt + ((size_t)gu * WC_PER_UNIT + WC_H) * WC_WORDS; target = (unsigned)(t + 1) * L.below; }
+            } else if (op.kind == OP_H) {
+                nkb = L.kb_h;
+                src = L.out_img + ((size_t)t * k.nu + gu) * nkb * kb_bytes;
+                if (t > 0) { cnt = cnt0 + ((size_t)gu * WC_PER_UNIT + WC_H) * WC_WORDS; target = (unsigned)t * L.n; }
+            } else {
+                nkb = L.kb_c;
+                src = L.m_img + (size_t)gu * nkb * kb_bytes;
+                cnt = cnt0 + ((size_t)gu * WC_PER_UNIT + WC_M) * WC_WORDS; target = (unsigned)(t + 1) * L.n;
+            }
+            if (cnt) {
+                bool ok = true;
+                if (lane == 0) ok = wv_wait_count(k, cnt, target, abort_flag);
+                if (!__shfl_sync(0xffffffffu, (int)ok, 0)) return false;
+                __syncwarp();
+            }
+            wv_fence_async_global();
+            for (int kb = 0; kb < nkb; ++kb) {
+                bool ok = true;
+                if (lane == 0) {
+                    ok = wv_wait(&ctl->a_empty[slot], phase ^ 1u, abort_flag);
+                    if (ok) ptx::mbar_arrive_expect_tx(&ctl->a_full[slot], kb_bytes * (uint32_t)k.nrep);
+                }
+                if (!__shfl_sync(0xffffffffu, (int)ok, 0)) return false;
+                if (copier)
+                    ptx::bulk_load_1d(a_ring + (size_t)slot * WV_A_SLOT + (size_t)lane * (WV_A_SLOT / k.nrep), src + (size_t)kb * kb_bytes, kb_bytes,
+                                      &ctl->a_full[slot]);
+                if (++slot == k.na) { slot = 0; phase ^= 1u; }
+            }
+            return true;
+        });
+    } else if (warp == 1) {
+        // ---------------- weights ----------------
+        if (lane == 0) {
+            int slot = 0; uint32_t phase = 0;
+            wv_walk(ctl, k.T, [&](const WaveOp &op, int) -> bool {
+                if (op.kind > OP_P) return true;
+                const int8_t *src;
+                uint32_t bytes;
+                int nkb;
+                if (op.kind == OP_P) {
+                    nkb = L.kb_c; bytes = (uint32_t)L.npadp * 128u;
+                    src = L.img_p + (size_t)(r.rank * L.ntp + op.tile) * nkb * bytes;
+                } else {
+                    nkb = op.kind == OP_X ? L.kb_i : L.kb_h; bytes = (uint32_t)L.npad * 128u;
+                    src = (op.kind == OP_X ? L.img_w : L.img_r) + (size_t)(r.rank * L.nt + op.tile) * nkb * bytes;
+                }
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!wv_wait(&ctl->b_empty[slot], phase ^ 1u, abort_flag)) return false;
+                    ptx::mbar_arrive_expect_tx(&ctl->b_full[slot], bytes);
+                    ptx::bulk_load_1d(b_ring + (size_t)slot * k.b_slot, src + (size_t)kb * bytes, bytes, &ctl->b_full[slot]);
+                    if (++slot == k.nb) { slot = 0; phase ^= 1u; }
+                }
+                return true;
+            });
+        }
+        __syncwarp();
+    } else if (warp == 2) {
+        // ---------------- MMAs ----------------
+        if (lane == 0) {
+            int sa = 0, sb = 0, job = 0;
+            uint32_t pa = 0, pb = 0;
+            const uint64_t a_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(a_ring)), b_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(b_ring));
+            wv_walk(ctl, k.T, [&](const WaveOp &op, int) -> bool {
+                if (op.kind > OP_P) return true;
+                const int k32 = op.kind == OP_X ? L.k32_i : op.kind == OP_H ? L.k32_h : L.k32_c;
+                const uint32_t idesc = ptx::idesc_i8(128, op.kind == OP_P ? L.npadp : L.npad);
+                const uint32_t d = tmem_base + (uint32_t)(job & 1) * WV_ACC_COLS;
+                if (!wv_wait(&ctl->t_empty[job & 1], ((uint32_t)(job >> 1) & 1u) ^ 1u, abort_flag)) return false;
+                ptx::tc_fence_after();
+                bool acc = false;
+                for (int left = k32; left > 0; left -= 4) {
+                    if (!wv_wait(&ctl->a_full[sa], pa, abort_flag) || !wv_wait(&ctl->b_full[sb], pb, abort_flag)) return false;
+                    ptx::tc_fence_after();
+                    const uint64_t ad = a_desc0 + (uint64_t)(sa * (WV_A_SLOT >> 4)), bd = b_desc0 + (uint64_t)(sb * (k.b_slot >> 4));
+                    const int nk = left < 4 ? left : 4;
+                    for (int i = 0; i < nk; ++i) { ptx::mma_i8_ss(d, ad + 2 * i, bd + 2 * i, idesc, acc); acc = true; }
+                    ptx::mma_commit(&ctl->a_empty[sa]);
+                    ptx::mma_commit(&ctl->b_empty[sb]);
+                    if (++sa == k.na) { sa = 0; pa ^= 1u; }
+                    if (++sb == k.nb) { sb = 0; pb ^= 1u; }
+                }
+                ptx::mma_commit(&ctl->t_full[job & 1]);
+                ++job;
+                return true;
+            });
+        }
+        __syncwarp();
+    } else if (warp >= WV_EPI_WARP0) {
+        // ---------------- epilogues and elementwise work ----------------
+        const int tid = threadIdx.x - 32 * WV_EPI_WARP0;
+        const int quarter = warp & 3, qpr = 4 / k.nrep;        // quarters of the lanes that hold one copy of the rows
+        const int row = (quarter % qpr) * 32 + lane, part = ((warp - WV_EPI_WARP0) >> 2) + 4 * (quarter / qpr), nparts = 4 * k.nrep;
+        const ActTabs at = make_act_tabs(ptx::smem_u32(s.tab), L.tab_lay);
+        WvPoint pt{abort_flag, &ctl->exit_at, 0};
+        if (TAB) wv_wait(&ctl->tab_full, 0, abort_flag);
+        int job = 0;
+        wv_walk(ctl, k.T, [&](const WaveOp &op, int t) -> bool {
+            const int u = op.u, rows = r.rows[u], gu = r.gu[u];
+            if (op.kind <= OP_P) {
+                const bool ok = wv_wait(&ctl->t_full[job & 1], (uint32_t)(job >> 1) & 1u, abort_flag);
+                if (__all_sync(0xffffffffu, ok)) {
+                    ptx::tc_fence_after();
+                    const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(job & 1) * WV_ACC_COLS;
+                    const bool valid = row < rows;
+                    uint4 *gb = r.g[u];
+                    uint4 *xb = gb + (size_t)(k.units == 1 ? 1 + (PEEP ? (t & 1) : 0) : (PEEP ? 1 : 0)) * r.pairs * rows;
+                    const int pair0 = op.tile * L.ppt;
+                    if (op.kind == OP_X)
+                        wv_gate_tile<G, LN, PEEP, false>(L, s, ta, pair0, gate_tile_pairs(op.tile), part, nparts, row, rows, valid, nullptr, xb, nullptr);
+                    else if (op.kind == OP_H)
+                        wv_gate_tile<G, LN, PEEP, true>(L, s, ta, pair0, gate_tile_pairs(op.tile), part, nparts, row, rows, valid, xb, gb, r.c[u]);
+                    else
+                        wv_proj_tile(k, L, s, r, ta, op.tile * L.opt, r.outs - op.tile * L.opt < L.opt ? r.outs - op.tile * L.opt : L.opt, part, nparts,
+                                     row, valid, L.out_img + ((size_t)(t + 1) * k.nu + gu) * L.kb_h * k.ra * 128, r.row0[u] + row, t, last_layer);
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(&ctl->t_empty[job & 1]);
+                }
+                ++job;
+                return true;                                   // (after an abort: on to the next meeting point)
+            }
+            unsigned *cnt = cnt0 + (size_t)gu * WC_PER_UNIT * WC_WORDS;
+            if (op.kind == OP_S) {
+                wv_epi_sync();                                 // gate sums and their statistics are complete in this block
+                if (!LN) return true;
+                constexpr unsigned ALL = (1u << G) - 1u;
+                wv_push_stats<G>(s, L.totals + ((size_t)(t & 1) * k.nu + gu) * k.ra * 8, rows, PEEP ? ALL & ~(1u << (G - 1)) : ALL, tid);
+                return wv_publish(cnt + WC_STATS * WC_WORDS, false, pt, tid);
+            }
+            if (op.kind == OP_B) return wv_elementwise<G, LN, PEEP, TAB>(k, L, s, r, at, u, t, last_layer, pt, tid);
+            return wv_publish(cnt + WC_H * WC_WORDS, true, pt, tid);        // OP_F: h^t of this block is written
+        });
+    }
+
+    // ---------------- teardown ----------------
+    ptx::cta_sync();
+    if (*abort_flag) {
+        // a wait ran out: give copies and MMAs in flight time to finish, then report
+        if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
+        for (int i = 0; i < 200; ++i) __nanosleep(500);
+    }
+    ptx::cta_sync();
+    if (warp == 2) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc(tmem_base, 512);
+    }
+}
+
+// ---- before the launch: operand images ---------------------------------------------------------------------------------
+
+__device__ __forceinline__ uint4 wv_load16(const int8_t *src, int valid)      // up to 16 bytes from any address, the rest zero
+{
+    if (valid >= 16 && ((uintptr_t)src & 15) == 0) return *reinterpret_cast<const uint4 *>(src);
+    uint32_t w[4] = {0, 0, 0, 0};
+    for (int j = 0; j < 16 && j < valid; ++j) w[j >> 2] |= (uint32_t)(uint8_t)src[j] << (8 * (j & 3));
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// The caller's x and h into activation images; counters, totals and status cleared.
+__global__ void k_wave_prepare(const __grid_constant__ WaveCall k, const int8_t *x, unsigned *zero, size_t zero_words)
+{
+    const size_t step = (size_t)gridDim.x * blockDim.x, first = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    auto put = [&](int8_t *img, int kbs, size_t block, int b, int chunk, const uint4 &v) {
+        // unit of row b: units are floor(i B / nu) .. floor((i + 1) B / nu)
+        int gu = (int)(((long long)(b + 1) * k.nu - 1) / k.B);
+        const int row = b - (int)((long long)gu * k.B / k.nu);
+        *reinterpret_cast<uint4 *>(img + (block * k.nu + gu) * kbs * k.ra * 128 + wv_img_off(row, chunk * 16, k.ra)) = v;
+    };
+    {
+        const WaveLayer &L = k.layer[0];
+        const int per = (L.I + 15) >> 4;
+        const size_t total = (size_t)k.T * k.B * per;
+        for (size_t i = first; i < total; i += step) {
+            const size_t rt = i / per;
+            const int chunk = (int)(i - rt * per), b = (int)(rt % k.B);
+            put(L.in_img, L.kb_i, rt / k.B, b, chunk, wv_load16(x + rt * L.I + chunk * 16, L.I - chunk * 16));
+        }
+    }
+    for (int l = 0; l < k.n_layers; ++l) {
+        const WaveLayer &L = k.layer[l];
+        const int per = (L.O + 15) >> 4;
+        for (size_t i = first; i < (size_t)k.B * per; i += step) {
+            const int b = (int)(i / per), chunk = (int)(i - (size_t)b * per);
+            put(L.out_img, L.kb_h, 0, b, chunk, wv_load16(k.h + L.h_off * k.B + (size_t)b * L.O + chunk * 16, L.O - chunk * 16));
+        }
+    }
+    for (size_t i = first; i < zero_words; i += step) zero[i] = 0u;
+    if (first == 0) *k.status = 0;
+}
+
+// A weight matrix into the tiles its blocks stream: [rank][tile][k-block][column][128 bytes], swizzled.  Gate matrices
+// (G > 0): column c of a tile is slot (c mod 2G) / 2, cell 2 (c / 2G) + c mod 2 of the tile.  W_proj (G = 0): plain rows.
+__global__ void k_wave_tile_weights(const int8_t *src, int8_t *dst, int G, int rows, int K, int n, int per_rank, int nt, int per_tile, int npad, int nkb)
+{
+    const size_t total = (size_t)n * nt * nkb * npad * 8;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const int chunk = (int)(i & 7);
+        size_t q = i >> 3;
+        const int c = (int)(q % npad); q /= npad;
+        const int kb = (int)(q % nkb); q /= nkb;
+        const int tile = (int)(q % nt), rank = (int)(q / nt);
+        int src_row = -1;
+        if (G > 0) {
+            const int pr = tile * per_tile + c / (2 * G), in = c % (2 * G);
+            const int u = 2 * (rank * per_rank + pr) + (in & 1);
+            if (c / (2 * G) < per_tile && pr < per_rank && u * G < rows) src_row = u * G + (in >> 1);
+        } else {
+            const int o = tile * per_tile + c;
+            if (c < per_tile && o < per_rank && rank * per_rank + o < rows) src_row = rank * per_rank + o;
+        }
+        const int k0 = kb * 128 + chunk * 16;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (src_row >= 0 && k0 < K) v = wv_load16(src + (size_t)src_row * K + k0, K - k0);
+        *reinterpret_cast<uint4 *>(dst + (((size_t)(rank * nt + tile) * nkb + kb) * npad + c) * 128 + ((chunk ^ (c & 7)) << 4)) = v;
+    }
+}
+
+int wv_round(int v, int m) { return (v + m - 1) / m * m; }
+
+template <bool TAB>
+const void *wave_kernel_of(int G, bool ln, bool peep)
+{
+    if (G == 4) {
+        if (ln) return peep ? (const void *)k_wave_sm100<4, true, true, TAB> : (const void *)k_wave_sm100<4, true, false, TAB>;
+        return peep ? (const void *)k_wave_sm100<4, false, true, TAB> : (const void *)k_wave_sm100<4, false, false, TAB>;
+    }
+    if (ln) return peep ? (const void *)k_wave_sm100<3, true, true, TAB> : (const void *)k_wave_sm100<3, true, false, TAB>;
+    return peep ? (const void *)k_wave_sm100<3, false, true, TAB> : (const void *)k_wave_sm100<3, false, false, TAB>;
+}
+
+}  // namespace
+
+struct WaveStack {
+    int n_layers = 0, rg = 1, max_T = 0, max_B = 0, max_smem = 0, grid = 0;
+    int G = 4;
+    bool ln = false, peep = false, tabs = false;
+    bool ragged = false;           // some dimension is not a multiple of 16
+    std::vector<WaveLayer> plan;
+    int max_ppc = 0, max_opc = 0, max_tab = 0, b_slot = 0;
+    unsigned *zero = nullptr;      // counters, abort word, totals: cleared before every call
+    size_t cnt_words = 0, tot_off = 0;
+    uint4 *gbuf = nullptr;
+    uint32_t *cbuf = nullptr;
+    std::vector<void *> owned;
+    unsigned dbg_missing = 0;
+    unsigned long long dbg_limit_ns = 0;
+};
+
+void wave_destroy(WaveStack *s)
+{
+    if (!s) return;
+    for (void *p : s->owned) cudaFree(p);
+    delete s;
+}
+
+// Rows a call of B rows is cut into: units of at most 128 rows, `rg` row groups times one or two units each.
+static void wave_units(int B, int rg, int &units, int &nu, int &ra)
+{
+    units = (B + rg - 1) / rg > 128 ? 2 : 1;
+    nu = rg * units;
+    ra = wv_round((B + nu - 1) / nu, 8);
+}
+
+// How many groups the rows of a batch are split into.  (Deep stacks: the layers already share out the SMs.)
+static int wave_row_groups(int n_layers, int max_B, int sm_count)
+{
+    int rg = 1;
+    while (rg > 1 && (rg > max_B || sm_count / (n_layers * rg) < 2)) rg >>= 1;
+    return rg;
+}
+
+// Plans the wavefront kernel for a handle; *out stays null when the stack does not qualify: layers of different variants,
+// a scale with a left shift where none is expected, or sums that could leave int32.
+int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B, int sm_count, WaveStack **out)
+{
+    *out = nullptr;
+    const int n = (int)lp.size();
+    if (n < 1 || n > WV_MAX_LAYERS || sm_count / n < 2) return QLSTM_OK;
+    for (const LayerParams *p : lp) {
+        if (p->G != lp[0]->G || ((p->flags ^ lp[0]->flags) & (F_LAYERNORM | F_PEEPHOLE))) return QLSTM_OK;
+        const bool proj = p->flags & F_PROJECTION, ln = p->flags & F_LAYERNORM, peep = p->flags & F_PEEPHOLE;
+        const long long lim = 0x7fffffffll;
+        for (int g = 0; g < p->G; ++g) {
+            if ((ln && p->eff_ln[g].shift > 0) || (peep && p->eff_c[g].shift > 0)) return QLSTM_OK;
+            const int xl = p->eff_x[g].shift > 0 ? p->eff_x[g].shift : 0, hl = p->eff_h[g].shift > 0 ? p->eff_h[g].shift : 0;
+            if (xl > 15 || ((p->I * 16256ll + p->max_bx) << xl) > lim) return QLSTM_OK;
+            if (hl > 15 || ((p->O * 16256ll + p->max_bh) << hl) > lim) return QLSTM_OK;
+        }
+        if (p->eff_m.shift > 0 || (proj && p->eff_proj.shift > 0)) return QLSTM_OK;
+        if (proj && p->C * 16256ll + p->max_bp > lim) return QLSTM_OK;
+    }
+    WaveStack *s = new WaveStack();
+    s->n_layers = n;
+    s->max_T = max_T;
+    s->max_B = max_B < 256 ? max_B : 256;
+    s->G = lp[0]->G;
+    s->ln = lp[0]->flags & F_LAYERNORM;
+    s->peep = lp[0]->flags & F_PEEPHOLE;
+    for (const LayerParams *p : lp) s->ragged = s->ragged || p->I % 16 || p->C % 16 || p->O % 16;
+    s->rg = wave_row_groups(n, s->max_B, sm_count);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&s->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    auto fail = [&](int rc) { wave_destroy(s); return rc; };
+    auto dalloc = [&](size_t bytes) -> void * {
+        void *d = nullptr;
+        if (cudaMalloc(&d, bytes ? bytes : 16) != cudaSuccess) return nullptr;
+        s->owned.push_back(d);
+        return d;
+    };
+    const size_t rows_alloc = (size_t)s->max_B + 8 * 2 * s->rg;      // rows of all units, each rounded up to 8
+    const int nu_max = 2 * s->rg;
+    const int per = sm_count / (n * s->rg);
+    long long h_off = 0, c_off = 0;
+    int cta = 0, prev_n = 0, prev_kb = 0;
+    int8_t *prev_img = nullptr;
+    s->tabs = true;
+    std::vector<std::pair<int, std::pair<uint8_t *, ActTabLayout>>> blobs;
+    size_t cnt_words = 0, tot_words = 0;
+    for (int l = 0; l < n; ++l) {
+        const LayerParams &p = *lp[l];
+        const bool proj = p.flags & F_PROJECTION;
+        WaveLayer L;
+        memset(&L, 0, sizeof(L));
+        L.I = p.I; L.C = p.C; L.O = p.O; L.flags = p.flags; L.m_bits = p.m_bits; L.zp_m = p.zp_m; L.zp_h = p.zp_h;
+        const int pairs = (p.C + 1) / 2, grain = p.G == 3 ? 2 : 1;
+        L.ppc = wv_round((pairs + per - 1) / per, grain);
+        L.n = (pairs + L.ppc - 1) / L.ppc;
+        L.opc = 0; L.ntp = 0; L.opt = 4; L.npadp = 16;
+        if (proj) {
+            // blocks without cells would only lengthen the exchanges: the projection keeps to the blocks that have some
+            L.opc = wv_round((p.O + L.n - 1) / L.n, 4);
+            L.ntp = (L.opc + 255) / 256;
+            L.opt = wv_round((L.opc + L.ntp - 1) / L.ntp, 4);
+            L.npadp = wv_round(L.opt, 16);
+        }
+        const int ppt_max = p.G == 4 ? 32 : 42;
+        L.nt = (L.ppc + ppt_max - 1) / ppt_max;
+        L.ppt = wv_round((L.ppc + L.nt - 1) / L.nt, grain);
+        L.npad = wv_round(L.ppt * 2 * p.G, 16);
+        if (L.npad > WV_ACC_COLS || L.npadp > WV_ACC_COLS || 2 * (4 * L.nt + L.ntp + 4) > WV_MAX_OPS) return fail(QLSTM_OK);
+        L.kb_i = (p.I + 127) / 128; L.kb_h = (p.O + 127) / 128; L.kb_c = (p.C + 127) / 128;
+        L.k32_i = (p.I + 31) / 32; L.k32_h = (p.O + 31) / 32; L.k32_c = (p.C + 31) / 32;
+        L.cta0 = cta;
+        cta += L.n * s->rg;
+        const size_t w_bytes = (size_t)L.n * L.nt * L.npad * 128;
+        int8_t *iw = (int8_t *)dalloc(w_bytes * L.kb_i), *ir = (int8_t *)dalloc(w_bytes * L.kb_h), *ip = nullptr;
+        if (!iw || !ir) return fail(QLSTM_ERR_NOMEM);
+        k_wave_tile_weights<<<2048, 256>>>(p.W, iw, p.G, p.N, p.I, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_i);
+        k_wave_tile_weights<<<2048, 256>>>(p.R, ir, p.G, p.N, p.O, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_h);
+        if (proj) {
+            ip = (int8_t *)dalloc((size_t)L.n * L.ntp * L.npadp * 128 * L.kb_c);
+            if (!ip) return fail(QLSTM_ERR_NOMEM);
+            k_wave_tile_weights<<<2048, 256>>>(p.Wproj, ip, 0, p.O, p.C, L.n, L.opc, L.ntp, L.opt, L.npadp, L.kb_c);
+        }
+        if (cudaGetLastError() != cudaSuccess) return fail(QLSTM_ERR_CUDA);
+        L.img_w = iw; L.img_r = ir; L.img_p = ip;
+        L.bx = p.bx; L.bh = p.bh; L.bln = p.bln; L.bp = p.bp; L.P = p.P; L.L = p.L;
+        for (int g = 0; g < p.G; ++g) {
+            L.x_left[g] = p.eff_x[g].shift > 0 ? p.eff_x[g].shift : 0;
+            L.h_left[g] = p.eff_h[g].shift > 0 ? p.eff_h[g].shift : 0;
+            L.f_x[g] = make_fast_scale(p.eff_x[g]); L.f_h[g] = make_fast_scale(p.eff_h[g]);
+            L.f_c[g] = make_fast_scale(p.eff_c[g]); L.f_ln[g] = make_fast_scale(p.eff_ln[g]);
+        }
+        L.f_m = make_fast_scale(p.eff_m); L.f_proj = make_fast_scale(p.eff_proj);
+        L.div_c = make_div_magic((uint32_t)p.C);
+        {
+            // q' L + b stays inside an int32 for |q'| <= limit + 1
+            const long long room = (0x7fffffffll - p.max_bln) / (p.max_L > 0 ? p.max_L : 1) - 2;
+            L.ln_limit = room < 0 ? 0.0f : (room > 65535 ? 65535.0f : (float)room);
+        }
+        L.in_img = l > 0 ? prev_img : (int8_t *)dalloc((size_t)max_T * rows_alloc * L.kb_i * 128);
+        L.out_img = (int8_t *)dalloc(((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
+        L.m_img = proj ? (int8_t *)dalloc(rows_alloc * L.kb_c * 128) : nullptr;
+        if (!L.in_img || !L.out_img || (proj && !L.m_img)) return fail(QLSTM_ERR_NOMEM);
+        if (proj && cudaMemset(L.m_img, 0, rows_alloc * L.kb_c * 128) != cudaSuccess) return fail(QLSTM_ERR_CUDA);
+        if (l > 0 && L.kb_i != prev_kb) return fail(QLSTM_OK);
+        prev_img = L.out_img; prev_kb = L.kb_h;
+        L.below = l > 0 ? prev_n : 0;
+        prev_n = L.n;
+        L.h_off = h_off; L.c_off = c_off;
+        h_off += p.O; c_off += p.C;
+        uint8_t *blob = nullptr;
+        ActTabLayout lay = {0, 0, 0, 0, 0, 0, 0};
+        bool have = false;
+        for (auto &b : blobs)
+            if (b.first == p.m_bits) { blob = b.second.first; lay = b.second.second; have = true; }
+        if (!have) {
+            if (!act_tables_build(p.m_bits, 92 * 1024, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
+            if (blob) s->owned.push_back(blob);
+            blobs.push_back({p.m_bits, {blob, lay}});
+        }
+        if (!blob) s->tabs = false;
+        L.tab = blob; L.tab_lay = lay;
+        s->max_tab = std::max(s->max_tab, (int)lay.bytes);
+        s->max_ppc = std::max(s->max_ppc, L.ppc);
+        s->max_opc = std::max(s->max_opc, wv_round(L.opc, 4));
+        s->b_slot = std::max(s->b_slot, std::max(L.npad, proj ? L.npadp : 0) * 128);
+        cnt_words += (size_t)nu_max * WC_PER_UNIT * WC_WORDS;
+        if (s->ln) tot_words += (size_t)2 * rows_alloc * 8 * 2;
+        s->plan.push_back(L);
+    }
+    s->grid = cta;
+    if (s->grid > sm_count) return fail(QLSTM_OK);
+    s->cnt_words = cnt_words + WC_WORDS;                             // + abort word
+    s->zero = (unsigned *)dalloc((s->cnt_words + tot_words) * sizeof(unsigned));
+    // gate buffers and cell states in global memory, for batches whose buffers do not fit in shared memory
+    const size_t cells = (size_t)s->grid * s->max_ppc * (((size_t)s->max_B + s->rg - 1) / s->rg + 2);
+    s->gbuf = (uint4 *)dalloc(cells * 3 * sizeof(uint4));
+    s->cbuf = (uint32_t *)dalloc(cells * sizeof(uint32_t));
+    if (!s->zero || !s->gbuf || !s->cbuf) return fail(QLSTM_ERR_NOMEM);
+    {
+        unsigned *c = s->zero;
+        long long *t = (long long *)(s->zero + s->cnt_words);
+        for (WaveLayer &L : s->plan) {
+            L.cnt = c; c += (size_t)nu_max * WC_PER_UNIT * WC_WORDS;
+            if (s->ln) { L.totals = t; t += (size_t)2 * rows_alloc * 8; }
+        }
+    }
+    for (int tab = 0; tab < 2; ++tab) {
+        const void *f = tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) return fail(QLSTM_OK);
+    }
+    // the smallest rings have to fit
+    if (wv_layout(2, 2, s->b_slot, s->max_ppc, s->max_opc, 0, 0).total > (size_t)s->max_smem) return fail(QLSTM_OK);
+    if (cudaDeviceSynchronize() != cudaSuccess) return fail(QLSTM_ERR_CUDA);
+    *out = s;
+    return QLSTM_OK;
+}
+
+bool wave_supported(const WaveStack *s, int T, int B) { return s && B >= 1 && B <= s->max_B && T >= 1 && T <= s->max_T; }
+
+bool wave_preferred(const WaveStack *s, int T, int B)
+{
+    if (!wave_supported(s, T, B)) return false;
+    return s->ragged || (s->n_layers >= 3 && B > 4);
+}
+
+void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns)
+{
+    if (!s) return;
+    s->dbg_missing = missing_arrivals;
+    s->dbg_limit_ns = missing_arrivals ? limit_ns : 0;
+}
+
+int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *h, int16_t *c, int8_t *y, int *status, bool tables, cudaStream_t st,
+                int *launches)
+{
+    WaveCall k;
+    memset(&k, 0, sizeof(k));
+    k.T = T; k.B = B; k.n_layers = s->n_layers; k.rg = s->rg;
+    wave_units(B, s->rg, k.units, k.nu, k.ra);
+    const int rows = (B + k.nu - 1) / k.nu;
+    k.nrep = rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
+    k.early = T >= 4 * s->n_layers;
+    k.nbuf = k.units == 1 ? (s->peep ? 3 : 2) : (s->peep ? 2 : 1);
+    k.max_ppc = s->max_ppc; k.max_opc = s->max_opc; k.b_slot = s->b_slot;
+    const size_t gates = (size_t)k.units * s->max_ppc * rows * (k.nbuf * 16 + 4);
+    auto total = [&](int na, int nb, bool tab, bool in_smem) {
+        return wv_layout(na, nb, s->b_slot, s->max_ppc, s->max_opc, tab ? s->max_tab : 0, in_smem ? gates : 0).total;
+    };
+    const size_t room = (size_t)s->max_smem;
+    k.tab = tables && s->tabs && rows * k.units >= 24 && total(2, 2, true, false) <= room;
+    k.gx_s = total(3, 3, k.tab, true) <= room;
+    k.na = 2; k.nb = 2;
+    while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
+    while (k.nb < WV_MAX_SLOTS && total(k.na, k.nb + 1, k.tab, k.gx_s) <= room) ++k.nb;
+    while (k.na < WV_MAX_SLOTS && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
+    k.max_tab = k.tab ? s->max_tab : 0;
+    k.h = h; k.c = c; k.y = y;
+    k.gbuf = s->gbuf; k.cbuf = s->cbuf;
+    k.abort_word = s->zero + s->cnt_words - WC_WORDS;
+    k.status = status;
+    k.limit_ns = s->dbg_limit_ns ? s->dbg_limit_ns : WV_WAIT_LIMIT_NS;
+    k.missing = s->dbg_missing;
+    for (int l = 0; l < s->n_layers; ++l) k.layer[l] = s->plan[l];
+    size_t zero_words = s->cnt_words;
+    if (s->ln) zero_words += (size_t)s->n_layers * 2 * ((size_t)s->max_B + 8 * 2 * s->rg) * 8 * 2;
+    const size_t items = (size_t)T * B * ((s->plan[0].I + 15) / 16);
+    const int blocks = (int)std::min<size_t>(1184, (items + 255) / 256 + 32);
+    k_wave_prepare<<<blocks, 256, 0, st>>>(k, x, s->zero, zero_words);
+    if (cudaGetLastError() != cudaSuccess) return QLSTM_ERR_CUDA;
+    void *args[] = {(void *)&k};
+    const void *f = k.tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
+    cudaError_t e = cudaLaunchCooperativeKernel(f, dim3(s->grid), dim3(WV_THREADS), args, total(k.na, k.nb, k.tab, k.gx_s), st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e == cudaErrorCooperativeLaunchTooLarge ? QLSTM_ERR_LAUNCH : QLSTM_ERR_CUDA;
+    }
+    if (launches) *launches = 2;
+    return QLSTM_OK;
+}
+
+}  // namespace ql

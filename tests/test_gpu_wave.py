@@ -1,0 +1,61 @@
+"""The wavefront kernel against the CPU oracle, bit for bit, at the edges of its tiles (needs a B200)."""
+import numpy as np
+import pytest
+
+from oracle import qlstm_ref as R
+from tests.gpu_util import run_gpu
+from workloads import make_workload, random_layer_stack
+
+pytestmark = pytest.mark.gpu
+
+WAVE = 8             # recurrent_impl: the wavefront kernel, forced
+
+VARIANTS = [dict(), dict(projection=True), dict(cifg=True), dict(peephole=True, cifg=True), dict(projection=True, layernorm=True),
+            dict(layernorm=True, cifg=True, projection=True), dict(projection=True, peephole=True, layernorm=True),
+            dict(peephole=True, layernorm=True, cifg=True)]
+
+
+def check(w):
+    h0, c0 = w.initial_state()
+    want = R.run(w.layers, w.x, h0, c0)
+    got = run_gpu(w, impl=(0, WAVE))
+    for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+        assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
+
+
+# one row; copies of the rows in the lanes end at 32 and 64; one unit ends at 128; two full units
+@pytest.mark.parametrize("B", [1, 31, 33, 64, 65, 128, 129, 256])
+@pytest.mark.parametrize("kw", VARIANTS, ids=lambda k: "+".join(sorted(k)) or "basic")
+def test_wave_variants(kw, B):
+    check(random_layer_stack(810 + B, 3, 48, 112, 64, T=6, B=B, **kw))
+
+
+# dimensions that no tile, vector or pair of cells divides
+@pytest.mark.parametrize("B", [3, 40, 131])
+@pytest.mark.parametrize("kw", VARIANTS, ids=lambda k: "+".join(sorted(k)) or "basic")
+def test_wave_odd_dimensions(kw, B):
+    check(random_layer_stack(820 + B, 2, 19, 37, 23, T=7, B=B, **kw))
+    check(random_layer_stack(830 + B, 4, 83, 301, 131, T=9, B=B, **kw))
+
+
+# several gate tiles per block, long K; calls shorter than four steps per layer and longer ones order X differently
+@pytest.mark.parametrize("index,kw", [(2, {}), (3, dict(batch=32, T=4)), (4, dict(batch=64, T=21)), (5, dict(batch=8, T=33)),
+                                      (5, dict(batch=256, T=3))])
+def test_wave_configs(index, kw):
+    check(make_workload(index, **kw))
+
+
+def test_wave_timeout_is_reported_and_the_handle_recovers():
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(9, 3, 48, 112, 64, projection=True, layernorm=True, T=5, B=40)
+    h0, c0 = w.initial_state()
+    want = R.run(w.layers, w.x, h0, c0)
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        q.debug_barrier_timeout(1, 3_000_000)
+        with pytest.raises(qlstm.QlstmError) as e:
+            run_gpu(w, handle=q, impl=(0, WAVE))
+        assert e.value.code == qlstm.binding.ERR_TIMEOUT
+        q.debug_barrier_timeout(0)
+        got = run_gpu(w, handle=q, impl=(0, WAVE))
+    for g, r in zip(got[:3], want[:3]):
+        assert np.array_equal(g, r)
