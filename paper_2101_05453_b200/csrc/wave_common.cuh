@@ -1,0 +1,229 @@
+// What the two wavefront kernels share: the description of a call, bounded waits, the exchanges between the blocks of a
+// group, and the fixed-point pieces of a step.  wave_sm100.cu has the overview.
+#pragma once
+
+#include "../../include/qlstm.h"
+#include "act_table.cuh"
+#include "fast_kernels.h"
+#include "sm100_ptx.cuh"
+
+namespace ql {
+
+constexpr int WV_THREADS = 640;
+constexpr int WV_EPI_WARP0 = 4;
+constexpr int WV_EPI = WV_THREADS - 32 * WV_EPI_WARP0;         // 512 epilogue threads
+constexpr int WV_MAX_LAYERS = 16;
+constexpr unsigned long long WV_WAIT_LIMIT_NS = 2000000000ull;
+
+// counters of one (layer, unit), each on a line of its own
+enum { WC_STATS = 0, WC_STATS2 = 1, WC_M = 2, WC_H = 3, WC_PER_UNIT = 4, WC_WORDS = 32 };
+
+struct WaveLayer {
+    int I, C, O;
+    uint32_t flags;
+    int m_bits, zp_m, zp_h;
+    int cta0, n;                   // first block of row group 0, blocks per (layer, row group)
+    int ppc;                       // cell pairs per block (wave_sm100.cu)
+    int nt, ppt, npad;             // gate tiles: count, pairs per tile, MMA columns
+    int opc, ntp, opt, npadp;      // outputs per block; projection tiles: count, outputs per tile, MMA columns
+    int cpc, ct, ctp, kpg;         // wave_small_sm100.cu: cells per block; cells of a tile, rounded up to 8; k-blocks per ring slot
+    int opp, kpp;                  // ... outputs of a projection tile rounded up to 8, k-blocks per ring slot
+    int kb_i, kb_h, kb_c;          // 128-byte k-blocks of the three products
+    int k32_i, k32_h, k32_c;       // K steps of 32
+    const int8_t *img_w, *img_r, *img_p;       // weights in the order and image in which the blocks stream them
+    const int32_t *bx, *bh, *bln, *bp;
+    const int16_t *P, *L;
+    int x_left[4], h_left[4];      // left shift before the rescale of the input / recurrent term (0 for scales below 1)
+    FastScale f_x[4], f_h[4], f_c[4], f_ln[4], f_m, f_proj;      // by gate slot
+    float ln_limit;                // layer-norm quotients below this keep q' L + b inside an int32
+    DivMagic div_c;
+    int8_t *in_img;                // [T][units][kb_i][ra][128] input activations
+    int8_t *out_img;               // [T + 1][units][kb_h][ra][128]: slot t + 1 holds h^t
+    int8_t *m_img;                 // [units][kb_c][ra][128]
+    long long *totals;             // [2][units][ra][4][2] layer-norm sums of the group
+    unsigned *cnt;                 // [units][WC_PER_UNIT][WC_WORDS]
+    int below;                     // blocks of the layer below, 0: none
+    long long h_off, c_off;        // of this layer in the caller's state, in units of one batch row
+    const uint8_t *tab;
+    ActTabLayout tab_lay;
+};
+
+struct WaveCall {
+    int T, B, n_layers, rg, units; // row groups; units of a row group
+    int nu, ra;                    // units in all, rows of an activation image's k-block
+    int nrep;                      // copies of a unit's rows in the 128 lanes
+    int early;                     // one unit: X(t + 1) before B(t) and P(t)
+    int tab;                       // memoised nonlinearities (resident in shared memory)
+    int na, nb, b_slot;            // ring depths, bytes of a weight slot
+    int max_cpc, max_kb_i, max_kb_h, max_kb_c;
+    int gx_s;                      // gate buffers in shared memory
+    int nbuf;                      // gate buffers per unit: [gate sums | X ...]
+    int max_ppc, max_opc, max_tab;
+    int8_t *h; int16_t *c; int8_t *y;
+    uint4 *gbuf;                   // [blocks][units][nbuf][max_ppc][max rows] gate buffers in global memory
+    uint32_t *cbuf;                // [blocks][units][max_ppc][max rows] cell states
+    unsigned *abort_word;
+    int *status;
+    unsigned long long limit_ns;
+    unsigned missing;
+    WaveLayer layer[WV_MAX_LAYERS];
+};
+
+// ---- waits ---------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ bool wv_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
+{
+    // each attempt parks the thread for up to 20 us; 100 000 attempts bound the wait to about 2 s
+    for (uint32_t i = 0; i < 100000u; ++i) {
+        if (ptx::mbar_try_wait_parked(bar, parity, 20000u)) return *abort_flag == 0;
+        if (*abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+__device__ __forceinline__ unsigned wv_ld_acquire(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long wv_timer()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)::"memory");
+    return t;
+}
+__device__ __forceinline__ void wv_fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
+// one thread: until *cnt has reached target (bounded); false once an abort is seen
+__device__ __forceinline__ bool wv_wait_count(const WaveCall &k, const unsigned *cnt, unsigned target, volatile int *abort_flag)
+{
+    target += k.missing;
+    if (wv_ld_acquire(cnt) >= target) return *abort_flag == 0;
+    const unsigned long long t0 = wv_timer();
+    unsigned spins = 0;
+    while (wv_ld_acquire(cnt) < target) {
+        if ((++spins & 31u) == 0u) {
+            if (*abort_flag) return false;
+            if (wv_ld_acquire(k.abort_word) != 0u) { *abort_flag = 1; return false; }
+            if (wv_timer() - t0 > k.limit_ns) { atomicExch(k.abort_word, 1u); *abort_flag = 1; return false; }
+        }
+    }
+    return *abort_flag == 0;
+}
+__device__ __forceinline__ void wv_epi_sync() { asm volatile("barrier.sync 1, 512;" ::: "memory"); }
+
+// ---- fixed-point pieces ----------------------------------------------------------------------------------------------
+__device__ __forceinline__ int32_t wv_lo(uint32_t w) { return (int32_t)(w << 16) >> 16; }
+__device__ __forceinline__ int32_t wv_hi(uint32_t w) { return (int32_t)w >> 16; }
+
+// byte offset of element (row, col) in a unit's activation image (see tile_off in recurrent_sm100.cu; k-blocks of ra rows)
+__device__ __forceinline__ uint32_t wv_img_off(int row, int col, int ra)
+{
+    return (uint32_t)((col >> 7) * (ra * 128) + (row << 7) + (((((col >> 4) & 7) ^ (row & 7)) << 4) | (col & 15)));
+}
+
+// ---- layer norm and nonlinearities -----------------------------------------------------------------------------------------------
+
+struct WvLnRow { int32_t mean; uint32_t sigma; float inv1024, off; };      // see ln_quotient_core in qmath.cuh
+
+__device__ __forceinline__ int4 wv_make_ln(long long sum, long long sq, const DivMagic &div)
+{
+    const LnRow r = make_ln_row(ln_stats_fast(sum, sq, div));
+    // sigma = 0: the quotient is 0; a divisor that no remainder reaches keeps the correction step from adding to it
+    const uint32_t sg = r.sigma ? r.sigma : 0xffffffffu;
+    const float off = (float)(r.sigma >> 1) * r.inv_sigma - 0.05f;
+    return make_int4(r.mean, (int)sg, __float_as_int(1024.0f * r.inv_sigma), __float_as_int(off));
+}
+
+// exact value for quotients beyond the fast range (a tiny sigma against a large deviation), out of line
+static __device__ __noinline__ int32_t wv_ln_slow(int32_t q, int4 row, int32_t Lw, int32_t b)
+{
+    const int32_t d = 1024 * q - row.x;
+    const uint32_t ad = (uint32_t)(d < 0 ? -d : d), sg = (uint32_t)row.y;
+    const uint64_t quo = sg == 0xffffffffu ? 0u : ((uint64_t)ad * 1024u + (sg >> 1)) / sg;
+    const int64_t qp = d < 0 ? -(int64_t)quo : (int64_t)quo;
+    return sat32_halves(qp * (int64_t)Lw + (int64_t)b);
+}
+
+// sat32(q' L + b) with q' = round(2^10 (2^10 q - mean) / sigma): fp32 estimate biased low by 0.05 (its error is below 0.02
+// for quotients under 2^16: four roundings of 2^-24 and 2^-25), one exact remainder test.  slow: the quotient is beyond
+// `limit` and the value is not usable.
+__device__ __forceinline__ int32_t wv_ln_fast(int32_t q, const int4 &row, int32_t Lw, int32_t b, float limit, bool &slow)
+{
+    const int32_t d = 1024 * q - row.x;
+    const uint32_t ad = (uint32_t)(d < 0 ? -d : d);
+    const float est = __fmaf_rn((float)ad, __int_as_float(row.z), __int_as_float(row.w));
+    slow = slow || !(est < limit);
+    uint32_t qe = __float2uint_rz(est);
+    const uint32_t sg = (uint32_t)row.y, half = sg == 0xffffffffu ? 0u : sg >> 1;
+    const uint32_t rem = (ad << 10) + half - qe * sg;
+    qe += rem >= sg ? 1u : 0u;
+    const int32_t qp = d < 0 ? -(int32_t)qe : (int32_t)qe;
+    return qp * Lw + b;
+}
+
+template <bool TAB>
+__device__ __forceinline__ int32_t wv_sigmoid(const ActTabs &at, int32_t x)
+{
+    if constexpr (TAB) return tab_sigmoid(at, x);
+    else return sigmoid_q_fast(x, 3);
+}
+template <bool TAB>
+__device__ __forceinline__ int32_t wv_tanh(const ActTabs &at, int32_t x)
+{
+    if constexpr (TAB) return tab_tanh_gate(at, x);
+    else return tanh_q_fast(x, 3);
+}
+template <bool TAB>
+__device__ __forceinline__ int32_t wv_hidden(const WaveLayer &L, const ActTabs &at, int32_t o, int32_t c_new)
+{
+    int32_t tc;
+    if constexpr (TAB) tc = tab_tanh_cell(at, c_new);
+    else tc = tanh_q_fast(c_new, L.m_bits);
+    return sat8(fast_rescale(o * tc, L.f_m) + L.zp_m);                     // Section 3.2.7
+}
+
+// The epilogue threads meet at named barriers, so they have to agree on where to leave after an abort: one thread looks at
+// the abort flag before the barrier of a meeting point and writes the point's number down; everybody leaves at the first
+// point that is not before it.
+struct WvPoint { volatile int *abort_flag, *exit_at; int n; };
+
+__device__ __forceinline__ bool wv_point(WvPoint &pt, int tid)
+{
+    if (tid == 0 && *pt.abort_flag) { if (*pt.exit_at > pt.n) *pt.exit_at = pt.n; }
+    wv_epi_sync();
+    const bool stay = *pt.exit_at > pt.n;
+    ++pt.n;
+    return stay;
+}
+// all epilogue threads: publish their writes and add one arrival; false: leave
+__device__ __forceinline__ bool wv_publish(unsigned *cnt, bool operands, WvPoint &pt, int tid)
+{
+    if (operands) wv_fence_async_global();
+    const bool stay = wv_point(pt, tid);
+    if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+    return stay;
+}
+// all epilogue threads: wait for the group; false: leave
+__device__ __forceinline__ bool wv_meet(const WaveCall &k, const unsigned *cnt, unsigned target, WvPoint &pt, int tid)
+{
+    if (tid == 0) wv_wait_count(k, cnt, target, pt.abort_flag);
+    return wv_point(pt, tid);
+}
+
+__device__ __forceinline__ uint4 wv_load16(const int8_t *src, int valid)      // up to 16 bytes from any address, the rest zero
+{
+    if (valid >= 16 && ((uintptr_t)src & 15) == 0) return *reinterpret_cast<const uint4 *>(src);
+    uint32_t w[4] = {0, 0, 0, 0};
+    for (int j = 0; j < 16 && j < valid; ++j) w[j >> 2] |= (uint32_t)(uint8_t)src[j] << (8 * (j & 3));
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__host__ __device__ inline size_t wv_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// wave_small_sm100.cu
+const void *wave_small_kernel(int G, bool ln, bool peep);
+size_t wave_small_smem(const WaveCall &k, int ns, bool peep);
+void wave_small_tile_weights(const int8_t *src, int8_t *dst, int G, int rows, int K, int n, int per_rank, int nt, int per_tile, int padded, int nkb, int kps);
+
+}  // namespace ql

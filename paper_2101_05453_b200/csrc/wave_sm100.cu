@@ -32,78 +32,19 @@
 #include <utility>
 #include <vector>
 
-#include "../../include/qlstm.h"
-#include "act_table.cuh"
-#include "fast_kernels.h"
-#include "sm100_ptx.cuh"
+#include "wave_common.cuh"
 
 namespace ql {
 
 namespace {
 
-constexpr int WV_THREADS = 640;
-constexpr int WV_EPI_WARP0 = 4;
-constexpr int WV_EPI = WV_THREADS - 32 * WV_EPI_WARP0;         // 512 epilogue threads
-constexpr int WV_MAX_LAYERS = 16;
 constexpr int WV_A_SLOT = 128 * 128;                           // one k-block of 128 activation rows
 constexpr int WV_MAX_SLOTS = 8;
 constexpr int WV_MAX_OPS = 96;
 constexpr int WV_ACC_COLS = 256;                               // columns of each of the two accumulators
-constexpr unsigned long long WV_WAIT_LIMIT_NS = 2000000000ull;
-
-// counters of one (layer, unit), each on a line of its own
-enum { WC_STATS = 0, WC_STATS2 = 1, WC_M = 2, WC_H = 3, WC_PER_UNIT = 4, WC_WORDS = 32 };
 
 enum { OP_X = 0, OP_H = 1, OP_P = 2, OP_S = 3, OP_B = 4, OP_F = 5 };
 struct WaveOp { uint8_t kind, u, tile, pad; };
-
-struct WaveLayer {
-    int I, C, O;
-    uint32_t flags;
-    int m_bits, zp_m, zp_h;
-    int cta0, n;                   // first block of row group 0, blocks per (layer, row group)
-    int ppc;                       // cell pairs per block
-    int nt, ppt, npad;             // gate tiles: count, pairs per tile, MMA columns
-    int opc, ntp, opt, npadp;      // outputs per block; projection tiles: count, outputs per tile, MMA columns
-    int kb_i, kb_h, kb_c;          // 128-byte k-blocks of the three products
-    int k32_i, k32_h, k32_c;       // K steps of 32
-    const int8_t *img_w, *img_r, *img_p;
-    const int32_t *bx, *bh, *bln, *bp;
-    const int16_t *P, *L;
-    int x_left[4], h_left[4];      // left shift before the rescale of the input / recurrent term (0 for scales below 1)
-    FastScale f_x[4], f_h[4], f_c[4], f_ln[4], f_m, f_proj;      // by gate slot
-    float ln_limit;                // layer-norm quotients below this keep q' L + b inside an int32
-    DivMagic div_c;
-    int8_t *in_img;                // [T][units][kb_i][ra][128] input activations
-    int8_t *out_img;               // [T + 1][units][kb_h][ra][128]: slot t + 1 holds h^t
-    int8_t *m_img;                 // [units][kb_c][ra][128]
-    long long *totals;             // [2][units][ra][4][2] layer-norm sums of the group
-    unsigned *cnt;                 // [units][WC_PER_UNIT][WC_WORDS]
-    int below;                     // blocks of the layer below, 0: none
-    long long h_off, c_off;        // of this layer in the caller's state, in units of one batch row
-    const uint8_t *tab;
-    ActTabLayout tab_lay;
-};
-
-struct WaveCall {
-    int T, B, n_layers, rg, units; // row groups; units of a row group
-    int nu, ra;                    // units in all, rows of an activation image's k-block
-    int nrep;                      // copies of a unit's rows in the 128 lanes
-    int early;                     // one unit: X(t + 1) before B(t) and P(t)
-    int tab;                       // memoised nonlinearities (resident in shared memory)
-    int na, nb, b_slot;            // ring depths, bytes of a weight slot
-    int gx_s;                      // gate buffers in shared memory
-    int nbuf;                      // gate buffers per unit: [gate sums | X ...]
-    int max_ppc, max_opc, max_tab;
-    int8_t *h; int16_t *c; int8_t *y;
-    uint4 *gbuf;                   // [blocks][units][nbuf][max_ppc][max rows] gate buffers in global memory
-    uint32_t *cbuf;                // [blocks][units][max_ppc][max rows] cell states
-    unsigned *abort_word;
-    int *status;
-    unsigned long long limit_ns;
-    unsigned missing;
-    WaveLayer layer[WV_MAX_LAYERS];
-};
 
 struct WaveCtl {
     uint64_t a_full[WV_MAX_SLOTS], a_empty[WV_MAX_SLOTS], b_full[WV_MAX_SLOTS], b_empty[WV_MAX_SLOTS];
@@ -114,59 +55,6 @@ struct WaveCtl {
     int n_ops, n_pro;              // operations of a step; of the prologue (X of step 0)
     WaveOp ops[WV_MAX_OPS];
 };
-
-// ---- waits ---------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ bool wv_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
-{
-    // each attempt parks the thread for up to 20 us; 100 000 attempts bound the wait to about 2 s
-    for (uint32_t i = 0; i < 100000u; ++i) {
-        if (ptx::mbar_try_wait_parked(bar, parity, 20000u)) return *abort_flag == 0;
-        if (*abort_flag) return false;
-    }
-    *abort_flag = 1;
-    return false;
-}
-__device__ __forceinline__ unsigned wv_ld_acquire(const unsigned *p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ unsigned long long wv_timer()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)::"memory");
-    return t;
-}
-__device__ __forceinline__ void wv_fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-
-// one thread: until *cnt has reached target (bounded); false once an abort is seen
-__device__ __forceinline__ bool wv_wait_count(const WaveCall &k, const unsigned *cnt, unsigned target, volatile int *abort_flag)
-{
-    target += k.missing;
-    if (wv_ld_acquire(cnt) >= target) return *abort_flag == 0;
-    const unsigned long long t0 = wv_timer();
-    unsigned spins = 0;
-    while (wv_ld_acquire(cnt) < target) {
-        if ((++spins & 31u) == 0u) {
-            if (*abort_flag) return false;
-            if (wv_ld_acquire(k.abort_word) != 0u) { *abort_flag = 1; return false; }
-            if (wv_timer() - t0 > k.limit_ns) { atomicExch(k.abort_word, 1u); *abort_flag = 1; return false; }
-        }
-    }
-    return *abort_flag == 0;
-}
-__device__ __forceinline__ void wv_epi_sync() { asm volatile("barrier.sync 1, 512;" ::: "memory"); }
-
-// ---- fixed-point pieces ----------------------------------------------------------------------------------------------
-__device__ __forceinline__ int32_t wv_lo(uint32_t w) { return (int32_t)(w << 16) >> 16; }
-__device__ __forceinline__ int32_t wv_hi(uint32_t w) { return (int32_t)w >> 16; }
-
-// byte offset of element (row, col) in a unit's activation image (see tile_off in recurrent_sm100.cu; k-blocks of ra rows)
-__device__ __forceinline__ uint32_t wv_img_off(int row, int col, int ra)
-{
-    return (uint32_t)((col >> 7) * (ra * 128) + (row << 7) + (((((col >> 4) & 7) ^ (row & 7)) << 4) | (col & 15)));
-}
 
 // What a block keeps in shared memory besides the rings.  Columns of a pair of cells: slot-major, [slot][cell of the pair].
 struct WaveSmem {
@@ -325,44 +213,6 @@ __device__ __forceinline__ void wv_proj_tile(const WaveCall &k, const WaveLayer 
 
 // ---- elementwise phase -----------------------------------------------------------------------------------------------
 
-struct WvLnRow { int32_t mean; uint32_t sigma; float inv1024, off; };      // see ln_quotient_core in qmath.cuh
-
-__device__ __forceinline__ int4 wv_make_ln(long long sum, long long sq, const DivMagic &div)
-{
-    const LnRow r = make_ln_row(ln_stats_fast(sum, sq, div));
-    // sigma = 0: the quotient is 0; a divisor that no remainder reaches keeps the correction step from adding to it
-    const uint32_t sg = r.sigma ? r.sigma : 0xffffffffu;
-    const float off = (float)(r.sigma >> 1) * r.inv_sigma - 0.05f;
-    return make_int4(r.mean, (int)sg, __float_as_int(1024.0f * r.inv_sigma), __float_as_int(off));
-}
-
-// exact value for quotients beyond the fast range (a tiny sigma against a large deviation), out of line
-__device__ __noinline__ int32_t wv_ln_slow(int32_t q, int4 row, int32_t Lw, int32_t b)
-{
-    const int32_t d = 1024 * q - row.x;
-    const uint32_t ad = (uint32_t)(d < 0 ? -d : d), sg = (uint32_t)row.y;
-    const uint64_t quo = sg == 0xffffffffu ? 0u : ((uint64_t)ad * 1024u + (sg >> 1)) / sg;
-    const int64_t qp = d < 0 ? -(int64_t)quo : (int64_t)quo;
-    return sat32_halves(qp * (int64_t)Lw + (int64_t)b);
-}
-
-// sat32(q' L + b) with q' = round(2^10 (2^10 q - mean) / sigma): fp32 estimate biased low by 0.05 (its error is below 0.02
-// for quotients under 2^16: four roundings of 2^-24 and 2^-25), one exact remainder test.  slow: the quotient is beyond
-// `limit` and the value is not usable.
-__device__ __forceinline__ int32_t wv_ln_fast(int32_t q, const int4 &row, int32_t Lw, int32_t b, float limit, bool &slow)
-{
-    const int32_t d = 1024 * q - row.x;
-    const uint32_t ad = (uint32_t)(d < 0 ? -d : d);
-    const float est = __fmaf_rn((float)ad, __int_as_float(row.z), __int_as_float(row.w));
-    slow = slow || !(est < limit);
-    uint32_t qe = __float2uint_rz(est);
-    const uint32_t sg = (uint32_t)row.y, half = sg == 0xffffffffu ? 0u : sg >> 1;
-    const uint32_t rem = (ad << 10) + half - qe * sg;
-    qe += rem >= sg ? 1u : 0u;
-    const int32_t qp = d < 0 ? -(int32_t)qe : (int32_t)qe;
-    return qp * Lw + b;
-}
-
 // The gate values of a pair after layer norm (slots in `mask`), in place.
 template <int G>
 __device__ __forceinline__ void wv_ln_pair(const WaveLayer &L, const WaveSmem &s, const int4 (&row)[4], int pr, unsigned mask, int32_t (&a)[4][2])
@@ -390,27 +240,6 @@ __device__ __forceinline__ void wv_ln_pair(const WaveLayer &L, const WaveSmem &s
 #pragma unroll
         for (int k = 0; k < 2; ++k)
             if ((mask >> g) & 1u) a[g][k] = sat16(fast_rescale(v[g][k], L.f_ln[g]));
-}
-
-template <bool TAB>
-__device__ __forceinline__ int32_t wv_sigmoid(const ActTabs &at, int32_t x)
-{
-    if constexpr (TAB) return tab_sigmoid(at, x);
-    else return sigmoid_q_fast(x, 3);
-}
-template <bool TAB>
-__device__ __forceinline__ int32_t wv_tanh(const ActTabs &at, int32_t x)
-{
-    if constexpr (TAB) return tab_tanh_gate(at, x);
-    else return tanh_q_fast(x, 3);
-}
-template <bool TAB>
-__device__ __forceinline__ int32_t wv_hidden(const WaveLayer &L, const ActTabs &at, int32_t o, int32_t c_new)
-{
-    int32_t tc;
-    if constexpr (TAB) tc = tab_tanh_cell(at, c_new);
-    else tc = tanh_q_fast(c_new, L.m_bits);
-    return sat8(fast_rescale(o * tc, L.f_m) + L.zp_m);                     // Section 3.2.7
 }
 
 // m of a pair of cells (h of a layer without a projection) to where the next product and the caller read it
@@ -468,34 +297,6 @@ __device__ __forceinline__ void wv_pull_stats(const WaveLayer &L, const WaveSmem
         s.ln[g * 128 + row] = wv_make_ln(v.x, v.y, L.div_c);
     }
 }
-// The epilogue threads meet at named barriers, so they have to agree on where to leave after an abort: one thread looks at
-// the abort flag before the barrier of a meeting point and writes the point's number down; everybody leaves at the first
-// point that is not before it.
-struct WvPoint { volatile int *abort_flag, *exit_at; int n; };
-
-__device__ __forceinline__ bool wv_point(WvPoint &pt, int tid)
-{
-    if (tid == 0 && *pt.abort_flag) { if (*pt.exit_at > pt.n) *pt.exit_at = pt.n; }
-    wv_epi_sync();
-    const bool stay = *pt.exit_at > pt.n;
-    ++pt.n;
-    return stay;
-}
-// all epilogue threads: publish their writes and add one arrival; false: leave
-__device__ __forceinline__ bool wv_publish(unsigned *cnt, bool operands, WvPoint &pt, int tid)
-{
-    if (operands) wv_fence_async_global();
-    const bool stay = wv_point(pt, tid);
-    if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
-    return stay;
-}
-// all epilogue threads: wait for the group; false: leave
-__device__ __forceinline__ bool wv_meet(const WaveCall &k, const unsigned *cnt, unsigned target, WvPoint &pt, int tid)
-{
-    if (tid == 0) wv_wait_count(k, cnt, target, pt.abort_flag);
-    return wv_point(pt, tid);
-}
-
 // Everything between the gate sums and m for one unit.  Tasks are (pair, row) with the row fastest, so that the gate
 // buffers are read as contiguous runs; a thread keeps one row, whose layer-norm constants stay in registers.
 template <int G, bool LN, bool PEEP, bool TAB>
@@ -654,8 +455,6 @@ __device__ __forceinline__ bool wv_walk(const WaveCtl *ctl, int T, F f)
         }
     return true;
 }
-
-__host__ __device__ inline size_t wv_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // shared memory of a block: [A slots][B slots][control][constants][statistics][tables][gate buffers, cell states]
 struct WvLayout { size_t b_ring, ctl, consts, st, ln, tab, gates, total; };
@@ -942,14 +741,6 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
 
 // ---- before the launch: operand images ---------------------------------------------------------------------------------
 
-__device__ __forceinline__ uint4 wv_load16(const int8_t *src, int valid)      // up to 16 bytes from any address, the rest zero
-{
-    if (valid >= 16 && ((uintptr_t)src & 15) == 0) return *reinterpret_cast<const uint4 *>(src);
-    uint32_t w[4] = {0, 0, 0, 0};
-    for (int j = 0; j < 16 && j < valid; ++j) w[j >> 2] |= (uint32_t)(uint8_t)src[j] << (8 * (j & 3));
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 // The caller's x and h into activation images; counters, totals and status cleared.
 __global__ void k_wave_prepare(const __grid_constant__ WaveCall k, const int8_t *x, unsigned *zero, size_t zero_words)
 {
@@ -1024,15 +815,24 @@ const void *wave_kernel_of(int G, bool ln, bool peep)
 
 }  // namespace
 
+// One way of sharing a stack out over the SMs: [0] batch as the M side (this file), [1] gate rows as the M side, for up to 32
+// rows per row group (wave_small_sm100.cu).
+struct WavePlan {
+    bool ok = false;
+    int rg = 1, grid = 0;
+    int max_ppc = 0, max_cpc = 0, max_opc = 0, b_slot = 0;
+    std::vector<WaveLayer> layer;
+};
+
 struct WaveStack {
-    int n_layers = 0, rg = 1, max_T = 0, max_B = 0, max_smem = 0, grid = 0;
+    int n_layers = 0, max_T = 0, max_B = 0, max_smem = 0;
     int G = 4;
     bool ln = false, peep = false, tabs = false;
     bool ragged = false;           // some dimension is not a multiple of 16
-    std::vector<WaveLayer> plan;
-    int max_ppc = 0, max_opc = 0, max_tab = 0, b_slot = 0;
+    WavePlan plan[2];
+    int max_tab = 0, max_kb_i = 0, max_kb_h = 0, max_kb_c = 0;
     unsigned *zero = nullptr;      // counters, abort word, totals: cleared before every call
-    size_t cnt_words = 0, tot_off = 0;
+    size_t cnt_words = 0, tot_words = 0;
     uint4 *gbuf = nullptr;
     uint32_t *cbuf = nullptr;
     std::vector<void *> owned;
@@ -1047,8 +847,20 @@ void wave_destroy(WaveStack *s)
     delete s;
 }
 
-// Rows a call of B rows is cut into: units of at most 128 rows, `rg` row groups times one or two units each.
-static void wave_units(int B, int rg, int &units, int &nu, int &ra)
+namespace {
+
+constexpr int WV_SMALL_ROWS = 32;
+
+void *wv_alloc(WaveStack *s, size_t bytes)
+{
+    void *d = nullptr;
+    if (cudaMalloc(&d, bytes ? bytes : 16) != cudaSuccess) return nullptr;
+    s->owned.push_back(d);
+    return d;
+}
+
+// Rows a call of B rows is cut into: `rg` row groups times one or two units of at most 128 rows each.
+void wave_units(int B, int rg, int &units, int &nu, int &ra)
 {
     units = (B + rg - 1) / rg > 128 ? 2 : 1;
     nu = rg * units;
@@ -1056,14 +868,71 @@ static void wave_units(int B, int rg, int &units, int &nu, int &ra)
 }
 
 // How many groups the rows of a batch are split into.  (Deep stacks: the layers already share out the SMs.)
-static int wave_row_groups(int n_layers, int max_B, int sm_count)
+int wave_row_groups(int mode, int n_layers, int max_B, int sm_count)
 {
     int rg = 1;
     while (rg > 1 && (rg > max_B || sm_count / (n_layers * rg) < 2)) rg >>= 1;
     return rg;
 }
 
-// Plans the wavefront kernel for a handle; *out stays null when the stack does not qualify: layers of different variants,
+// Shares of the blocks and weight images of one layer under plan `mode`; a qlstm_error.  L.n = 0: the plan does not work.
+int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, WaveLayer &L)
+{
+    const bool proj = p.flags & F_PROJECTION;
+    L.opc = 0; L.ntp = 0; L.opt = 4; L.npadp = 16; L.opp = 8; L.kpp = 1;
+    // blocks without cells would only lengthen the exchanges: the projection keeps to the blocks that have some
+    if (mode == 0) {
+        const int pairs = (p.C + 1) / 2, grain = p.G == 3 ? 2 : 1, ppt_max = p.G == 4 ? 32 : 42;
+        L.ppc = wv_round((pairs + per - 1) / per, grain);
+        L.n = (pairs + L.ppc - 1) / L.ppc;
+        L.nt = (L.ppc + ppt_max - 1) / ppt_max;
+        L.ppt = wv_round((L.ppc + L.nt - 1) / L.nt, grain);
+        L.npad = wv_round(L.ppt * 2 * p.G, 16);
+        if (proj) {
+            L.opc = wv_round((p.O + L.n - 1) / L.n, 4);
+            L.ntp = (L.opc + 255) / 256;
+            L.opt = wv_round((L.opc + L.ntp - 1) / L.ntp, 4);
+            L.npadp = wv_round(L.opt, 16);
+        }
+        if (L.npad > WV_ACC_COLS || L.npadp > WV_ACC_COLS || 2 * (4 * L.nt + L.ntp + 4) > WV_MAX_OPS) { L.n = 0; return QLSTM_OK; }
+    } else {
+        L.cpc = (p.C + per - 1) / per;
+        L.n = (p.C + L.cpc - 1) / L.cpc;
+        L.nt = (L.cpc + 31) / 32;
+        L.ct = (L.cpc + L.nt - 1) / L.nt;
+        L.ctp = wv_round(L.ct, 8);
+        L.kpg = 32 / L.ctp;
+        if (proj) {
+            L.opc = (p.O + L.n - 1) / L.n;
+            L.ntp = (L.opc + 127) / 128;
+            L.opt = (L.opc + L.ntp - 1) / L.ntp;
+            L.opp = wv_round(L.opt, 8);
+            L.kpp = 128 / L.opp;
+        }
+        if (L.nt > 8 || (2 * L.nt + L.ntp) * 8 > 512) { L.n = 0; return QLSTM_OK; }
+    }
+    const size_t row_bytes = mode == 0 ? (size_t)L.n * L.nt * L.npad * 128 : (size_t)L.n * L.nt * p.G * L.ctp * 128;
+    auto kbs = [&](int kb) { return mode == 0 ? kb : wv_round(kb, L.kpg); };
+    int8_t *iw = (int8_t *)wv_alloc(s, row_bytes * kbs(L.kb_i)), *ir = (int8_t *)wv_alloc(s, row_bytes * kbs(L.kb_h)), *ip = nullptr;
+    if (proj) ip = (int8_t *)wv_alloc(s, (size_t)L.n * L.ntp * (mode == 0 ? L.npadp : L.opp) * 128 * L.kb_c);
+    if (!iw || !ir || (proj && !ip)) return QLSTM_ERR_NOMEM;
+    if (mode == 0) {
+        k_wave_tile_weights<<<2048, 256>>>(p.W, iw, p.G, p.N, p.I, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_i);
+        k_wave_tile_weights<<<2048, 256>>>(p.R, ir, p.G, p.N, p.O, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_h);
+        if (proj) k_wave_tile_weights<<<2048, 256>>>(p.Wproj, ip, 0, p.O, p.C, L.n, L.opc, L.ntp, L.opt, L.npadp, L.kb_c);
+    } else {
+        wave_small_tile_weights(p.W, iw, p.G, p.N, p.I, L.n, L.cpc, L.nt, L.ct, L.ctp, L.kb_i, L.kpg);
+        wave_small_tile_weights(p.R, ir, p.G, p.N, p.O, L.n, L.cpc, L.nt, L.ct, L.ctp, L.kb_h, L.kpg);
+        if (proj) wave_small_tile_weights(p.Wproj, ip, 0, p.O, p.C, L.n, L.opc, L.ntp, L.opt, L.opp, L.kb_c, L.kpp);
+    }
+    if (cudaGetLastError() != cudaSuccess) return QLSTM_ERR_CUDA;
+    L.img_w = iw; L.img_r = ir; L.img_p = ip;
+    return QLSTM_OK;
+}
+
+}  // namespace
+
+// Plans the wavefront kernels for a handle; *out stays null when the stack does not qualify: layers of different variants,
 // a scale with a left shift where none is expected, or sums that could leave int32.
 int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B, int sm_count, WaveStack **out)
 {
@@ -1091,64 +960,35 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
     s->ln = lp[0]->flags & F_LAYERNORM;
     s->peep = lp[0]->flags & F_PEEPHOLE;
     for (const LayerParams *p : lp) s->ragged = s->ragged || p->I % 16 || p->C % 16 || p->O % 16;
-    s->rg = wave_row_groups(n, s->max_B, sm_count);
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&s->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     auto fail = [&](int rc) { wave_destroy(s); return rc; };
-    auto dalloc = [&](size_t bytes) -> void * {
-        void *d = nullptr;
-        if (cudaMalloc(&d, bytes ? bytes : 16) != cudaSuccess) return nullptr;
-        s->owned.push_back(d);
-        return d;
-    };
-    const size_t rows_alloc = (size_t)s->max_B + 8 * 2 * s->rg;      // rows of all units, each rounded up to 8
-    const int nu_max = 2 * s->rg;
-    const int per = sm_count / (n * s->rg);
+    int nu_max = 1;
+    for (int mode = 0; mode < 2; ++mode) {
+        WavePlan &pl = s->plan[mode];
+        pl.rg = wave_row_groups(mode, n, s->max_B, sm_count);
+        nu_max = std::max(nu_max, (mode == 0 ? 2 : 1) * pl.rg);
+    }
+    s->plan[1].ok = true;                                            // [0] only where [1] does not cover every batch
+    s->plan[0].ok = (s->max_B + s->plan[1].rg - 1) / s->plan[1].rg > WV_SMALL_ROWS;
+    const size_t rows_alloc = (size_t)s->max_B + 8 * nu_max;         // rows of all units, each rounded up to 8
     long long h_off = 0, c_off = 0;
-    int cta = 0, prev_n = 0, prev_kb = 0;
     int8_t *prev_img = nullptr;
+    int prev_n[2] = {0, 0};
     s->tabs = true;
     std::vector<std::pair<int, std::pair<uint8_t *, ActTabLayout>>> blobs;
-    size_t cnt_words = 0, tot_words = 0;
     for (int l = 0; l < n; ++l) {
         const LayerParams &p = *lp[l];
         const bool proj = p.flags & F_PROJECTION;
         WaveLayer L;
         memset(&L, 0, sizeof(L));
         L.I = p.I; L.C = p.C; L.O = p.O; L.flags = p.flags; L.m_bits = p.m_bits; L.zp_m = p.zp_m; L.zp_h = p.zp_h;
-        const int pairs = (p.C + 1) / 2, grain = p.G == 3 ? 2 : 1;
-        L.ppc = wv_round((pairs + per - 1) / per, grain);
-        L.n = (pairs + L.ppc - 1) / L.ppc;
-        L.opc = 0; L.ntp = 0; L.opt = 4; L.npadp = 16;
-        if (proj) {
-            // blocks without cells would only lengthen the exchanges: the projection keeps to the blocks that have some
-            L.opc = wv_round((p.O + L.n - 1) / L.n, 4);
-            L.ntp = (L.opc + 255) / 256;
-            L.opt = wv_round((L.opc + L.ntp - 1) / L.ntp, 4);
-            L.npadp = wv_round(L.opt, 16);
-        }
-        const int ppt_max = p.G == 4 ? 32 : 42;
-        L.nt = (L.ppc + ppt_max - 1) / ppt_max;
-        L.ppt = wv_round((L.ppc + L.nt - 1) / L.nt, grain);
-        L.npad = wv_round(L.ppt * 2 * p.G, 16);
-        if (L.npad > WV_ACC_COLS || L.npadp > WV_ACC_COLS || 2 * (4 * L.nt + L.ntp + 4) > WV_MAX_OPS) return fail(QLSTM_OK);
         L.kb_i = (p.I + 127) / 128; L.kb_h = (p.O + 127) / 128; L.kb_c = (p.C + 127) / 128;
         L.k32_i = (p.I + 31) / 32; L.k32_h = (p.O + 31) / 32; L.k32_c = (p.C + 31) / 32;
-        L.cta0 = cta;
-        cta += L.n * s->rg;
-        const size_t w_bytes = (size_t)L.n * L.nt * L.npad * 128;
-        int8_t *iw = (int8_t *)dalloc(w_bytes * L.kb_i), *ir = (int8_t *)dalloc(w_bytes * L.kb_h), *ip = nullptr;
-        if (!iw || !ir) return fail(QLSTM_ERR_NOMEM);
-        k_wave_tile_weights<<<2048, 256>>>(p.W, iw, p.G, p.N, p.I, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_i);
-        k_wave_tile_weights<<<2048, 256>>>(p.R, ir, p.G, p.N, p.O, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_h);
-        if (proj) {
-            ip = (int8_t *)dalloc((size_t)L.n * L.ntp * L.npadp * 128 * L.kb_c);
-            if (!ip) return fail(QLSTM_ERR_NOMEM);
-            k_wave_tile_weights<<<2048, 256>>>(p.Wproj, ip, 0, p.O, p.C, L.n, L.opc, L.ntp, L.opt, L.npadp, L.kb_c);
-        }
-        if (cudaGetLastError() != cudaSuccess) return fail(QLSTM_ERR_CUDA);
-        L.img_w = iw; L.img_r = ir; L.img_p = ip;
+        s->max_kb_i = std::max(s->max_kb_i, L.kb_i);
+        s->max_kb_h = std::max(s->max_kb_h, L.kb_h);
+        if (proj) s->max_kb_c = std::max(s->max_kb_c, L.kb_c);
         L.bx = p.bx; L.bh = p.bh; L.bln = p.bln; L.bp = p.bp; L.P = p.P; L.L = p.L;
         for (int g = 0; g < p.G; ++g) {
             L.x_left[g] = p.eff_x[g].shift > 0 ? p.eff_x[g].shift : 0;
@@ -1163,71 +1003,138 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
             const long long room = (0x7fffffffll - p.max_bln) / (p.max_L > 0 ? p.max_L : 1) - 2;
             L.ln_limit = room < 0 ? 0.0f : (room > 65535 ? 65535.0f : (float)room);
         }
-        L.in_img = l > 0 ? prev_img : (int8_t *)dalloc((size_t)max_T * rows_alloc * L.kb_i * 128);
-        L.out_img = (int8_t *)dalloc(((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
-        L.m_img = proj ? (int8_t *)dalloc(rows_alloc * L.kb_c * 128) : nullptr;
+        L.in_img = l > 0 ? prev_img : (int8_t *)wv_alloc(s, (size_t)max_T * rows_alloc * L.kb_i * 128);
+        L.out_img = (int8_t *)wv_alloc(s, ((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
+        L.m_img = proj ? (int8_t *)wv_alloc(s, rows_alloc * L.kb_c * 128) : nullptr;
         if (!L.in_img || !L.out_img || (proj && !L.m_img)) return fail(QLSTM_ERR_NOMEM);
         if (proj && cudaMemset(L.m_img, 0, rows_alloc * L.kb_c * 128) != cudaSuccess) return fail(QLSTM_ERR_CUDA);
-        if (l > 0 && L.kb_i != prev_kb) return fail(QLSTM_OK);
-        prev_img = L.out_img; prev_kb = L.kb_h;
-        L.below = l > 0 ? prev_n : 0;
-        prev_n = L.n;
+        prev_img = L.out_img;
         L.h_off = h_off; L.c_off = c_off;
         h_off += p.O; c_off += p.C;
         uint8_t *blob = nullptr;
         ActTabLayout lay = {0, 0, 0, 0, 0, 0, 0};
-        bool have = false;
-        for (auto &b : blobs)
-            if (b.first == p.m_bits) { blob = b.second.first; lay = b.second.second; have = true; }
-        if (!have) {
-            if (!act_tables_build(p.m_bits, 92 * 1024, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
-            if (blob) s->owned.push_back(blob);
-            blobs.push_back({p.m_bits, {blob, lay}});
+        if (s->plan[0].ok) {
+            bool have = false;
+            for (auto &b : blobs)
+                if (b.first == p.m_bits) { blob = b.second.first; lay = b.second.second; have = true; }
+            if (!have) {
+                if (!act_tables_build(p.m_bits, 92 * 1024, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
+                if (blob) s->owned.push_back(blob);
+                blobs.push_back({p.m_bits, {blob, lay}});
+            }
         }
         if (!blob) s->tabs = false;
         L.tab = blob; L.tab_lay = lay;
         s->max_tab = std::max(s->max_tab, (int)lay.bytes);
-        s->max_ppc = std::max(s->max_ppc, L.ppc);
-        s->max_opc = std::max(s->max_opc, wv_round(L.opc, 4));
-        s->b_slot = std::max(s->b_slot, std::max(L.npad, proj ? L.npadp : 0) * 128);
-        cnt_words += (size_t)nu_max * WC_PER_UNIT * WC_WORDS;
-        if (s->ln) tot_words += (size_t)2 * rows_alloc * 8 * 2;
-        s->plan.push_back(L);
+        for (int mode = 0; mode < 2; ++mode) {
+            WavePlan &pl = s->plan[mode];
+            if (!pl.ok) continue;
+            WaveLayer M = L;
+            const int rc = wave_share_layer(s, mode, p, sm_count / (n * pl.rg), M);
+            if (rc != QLSTM_OK) return fail(rc);
+            if (M.n == 0) { pl.ok = false; continue; }
+            M.cta0 = pl.grid;
+            pl.grid += M.n * pl.rg;
+            M.below = l > 0 ? prev_n[mode] : 0;
+            prev_n[mode] = M.n;
+            pl.max_ppc = std::max(pl.max_ppc, M.ppc);
+            pl.max_cpc = std::max(pl.max_cpc, wv_round(M.cpc, 2));
+            pl.max_opc = std::max(pl.max_opc, wv_round(M.opc, 4));
+            pl.b_slot = mode == 1 ? 128 * 128 : std::max(pl.b_slot, std::max(M.npad, proj ? M.npadp : 0) * 128);
+            pl.layer.push_back(M);
+        }
     }
-    s->grid = cta;
-    if (s->grid > sm_count) return fail(QLSTM_OK);
-    s->cnt_words = cnt_words + WC_WORDS;                             // + abort word
-    s->zero = (unsigned *)dalloc((s->cnt_words + tot_words) * sizeof(unsigned));
-    // gate buffers and cell states in global memory, for batches whose buffers do not fit in shared memory
-    const size_t cells = (size_t)s->grid * s->max_ppc * (((size_t)s->max_B + s->rg - 1) / s->rg + 2);
-    s->gbuf = (uint4 *)dalloc(cells * 3 * sizeof(uint4));
-    s->cbuf = (uint32_t *)dalloc(cells * sizeof(uint32_t));
-    if (!s->zero || !s->gbuf || !s->cbuf) return fail(QLSTM_ERR_NOMEM);
-    {
+    s->cnt_words = (size_t)n * nu_max * WC_PER_UNIT * WC_WORDS + WC_WORDS;      // + abort word
+    s->tot_words = s->ln ? (size_t)n * 2 * rows_alloc * 8 * 2 : 0;
+    s->zero = (unsigned *)wv_alloc(s, (s->cnt_words + s->tot_words) * sizeof(unsigned));
+    if (!s->zero) return fail(QLSTM_ERR_NOMEM);
+    for (WavePlan &pl : s->plan) {
         unsigned *c = s->zero;
         long long *t = (long long *)(s->zero + s->cnt_words);
-        for (WaveLayer &L : s->plan) {
+        for (WaveLayer &L : pl.layer) {
             L.cnt = c; c += (size_t)nu_max * WC_PER_UNIT * WC_WORDS;
             if (s->ln) { L.totals = t; t += (size_t)2 * rows_alloc * 8; }
         }
     }
-    for (int tab = 0; tab < 2; ++tab) {
-        const void *f = tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) return fail(QLSTM_OK);
+    WavePlan &big = s->plan[0], &small = s->plan[1];
+    if (big.ok && wv_layout(2, 2, big.b_slot, big.max_ppc, big.max_opc, 0, 0).total > (size_t)s->max_smem) big.ok = false;
+    if (big.ok) {
+        // gate buffers and cell states in global memory, for batches whose buffers do not fit in shared memory
+        const size_t cells = (size_t)big.grid * big.max_ppc * (((size_t)s->max_B + big.rg - 1) / big.rg + 2);
+        s->gbuf = (uint4 *)wv_alloc(s, cells * 3 * sizeof(uint4));
+        s->cbuf = (uint32_t *)wv_alloc(s, cells * sizeof(uint32_t));
+        if (!s->gbuf || !s->cbuf) return fail(QLSTM_ERR_NOMEM);
+        for (int tab = 0; tab < 2; ++tab) {
+            const void *f = tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
+            if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) big.ok = false;
+        }
     }
-    // the smallest rings have to fit
-    if (wv_layout(2, 2, s->b_slot, s->max_ppc, s->max_opc, 0, 0).total > (size_t)s->max_smem) return fail(QLSTM_OK);
+    if (small.ok && cudaFuncSetAttribute(wave_small_kernel(s->G, s->ln, s->peep), cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess)
+        small.ok = false;
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(QLSTM_ERR_CUDA);
+    if (!big.ok && !small.ok) return fail(QLSTM_OK);
     *out = s;
     return QLSTM_OK;
 }
 
-bool wave_supported(const WaveStack *s, int T, int B) { return s && B >= 1 && B <= s->max_B && T >= 1 && T <= s->max_T; }
+// The description of a call under plan `mode`; false if the plan cannot take it.
+static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool tables, WaveCall &k, size_t &smem)
+{
+    const WavePlan &pl = s->plan[mode];
+    if (!pl.ok) return false;
+    memset(&k, 0, sizeof(k));
+    k.T = T; k.B = B; k.n_layers = s->n_layers; k.rg = pl.rg;
+    wave_units(B, pl.rg, k.units, k.nu, k.ra);
+    const int rows = (B + k.nu - 1) / k.nu;
+    k.early = T >= 4 * s->n_layers;
+    k.max_ppc = pl.max_ppc; k.max_cpc = pl.max_cpc; k.max_opc = pl.max_opc; k.b_slot = pl.b_slot;
+    k.max_kb_i = s->max_kb_i; k.max_kb_h = s->max_kb_h; k.max_kb_c = s->max_kb_c;
+    const size_t room = (size_t)s->max_smem;
+    if (mode == 1) {
+        if (rows > WV_SMALL_ROWS) return false;
+        for (const WaveLayer &L : pl.layer)
+            if ((2 * L.nt + L.ntp) * k.ra > 512) return false;
+        k.nb = 16;
+        while (k.nb > 3 && wave_small_smem(k, k.nb, s->peep) > room) --k.nb;
+        smem = wave_small_smem(k, k.nb, s->peep);
+        return smem <= room;
+    }
+    k.nrep = rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
+    k.nbuf = k.units == 1 ? (s->peep ? 3 : 2) : (s->peep ? 2 : 1);
+    const size_t gates = (size_t)k.units * pl.max_ppc * rows * (k.nbuf * 16 + 4);
+    auto total = [&](int na, int nb, bool tab, bool in_smem) {
+        return wv_layout(na, nb, pl.b_slot, pl.max_ppc, pl.max_opc, tab ? s->max_tab : 0, in_smem ? gates : 0).total;
+    };
+    k.tab = tables && s->tabs && rows * k.units >= 24 && total(2, 2, true, false) <= room;
+    k.gx_s = total(3, 3, k.tab, true) <= room;
+    k.na = 2; k.nb = 2;
+    while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
+    while (k.nb < WV_MAX_SLOTS && total(k.na, k.nb + 1, k.tab, k.gx_s) <= room) ++k.nb;
+    while (k.na < WV_MAX_SLOTS && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
+    k.max_tab = k.tab ? s->max_tab : 0;
+    smem = total(k.na, k.nb, k.tab, k.gx_s);
+    return true;
+}
+
+static int wave_mode(const WaveStack *s, int T, int B, bool tables, WaveCall &k, size_t &smem)
+{
+    if (!s || B < 1 || B > s->max_B || T < 1 || T > s->max_T) return -1;
+    for (int mode = 1; mode >= 0; --mode)
+        if (wave_describe(s, mode, T, B, tables, k, smem)) return mode;
+    return -1;
+}
+
+bool wave_supported(const WaveStack *s, int T, int B)
+{
+    WaveCall k;
+    size_t smem;
+    return wave_mode(s, T, B, true, k, smem) >= 0;
+}
 
 bool wave_preferred(const WaveStack *s, int T, int B)
 {
     if (!wave_supported(s, T, B)) return false;
-    return s->ragged || (s->n_layers >= 3 && B > 4);
+    return s->ragged || (B > 4 && (s->n_layers >= 3 || (s->n_layers == 2 && B <= WV_SMALL_ROWS)));
 }
 
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns)
@@ -1241,42 +1148,25 @@ int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *h, int16_t 
                 int *launches)
 {
     WaveCall k;
-    memset(&k, 0, sizeof(k));
-    k.T = T; k.B = B; k.n_layers = s->n_layers; k.rg = s->rg;
-    wave_units(B, s->rg, k.units, k.nu, k.ra);
-    const int rows = (B + k.nu - 1) / k.nu;
-    k.nrep = rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
-    k.early = T >= 4 * s->n_layers;
-    k.nbuf = k.units == 1 ? (s->peep ? 3 : 2) : (s->peep ? 2 : 1);
-    k.max_ppc = s->max_ppc; k.max_opc = s->max_opc; k.b_slot = s->b_slot;
-    const size_t gates = (size_t)k.units * s->max_ppc * rows * (k.nbuf * 16 + 4);
-    auto total = [&](int na, int nb, bool tab, bool in_smem) {
-        return wv_layout(na, nb, s->b_slot, s->max_ppc, s->max_opc, tab ? s->max_tab : 0, in_smem ? gates : 0).total;
-    };
-    const size_t room = (size_t)s->max_smem;
-    k.tab = tables && s->tabs && rows * k.units >= 24 && total(2, 2, true, false) <= room;
-    k.gx_s = total(3, 3, k.tab, true) <= room;
-    k.na = 2; k.nb = 2;
-    while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
-    while (k.nb < WV_MAX_SLOTS && total(k.na, k.nb + 1, k.tab, k.gx_s) <= room) ++k.nb;
-    while (k.na < WV_MAX_SLOTS && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
-    k.max_tab = k.tab ? s->max_tab : 0;
+    size_t smem = 0;
+    const int mode = wave_mode(s, T, B, tables, k, smem);
+    if (mode < 0) return QLSTM_ERR_DIM;
+    const WavePlan &pl = s->plan[mode];
     k.h = h; k.c = c; k.y = y;
     k.gbuf = s->gbuf; k.cbuf = s->cbuf;
     k.abort_word = s->zero + s->cnt_words - WC_WORDS;
     k.status = status;
     k.limit_ns = s->dbg_limit_ns ? s->dbg_limit_ns : WV_WAIT_LIMIT_NS;
     k.missing = s->dbg_missing;
-    for (int l = 0; l < s->n_layers; ++l) k.layer[l] = s->plan[l];
-    size_t zero_words = s->cnt_words;
-    if (s->ln) zero_words += (size_t)s->n_layers * 2 * ((size_t)s->max_B + 8 * 2 * s->rg) * 8 * 2;
-    const size_t items = (size_t)T * B * ((s->plan[0].I + 15) / 16);
+    for (int l = 0; l < s->n_layers; ++l) k.layer[l] = pl.layer[l];
+    const size_t items = (size_t)T * B * ((pl.layer[0].I + 15) / 16);
     const int blocks = (int)std::min<size_t>(1184, (items + 255) / 256 + 32);
-    k_wave_prepare<<<blocks, 256, 0, st>>>(k, x, s->zero, zero_words);
+    k_wave_prepare<<<blocks, 256, 0, st>>>(k, x, s->zero, s->cnt_words + s->tot_words);
     if (cudaGetLastError() != cudaSuccess) return QLSTM_ERR_CUDA;
     void *args[] = {(void *)&k};
-    const void *f = k.tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
-    cudaError_t e = cudaLaunchCooperativeKernel(f, dim3(s->grid), dim3(WV_THREADS), args, total(k.na, k.nb, k.tab, k.gx_s), st);
+    const void *f = mode == 1 ? wave_small_kernel(s->G, s->ln, s->peep)
+                              : (k.tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep));
+    cudaError_t e = cudaLaunchCooperativeKernel(f, dim3(pl.grid), dim3(WV_THREADS), args, smem, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e == cudaErrorCooperativeLaunchTooLarge ? QLSTM_ERR_LAUNCH : QLSTM_ERR_CUDA;

@@ -1,0 +1,588 @@
+// Wavefront kernel for units of up to 32 batch rows.  The same schedule and the same exchanges as wave_sm100.cu (see the
+// overview there), with the roles of the MMA operands swapped: the gate rows are the M side (128 tensor-memory lanes),
+// the batch rows the N side (8 to 32 columns).  With so few rows a step is bound by the stream of weights and by its chain
+// of exchanges, so the point of this form is that nothing else takes time:
+//   - every lane holds a gate row, whatever the batch (with the batch as M, one row would use one lane of 128);
+//   - a layer's input, its h and its m are a few kilobytes and arrive with one copy each;
+//   - all accumulators of a step fit in tensor memory side by side, so X(t + 1) is accumulated as soon as the gate sums of
+//     step t have been read, and is only rescaled together with H(t + 1).
+// A gate tile holds up to 32 cells, gate slot g in the lanes 32 g .. 32 g + 31: a warp's lanes share a gate and its scales,
+// and a row's layer-norm sums over a tile are warp-wide reductions.
+#include <cstring>
+
+#include "wave_common.cuh"
+
+namespace ql {
+
+namespace {
+
+constexpr int WS_SLOTS = 16;
+constexpr int WS_MAX_TILES = 8;
+constexpr int WS_ROWS = 32;
+
+struct WsCtl {
+    uint64_t w_full[WS_SLOTS], w_empty[WS_SLOTS];
+    uint64_t op_full[3], op_empty[3];          // operands x, h, m
+    uint64_t gate_full[WS_MAX_TILES], acc_empty, p_full, p_empty;
+    uint32_t tmem_base;
+    int abort_flag, exit_at;
+};
+
+// [weight ring][x][h][m][control][constants][statistics][gates][cell states]
+struct WsLayout { size_t act[3], ctl, consts, st, ln, gates, c, total; };
+
+__host__ __device__ inline WsLayout ws_layout(const WaveCall &k, int ns, int rows, bool peep)
+{
+    WsLayout l;
+    l.act[0] = (size_t)ns * k.b_slot;
+    l.act[1] = l.act[0] + (size_t)k.max_kb_i * k.ra * 128;
+    l.act[2] = l.act[1] + (size_t)k.max_kb_h * k.ra * 128;
+    l.ctl = l.act[2] + (size_t)k.max_kb_c * k.ra * 128;
+    l.consts = l.ctl + wv_up(sizeof(WsCtl), 16);
+    l.st = l.consts + wv_up((size_t)k.max_cpc * 4 * (3 * 4 + 2 * 2) + (size_t)k.max_opc * 4, 16);
+    l.ln = l.st + 12 * WS_ROWS * 4;
+    l.gates = l.ln + 4 * WS_ROWS * 16;
+    l.c = l.gates + wv_up((size_t)(peep ? 5 : 4) * rows * k.max_cpc * 2, 16);
+    l.total = l.c + wv_up((size_t)rows * k.max_cpc * 2, 16);
+    // an MMA reads 128 rows of 128 bytes from where its k-block starts, whatever the tile holds
+    if (l.total < l.act[0] + 128 * 128) l.total = l.act[0] + 128 * 128;
+    l.total += 1024;                           // alignment of the ring
+    return l;
+}
+
+struct WsSmem {
+    int32_t *bx, *bh, *bln;        // [4][cpc]
+    int16_t *L, *P;                // [4][cpc]
+    int32_t *bp;                   // [opc]
+    uint32_t *st;                  // [4][3][32] layer-norm sums: sum, low 20 bits and rest of the squares
+    int4 *ln;                      // [4][32]
+    int16_t *g;                    // [slot][row][cpc] gate sums; slot 4: X of the output gate (peephole)
+    int16_t *c;                    // [row][cpc]
+};
+
+struct WsRole {
+    int li, rank;
+    int u0, cells, o_lo, outs;
+    int row0, rows, gu;
+};
+
+// Gate sums of one tile, one lane per cell, for the gate `g` of this warp.
+template <int G, bool LN, bool PEEP>
+__device__ __forceinline__ void ws_gate_tile(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, uint32_t tx, uint32_t th,
+                                             int tile, int g, int lane)
+{
+    constexpr int SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
+    const int cpc = L.cpc, ul = tile * L.ct + lane, rows = r.rows;
+    const bool in = lane < L.ct && ul < r.cells;
+    const int i0 = g * cpc + (in ? ul : 0);
+    const int32_t bx = s.bx[i0], bh = s.bh[i0], P = PEEP ? (int32_t)s.P[i0] : 0;
+    const FastScale fx = L.f_x[g], fh = L.f_h[g];
+    const int xl = L.x_left[g], hl = L.h_left[g];
+    const bool is_o = PEEP && g == SO;                         // warp-uniform
+    uint32_t my_sum = 0, my_lo = 0, my_hi = 0;                 // lane b keeps the sums of row b
+#pragma unroll 1
+    for (int r0 = 0; r0 < rows; r0 += 8) {
+        uint32_t x[8], h[8];
+        __syncwarp();
+        ptx::tmem_ld_32x8(tx + (uint32_t)r0, x);
+        ptx::tmem_ld_32x8(th + (uint32_t)r0, h);
+        ptx::tmem_ld_wait();
+        int32_t v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int32_t X = sat16(fast_rescale(((int32_t)x[e] + bx) << xl, fx));
+            const int32_t H = sat16(fast_rescale(((int32_t)h[e] + bh) << hl, fh));
+            v[e] = X + H;
+            if (PEEP) {
+                if (is_o) {
+                    if (in && r0 + e < rows) s.g[(4 * rows + r0 + e) * cpc + ul] = (int16_t)X;
+                    v[e] = H;                                  // X + H + P c^t once c^t exists
+                } else if (g != SZ) {
+                    const int32_t c_old = (in && r0 + e < rows) ? s.c[(r0 + e) * cpc + ul] : 0;
+                    v[e] += sat16(fast_rescale(P * c_old, L.f_c[g]));
+                }
+            }
+            v[e] = in ? sat16(v[e]) : 0;
+            if (in && r0 + e < rows) s.g[(g * rows + r0 + e) * cpc + ul] = (int16_t)v[e];
+        }
+        if (LN && !is_o) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const uint32_t sq = (uint32_t)(v[e] * v[e]);
+                const uint32_t a = (uint32_t)__reduce_add_sync(0xffffffffu, v[e]);
+                const uint32_t lo = __reduce_add_sync(0xffffffffu, sq & 0xfffffu), hi = __reduce_add_sync(0xffffffffu, sq >> 20);
+                if (lane == r0 + e) { my_sum = a; my_lo = lo; my_hi = hi; }
+            }
+        }
+    }
+    if (LN && !is_o && lane < rows) {
+        uint32_t *st = s.st + g * 3 * WS_ROWS + lane;
+        atomicAdd(st, my_sum);
+        atomicAdd(st + WS_ROWS, my_lo);
+        atomicAdd(st + 2 * WS_ROWS, my_hi);
+    }
+}
+
+template <int G>
+__device__ __forceinline__ void ws_push_stats(const WsSmem &s, long long *totals, int rows, unsigned mask, int tid)
+{
+    const int g = tid >> 5, row = tid & 31;
+    if (g < G && row < rows && ((mask >> g) & 1u)) {
+        uint32_t *st = s.st + g * 3 * WS_ROWS + row;
+        const long long sum = (long long)(int32_t)st[0];
+        const unsigned long long sq = ((unsigned long long)st[2 * WS_ROWS] << 20) + st[WS_ROWS];
+        st[0] = st[WS_ROWS] = st[2 * WS_ROWS] = 0u;
+        unsigned long long *dst = reinterpret_cast<unsigned long long *>(totals + (size_t)(row * 4 + g) * 2);
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"((unsigned long long)sum) : "memory");
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst + 1), "l"(sq) : "memory");
+    }
+}
+template <int G>
+__device__ __forceinline__ void ws_pull_stats(const WaveLayer &L, const WsSmem &s, const long long *totals, int rows, unsigned mask, int tid)
+{
+    const int g = tid >> 5, row = tid & 31;
+    if (g < G && row < rows && ((mask >> g) & 1u)) {
+        const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(totals + (size_t)(row * 4 + g) * 2));
+        s.ln[g * WS_ROWS + row] = wv_make_ln(v.x, v.y, L.div_c);
+    }
+}
+
+// layer norm of the gate slots in `mask` of one cell, in place
+template <int G>
+__device__ __forceinline__ void ws_ln_cell(const WaveLayer &L, const WsSmem &s, int row, int ul, unsigned mask, int32_t (&a)[4])
+{
+    int32_t v[4];
+    bool slow = false;
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+        if ((mask >> g) & 1u) v[g] = wv_ln_fast(a[g], s.ln[g * WS_ROWS + row], s.L[g * L.cpc + ul], s.bln[g * L.cpc + ul], L.ln_limit, slow);
+    if (slow) {
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if ((mask >> g) & 1u) v[g] = wv_ln_slow(a[g], s.ln[g * WS_ROWS + row], s.L[g * L.cpc + ul], s.bln[g * L.cpc + ul]);
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+        if ((mask >> g) & 1u) a[g] = sat16(fast_rescale(v[g], L.f_ln[g]));
+}
+
+// m of one cell (h of a layer without a projection)
+__device__ __forceinline__ void ws_store_m(const WaveCall &k, const WaveLayer &L, int8_t *img_unit, int row, int u, int b, int t, int32_t m, bool last_layer)
+{
+    img_unit[wv_img_off(row, u, k.ra)] = (int8_t)m;
+    if (L.flags & F_PROJECTION) return;
+    if (last_layer) k.y[((size_t)t * k.B + b) * L.O + u] = (int8_t)m;
+    if (t == k.T - 1) k.h[L.h_off * k.B + (size_t)b * L.O + u] = (int8_t)m;
+}
+
+// Everything between the gate sums and m, one cell per task, consecutive threads on consecutive cells of a row.
+template <int G, bool LN, bool PEEP>
+__device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, int t, bool last_layer, WvPoint &pt,
+                                               int tid)
+{
+    constexpr int SI = 0, SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
+    constexpr unsigned ALL = (1u << G) - 1u;
+    const int rows = r.rows, cells = r.cells, cpc = L.cpc, n_tasks = rows * cells;
+    unsigned *cnt = L.cnt + (size_t)r.gu * WC_PER_UNIT * WC_WORDS;
+    long long *tot = L.totals ? L.totals + ((size_t)(t & 1) * k.nu + r.gu) * k.ra * 8 : nullptr;
+    if (LN) {
+        ws_push_stats<G>(s, tot, rows, PEEP ? ALL & ~(1u << SO) : ALL, tid);
+        if (!wv_publish(cnt + WC_STATS * WC_WORDS, false, pt, tid)) return false;
+        if (!wv_meet(k, cnt + WC_STATS * WC_WORDS, (unsigned)(t + 1) * L.n, pt, tid)) return false;
+        ws_pull_stats<G>(L, s, tot, rows, PEEP ? ALL & ~(1u << SO) : ALL, tid);
+        // the other set of totals was read by everyone before this step's sums were complete: cleared for the next step
+        long long *next = L.totals + ((size_t)((t + 1) & 1) * k.nu + r.gu) * k.ra * 8;
+        for (int i = r.rank * WV_EPI + tid; i < rows * 8; i += L.n * WV_EPI) next[i] = 0;
+        wv_epi_sync();
+    }
+    int8_t *img = (L.flags & F_PROJECTION) ? L.m_img + (size_t)r.gu * L.kb_c * k.ra * 128
+                                           : L.out_img + ((size_t)(t + 1) * k.nu + r.gu) * L.kb_h * k.ra * 128;
+    const bool fin = t == k.T - 1;
+#pragma unroll 1
+    for (int i = tid; i < n_tasks; i += WV_EPI) {
+        const int row = i / cells, ul = i - row * cells, u = r.u0 + ul, b = r.row0 + row;
+        int32_t a[4];
+#pragma unroll
+        for (int g = 0; g < G; ++g) a[g] = s.g[(g * rows + row) * cpc + ul];
+        if (LN) ws_ln_cell<G>(L, s, row, ul, PEEP ? ALL & ~(1u << SO) : ALL, a);
+        const int32_t f = sigmoid_q_fast(a[SF], 3), z = tanh_q_fast(a[SZ], 3);
+        int32_t ig;
+        if (G == 4) ig = sigmoid_q_fast(a[SI], 3);
+        else { ig = 32768 - f; if (ig > 32767) ig = 32767; }               // coupled input gate, Section 3.2.9
+        const int32_t c_new = cell_update_fast(ig, z, f, s.c[row * cpc + ul], L.m_bits);
+        s.c[row * cpc + ul] = (int16_t)c_new;
+        if (fin) k.c[L.c_off * k.B + (size_t)b * L.C + u] = (int16_t)c_new;
+        int32_t ao = a[SO];
+        if (PEEP) {
+            ao = sat16((int32_t)s.g[(4 * rows + row) * cpc + ul] + a[SO] + sat16(fast_rescale((int32_t)s.P[SO * cpc + ul] * c_new, L.f_c[SO])));   // Eq. 5
+            if (LN) {
+                s.g[(SO * rows + row) * cpc + ul] = (int16_t)ao;           // waits for the row's statistics
+                uint32_t *st = s.st + SO * 3 * WS_ROWS + row;
+                const uint32_t sq = (uint32_t)(ao * ao);
+                atomicAdd(st, (uint32_t)ao);
+                atomicAdd(st + WS_ROWS, sq & 0xfffffu);
+                atomicAdd(st + 2 * WS_ROWS, sq >> 20);
+                continue;
+            }
+        }
+        const int32_t tc = tanh_q_fast(c_new, L.m_bits);
+        ws_store_m(k, L, img, row, u, b, t, sat8(fast_rescale(sigmoid_q_fast(ao, 3) * tc, L.f_m) + L.zp_m), last_layer);
+    }
+    if (LN && PEEP) {
+        wv_epi_sync();
+        ws_push_stats<G>(s, tot, rows, 1u << SO, tid);
+        if (!wv_publish(cnt + WC_STATS2 * WC_WORDS, false, pt, tid)) return false;
+        if (!wv_meet(k, cnt + WC_STATS2 * WC_WORDS, (unsigned)(t + 1) * L.n, pt, tid)) return false;
+        ws_pull_stats<G>(L, s, tot, rows, 1u << SO, tid);
+        wv_epi_sync();
+#pragma unroll 1
+        for (int i = tid; i < n_tasks; i += WV_EPI) {
+            const int row = i / cells, ul = i - row * cells;
+            int32_t a[4] = {0, 0, 0, 0};
+            a[SO] = s.g[(SO * rows + row) * cpc + ul];
+            ws_ln_cell<G>(L, s, row, ul, 1u << SO, a);
+            const int32_t tc = tanh_q_fast(s.c[row * cpc + ul], L.m_bits);
+            ws_store_m(k, L, img, row, r.u0 + ul, r.row0 + row, t, sat8(fast_rescale(sigmoid_q_fast(a[SO], 3) * tc, L.f_m) + L.zp_m), last_layer);
+        }
+    }
+    return wv_publish(cnt + ((L.flags & F_PROJECTION) ? WC_M : WC_H) * WC_WORDS, true, pt, tid);
+}
+
+// One projection tile: a lane is an output, the four warps of a lane quarter share the rows.
+__device__ __forceinline__ void ws_proj_tile(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, uint32_t tp, int o_first, int no,
+                                             int quarter, int wq, int lane, int8_t *out_unit, int t, bool last_layer)
+{
+    const int j = quarter * 32 + lane, col = r.o_lo + o_first + j;
+    const bool in = j < no;
+    if (quarter * 32 >= no) return;                            // warp-uniform
+    const int32_t bias = in ? s.bp[o_first + j] : 0;
+    const bool fin = t == k.T - 1;
+#pragma unroll 1
+    for (int r0 = 8 * wq; r0 < r.rows; r0 += 32) {
+        uint32_t a[8];
+        __syncwarp();
+        ptx::tmem_ld_32x8(tp + (uint32_t)r0, a);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int row = r0 + e, b = r.row0 + row;
+            const int8_t h = (int8_t)sat8(fast_rescale((int32_t)a[e] + bias, L.f_proj) + L.zp_h);
+            if (in && row < r.rows) {
+                out_unit[wv_img_off(row, col, k.ra)] = h;
+                if (last_layer) k.y[((size_t)t * k.B + b) * L.O + col] = h;
+                if (fin) k.h[L.h_off * k.B + (size_t)b * L.O + col] = h;
+            }
+        }
+    }
+}
+
+template <int G, bool LN, bool PEEP>
+__global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid_constant__ WaveCall k)
+{
+    extern __shared__ uint8_t ws_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)ws_raw + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = blockIdx.x;
+    WsRole r;
+    r.li = -1;
+    for (int l = 0; l < k.n_layers; ++l)
+        if (cta >= k.layer[l].cta0 && cta < k.layer[l].cta0 + k.layer[l].n * k.rg) r.li = l;
+    if (r.li < 0) return;
+    const WaveLayer &L = k.layer[r.li];
+    const bool proj = (L.flags & F_PROJECTION) != 0, last_layer = r.li == k.n_layers - 1;
+    r.gu = (cta - L.cta0) / L.n;
+    r.rank = cta - L.cta0 - r.gu * L.n;
+    r.u0 = r.rank * L.cpc;
+    r.cells = L.C - r.u0 < L.cpc ? L.C - r.u0 : L.cpc;
+    r.o_lo = r.rank * L.opc;
+    r.outs = proj ? (L.O - r.o_lo < L.opc ? L.O - r.o_lo : L.opc) : 0;
+    if (r.outs < 0) r.outs = 0;
+    r.row0 = (int)((long long)r.gu * k.B / k.nu);
+    r.rows = (int)((long long)(r.gu + 1) * k.B / k.nu) - r.row0;
+    if (r.rows == 0) return;                                   // fewer rows than row groups: this group is idle
+
+    const WsLayout lay = ws_layout(k, k.nb, (k.B + k.nu - 1) / k.nu, PEEP);
+    WsCtl *ctl = reinterpret_cast<WsCtl *>(smem + lay.ctl);
+    volatile int *abort_flag = &ctl->abort_flag;
+    WsSmem s;
+    {
+        uint8_t *p = smem + lay.consts;
+        const size_t q = (size_t)k.max_cpc * 4;
+        s.bx = (int32_t *)p;  p += q * 4;
+        s.bh = (int32_t *)p;  p += q * 4;
+        s.bln = (int32_t *)p; p += q * 4;
+        s.bp = (int32_t *)p;  p += (size_t)k.max_opc * 4;
+        s.L = (int16_t *)p;   p += q * 2;
+        s.P = (int16_t *)p;
+        s.st = (uint32_t *)(smem + lay.st);
+        s.ln = (int4 *)(smem + lay.ln);
+        s.g = (int16_t *)(smem + lay.gates);
+        s.c = (int16_t *)(smem + lay.c);
+    }
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < WS_SLOTS; ++i) { ptx::mbar_init(&ctl->w_full[i], 1); ptx::mbar_init(&ctl->w_empty[i], 1); }
+        for (int i = 0; i < 3; ++i) { ptx::mbar_init(&ctl->op_full[i], 1); ptx::mbar_init(&ctl->op_empty[i], 1); }
+        for (int i = 0; i < WS_MAX_TILES; ++i) ptx::mbar_init(&ctl->gate_full[i], 1);
+        ptx::mbar_init(&ctl->acc_empty, WV_EPI / 32);
+        ptx::mbar_init(&ctl->p_full, 1);
+        ptx::mbar_init(&ctl->p_empty, WV_EPI / 32);
+        ctl->abort_flag = 0;
+        ctl->exit_at = 0x7fffffff;
+        ptx::fence_barrier_init();
+    }
+    if (warp == 2) {
+        ptx::tmem_alloc(&ctl->tmem_base, 512);
+        ptx::tmem_relinquish();
+    }
+    for (int i = threadIdx.x; i < 4 * L.cpc; i += WV_THREADS) {
+        const int g = i / L.cpc, u = r.u0 + i - g * L.cpc;
+        const bool in = g < G && i - g * L.cpc < r.cells;
+        const int n = u * G + g;
+        s.bx[i] = in ? L.bx[n] : 0;
+        s.bh[i] = in ? L.bh[n] : 0;
+        s.bln[i] = in && LN ? L.bln[n] : 0;
+        s.L[i] = in && LN ? L.L[n] : (int16_t)0;
+        s.P[i] = in && PEEP ? L.P[n] : (int16_t)0;
+    }
+    for (int i = threadIdx.x; i < r.outs; i += WV_THREADS) s.bp[i] = L.bp[r.o_lo + i];
+    for (int i = threadIdx.x; i < 12 * WS_ROWS; i += WV_THREADS) s.st[i] = 0u;
+    for (int i = threadIdx.x; i < r.rows * r.cells; i += WV_THREADS) {
+        const int row = i / r.cells, ul = i - row * r.cells;
+        s.c[row * L.cpc + ul] = k.c[L.c_off * k.B + (size_t)(r.row0 + row) * L.C + r.u0 + ul];
+    }
+    ptx::tc_fence_before();
+    ptx::cta_sync();
+    ptx::tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    const int nt = (r.cells + L.ct - 1) / L.ct, ntp = proj ? (r.outs + L.opt - 1) / L.opt : 0, nr = k.ra, T = k.T;
+    // accumulators: X tiles, H tiles, projection tiles
+    const uint32_t col_h = (uint32_t)(nt * nr), col_p = (uint32_t)(2 * nt * nr);
+    unsigned *cnt0 = L.cnt + (size_t)r.gu * WC_PER_UNIT * WC_WORDS;
+    // the order of a step's products, which the three service warps share: X of step 0, then per step
+    // H(t), X(t + 1), P(t) - or P before X in calls too short to be ahead of the layer below
+    auto walk = [&](auto f) -> bool {
+        if (!f(0, 0)) return false;
+        for (int t = 0; t < T; ++t) {
+            if (!f(1, t)) return false;
+            if (k.early && t + 1 < T && !f(0, t + 1)) return false;
+            if (ntp > 0 && !f(2, t)) return false;
+            if (!k.early && t + 1 < T && !f(0, t + 1)) return false;
+        }
+        return true;
+    };
+
+    if (warp == 0) {
+        // ---------------- operands: x, h, m of a unit, each one contiguous copy ----------------
+        if (lane == 0) {
+            walk([&](int op, int t) -> bool {
+                const unsigned *cnt = nullptr;
+                unsigned target = 0;
+                const int8_t *src;
+                uint32_t bytes = (uint32_t)nr * 128u;
+                if (op == 0) {
+                    bytes *= (uint32_t)L.kb_i;
+                    src = L.in_img + ((size_t)(t + (L.below ? 1 : 0)) * k.nu + r.gu) * bytes;
+                    if (L.below) { cnt = k.layer[r.li - 1].cnt + ((size_t)r.gu * WC_PER_UNIT + WC_H) * WC_WORDS; target = (unsigned)(t + 1) * L.below; }
+                } else if (op == 1) {
+                    bytes *= (uint32_t)L.kb_h;
+                    src = L.out_img + ((size_t)t * k.nu + r.gu) * bytes;
+                    if (t > 0) { cnt = cnt0 + WC_H * WC_WORDS; target = (unsigned)t * L.n; }
+                } else {
+                    bytes *= (uint32_t)L.kb_c;
+                    src = L.m_img + (size_t)r.gu * bytes;
+                    cnt = cnt0 + WC_M * WC_WORDS; target = (unsigned)(t + 1) * L.n;
+                }
+                if (cnt && !wv_wait_count(k, cnt, target, abort_flag)) return false;
+                if (!wv_wait(&ctl->op_empty[op], ((uint32_t)t & 1u) ^ 1u, abort_flag)) return false;
+                wv_fence_async_global();
+                ptx::mbar_arrive_expect_tx(&ctl->op_full[op], bytes);
+                ptx::bulk_load_1d(smem + lay.act[op], src, bytes, &ctl->op_full[op]);
+                return true;
+            });
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---------------- weights ----------------
+        int slot = 0; uint32_t phase = 0;
+        const int whole = L.kpg * L.ctp == 32;                 // a slot is one contiguous piece
+        auto put = [&](const int8_t *src, uint32_t bytes, int pieces) -> bool {
+            bool ok = true;
+            if (lane == 0) {
+                ok = wv_wait(&ctl->w_empty[slot], phase ^ 1u, abort_flag);
+                if (ok) ptx::mbar_arrive_expect_tx(&ctl->w_full[slot], bytes * (uint32_t)pieces);
+            }
+            if (!__shfl_sync(0xffffffffu, (int)ok, 0)) return false;
+            __syncwarp();
+            if (lane < pieces)
+                ptx::bulk_load_1d(smem + (size_t)slot * k.b_slot + (size_t)lane * 4096, src + (size_t)lane * bytes, bytes, &ctl->w_full[slot]);
+            if (++slot == k.nb) { slot = 0; phase ^= 1u; }
+            return true;
+        };
+        walk([&](int op, int) -> bool {
+            if (op == 2) {
+                for (int j = 0; j < ntp; ++j) {
+                    const int8_t *src = L.img_p + (size_t)(r.rank * L.ntp + j) * L.kb_c * L.opp * 128;
+                    for (int kb = 0; kb < L.kb_c; kb += L.kpp) {
+                        const int n = L.kb_c - kb < L.kpp ? L.kb_c - kb : L.kpp;
+                        if (!put(src + (size_t)kb * L.opp * 128, (uint32_t)(n * L.opp * 128), 1)) return false;
+                    }
+                }
+                return true;
+            }
+            const int nch = ((op == 0 ? L.kb_i : L.kb_h) + L.kpg - 1) / L.kpg;
+            const uint32_t piece = (uint32_t)(L.kpg * L.ctp * 128);
+            for (int i = 0; i < nt; ++i) {
+                const int8_t *src = (op == 0 ? L.img_w : L.img_r) + (size_t)(r.rank * L.nt + i) * nch * G * piece;
+                for (int ch = 0; ch < nch; ++ch)
+                    if (!put(src + (size_t)ch * G * piece, whole ? G * piece : piece, whole ? 1 : G)) return false;
+            }
+            return true;
+        });
+    } else if (warp == 2) {
+        // ---------------- MMAs: weights x operand ----------------
+        if (lane == 0) {
+            int slot = 0; uint32_t phase = 0;
+            const uint64_t w_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem));
+            const uint32_t idesc = ptx::idesc_i8(128, nr);
+            // one tile: nkb k-blocks, kps of them per ring slot, kb_bytes apart
+            auto tile = [&](uint32_t d, int op, int nkb, int k32, int kps, uint32_t kb_bytes) -> bool {
+                uint64_t bd = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + lay.act[op]));
+                bool acc = false;
+                for (int kb = 0; kb < nkb;) {
+                    if (!wv_wait(&ctl->w_full[slot], phase, abort_flag)) return false;
+                    ptx::tc_fence_after();
+                    uint64_t ad = w_desc0 + (uint64_t)((uint32_t)slot * ((uint32_t)k.b_slot >> 4));
+                    for (int i = 0; i < kps && kb < nkb; ++i, ++kb) {
+                        const int left = k32 - 4 * kb, nk = left < 4 ? left : 4;
+                        for (int q = 0; q < nk; ++q) { ptx::mma_i8_ss(d, ad + 2 * q, bd + 2 * q, idesc, acc); acc = true; }
+                        ad += kb_bytes >> 4;
+                        bd += (uint32_t)nr * 128u >> 4;
+                    }
+                    ptx::mma_commit(&ctl->w_empty[slot]);
+                    if (++slot == k.nb) { slot = 0; phase ^= 1u; }
+                }
+                return true;
+            };
+            walk([&](int op, int t) -> bool {
+                const uint32_t par = (uint32_t)t & 1u;
+                // the gate accumulators of the step before have been read (X(t) waits for step t - 1 as well)
+                if (op != 2 && t > 0 && !wv_wait(&ctl->acc_empty, par ^ 1u, abort_flag)) return false;
+                if (op == 2 && t > 0 && !wv_wait(&ctl->p_empty, par ^ 1u, abort_flag)) return false;
+                if (!wv_wait(&ctl->op_full[op], par, abort_flag)) return false;
+                ptx::tc_fence_after();
+                if (op == 2) {
+                    for (int j = 0; j < ntp; ++j)
+                        if (!tile(tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.k32_c, L.kpp, (uint32_t)L.opp * 128u)) return false;
+                    ptx::mma_commit(&ctl->p_full);
+                } else {
+                    for (int i = 0; i < nt; ++i) {
+                        if (!tile(tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, op ? L.k32_h : L.k32_i, L.kpg,
+                                  (uint32_t)L.ctp * 128u))
+                            return false;
+                        if (op == 1) ptx::mma_commit(&ctl->gate_full[i]);      // (X of this step was issued before)
+                    }
+                }
+                ptx::mma_commit(&ctl->op_empty[op]);
+                return true;
+            });
+        }
+        __syncwarp();
+    } else if (warp >= WV_EPI_WARP0) {
+        // ---------------- epilogues and elementwise work ----------------
+        const int tid = threadIdx.x - 32 * WV_EPI_WARP0, quarter = warp & 3, wq = (warp - WV_EPI_WARP0) >> 2;
+        const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        WvPoint pt{abort_flag, &ctl->exit_at, 0};
+        bool stay = true;
+        for (int t = 0; t < T && stay; ++t) {
+            const uint32_t par = (uint32_t)t & 1u;
+            for (int i = wq; i < nt; i += 4) {
+                if (quarter >= G) break;
+                if (!__all_sync(0xffffffffu, wv_wait(&ctl->gate_full[i], par, abort_flag))) break;   // (on to the next meeting point)
+                ptx::tc_fence_after();
+                ws_gate_tile<G, LN, PEEP>(k, L, s, r, tq + (uint32_t)(i * nr), tq + col_h + (uint32_t)(i * nr), i, quarter, lane);
+            }
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&ctl->acc_empty);
+            wv_epi_sync();
+            stay = ws_elementwise<G, LN, PEEP>(k, L, s, r, t, last_layer, pt, tid);
+            if (!stay || !proj) continue;
+            if (ntp > 0 && __all_sync(0xffffffffu, wv_wait(&ctl->p_full, par, abort_flag))) {
+                ptx::tc_fence_after();
+                for (int j = 0; j < ntp; ++j) {
+                    const int left = r.outs - j * L.opt;
+                    ws_proj_tile(k, L, s, r, tq + col_p + (uint32_t)(j * nr), j * L.opt, left < L.opt ? left : L.opt, quarter, wq, lane,
+                                 L.out_img + ((size_t)(t + 1) * k.nu + r.gu) * L.kb_h * k.ra * 128, t, last_layer);
+                }
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&ctl->p_empty);
+            }
+            stay = wv_publish(cnt0 + WC_H * WC_WORDS, true, pt, tid);
+        }
+    }
+
+    // ---------------- teardown ----------------
+    ptx::cta_sync();
+    if (*abort_flag) {
+        // a wait ran out: give copies and MMAs in flight time to finish, then report
+        if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
+        for (int i = 0; i < 200; ++i) __nanosleep(500);
+    }
+    ptx::cta_sync();
+    if (warp == 2) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc(tmem_base, 512);
+    }
+}
+
+// A weight matrix into the tiles its blocks stream.  Gate matrices (G > 0): [rank][tile][chunk of kps k-blocks][gate][k-block]
+// [ctp cells][128 bytes]; W_proj (G = 0): [rank][tile][k-block][opp outputs][128 bytes]; 16-byte pieces swizzled by row mod 8.
+__global__ void k_wave_small_tile_weights(const int8_t *src, int8_t *dst, int G, int rows, int K, int n, int per_rank, int nt, int per_tile, int padded,
+                                          int nkb, int kps)
+{
+    const int gates = G > 0 ? G : 1, nch = (nkb + kps - 1) / kps, kbs = G > 0 ? nch * kps : nkb;
+    const size_t total = (size_t)n * nt * kbs * gates * padded * 8;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const int piece = (int)(i & 7);
+        size_t q = i >> 3;
+        const int c = (int)(q % padded); q /= padded;
+        int kb, g = 0, tile, rank;
+        if (G > 0) {
+            const int kk = (int)(q % kps); q /= kps;
+            g = (int)(q % G); q /= G;
+            kb = (int)(q % nch) * kps + kk; q /= nch;
+        } else {
+            kb = (int)(q % nkb); q /= nkb;
+        }
+        tile = (int)(q % nt); rank = (int)(q / nt);
+        const int u = tile * per_tile + c;                     // cell or output within the block
+        int src_row = -1;
+        if (c < per_tile && u < per_rank && (size_t)(rank * per_rank + u) * gates < (size_t)rows) src_row = (rank * per_rank + u) * gates + g;
+        const int k0 = kb * 128 + piece * 16;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (src_row >= 0 && k0 < K) v = wv_load16(src + (size_t)src_row * K + k0, K - k0);
+        *reinterpret_cast<uint4 *>(dst + (i >> 3) * 128 + ((piece ^ (c & 7)) << 4)) = v;
+    }
+}
+
+}  // namespace
+
+void wave_small_tile_weights(const int8_t *src, int8_t *dst, int G, int rows, int K, int n, int per_rank, int nt, int per_tile, int padded, int nkb, int kps)
+{
+    k_wave_small_tile_weights<<<2048, 256>>>(src, dst, G, rows, K, n, per_rank, nt, per_tile, padded, nkb, kps);
+}
+
+const void *wave_small_kernel(int G, bool ln, bool peep)
+{
+    if (G == 4) {
+        if (ln) return peep ? (const void *)k_wave_small_sm100<4, true, true> : (const void *)k_wave_small_sm100<4, true, false>;
+        return peep ? (const void *)k_wave_small_sm100<4, false, true> : (const void *)k_wave_small_sm100<4, false, false>;
+    }
+    if (ln) return peep ? (const void *)k_wave_small_sm100<3, true, true> : (const void *)k_wave_small_sm100<3, true, false>;
+    return peep ? (const void *)k_wave_small_sm100<3, false, true> : (const void *)k_wave_small_sm100<3, false, false>;
+}
+
+// shared memory of a launch with ns ring slots
+size_t wave_small_smem(const WaveCall &k, int ns, bool peep) { return ws_layout(k, ns, (k.B + k.nu - 1) / k.nu, peep).total; }
+
+}  // namespace ql

@@ -23,8 +23,8 @@ def check(w):
         assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
 
 
-# one row; copies of the rows in the lanes end at 32 and 64; one unit ends at 128; two full units
-@pytest.mark.parametrize("B", [1, 31, 33, 64, 65, 128, 129, 256])
+# one row; MMA columns of eight and 32 rows; copies of the rows in the lanes end at 64; one unit ends at 128; two full units
+@pytest.mark.parametrize("B", [1, 8, 9, 32, 33, 64, 65, 128, 129, 256])
 @pytest.mark.parametrize("kw", VARIANTS, ids=lambda k: "+".join(sorted(k)) or "basic")
 def test_wave_variants(kw, B):
     check(random_layer_stack(810 + B, 3, 48, 112, 64, T=6, B=B, **kw))
