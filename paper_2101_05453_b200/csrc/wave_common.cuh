@@ -29,7 +29,6 @@ struct WaveLayer {
     int cpc, ct, ctp, kpg;         // wave_small_sm100.cu: cells per block; cells of a tile, rounded up to 8; k-blocks per ring slot
     int opp, kpp;                  // ... outputs of a projection tile rounded up to 8, k-blocks per ring slot
     int kb_i, kb_h, kb_c;          // 128-byte k-blocks of the three products
-    int k32_i, k32_h, k32_c;       // K steps of 32
     const int8_t *img_w, *img_r, *img_p;       // weights in the order and image in which the blocks stream them
     const int32_t *bx, *bh, *bln, *bp;
     const int16_t *P, *L;
@@ -74,7 +73,7 @@ __device__ __forceinline__ bool wv_wait(uint64_t *bar, uint32_t parity, volatile
 {
     // each attempt parks the thread for up to 20 us; 100 000 attempts bound the wait to about 2 s
     for (uint32_t i = 0; i < 100000u; ++i) {
-        if (ptx::mbar_try_wait_parked(bar, parity, 20000u)) return *abort_flag == 0;
+        if (ptx::mbar_try_wait_parked(bar, parity, 20000u)) return true;
         if (*abort_flag) return false;
     }
     *abort_flag = 1;
@@ -111,6 +110,39 @@ __device__ __forceinline__ bool wv_wait_count(const WaveCall &k, const unsigned 
     return *abort_flag == 0;
 }
 __device__ __forceinline__ void wv_epi_sync() { asm volatile("barrier.sync 1, 512;" ::: "memory"); }
+
+// The same for a whole warp that stays together.
+__device__ __forceinline__ bool wv_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
+{
+    return __all_sync(0xffffffffu, wv_wait(bar, parity, abort_flag));
+}
+
+// The MMAs of nkb consecutive k-blocks (128 bytes of K each; both operands are zero-padded to that), a_step and b_step
+// apart, by one elected lane of a warp that stays together.  The instruction wants its operands in uniform registers: in a
+// rolled loop under a divergent branch an MMA took 200 cycles of issue, written like this 50 to 75 (N <= 128; the tensor core
+// itself needs 50 at N <= 64 and 127 at N = 256).
+__device__ __forceinline__ void wv_mma_kblocks(uint32_t d, uint64_t a, uint64_t b, uint32_t a_step, uint32_t b_step, int nkb, uint32_t idesc, bool fresh,
+                                               uint64_t *bar0, uint64_t *bar1)
+{
+    if (ptx::elect_one()) {
+        for (int i = 0; i < nkb; ++i) {
+            ptx::mma_i8_ss(d, a, b, idesc, !(fresh && i == 0));
+            ptx::mma_i8_ss(d, a + 2, b + 2, idesc, true);
+            ptx::mma_i8_ss(d, a + 4, b + 4, idesc, true);
+            ptx::mma_i8_ss(d, a + 6, b + 6, idesc, true);
+            a += a_step;
+            b += b_step;
+        }
+        ptx::mma_commit(bar0);
+        if (bar1) ptx::mma_commit(bar1);
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ void wv_commit(uint64_t *bar)
+{
+    if (ptx::elect_one()) ptx::mma_commit(bar);
+    __syncwarp();
+}
 
 // ---- fixed-point pieces ----------------------------------------------------------------------------------------------
 __device__ __forceinline__ int32_t wv_lo(uint32_t w) { return (int32_t)(w << 16) >> 16; }

@@ -649,35 +649,29 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
         __syncwarp();
     } else if (warp == 2) {
         // ---------------- MMAs ----------------
-        if (lane == 0) {
-            int sa = 0, sb = 0, job = 0;
-            uint32_t pa = 0, pb = 0;
-            const uint64_t a_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(a_ring)), b_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(b_ring));
-            wv_walk(ctl, k.T, [&](const WaveOp &op, int) -> bool {
-                if (op.kind > OP_P) return true;
-                const int k32 = op.kind == OP_X ? L.k32_i : op.kind == OP_H ? L.k32_h : L.k32_c;
-                const uint32_t idesc = ptx::idesc_i8(128, op.kind == OP_P ? L.npadp : L.npad);
-                const uint32_t d = tmem_base + (uint32_t)(job & 1) * WV_ACC_COLS;
-                if (!wv_wait(&ctl->t_empty[job & 1], ((uint32_t)(job >> 1) & 1u) ^ 1u, abort_flag)) return false;
+        int sa = 0, sb = 0, job = 0;
+        uint32_t pa = 0, pb = 0;
+        const uint64_t a_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(a_ring)), b_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(b_ring));
+        wv_walk(ctl, k.T, [&](const WaveOp &op, int) -> bool {
+            if (op.kind > OP_P) return true;
+            const int nkb = op.kind == OP_X ? L.kb_i : op.kind == OP_H ? L.kb_h : L.kb_c;
+            const uint32_t idesc = ptx::idesc_i8(128, op.kind == OP_P ? L.npadp : L.npad);
+            const uint32_t d = tmem_base + (uint32_t)(job & 1) * WV_ACC_COLS;
+            if (!wv_wait_warp(&ctl->t_empty[job & 1], ((uint32_t)(job >> 1) & 1u) ^ 1u, abort_flag)) return false;
+            ptx::tc_fence_after();
+            for (int kb = 0; kb < nkb; ++kb) {
+                const bool ok = wv_wait(&ctl->a_full[sa], pa, abort_flag) && wv_wait(&ctl->b_full[sb], pb, abort_flag);
+                if (!__all_sync(0xffffffffu, ok)) return false;
                 ptx::tc_fence_after();
-                bool acc = false;
-                for (int left = k32; left > 0; left -= 4) {
-                    if (!wv_wait(&ctl->a_full[sa], pa, abort_flag) || !wv_wait(&ctl->b_full[sb], pb, abort_flag)) return false;
-                    ptx::tc_fence_after();
-                    const uint64_t ad = a_desc0 + (uint64_t)(sa * (WV_A_SLOT >> 4)), bd = b_desc0 + (uint64_t)(sb * (k.b_slot >> 4));
-                    const int nk = left < 4 ? left : 4;
-                    for (int i = 0; i < nk; ++i) { ptx::mma_i8_ss(d, ad + 2 * i, bd + 2 * i, idesc, acc); acc = true; }
-                    ptx::mma_commit(&ctl->a_empty[sa]);
-                    ptx::mma_commit(&ctl->b_empty[sb]);
-                    if (++sa == k.na) { sa = 0; pa ^= 1u; }
-                    if (++sb == k.nb) { sb = 0; pb ^= 1u; }
-                }
-                ptx::mma_commit(&ctl->t_full[job & 1]);
-                ++job;
-                return true;
-            });
-        }
-        __syncwarp();
+                wv_mma_kblocks(d, a_desc0 + (uint64_t)(sa * (WV_A_SLOT >> 4)), b_desc0 + (uint64_t)(sb * (k.b_slot >> 4)), 0, 0, 1, idesc, kb == 0,
+                               &ctl->a_empty[sa], &ctl->b_empty[sb]);
+                if (++sa == k.na) { sa = 0; pa ^= 1u; }
+                if (++sb == k.nb) { sb = 0; pb ^= 1u; }
+            }
+            wv_commit(&ctl->t_full[job & 1]);
+            ++job;
+            return true;
+        });
     } else if (warp >= WV_EPI_WARP0) {
         // ---------------- epilogues and elementwise work ----------------
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0;
@@ -985,7 +979,6 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
         memset(&L, 0, sizeof(L));
         L.I = p.I; L.C = p.C; L.O = p.O; L.flags = p.flags; L.m_bits = p.m_bits; L.zp_m = p.zp_m; L.zp_h = p.zp_h;
         L.kb_i = (p.I + 127) / 128; L.kb_h = (p.O + 127) / 128; L.kb_c = (p.C + 127) / 128;
-        L.k32_i = (p.I + 31) / 32; L.k32_h = (p.O + 31) / 32; L.k32_c = (p.C + 31) / 32;
         s->max_kb_i = std::max(s->max_kb_i, L.kb_i);
         s->max_kb_h = std::max(s->max_kb_h, L.kb_h);
         if (proj) s->max_kb_c = std::max(s->max_kb_c, L.kb_c);

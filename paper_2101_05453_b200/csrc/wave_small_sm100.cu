@@ -439,53 +439,42 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         });
     } else if (warp == 2) {
         // ---------------- MMAs: weights x operand ----------------
-        if (lane == 0) {
-            int slot = 0; uint32_t phase = 0;
-            const uint64_t w_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem));
-            const uint32_t idesc = ptx::idesc_i8(128, nr);
-            // one tile: nkb k-blocks, kps of them per ring slot, kb_bytes apart
-            auto tile = [&](uint32_t d, int op, int nkb, int k32, int kps, uint32_t kb_bytes) -> bool {
-                uint64_t bd = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + lay.act[op]));
-                bool acc = false;
-                for (int kb = 0; kb < nkb;) {
-                    if (!wv_wait(&ctl->w_full[slot], phase, abort_flag)) return false;
-                    ptx::tc_fence_after();
-                    uint64_t ad = w_desc0 + (uint64_t)((uint32_t)slot * ((uint32_t)k.b_slot >> 4));
-                    for (int i = 0; i < kps && kb < nkb; ++i, ++kb) {
-                        const int left = k32 - 4 * kb, nk = left < 4 ? left : 4;
-                        for (int q = 0; q < nk; ++q) { ptx::mma_i8_ss(d, ad + 2 * q, bd + 2 * q, idesc, acc); acc = true; }
-                        ad += kb_bytes >> 4;
-                        bd += (uint32_t)nr * 128u >> 4;
-                    }
-                    ptx::mma_commit(&ctl->w_empty[slot]);
-                    if (++slot == k.nb) { slot = 0; phase ^= 1u; }
-                }
-                return true;
-            };
-            walk([&](int op, int t) -> bool {
-                const uint32_t par = (uint32_t)t & 1u;
-                // the gate accumulators of the step before have been read (X(t) waits for step t - 1 as well)
-                if (op != 2 && t > 0 && !wv_wait(&ctl->acc_empty, par ^ 1u, abort_flag)) return false;
-                if (op == 2 && t > 0 && !wv_wait(&ctl->p_empty, par ^ 1u, abort_flag)) return false;
-                if (!wv_wait(&ctl->op_full[op], par, abort_flag)) return false;
+        int slot = 0; uint32_t phase = 0;
+        const uint64_t w_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem));
+        const uint32_t idesc = ptx::idesc_i8(128, nr), b_step = (uint32_t)nr * 128u >> 4;
+        // one tile: nkb k-blocks, kps of them per ring slot, kb_bytes apart
+        auto tile = [&](uint32_t d, int op, int nkb, int kps, uint32_t kb_bytes) -> bool {
+            uint64_t bd = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + lay.act[op]));
+            for (int kb = 0; kb < nkb; kb += kps) {
+                if (!wv_wait_warp(&ctl->w_full[slot], phase, abort_flag)) return false;
                 ptx::tc_fence_after();
-                if (op == 2) {
-                    for (int j = 0; j < ntp; ++j)
-                        if (!tile(tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.k32_c, L.kpp, (uint32_t)L.opp * 128u)) return false;
-                    ptx::mma_commit(&ctl->p_full);
-                } else {
-                    for (int i = 0; i < nt; ++i) {
-                        if (!tile(tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, op ? L.k32_h : L.k32_i, L.kpg,
-                                  (uint32_t)L.ctp * 128u))
-                            return false;
-                        if (op == 1) ptx::mma_commit(&ctl->gate_full[i]);      // (X of this step was issued before)
-                    }
+                wv_mma_kblocks(d, w_desc0 + (uint64_t)((uint32_t)slot * ((uint32_t)k.b_slot >> 4)), bd, kb_bytes >> 4, b_step,
+                               nkb - kb < kps ? nkb - kb : kps, idesc, kb == 0, &ctl->w_empty[slot], nullptr);
+                bd += (uint64_t)(b_step * (uint32_t)kps);
+                if (++slot == k.nb) { slot = 0; phase ^= 1u; }
+            }
+            return true;
+        };
+        walk([&](int op, int t) -> bool {
+            const uint32_t par = (uint32_t)t & 1u;
+            // the gate accumulators of the step before have been read (X(t) waits for step t - 1 as well)
+            if (op != 2 && t > 0 && !wv_wait_warp(&ctl->acc_empty, par ^ 1u, abort_flag)) return false;
+            if (op == 2 && t > 0 && !wv_wait_warp(&ctl->p_empty, par ^ 1u, abort_flag)) return false;
+            if (!wv_wait_warp(&ctl->op_full[op], par, abort_flag)) return false;
+            ptx::tc_fence_after();
+            if (op == 2) {
+                for (int j = 0; j < ntp; ++j)
+                    if (!tile(tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.kpp, (uint32_t)L.opp * 128u)) return false;
+                wv_commit(&ctl->p_full);
+            } else {
+                for (int i = 0; i < nt; ++i) {
+                    if (!tile(tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u)) return false;
+                    if (op == 1) wv_commit(&ctl->gate_full[i]);      // (X of this step was issued before)
                 }
-                ptx::mma_commit(&ctl->op_empty[op]);
-                return true;
-            });
-        }
-        __syncwarp();
+            }
+            wv_commit(&ctl->op_empty[op]);
+            return true;
+        });
     } else if (warp >= WV_EPI_WARP0) {
         // ---------------- epilogues and elementwise work ----------------
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0, quarter = warp & 3, wq = (warp - WV_EPI_WARP0) >> 2;
