@@ -13,6 +13,7 @@ constexpr int WV_THREADS = 640;
 constexpr int WV_EPI_WARP0 = 4;
 constexpr int WV_EPI = WV_THREADS - 32 * WV_EPI_WARP0;         // 512 epilogue threads
 constexpr int WV_MAX_LAYERS = 16;
+constexpr int WS_SLOT_ROWS = 256;              // wave_small_sm100.cu: 128-byte rows of a weight slot
 constexpr unsigned long long WV_WAIT_LIMIT_NS = 2000000000ull;
 
 // counters of one (layer, unit), each on a line of its own
@@ -26,7 +27,7 @@ struct WaveLayer {
     int ppc;                       // cell pairs per block (wave_sm100.cu)
     int nt, ppt, npad;             // gate tiles: count, pairs per tile, MMA columns
     int opc, ntp, opt, npadp;      // outputs per block; projection tiles: count, outputs per tile, MMA columns
-    int cpc, ct, ctp, kpg;         // wave_small_sm100.cu: cells per block; cells of a tile, rounded up to 8; k-blocks per ring slot
+    int cpc, ct, ctp, kpg;         // wave_small_sm100.cu: cells per block; cells of a tile, rounded up; k-blocks per chunk
     int opp, kpp;                  // ... outputs of a projection tile rounded up to 8, k-blocks per ring slot
     int kb_i, kb_h, kb_c;          // 128-byte k-blocks of the three products
     const int8_t *img_w, *img_r, *img_p;       // weights in the order and image in which the blocks stream them
@@ -117,26 +118,15 @@ __device__ __forceinline__ bool wv_wait_warp(uint64_t *bar, uint32_t parity, vol
     return __all_sync(0xffffffffu, wv_wait(bar, parity, abort_flag));
 }
 
-// The MMAs of nkb consecutive k-blocks (128 bytes of K each; both operands are zero-padded to that), a_step and b_step
-// apart, by one elected lane of a warp that stays together.  The instruction wants its operands in uniform registers: in a
-// rolled loop under a divergent branch an MMA took 200 cycles of issue, written like this 50 to 75 (N <= 128; the tensor core
-// itself needs 50 at N <= 64 and 127 at N = 256).
-__device__ __forceinline__ void wv_mma_kblocks(uint32_t d, uint64_t a, uint64_t b, uint32_t a_step, uint32_t b_step, int nkb, uint32_t idesc, bool fresh,
-                                               uint64_t *bar0, uint64_t *bar1)
+// The four MMAs of one k-block (128 bytes of K; both operands are zero-padded to that), by an elected lane of a warp that
+// stays together.  The instruction wants its operands in uniform registers: in a rolled loop under a divergent branch an MMA
+// took 200 cycles of issue, written like this 50 to 75 (N <= 128; the tensor core itself needs 50 at N <= 64 and 127 at N = 256).
+__device__ __forceinline__ void wv_mma_kblock(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool fresh)
 {
-    if (ptx::elect_one()) {
-        for (int i = 0; i < nkb; ++i) {
-            ptx::mma_i8_ss(d, a, b, idesc, !(fresh && i == 0));
-            ptx::mma_i8_ss(d, a + 2, b + 2, idesc, true);
-            ptx::mma_i8_ss(d, a + 4, b + 4, idesc, true);
-            ptx::mma_i8_ss(d, a + 6, b + 6, idesc, true);
-            a += a_step;
-            b += b_step;
-        }
-        ptx::mma_commit(bar0);
-        if (bar1) ptx::mma_commit(bar1);
-    }
-    __syncwarp();
+    ptx::mma_i8_ss(d, a, b, idesc, !fresh);
+    ptx::mma_i8_ss(d, a + 2, b + 2, idesc, true);
+    ptx::mma_i8_ss(d, a + 4, b + 4, idesc, true);
+    ptx::mma_i8_ss(d, a + 6, b + 6, idesc, true);
 }
 __device__ __forceinline__ void wv_commit(uint64_t *bar)
 {

@@ -663,8 +663,12 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
                 const bool ok = wv_wait(&ctl->a_full[sa], pa, abort_flag) && wv_wait(&ctl->b_full[sb], pb, abort_flag);
                 if (!__all_sync(0xffffffffu, ok)) return false;
                 ptx::tc_fence_after();
-                wv_mma_kblocks(d, a_desc0 + (uint64_t)(sa * (WV_A_SLOT >> 4)), b_desc0 + (uint64_t)(sb * (k.b_slot >> 4)), 0, 0, 1, idesc, kb == 0,
-                               &ctl->a_empty[sa], &ctl->b_empty[sb]);
+                if (ptx::elect_one()) {
+                    wv_mma_kblock(d, a_desc0 + (uint64_t)(sa * (WV_A_SLOT >> 4)), b_desc0 + (uint64_t)(sb * (k.b_slot >> 4)), idesc, kb == 0);
+                    ptx::mma_commit(&ctl->a_empty[sa]);
+                    ptx::mma_commit(&ctl->b_empty[sb]);
+                }
+                __syncwarp();
                 if (++sa == k.na) { sa = 0; pa ^= 1u; }
                 if (++sb == k.nb) { sb = 0; pb ^= 1u; }
             }
@@ -894,14 +898,14 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
         L.n = (p.C + L.cpc - 1) / L.cpc;
         L.nt = (L.cpc + 31) / 32;
         L.ct = (L.cpc + L.nt - 1) / L.nt;
-        L.ctp = wv_round(L.ct, 8);
+        L.ctp = L.ct <= 8 ? 8 : L.ct <= 16 ? 16 : 32;                // (a chunk's gates are 32 rows apart and leave no gaps)
         L.kpg = 32 / L.ctp;
         if (proj) {
             L.opc = (p.O + L.n - 1) / L.n;
             L.ntp = (L.opc + 127) / 128;
             L.opt = (L.opc + L.ntp - 1) / L.ntp;
             L.opp = wv_round(L.opt, 8);
-            L.kpp = 128 / L.opp;
+            L.kpp = WS_SLOT_ROWS / L.opp;
         }
         if (L.nt > 8 || (2 * L.nt + L.ntp) * 8 > 512) { L.n = 0; return QLSTM_OK; }
     }
@@ -1033,7 +1037,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
             pl.max_ppc = std::max(pl.max_ppc, M.ppc);
             pl.max_cpc = std::max(pl.max_cpc, wv_round(M.cpc, 2));
             pl.max_opc = std::max(pl.max_opc, wv_round(M.opc, 4));
-            pl.b_slot = mode == 1 ? 128 * 128 : std::max(pl.b_slot, std::max(M.npad, proj ? M.npadp : 0) * 128);
+            pl.b_slot = mode == 1 ? WS_SLOT_ROWS * 128 : std::max(pl.b_slot, std::max(M.npad, proj ? M.npadp : 0) * 128);
             pl.layer.push_back(M);
         }
     }
@@ -1087,7 +1091,7 @@ static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool table
         if (rows > WV_SMALL_ROWS) return false;
         for (const WaveLayer &L : pl.layer)
             if ((2 * L.nt + L.ntp) * k.ra > 512) return false;
-        k.nb = 16;
+        k.nb = 8;
         while (k.nb > 3 && wave_small_smem(k, k.nb, s->peep) > room) --k.nb;
         smem = wave_small_smem(k, k.nb, s->peep);
         return smem <= room;

@@ -16,7 +16,9 @@ namespace ql {
 
 namespace {
 
-constexpr int WS_SLOTS = 16;
+constexpr int WS_SLOTS = 8;
+constexpr int WS_CHUNKS = 2;                   // gate chunks of a slot: a copy of 32 KB streams at 125 KB/us, one of 16 KB at 80, one
+                                               // of 4 KB at 21 (about 0.2 us of the copying thread each)
 constexpr int WS_MAX_TILES = 8;
 constexpr int WS_ROWS = 32;
 
@@ -402,55 +404,59 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- weights ----------------
-        int slot = 0; uint32_t phase = 0;
-        const int whole = L.kpg * L.ctp == 32;                 // a slot is one contiguous piece
-        auto put = [&](const int8_t *src, uint32_t bytes, int pieces) -> bool {
-            bool ok = true;
-            if (lane == 0) {
-                ok = wv_wait(&ctl->w_empty[slot], phase ^ 1u, abort_flag);
-                if (ok) ptx::mbar_arrive_expect_tx(&ctl->w_full[slot], bytes * (uint32_t)pieces);
-            }
-            if (!__shfl_sync(0xffffffffu, (int)ok, 0)) return false;
-            __syncwarp();
-            if (lane < pieces)
-                ptx::bulk_load_1d(smem + (size_t)slot * k.b_slot + (size_t)lane * 4096, src + (size_t)lane * bytes, bytes, &ctl->w_full[slot]);
-            if (++slot == k.nb) { slot = 0; phase ^= 1u; }
-            return true;
-        };
-        walk([&](int op, int) -> bool {
-            if (op == 2) {
-                for (int j = 0; j < ntp; ++j) {
-                    const int8_t *src = L.img_p + (size_t)(r.rank * L.ntp + j) * L.kb_c * L.opp * 128;
-                    for (int kb = 0; kb < L.kb_c; kb += L.kpp) {
-                        const int n = L.kb_c - kb < L.kpp ? L.kb_c - kb : L.kpp;
-                        if (!put(src + (size_t)kb * L.opp * 128, (uint32_t)(n * L.opp * 128), 1)) return false;
-                    }
+        if (lane == 0) {
+            int slot = 0; uint32_t phase = 0;
+            // `total` bytes from src, a slot's worth (`most`) at a time
+            auto put = [&](const int8_t *src, uint32_t total, uint32_t most) -> bool {
+                for (uint32_t done = 0; done < total; done += most) {
+                    const uint32_t bytes = total - done < most ? total - done : most;
+                    if (!wv_wait(&ctl->w_empty[slot], phase ^ 1u, abort_flag)) return false;
+                    ptx::mbar_arrive_expect_tx(&ctl->w_full[slot], bytes);
+                    ptx::bulk_load_1d(smem + (size_t)slot * k.b_slot, src + done, bytes, &ctl->w_full[slot]);
+                    if (++slot == k.nb) { slot = 0; phase ^= 1u; }
                 }
                 return true;
-            }
-            const int nch = ((op == 0 ? L.kb_i : L.kb_h) + L.kpg - 1) / L.kpg;
-            const uint32_t piece = (uint32_t)(L.kpg * L.ctp * 128);
-            for (int i = 0; i < nt; ++i) {
-                const int8_t *src = (op == 0 ? L.img_w : L.img_r) + (size_t)(r.rank * L.nt + i) * nch * G * piece;
-                for (int ch = 0; ch < nch; ++ch)
-                    if (!put(src + (size_t)ch * G * piece, whole ? G * piece : piece, whole ? 1 : G)) return false;
-            }
-            return true;
-        });
+            };
+            walk([&](int op, int) -> bool {
+                if (op == 2) {
+                    const uint32_t total = (uint32_t)(L.kb_c * L.opp * 128);
+                    for (int j = 0; j < ntp; ++j)
+                        if (!put(L.img_p + (size_t)(r.rank * L.ntp + j) * total, total, (uint32_t)(L.kpp * L.opp * 128))) return false;
+                    return true;
+                }
+                const uint32_t total = (uint32_t)((((op == 0 ? L.kb_i : L.kb_h) + L.kpg - 1) / L.kpg) * G * 4096);
+                for (int i = 0; i < nt; ++i)
+                    if (!put((op == 0 ? L.img_w : L.img_r) + (size_t)(r.rank * L.nt + i) * total, total, WS_CHUNKS * G * 4096u)) return false;
+                return true;
+            });
+        }
+        __syncwarp();
     } else if (warp == 2) {
         // ---------------- MMAs: weights x operand ----------------
         int slot = 0; uint32_t phase = 0;
         const uint64_t w_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem));
         const uint32_t idesc = ptx::idesc_i8(128, nr), b_step = (uint32_t)nr * 128u >> 4;
-        // one tile: nkb k-blocks, kps of them per ring slot, kb_bytes apart
-        auto tile = [&](uint32_t d, int op, int nkb, int kps, uint32_t kb_bytes) -> bool {
-            uint64_t bd = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + lay.act[op]));
-            for (int kb = 0; kb < nkb; kb += kps) {
+        // one tile of nkb k-blocks: kpc of them per chunk (kb_bytes apart), the chunks of a ring slot chunk_bytes apart
+        auto tile = [&](uint32_t d, int op, int nkb, int kpc, uint32_t kb_bytes, int n_chunks, uint32_t chunk_bytes) -> bool {
+            const uint64_t b_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + lay.act[op]));
+            for (int kb0 = 0; kb0 < nkb; kb0 += kpc * n_chunks) {
                 if (!wv_wait_warp(&ctl->w_full[slot], phase, abort_flag)) return false;
                 ptx::tc_fence_after();
-                wv_mma_kblocks(d, w_desc0 + (uint64_t)((uint32_t)slot * ((uint32_t)k.b_slot >> 4)), bd, kb_bytes >> 4, b_step,
-                               nkb - kb < kps ? nkb - kb : kps, idesc, kb == 0, &ctl->w_empty[slot], nullptr);
-                bd += (uint64_t)(b_step * (uint32_t)kps);
+                if (ptx::elect_one()) {
+                    uint64_t ac = w_desc0 + (uint64_t)((uint32_t)slot * ((uint32_t)k.b_slot >> 4));
+                    uint64_t bd = b_desc0 + (uint64_t)(b_step * (uint32_t)kb0);
+                    int kb = kb0;
+                    for (int c = 0; c < n_chunks; ++c, ac += chunk_bytes >> 4) {
+                        uint64_t ad = ac;
+                        for (int i = 0; i < kpc && kb < nkb; ++i, ++kb) {
+                            wv_mma_kblock(d, ad, bd, idesc, kb == 0);
+                            ad += kb_bytes >> 4;
+                            bd += b_step;
+                        }
+                    }
+                    ptx::mma_commit(&ctl->w_empty[slot]);
+                }
+                __syncwarp();
                 if (++slot == k.nb) { slot = 0; phase ^= 1u; }
             }
             return true;
@@ -464,11 +470,13 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
             ptx::tc_fence_after();
             if (op == 2) {
                 for (int j = 0; j < ntp; ++j)
-                    if (!tile(tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.kpp, (uint32_t)L.opp * 128u)) return false;
+                    if (!tile(tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.kpp, (uint32_t)L.opp * 128u, 1, 0u)) return false;
                 wv_commit(&ctl->p_full);
             } else {
                 for (int i = 0; i < nt; ++i) {
-                    if (!tile(tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u)) return false;
+                    if (!tile(tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u, WS_CHUNKS,
+                              G * 4096u))
+                        return false;
                     if (op == 1) wv_commit(&ctl->gate_full[i]);      // (X of this step was issued before)
                 }
             }
