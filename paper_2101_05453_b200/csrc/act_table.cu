@@ -63,28 +63,32 @@ bool pack_quads(const int32_t *v, int amax, std::vector<uint32_t> &out)
     return true;
 }
 
+// quotients of the definition for |x| = 0 .. 32768: sigmoid, gate tanh, cell tanh; bad: they are not symmetric
+bool act_domain(int m_cell, std::vector<int32_t> &v, bool &bad_out)
+{
+    int32_t *v_dev = nullptr;
+    if (cudaMalloc(&v_dev, (3 * ACT_DOMAIN + 1) * sizeof(int32_t)) != cudaSuccess) return false;
+    int *bad_dev = v_dev + 3 * ACT_DOMAIN;
+    v.resize((size_t)3 * ACT_DOMAIN + 1);
+    bool ok = cudaMemset(bad_dev, 0, sizeof(int)) == cudaSuccess;
+    if (ok) {
+        k_act_domain<<<(ACT_DOMAIN + 255) / 256, 256>>>(m_cell, v_dev, bad_dev);
+        ok = cudaGetLastError() == cudaSuccess && cudaMemcpy(v.data(), v_dev, v.size() * sizeof(int32_t), cudaMemcpyDeviceToHost) == cudaSuccess;
+    }
+    cudaFree(v_dev);
+    bad_out = v.back() != 0;
+    return ok;
+}
+
 }  // namespace
 
 bool act_tables_build(int m_cell, size_t max_bytes, uint8_t **blob_dev, ActTabLayout *lay)
 {
     *blob_dev = nullptr;
     *lay = ActTabLayout{0, 0, 0, 0, 0, 0, 0};
-    int32_t *v_dev = nullptr;
-    int *bad_dev = nullptr;
-    if (cudaMalloc(&v_dev, 3 * ACT_DOMAIN * sizeof(int32_t)) != cudaSuccess) return false;
-    if (cudaMalloc(&bad_dev, sizeof(int)) != cudaSuccess) { cudaFree(v_dev); return false; }
-    std::vector<int32_t> v((size_t)3 * ACT_DOMAIN);
-    int bad = 0;
-    bool ok = cudaMemset(bad_dev, 0, sizeof(int)) == cudaSuccess;
-    if (ok) {
-        k_act_domain<<<(ACT_DOMAIN + 255) / 256, 256>>>(m_cell, v_dev, bad_dev);
-        ok = cudaGetLastError() == cudaSuccess &&
-             cudaMemcpy(v.data(), v_dev, v.size() * sizeof(int32_t), cudaMemcpyDeviceToHost) == cudaSuccess &&
-             cudaMemcpy(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess;
-    }
-    cudaFree(v_dev);
-    cudaFree(bad_dev);
-    if (!ok) return false;
+    std::vector<int32_t> v;
+    bool bad = false;
+    if (!act_domain(m_cell, v, bad)) return false;
     if (bad) return true;
     const int32_t *sg = v.data(), *tz = sg + ACT_DOMAIN, *tc = tz + ACT_DOMAIN;
     for (int a = 0; a < ACT_DOMAIN; ++a)
@@ -132,6 +136,98 @@ bool act_tables_build(int m_cell, size_t max_bytes, uint8_t **blob_dev, ActTabLa
     if (cudaMemcpy(d, blob.data(), L.bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(d); return false; }
     *blob_dev = d;
     *lay = L;
+    return true;
+}
+
+namespace {
+
+// the entry of 2^sh consecutive inputs, f their values; every slope that can fit lies within 1 / (2^sh - 1) of the secant's
+bool find_line(const int32_t *f, int sh, int k, int32_t &entry)
+{
+    const int n = 1 << sh;
+    const int64_t rise = ((int64_t)(f[n - 1] - f[0]) << 16) / (n > 1 ? n - 1 : 1);
+    const int64_t s0 = rise >> k, reach = ((65536 / (n > 1 ? n - 1 : 1)) >> k) + 2;
+    for (int64_t d = 0; d < 2 * reach; ++d) {
+        const int64_t s = s0 + ((d & 1) ? (d + 1) / 2 : -d / 2);
+        if (s < 0 || s > 1023) continue;
+        int64_t lo = INT64_MIN, hi = INT64_MAX;
+        for (int j = 0; j < n; ++j) {
+            const int64_t a = ((int64_t)f[j] << 16) - ((s << k) * j), b = a + 65535;
+            lo = lo > a ? lo : a;
+            hi = hi < b ? hi : b;
+        }
+        const int64_t e = lo + ((s - lo) & 1023);
+        if (e > hi || e < INT32_MIN || e + ((s << k) * (n - 1)) > INT32_MAX) continue;
+        bool ok = true;
+        for (int j = 0; j < n && ok; ++j) ok = act_line_value((int32_t)e, j, sh, k) == f[j];
+        if (!ok) continue;
+        entry = (int32_t)e;
+        return true;
+    }
+    return false;
+}
+
+// the entries of all segments that meet [lo, hi]; f: values of x = -32768 .. 32767
+bool build_lines(const std::vector<int32_t> &f, int lo, int hi, int sh, int k, std::vector<int32_t> &out)
+{
+    out.clear();
+    for (int seg = lo >> sh; seg <= (hi >> sh); ++seg) {
+        int32_t e;
+        if (!find_line(&f[(size_t)(seg * (1 << sh) + 32768)], sh, k, e)) return false;
+        out.push_back(e);
+    }
+    return true;
+}
+
+}  // namespace
+
+bool act_lines_build(int m_cell, uint8_t **blob_dev, ActLineLayout *lay)
+{
+    *blob_dev = nullptr;
+    *lay = ActLineLayout{0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    std::vector<int32_t> v;
+    bool bad = false;
+    if (!act_domain(m_cell, v, bad)) return false;
+    if (bad) return true;
+    // values over the signed domain, as the definition's last step forms them
+    std::vector<int32_t> f[3];
+    for (int t = 0; t < 3; ++t) {
+        f[t].resize(65536);
+        for (int x = -32768; x < 32768; ++x) {
+            const int32_t q = v[(size_t)t * ACT_DOMAIN + (x < 0 ? -x : x)];
+            f[t][x + 32768] = x >= 0 ? (q < 32767 ? q : 32767) : (t == 0 ? 32768 - q : -q);
+        }
+    }
+    std::vector<int32_t> sig, tz, tc;
+    auto range = [](const std::vector<int32_t> &g, int &lo, int &hi) {
+        lo = -32768; hi = 32767;
+        while (lo < hi && g[lo + 1 + 32768] == g[lo + 32768]) ++lo;
+        while (hi > lo && g[hi - 1 + 32768] == g[hi + 32768]) --hi;
+    };
+    if (!build_lines(f[0], -32768, 32767, ACT_SIG_SH, ACT_SIG_K, sig)) return true;
+    range(f[1], lay->tz_lo, lay->tz_hi);
+    if (!build_lines(f[1], lay->tz_lo, lay->tz_hi, ACT_TZ_SH, ACT_TZ_K, tz)) return true;
+    range(f[2], lay->tc_lo, lay->tc_hi);
+    lay->tc_sh = -1;
+    if (m_cell == 3) { lay->tc_sh = ACT_TZ_SH; lay->tc_k = ACT_TZ_K; }
+    for (int sh = 4; sh >= 0 && lay->tc_sh < 0; --sh)
+        for (int k = 8; k <= 12 && lay->tc_sh < 0; ++k)
+            if (build_lines(f[2], lay->tc_lo, lay->tc_hi, sh, k, tc)) { lay->tc_sh = sh; lay->tc_k = k; }
+    if (lay->tc_sh < 0) return true;
+    const uint32_t tz_off = pad16(sig.size() * 4), tc_off = m_cell == 3 ? tz_off : tz_off + pad16(tz.size() * 4);
+    const uint32_t bytes = tz_off + pad16(tz.size() * 4) + pad16(tc.size() * 4);
+    lay->sig_at = 4u * (32768u >> ACT_SIG_SH);
+    lay->tz_at = tz_off - 4u * (uint32_t)(lay->tz_lo >> ACT_TZ_SH);
+    lay->tc_at = tc_off - 4u * (uint32_t)(lay->tc_lo >> lay->tc_sh);
+    std::vector<uint8_t> blob(bytes, 0);
+    memcpy(blob.data(), sig.data(), sig.size() * 4);
+    memcpy(blob.data() + tz_off, tz.data(), tz.size() * 4);
+    if (m_cell != 3) memcpy(blob.data() + tc_off, tc.data(), tc.size() * 4);
+    uint8_t *d = nullptr;
+    if (cudaMalloc(&d, bytes) != cudaSuccess) return false;
+    if (cudaMemcpy(d, blob.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(d); return false; }
+    *blob_dev = d;
+    lay->bytes = bytes;
     return true;
 }
 

@@ -108,4 +108,53 @@ __device__ __forceinline__ int32_t tab_tanh_cell(const ActTabs &t, int32_t x)
 // false only on a CUDA error.
 bool act_tables_build(int m_cell, size_t max_bytes, uint8_t **blob_dev, ActTabLayout *lay);
 
+// ---- piecewise-linear form, for the wavefront kernels ----------------------------------------------------------------
+//
+// The same memoised values over the signed domain, one 32-bit entry e per 2^sh consecutive inputs:
+//   f(x) = (e + ((e mod 2^10) << k) * (x mod 2^sh)) >> 16,   e the entry of x >> sh
+// The slope sits in the low bits of the entry, which the value never sees.  Every entry is searched for and checked against
+// all of its inputs when the tables are built, so the result is the definition's value for every int16.  Half the memory of
+// the packed form and no sign cases: 8 instructions per sigmoid, 10 per tanh.  Sigmoid: sh = 4, k = 8 (16 KB); the z gate's
+// tanh: sh = 3, k = 10; the cell's: the longest segments that its own Q_{m.15-m} allows.  Outside [lo, hi] tanh is constant.
+constexpr int ACT_SIG_SH = 4, ACT_SIG_K = 8, ACT_TZ_SH = 3, ACT_TZ_K = 10;
+
+struct ActLineLayout {
+    uint32_t bytes;              // whole blob, a multiple of 16; 0: no tables
+    uint32_t sig_at, tz_at, tc_at;      // byte offsets of the entries of x = 0
+    int32_t tz_lo, tz_hi, tc_lo, tc_hi, tc_sh, tc_k;
+};
+
+struct ActLines {
+    uint32_t sig, tz, tc;        // shared-memory addresses of the entries of x = 0
+    int32_t tz_lo, tz_hi, tc_lo, tc_hi, tc_sh, tc_k;
+};
+
+__device__ __forceinline__ ActLines make_act_lines(uint32_t blob_smem_addr, const ActLineLayout &l)
+{
+    return ActLines{blob_smem_addr + l.sig_at, blob_smem_addr + l.tz_at, blob_smem_addr + l.tc_at, l.tz_lo, l.tz_hi, l.tc_lo, l.tc_hi, l.tc_sh, l.tc_k};
+}
+
+__host__ __device__ __forceinline__ int32_t act_line_value(int32_t e, int32_t x, int sh, int k)
+{
+    return (e + (((e & 1023) * (x & ((1 << sh) - 1))) << k)) >> 16;
+}
+__device__ __forceinline__ int32_t line_sigmoid(const ActLines &t, int32_t x)
+{
+    return act_line_value((int32_t)lds_u32(t.sig + (uint32_t)((x >> ACT_SIG_SH) << 2)), x, ACT_SIG_SH, ACT_SIG_K);
+}
+__device__ __forceinline__ int32_t line_tanh_gate(const ActLines &t, int32_t x)
+{
+    x = x < t.tz_lo ? t.tz_lo : (x > t.tz_hi ? t.tz_hi : x);
+    return act_line_value((int32_t)lds_u32(t.tz + (uint32_t)((x >> ACT_TZ_SH) << 2)), x, ACT_TZ_SH, ACT_TZ_K);
+}
+__device__ __forceinline__ int32_t line_tanh_cell(const ActLines &t, int32_t x)
+{
+    x = x < t.tc_lo ? t.tc_lo : (x > t.tc_hi ? t.tc_hi : x);
+    return act_line_value((int32_t)lds_u32(t.tc + (uint32_t)((x >> t.tc_sh) << 2)), x, t.tc_sh, t.tc_k);
+}
+
+// Builds the blob for a cell format; *blob_dev = nullptr and lay->bytes = 0 when some input has no entry that yields its value
+// (the caller then evaluates the definition); false only on a CUDA error.
+bool act_lines_build(int m_cell, uint8_t **blob_dev, ActLineLayout *lay);
+
 }  // namespace ql

@@ -35,8 +35,8 @@ struct WaveLayer {
     const int16_t *P, *L;
     int x_left[4], h_left[4];      // left shift before the rescale of the input / recurrent term (0 for scales below 1)
     FastScale f_x[4], f_h[4], f_c[4], f_ln[4], f_m, f_proj;      // by gate slot
-    float ln_limit;                // layer-norm quotients below this keep q' L + b inside an int32
-    DivMagic div_c;
+    double inv_c;                  // (1 + 2^-46) / C
+    uint32_t sigma_min;            // layer norm: from this sigma on every quotient is below 2^16 and q' L + b inside an int32
     int8_t *in_img;                // [T][units][kb_i][ra][128] input activations
     int8_t *out_img;               // [T + 1][units][kb_h][ra][128]: slot t + 1 holds h^t
     int8_t *m_img;                 // [units][kb_c][ra][128]
@@ -45,7 +45,7 @@ struct WaveLayer {
     int below;                     // blocks of the layer below, 0: none
     long long h_off, c_off;        // of this layer in the caller's state, in units of one batch row
     const uint8_t *tab;
-    ActTabLayout tab_lay;
+    ActLineLayout tab_lay;
 };
 
 struct WaveCall {
@@ -146,61 +146,87 @@ __device__ __forceinline__ uint32_t wv_img_off(int row, int col, int ra)
 
 // ---- layer norm and nonlinearities -----------------------------------------------------------------------------------------------
 
-struct WvLnRow { int32_t mean; uint32_t sigma; float inv1024, off; };      // see ln_quotient_core in qmath.cuh
+// Layer-norm constants of one (row, gate).  The quotient q' = round(2^10 (2^10 q - mean) / sigma) (ties away from zero) is one
+// fp64 multiply-add: the product of the exact 2^10 q - mean with inv = 2^10 / sigma (1 + 2^-48) is off by a relative 2^-47 at
+// most, always outwards - ties, |q'| >= 1/2, move by more than inv's rounding errors (2^-51) can take back, and other quotients
+// below 2^16 stay on their side, since they are 1 / (2 sigma) >= 2^-27 away from a tie.  The added 1.5 * 2^52 leaves the
+// rounded quotient in the low word.  (An fp32 estimate with an exact remainder test took three times the instructions.)
+struct alignas(16) WvLnRow {
+    double inv;
+    uint32_t off;                  // 2^31 - mean
+    uint32_t sigma;                // top bit: quotients of this row may leave the fast range
+};
+constexpr uint32_t WV_LN_SLOW = 0x80000000u;
 
-__device__ __forceinline__ int4 wv_make_ln(long long sum, long long sq, const DivMagic &div)
+// Statistics as ln_stats_fast (qmath.cuh), the divisions by n as fp64 multiplications by inv_n = (1 + 2^-46) / n: sums below
+// 2^43 and n < 2^13 keep every quotient 2^-14 from the next tie or integer, and the bias moves it by less than 2^-16.
+__device__ __forceinline__ WvLnRow wv_make_ln(long long sum, long long sq, int n, double inv_n, uint32_t sigma_min)
 {
-    const LnRow r = make_ln_row(ln_stats_fast(sum, sq, div));
-    // sigma = 0: the quotient is 0; a divisor that no remainder reaches keeps the correction step from adding to it
-    const uint32_t sg = r.sigma ? r.sigma : 0xffffffffu;
-    const float off = (float)(r.sigma >> 1) * r.inv_sigma - 0.05f;
-    return make_int4(r.mean, (int)sg, __float_as_int(1024.0f * r.inv_sigma), __float_as_int(off));
+    const int32_t mean = __double2loint(__fma_rn(1024.0 * (double)(int32_t)sum, inv_n, 6755399441055744.0));
+    // round(sq 2^20 / n) = floor(sq / n) 2^20 + floor(((sq mod n) 2^20 + n / 2) / n)
+    const uint32_t q1 = (uint32_t)__double2loint(__fma_rd((double)sq, inv_n, 4503599627370496.0));
+    const uint32_t r1 = (uint32_t)sq - q1 * (uint32_t)n;
+    const uint32_t m2 = (uint32_t)__double2loint(__fma_rd((double)(((uint64_t)r1 << 20) + (uint64_t)(n >> 1)), inv_n, 4503599627370496.0));
+    long long var = (long long)(((uint64_t)q1 << 20) + m2) - (long long)mean * mean;
+    if (var < 0) var = 0;
+    // integer root: fp32 estimate (within 4), one Newton step in fp64 (within 2^-18), exact correction
+    const double v = (double)var;
+    const float s0 = __fsqrt_rn((float)var);
+    const double e = __fma_rn(-(double)s0, (double)s0, v);
+    const float es = s0 > 0.0f ? __fdividef((float)e, 2.0f * s0) : 0.0f;
+    uint32_t sigma = (uint32_t)((double)s0 + (double)es);
+    if ((long long)sigma * sigma > var) --sigma;
+    else if ((long long)(sigma + 1u) * (sigma + 1u) <= var) ++sigma;
+    WvLnRow r;
+    r.off = 0x80000000u - (uint32_t)mean;
+    r.inv = 0.0;                                               // sigma = 0: the quotient is 0
+    if (sigma) {
+        const double d = (double)sigma;
+        double x = (double)rcp_est((float)sigma);              // two Newton steps from 2^-22: 2^-43, then full precision
+        x = __fma_rn(x, __fma_rn(-d, x, 1.0), x);
+        x = __fma_rn(x, __fma_rn(-d, x, 1.0), x);
+        r.inv = x * (1024.0 * (1.0 + 0x1p-48));
+        if (sigma < sigma_min) sigma |= WV_LN_SLOW;
+    }
+    r.sigma = sigma;
+    return r;
 }
 
-// exact value for quotients beyond the fast range (a tiny sigma against a large deviation), out of line
-static __device__ __noinline__ int32_t wv_ln_slow(int32_t q, int4 row, int32_t Lw, int32_t b)
+// sat32(q' L + b) where q' and the product are known to be in range
+__device__ __forceinline__ int32_t wv_ln_fast(int32_t q, double inv, uint32_t off, int32_t Lw, int32_t b)
 {
-    const int32_t d = 1024 * q - row.x;
-    const uint32_t ad = (uint32_t)(d < 0 ? -d : d), sg = (uint32_t)row.y;
-    const uint64_t quo = sg == 0xffffffffu ? 0u : ((uint64_t)ad * 1024u + (sg >> 1)) / sg;
+    // 2^52 + 2^31 + 2^10 q - mean, whose low word is one integer multiply-add
+    const double d = __dadd_rn(__hiloint2double(0x43300000, (int)((uint32_t)(q * 1024) + off)), -4503601774854144.0);
+    return __double2loint(__fma_rn(d, inv, 6755399441055744.0)) * Lw + b;
+}
+
+// the same for any row, by division, out of line
+static __device__ __noinline__ int32_t wv_ln_slow(int32_t q, WvLnRow row, int32_t Lw, int32_t b)
+{
+    const int32_t d = 1024 * q - (int32_t)(0x80000000u - row.off);
+    const uint32_t ad = (uint32_t)(d < 0 ? -d : d), sg = row.sigma & ~WV_LN_SLOW;
+    const uint64_t quo = sg == 0u ? 0u : ((uint64_t)ad * 1024u + (sg >> 1)) / sg;
     const int64_t qp = d < 0 ? -(int64_t)quo : (int64_t)quo;
     return sat32_halves(qp * (int64_t)Lw + (int64_t)b);
 }
 
-// sat32(q' L + b) with q' = round(2^10 (2^10 q - mean) / sigma): fp32 estimate biased low by 0.05 (its error is below 0.02
-// for quotients under 2^16: four roundings of 2^-24 and 2^-25), one exact remainder test.  slow: the quotient is beyond
-// `limit` and the value is not usable.
-__device__ __forceinline__ int32_t wv_ln_fast(int32_t q, const int4 &row, int32_t Lw, int32_t b, float limit, bool &slow)
-{
-    const int32_t d = 1024 * q - row.x;
-    const uint32_t ad = (uint32_t)(d < 0 ? -d : d);
-    const float est = __fmaf_rn((float)ad, __int_as_float(row.z), __int_as_float(row.w));
-    slow = slow || !(est < limit);
-    uint32_t qe = __float2uint_rz(est);
-    const uint32_t sg = (uint32_t)row.y, half = sg == 0xffffffffu ? 0u : sg >> 1;
-    const uint32_t rem = (ad << 10) + half - qe * sg;
-    qe += rem >= sg ? 1u : 0u;
-    const int32_t qp = d < 0 ? -(int32_t)qe : (int32_t)qe;
-    return qp * Lw + b;
-}
-
 template <bool TAB>
-__device__ __forceinline__ int32_t wv_sigmoid(const ActTabs &at, int32_t x)
+__device__ __forceinline__ int32_t wv_sigmoid(const ActLines &at, int32_t x)
 {
-    if constexpr (TAB) return tab_sigmoid(at, x);
+    if constexpr (TAB) return line_sigmoid(at, x);
     else return sigmoid_q_fast(x, 3);
 }
 template <bool TAB>
-__device__ __forceinline__ int32_t wv_tanh(const ActTabs &at, int32_t x)
+__device__ __forceinline__ int32_t wv_tanh(const ActLines &at, int32_t x)
 {
-    if constexpr (TAB) return tab_tanh_gate(at, x);
+    if constexpr (TAB) return line_tanh_gate(at, x);
     else return tanh_q_fast(x, 3);
 }
 template <bool TAB>
-__device__ __forceinline__ int32_t wv_hidden(const WaveLayer &L, const ActTabs &at, int32_t o, int32_t c_new)
+__device__ __forceinline__ int32_t wv_hidden(const WaveLayer &L, const ActLines &at, int32_t o, int32_t c_new)
 {
     int32_t tc;
-    if constexpr (TAB) tc = tab_tanh_cell(at, c_new);
+    if constexpr (TAB) tc = line_tanh_cell(at, c_new);
     else tc = tanh_q_fast(c_new, L.m_bits);
     return sat8(fast_rescale(o * tc, L.f_m) + L.zp_m);                     // Section 3.2.7
 }

@@ -62,7 +62,7 @@ struct WaveSmem {
     int16_t *L, *P;                // [ppc][8]
     int32_t *bp;                   // [opc]
     uint32_t *st;                  // [4 slots][3][128] layer-norm sums of the block: sum, low 20 bits and rest of the squares
-    int4 *ln;                      // [4 slots][128] mean, sigma, 1024 / sigma, estimate's offset
+    WvLnRow *ln;                   // [4 slots][128]
     uint8_t *tab;
 };
 
@@ -213,27 +213,42 @@ __device__ __forceinline__ void wv_proj_tile(const WaveCall &k, const WaveLayer 
 
 // ---- elementwise phase -----------------------------------------------------------------------------------------------
 
+// Layer-norm constants of a thread's row in registers: those that the fast form needs.
+struct WvLnRegs { double inv[4]; uint32_t off[4]; bool slow; };
+
+template <int G>
+__device__ __forceinline__ void wv_load_ln(const WaveSmem &s, int row, unsigned mask, WvLnRegs &r)
+{
+    uint32_t any = 0;
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+        if ((mask >> g) & 1u) {
+            const WvLnRow v = s.ln[g * 128 + row];
+            r.inv[g] = v.inv; r.off[g] = v.off; any |= v.sigma;
+        }
+    r.slow = (any & WV_LN_SLOW) != 0u;
+}
+
 // The gate values of a pair after layer norm (slots in `mask`), in place.
 template <int G>
-__device__ __forceinline__ void wv_ln_pair(const WaveLayer &L, const WaveSmem &s, const int4 (&row)[4], int pr, unsigned mask, int32_t (&a)[4][2])
+__device__ __forceinline__ void wv_ln_pair(const WaveLayer &L, const WaveSmem &s, const WvLnRegs &r, int row, int pr, unsigned mask, int32_t (&a)[4][2])
 {
     const uint4 lw = *reinterpret_cast<const uint4 *>(s.L + pr * 8);
     const uint32_t lws[4] = {lw.x, lw.y, lw.z, lw.w};
     const int4 b0 = *reinterpret_cast<const int4 *>(s.bln + pr * 8), b1 = *reinterpret_cast<const int4 *>(s.bln + pr * 8 + 4);
     const int32_t bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
     int32_t v[4][2];
-    bool slow = false;
 #pragma unroll
     for (int g = 0; g < G; ++g)
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if ((mask >> g) & 1u) v[g][k] = wv_ln_fast(a[g][k], row[g], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k], L.ln_limit, slow);
-    if (slow) {
+            if ((mask >> g) & 1u) v[g][k] = wv_ln_fast(a[g][k], r.inv[g], r.off[g], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k]);
+    if (r.slow) {
 #pragma unroll
         for (int g = 0; g < G; ++g)
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                if ((mask >> g) & 1u) v[g][k] = wv_ln_slow(a[g][k], row[g], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k]);
+                if ((mask >> g) & 1u) v[g][k] = wv_ln_slow(a[g][k], s.ln[g * 128 + row], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k]);
     }
 #pragma unroll
     for (int g = 0; g < G; ++g)
@@ -294,13 +309,13 @@ __device__ __forceinline__ void wv_pull_stats(const WaveLayer &L, const WaveSmem
         const int g = i / rows, row = i - g * rows;
         if (!((mask >> g) & 1u)) continue;
         const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(totals + (size_t)(row * 4 + g) * 2));
-        s.ln[g * 128 + row] = wv_make_ln(v.x, v.y, L.div_c);
+        s.ln[g * 128 + row] = wv_make_ln(v.x, v.y, L.C, L.inv_c, L.sigma_min);
     }
 }
 // Everything between the gate sums and m for one unit.  Tasks are (pair, row) with the row fastest, so that the gate
 // buffers are read as contiguous runs; a thread keeps one row, whose layer-norm constants stay in registers.
 template <int G, bool LN, bool PEEP, bool TAB>
-__device__ __forceinline__ bool wv_elementwise(const WaveCall &k, const WaveLayer &L, const WaveSmem &s, const WaveRole &r, const ActTabs &at, int u,
+__device__ __forceinline__ bool wv_elementwise(const WaveCall &k, const WaveLayer &L, const WaveSmem &s, const WaveRole &r, const ActLines &at, int u,
                                                int t, bool last_layer, WvPoint &pt, int tid)
 {
     constexpr int SI = 0, SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
@@ -326,11 +341,8 @@ __device__ __forceinline__ bool wv_elementwise(const WaveCall &k, const WaveLaye
     int8_t *img = (L.flags & F_PROJECTION) ? L.m_img + (size_t)gu * L.kb_c * k.ra * 128
                                            : L.out_img + ((size_t)(t + 1) * k.nu + gu) * L.kb_h * k.ra * 128;
     const bool fin = t == k.T - 1;
-    int4 lr[4] = {};
-    if (LN && p0 < per) {
-#pragma unroll
-        for (int g = 0; g < G; ++g) lr[g] = s.ln[g * 128 + row];
-    }
+    WvLnRegs lr = {};
+    if (LN && p0 < per) wv_load_ln<G>(s, row, PEEP ? ALL & ~(1u << SO) : ALL, lr);
     if (p0 < per) {
 #pragma unroll 1
         for (int pr = p0; pr < r.pairs; pr += per) {
@@ -340,7 +352,7 @@ __device__ __forceinline__ bool wv_elementwise(const WaveCall &k, const WaveLaye
             int32_t a[4][2];
 #pragma unroll
             for (int g = 0; g < G; ++g) { a[g][0] = wv_lo(gw[g]); a[g][1] = wv_hi(gw[g]); }
-            if (LN) wv_ln_pair<G>(L, s, lr, pr, PEEP ? ALL & ~(1u << SO) : ALL, a);
+            if (LN) wv_ln_pair<G>(L, s, lr, row, pr, PEEP ? ALL & ~(1u << SO) : ALL, a);
             const int32_t c_old[2] = {wv_lo(cw), wv_hi(cw)};
             int32_t c_new[2];
 #pragma unroll
@@ -389,14 +401,14 @@ __device__ __forceinline__ bool wv_elementwise(const WaveCall &k, const WaveLaye
         wv_pull_stats<G>(L, s, tot, rows, 1u << SO, tid);
         wv_epi_sync();
         if (p0 < per) {
-            lr[SO] = s.ln[SO * 128 + row];
+            wv_load_ln<G>(s, row, 1u << SO, lr);
 #pragma unroll 1
             for (int pr = p0; pr < r.pairs; pr += per) {
                 const uint32_t gw = reinterpret_cast<const uint32_t *>(&g_s[pr * rows + row])[SO];
                 const uint32_t cw = c_s[pr * rows + row];
                 int32_t a[4][2] = {};
                 a[SO][0] = wv_lo(gw); a[SO][1] = wv_hi(gw);
-                wv_ln_pair<G>(L, s, lr, pr, 1u << SO, a);
+                wv_ln_pair<G>(L, s, lr, row, pr, 1u << SO, a);
                 const int32_t m0 = wv_hidden<TAB>(L, at, wv_sigmoid<TAB>(at, a[SO][0]), wv_lo(cw));
                 const int32_t m1 = wv_hidden<TAB>(L, at, wv_sigmoid<TAB>(at, a[SO][1]), wv_hi(cw));
                 wv_store_m(k, L, img, row, r.u0 + 2 * pr, b, t, m0, m1, last_layer);
@@ -490,7 +502,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
         s.P = (int16_t *)p;   p += (size_t)k.max_ppc * 16;
         s.bp = (int32_t *)p;
         s.st = (uint32_t *)(smem + lay.st);
-        s.ln = (int4 *)(smem + lay.ln);
+        s.ln = (WvLnRow *)(smem + lay.ln);
         s.tab = smem + lay.tab;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = blockIdx.x;
@@ -681,7 +693,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0;
         const int quarter = warp & 3, qpr = 4 / k.nrep;        // quarters of the lanes that hold one copy of the rows
         const int row = (quarter % qpr) * 32 + lane, part = ((warp - WV_EPI_WARP0) >> 2) + 4 * (quarter / qpr), nparts = 4 * k.nrep;
-        const ActTabs at = make_act_tabs(ptx::smem_u32(s.tab), L.tab_lay);
+        const ActLines at = make_act_lines(ptx::smem_u32(s.tab), L.tab_lay);
         WvPoint pt{abort_flag, &ctl->exit_at, 0};
         if (TAB) wv_wait(&ctl->tab_full, 0, abort_flag);
         int job = 0;
@@ -975,7 +987,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
     int8_t *prev_img = nullptr;
     int prev_n[2] = {0, 0};
     s->tabs = true;
-    std::vector<std::pair<int, std::pair<uint8_t *, ActTabLayout>>> blobs;
+    std::vector<std::pair<int, std::pair<uint8_t *, ActLineLayout>>> blobs;
     for (int l = 0; l < n; ++l) {
         const LayerParams &p = *lp[l];
         const bool proj = p.flags & F_PROJECTION;
@@ -994,11 +1006,11 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
             L.f_c[g] = make_fast_scale(p.eff_c[g]); L.f_ln[g] = make_fast_scale(p.eff_ln[g]);
         }
         L.f_m = make_fast_scale(p.eff_m); L.f_proj = make_fast_scale(p.eff_proj);
-        L.div_c = make_div_magic((uint32_t)p.C);
+        L.inv_c = (1.0 + 0x1p-46) / p.C;
         {
-            // q' L + b stays inside an int32 for |q'| <= limit + 1
-            const long long room = (0x7fffffffll - p.max_bln) / (p.max_L > 0 ? p.max_L : 1) - 2;
-            L.ln_limit = room < 0 ? 0.0f : (room > 65535 ? 65535.0f : (float)room);
+            // q' L + b stays inside an int32 for |q'| <= room, and |2^10 (2^10 q - mean)| <= 2^36
+            const long long room = std::min(65535ll, (0x7fffffffll - p.max_bln) / (p.max_L > 0 ? p.max_L : 1)) - 1;
+            L.sigma_min = room < 64 ? 0x7fffffffu : (uint32_t)((1ll << 36) / room + 1);
         }
         L.in_img = l > 0 ? prev_img : (int8_t *)wv_alloc(s, (size_t)max_T * rows_alloc * L.kb_i * 128);
         L.out_img = (int8_t *)wv_alloc(s, ((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
@@ -1009,16 +1021,14 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
         L.h_off = h_off; L.c_off = c_off;
         h_off += p.O; c_off += p.C;
         uint8_t *blob = nullptr;
-        ActTabLayout lay = {0, 0, 0, 0, 0, 0, 0};
-        if (s->plan[0].ok) {
-            bool have = false;
-            for (auto &b : blobs)
-                if (b.first == p.m_bits) { blob = b.second.first; lay = b.second.second; have = true; }
-            if (!have) {
-                if (!act_tables_build(p.m_bits, 92 * 1024, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
-                if (blob) s->owned.push_back(blob);
-                blobs.push_back({p.m_bits, {blob, lay}});
-            }
+        ActLineLayout lay = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+        bool have = false;
+        for (auto &b : blobs)
+            if (b.first == p.m_bits) { blob = b.second.first; lay = b.second.second; have = true; }
+        if (!have) {
+            if (!act_lines_build(p.m_bits, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
+            if (blob) s->owned.push_back(blob);
+            blobs.push_back({p.m_bits, {blob, lay}});
         }
         if (!blob) s->tabs = false;
         L.tab = blob; L.tab_lay = lay;
@@ -1088,7 +1098,8 @@ static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool table
     k.max_kb_i = s->max_kb_i; k.max_kb_h = s->max_kb_h; k.max_kb_c = s->max_kb_c;
     const size_t room = (size_t)s->max_smem;
     if (mode == 1) {
-        if (rows > WV_SMALL_ROWS) return false;
+        if (rows > WV_SMALL_ROWS || !tables || !s->tabs) return false;
+        k.max_tab = s->max_tab;
         for (const WaveLayer &L : pl.layer)
             if ((2 * L.nt + L.ntp) * k.ra > 512) return false;
         k.nb = 8;
@@ -1102,7 +1113,7 @@ static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool table
     auto total = [&](int na, int nb, bool tab, bool in_smem) {
         return wv_layout(na, nb, pl.b_slot, pl.max_ppc, pl.max_opc, tab ? s->max_tab : 0, in_smem ? gates : 0).total;
     };
-    k.tab = tables && s->tabs && rows * k.units >= 24 && total(2, 2, true, false) <= room;
+    k.tab = tables && s->tabs && total(2, 2, true, false) <= room;
     k.gx_s = total(3, 3, k.tab, true) <= room;
     k.na = 2; k.nb = 2;
     while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;

@@ -25,13 +25,13 @@ constexpr int WS_ROWS = 32;
 struct WsCtl {
     uint64_t w_full[WS_SLOTS], w_empty[WS_SLOTS];
     uint64_t op_full[3], op_empty[3];          // operands x, h, m
-    uint64_t gate_full[WS_MAX_TILES], acc_empty, p_full, p_empty;
+    uint64_t gate_full[WS_MAX_TILES], acc_empty, p_full, p_empty, tab_full;
     uint32_t tmem_base;
     int abort_flag, exit_at;
 };
 
-// [weight ring][x][h][m][control][constants][statistics][gates][cell states]
-struct WsLayout { size_t act[3], ctl, consts, st, ln, gates, c, total; };
+// [weight ring][x][h][m][control][constants][statistics][tables][gates][cell states]
+struct WsLayout { size_t act[3], ctl, consts, st, ln, tab, gates, c, total; };
 
 __host__ __device__ inline WsLayout ws_layout(const WaveCall &k, int ns, int rows, bool peep)
 {
@@ -43,7 +43,8 @@ __host__ __device__ inline WsLayout ws_layout(const WaveCall &k, int ns, int row
     l.consts = l.ctl + wv_up(sizeof(WsCtl), 16);
     l.st = l.consts + wv_up((size_t)k.max_cpc * 4 * (3 * 4 + 2 * 2) + (size_t)k.max_opc * 4, 16);
     l.ln = l.st + 12 * WS_ROWS * 4;
-    l.gates = l.ln + 4 * WS_ROWS * 16;
+    l.tab = l.ln + 4 * WS_ROWS * 16;
+    l.gates = l.tab + wv_up((size_t)k.max_tab, 16);
     l.c = l.gates + wv_up((size_t)(peep ? 5 : 4) * rows * k.max_cpc * 2, 16);
     l.total = l.c + wv_up((size_t)rows * k.max_cpc * 2, 16);
     // an MMA reads 128 rows of 128 bytes from where its k-block starts, whatever the tile holds
@@ -57,7 +58,7 @@ struct WsSmem {
     int16_t *L, *P;                // [4][cpc]
     int32_t *bp;                   // [opc]
     uint32_t *st;                  // [4][3][32] layer-norm sums: sum, low 20 bits and rest of the squares
-    int4 *ln;                      // [4][32]
+    WvLnRow *ln;                   // [4][32]
     int16_t *g;                    // [slot][row][cpc] gate sums; slot 4: X of the output gate (peephole)
     int16_t *c;                    // [row][cpc]
 };
@@ -68,10 +69,10 @@ struct WsRole {
     int row0, rows, gu;
 };
 
-// Gate sums of one tile, one lane per cell, for the gate `g` of this warp.
+// Gate sums of eight rows from r0 of one tile, one lane per cell, for the gate `g` of this warp.
 template <int G, bool LN, bool PEEP>
 __device__ __forceinline__ void ws_gate_tile(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, uint32_t tx, uint32_t th,
-                                             int tile, int g, int lane)
+                                             int tile, int g, int r0, int lane)
 {
     constexpr int SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
     const int cpc = L.cpc, ul = tile * L.ct + lane, rows = r.rows;
@@ -81,47 +82,47 @@ __device__ __forceinline__ void ws_gate_tile(const WaveCall &k, const WaveLayer 
     const FastScale fx = L.f_x[g], fh = L.f_h[g];
     const int xl = L.x_left[g], hl = L.h_left[g];
     const bool is_o = PEEP && g == SO;                         // warp-uniform
-    uint32_t my_sum = 0, my_lo = 0, my_hi = 0;                 // lane b keeps the sums of row b
-#pragma unroll 1
-    for (int r0 = 0; r0 < rows; r0 += 8) {
-        uint32_t x[8], h[8];
-        __syncwarp();
-        ptx::tmem_ld_32x8(tx + (uint32_t)r0, x);
-        ptx::tmem_ld_32x8(th + (uint32_t)r0, h);
-        ptx::tmem_ld_wait();
-        int32_t v[8];
+    uint32_t x[8], h[8];
+    __syncwarp();
+    ptx::tmem_ld_32x8(tx + (uint32_t)r0, x);
+    ptx::tmem_ld_32x8(th + (uint32_t)r0, h);
+    ptx::tmem_ld_wait();
+    int32_t v[8];
+    const int ne = rows - r0 < 8 ? rows - r0 : 8;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        if (e >= ne) break;
+        const int32_t X = sat16(fast_rescale(((int32_t)x[e] + bx) << xl, fx));
+        const int32_t H = sat16(fast_rescale(((int32_t)h[e] + bh) << hl, fh));
+        v[e] = X + H;
+        if (PEEP) {
+            if (is_o) {
+                if (in) s.g[(4 * rows + r0 + e) * cpc + ul] = (int16_t)X;
+                v[e] = H;                                  // X + H + P c^t once c^t exists
+            } else if (g != SZ) {
+                const int32_t c_old = in ? s.c[(r0 + e) * cpc + ul] : 0;
+                v[e] += sat16(fast_rescale(P * c_old, L.f_c[g]));
+            }
+        }
+        v[e] = in ? sat16(v[e]) : 0;
+        if (in) s.g[(g * rows + r0 + e) * cpc + ul] = (int16_t)v[e];
+    }
+    if (LN && !is_o) {
+        uint32_t my_sum = 0, my_lo = 0, my_hi = 0;             // lane e keeps the sums of row r0 + e
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const int32_t X = sat16(fast_rescale(((int32_t)x[e] + bx) << xl, fx));
-            const int32_t H = sat16(fast_rescale(((int32_t)h[e] + bh) << hl, fh));
-            v[e] = X + H;
-            if (PEEP) {
-                if (is_o) {
-                    if (in && r0 + e < rows) s.g[(4 * rows + r0 + e) * cpc + ul] = (int16_t)X;
-                    v[e] = H;                                  // X + H + P c^t once c^t exists
-                } else if (g != SZ) {
-                    const int32_t c_old = (in && r0 + e < rows) ? s.c[(r0 + e) * cpc + ul] : 0;
-                    v[e] += sat16(fast_rescale(P * c_old, L.f_c[g]));
-                }
-            }
-            v[e] = in ? sat16(v[e]) : 0;
-            if (in && r0 + e < rows) s.g[(g * rows + r0 + e) * cpc + ul] = (int16_t)v[e];
+            if (e >= ne) break;
+            const uint32_t sq = (uint32_t)(v[e] * v[e]);
+            const uint32_t a = (uint32_t)__reduce_add_sync(0xffffffffu, v[e]);
+            const uint32_t lo = __reduce_add_sync(0xffffffffu, sq & 0xfffffu), hi = __reduce_add_sync(0xffffffffu, sq >> 20);
+            if (lane == e) { my_sum = a; my_lo = lo; my_hi = hi; }
         }
-        if (LN && !is_o) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint32_t sq = (uint32_t)(v[e] * v[e]);
-                const uint32_t a = (uint32_t)__reduce_add_sync(0xffffffffu, v[e]);
-                const uint32_t lo = __reduce_add_sync(0xffffffffu, sq & 0xfffffu), hi = __reduce_add_sync(0xffffffffu, sq >> 20);
-                if (lane == r0 + e) { my_sum = a; my_lo = lo; my_hi = hi; }
-            }
+        if (lane < ne) {
+            uint32_t *st = s.st + g * 3 * WS_ROWS + r0 + lane;
+            atomicAdd(st, my_sum);
+            atomicAdd(st + WS_ROWS, my_lo);
+            atomicAdd(st + 2 * WS_ROWS, my_hi);
         }
-    }
-    if (LN && !is_o && lane < rows) {
-        uint32_t *st = s.st + g * 3 * WS_ROWS + lane;
-        atomicAdd(st, my_sum);
-        atomicAdd(st + WS_ROWS, my_lo);
-        atomicAdd(st + 2 * WS_ROWS, my_hi);
     }
 }
 
@@ -145,7 +146,7 @@ __device__ __forceinline__ void ws_pull_stats(const WaveLayer &L, const WsSmem &
     const int g = tid >> 5, row = tid & 31;
     if (g < G && row < rows && ((mask >> g) & 1u)) {
         const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(totals + (size_t)(row * 4 + g) * 2));
-        s.ln[g * WS_ROWS + row] = wv_make_ln(v.x, v.y, L.div_c);
+        s.ln[g * WS_ROWS + row] = wv_make_ln(v.x, v.y, L.C, L.inv_c, L.sigma_min);
     }
 }
 
@@ -154,11 +155,15 @@ template <int G>
 __device__ __forceinline__ void ws_ln_cell(const WaveLayer &L, const WsSmem &s, int row, int ul, unsigned mask, int32_t (&a)[4])
 {
     int32_t v[4];
-    bool slow = false;
+    uint32_t any = 0;
 #pragma unroll
     for (int g = 0; g < G; ++g)
-        if ((mask >> g) & 1u) v[g] = wv_ln_fast(a[g], s.ln[g * WS_ROWS + row], s.L[g * L.cpc + ul], s.bln[g * L.cpc + ul], L.ln_limit, slow);
-    if (slow) {
+        if ((mask >> g) & 1u) {
+            const WvLnRow r = s.ln[g * WS_ROWS + row];
+            any |= r.sigma;
+            v[g] = wv_ln_fast(a[g], r.inv, r.off, s.L[g * L.cpc + ul], s.bln[g * L.cpc + ul]);
+        }
+    if (any & WV_LN_SLOW) {
 #pragma unroll
         for (int g = 0; g < G; ++g)
             if ((mask >> g) & 1u) v[g] = wv_ln_slow(a[g], s.ln[g * WS_ROWS + row], s.L[g * L.cpc + ul], s.bln[g * L.cpc + ul]);
@@ -179,8 +184,8 @@ __device__ __forceinline__ void ws_store_m(const WaveCall &k, const WaveLayer &L
 
 // Everything between the gate sums and m, one cell per task, consecutive threads on consecutive cells of a row.
 template <int G, bool LN, bool PEEP>
-__device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, int t, bool last_layer, WvPoint &pt,
-                                               int tid)
+__device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, const ActLines &at, int t, bool last_layer,
+                                               WvPoint &pt, int tid)
 {
     constexpr int SI = 0, SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
     constexpr unsigned ALL = (1u << G) - 1u;
@@ -200,16 +205,17 @@ __device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLaye
     int8_t *img = (L.flags & F_PROJECTION) ? L.m_img + (size_t)r.gu * L.kb_c * k.ra * 128
                                            : L.out_img + ((size_t)(t + 1) * k.nu + r.gu) * L.kb_h * k.ra * 128;
     const bool fin = t == k.T - 1;
+    const float inv_cells = 1.0f / (float)cells;               // (i + 1/2) / cells is 2^-9 or more away from an integer
 #pragma unroll 1
     for (int i = tid; i < n_tasks; i += WV_EPI) {
-        const int row = i / cells, ul = i - row * cells, u = r.u0 + ul, b = r.row0 + row;
+        const int row = (int)(((float)i + 0.5f) * inv_cells), ul = i - row * cells, u = r.u0 + ul, b = r.row0 + row;
         int32_t a[4];
 #pragma unroll
         for (int g = 0; g < G; ++g) a[g] = s.g[(g * rows + row) * cpc + ul];
         if (LN) ws_ln_cell<G>(L, s, row, ul, PEEP ? ALL & ~(1u << SO) : ALL, a);
-        const int32_t f = sigmoid_q_fast(a[SF], 3), z = tanh_q_fast(a[SZ], 3);
+        const int32_t f = line_sigmoid(at, a[SF]), z = line_tanh_gate(at, a[SZ]);
         int32_t ig;
-        if (G == 4) ig = sigmoid_q_fast(a[SI], 3);
+        if (G == 4) ig = line_sigmoid(at, a[SI]);
         else { ig = 32768 - f; if (ig > 32767) ig = 32767; }               // coupled input gate, Section 3.2.9
         const int32_t c_new = cell_update_fast(ig, z, f, s.c[row * cpc + ul], L.m_bits);
         s.c[row * cpc + ul] = (int16_t)c_new;
@@ -227,8 +233,7 @@ __device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLaye
                 continue;
             }
         }
-        const int32_t tc = tanh_q_fast(c_new, L.m_bits);
-        ws_store_m(k, L, img, row, u, b, t, sat8(fast_rescale(sigmoid_q_fast(ao, 3) * tc, L.f_m) + L.zp_m), last_layer);
+        ws_store_m(k, L, img, row, u, b, t, wv_hidden<true>(L, at, line_sigmoid(at, ao), c_new), last_layer);
     }
     if (LN && PEEP) {
         wv_epi_sync();
@@ -239,12 +244,11 @@ __device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLaye
         wv_epi_sync();
 #pragma unroll 1
         for (int i = tid; i < n_tasks; i += WV_EPI) {
-            const int row = i / cells, ul = i - row * cells;
+            const int row = (int)(((float)i + 0.5f) * inv_cells), ul = i - row * cells;
             int32_t a[4] = {0, 0, 0, 0};
             a[SO] = s.g[(SO * rows + row) * cpc + ul];
             ws_ln_cell<G>(L, s, row, ul, 1u << SO, a);
-            const int32_t tc = tanh_q_fast(s.c[row * cpc + ul], L.m_bits);
-            ws_store_m(k, L, img, row, r.u0 + ul, r.row0 + row, t, sat8(fast_rescale(sigmoid_q_fast(a[SO], 3) * tc, L.f_m) + L.zp_m), last_layer);
+            ws_store_m(k, L, img, row, r.u0 + ul, r.row0 + row, t, wv_hidden<true>(L, at, line_sigmoid(at, a[SO]), s.c[row * cpc + ul]), last_layer);
         }
     }
     return wv_publish(cnt + ((L.flags & F_PROJECTION) ? WC_M : WC_H) * WC_WORDS, true, pt, tid);
@@ -316,20 +320,23 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         s.L = (int16_t *)p;   p += q * 2;
         s.P = (int16_t *)p;
         s.st = (uint32_t *)(smem + lay.st);
-        s.ln = (int4 *)(smem + lay.ln);
+        s.ln = (WvLnRow *)(smem + lay.ln);
         s.g = (int16_t *)(smem + lay.gates);
         s.c = (int16_t *)(smem + lay.c);
     }
     if (threadIdx.x == 0) {
-        for (int i = 0; i < WS_SLOTS; ++i) { ptx::mbar_init(&ctl->w_full[i], 1); ptx::mbar_init(&ctl->w_empty[i], 1); }
-        for (int i = 0; i < 3; ++i) { ptx::mbar_init(&ctl->op_full[i], 1); ptx::mbar_init(&ctl->op_empty[i], 1); }
+        for (int i = 0; i < WS_SLOTS; ++i) { ptx::mbar_init(&ctl->w_full[i], 1); ptx::mbar_init(&ctl->w_empty[i], 2); }
+        for (int i = 0; i < 3; ++i) { ptx::mbar_init(&ctl->op_full[i], 1); ptx::mbar_init(&ctl->op_empty[i], 2); }
         for (int i = 0; i < WS_MAX_TILES; ++i) ptx::mbar_init(&ctl->gate_full[i], 1);
         ptx::mbar_init(&ctl->acc_empty, WV_EPI / 32);
-        ptx::mbar_init(&ctl->p_full, 1);
+        ptx::mbar_init(&ctl->p_full, 2);
         ptx::mbar_init(&ctl->p_empty, WV_EPI / 32);
+        ptx::mbar_init(&ctl->tab_full, 1);
         ctl->abort_flag = 0;
         ctl->exit_at = 0x7fffffff;
         ptx::fence_barrier_init();
+        ptx::mbar_arrive_expect_tx(&ctl->tab_full, L.tab_lay.bytes);
+        ptx::bulk_load_1d(smem + lay.tab, L.tab, L.tab_lay.bytes, &ctl->tab_full);
     }
     if (warp == 2) {
         ptx::tmem_alloc(&ctl->tmem_base, 512);
@@ -431,18 +438,23 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
             });
         }
         __syncwarp();
-    } else if (warp == 2) {
+    } else if (warp < WV_EPI_WARP0) {
         // ---------------- MMAs: weights x operand ----------------
+        // Two warps take the tiles in turn: the waits and loop overhead around a slot (about 300 cycles) pass under the
+        // other's MMAs.  Both watch every slot (a parity wait must not skip a round).  A gate tile's X and H have one issuer.
+        const int me = warp - 2;
         int slot = 0; uint32_t phase = 0;
         const uint64_t w_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem));
         const uint32_t idesc = ptx::idesc_i8(128, nr), b_step = (uint32_t)nr * 128u >> 4;
         // one tile of nkb k-blocks: kpc of them per chunk (kb_bytes apart), the chunks of a ring slot chunk_bytes apart
-        auto tile = [&](uint32_t d, int op, int nkb, int kpc, uint32_t kb_bytes, int n_chunks, uint32_t chunk_bytes) -> bool {
+        auto tile = [&](bool mine, uint32_t d, int op, int nkb, int kpc, uint32_t kb_bytes, int n_chunks, uint32_t chunk_bytes) -> bool {
             const uint64_t b_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + lay.act[op]));
             for (int kb0 = 0; kb0 < nkb; kb0 += kpc * n_chunks) {
                 if (!wv_wait_warp(&ctl->w_full[slot], phase, abort_flag)) return false;
                 ptx::tc_fence_after();
-                if (ptx::elect_one()) {
+                if (!mine) {
+                    if (lane == 0) ptx::mbar_arrive(&ctl->w_empty[slot]);
+                } else if (ptx::elect_one()) {
                     uint64_t ac = w_desc0 + (uint64_t)((uint32_t)slot * ((uint32_t)k.b_slot >> 4));
                     uint64_t bd = b_desc0 + (uint64_t)(b_step * (uint32_t)kb0);
                     int kb = kb0;
@@ -470,14 +482,14 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
             ptx::tc_fence_after();
             if (op == 2) {
                 for (int j = 0; j < ntp; ++j)
-                    if (!tile(tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.kpp, (uint32_t)L.opp * 128u, 1, 0u)) return false;
+                    if (!tile((j & 1) != me, tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.kpp, (uint32_t)L.opp * 128u, 1, 0u)) return false;
                 wv_commit(&ctl->p_full);
             } else {
                 for (int i = 0; i < nt; ++i) {
-                    if (!tile(tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u, WS_CHUNKS,
+                    if (!tile((i & 1) == me, tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u, WS_CHUNKS,
                               G * 4096u))
                         return false;
-                    if (op == 1) wv_commit(&ctl->gate_full[i]);      // (X of this step was issued before)
+                    if (op == 1 && (i & 1) == me) wv_commit(&ctl->gate_full[i]);      // (X of this step was issued before)
                 }
             }
             wv_commit(&ctl->op_empty[op]);
@@ -488,20 +500,31 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0, quarter = warp & 3, wq = (warp - WV_EPI_WARP0) >> 2;
         const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16);
         WvPoint pt{abort_flag, &ctl->exit_at, 0};
+        const ActLines at = make_act_lines(ptx::smem_u32(smem + lay.tab), L.tab_lay);
+        wv_wait(&ctl->tab_full, 0, abort_flag);
         bool stay = true;
         for (int t = 0; t < T && stay; ++t) {
             const uint32_t par = (uint32_t)t & 1u;
-            for (int i = wq; i < nt; i += 4) {
-                if (quarter >= G) break;
-                if (!__all_sync(0xffffffffu, wv_wait(&ctl->gate_full[i], par, abort_flag))) break;   // (on to the next meeting point)
-                ptx::tc_fence_after();
-                ws_gate_tile<G, LN, PEEP>(k, L, s, r, tq + (uint32_t)(i * nr), tq + col_h + (uint32_t)(i * nr), i, quarter, lane);
+            // pieces of (tile, eight rows), dealt to the four warps of a lane quarter
+            for (int i = 0, q = 0; i < nt && quarter < G; ++i) {
+                bool seen = false, ok = true;
+                for (int r0 = 0; r0 < r.rows && ok; r0 += 8, ++q) {
+                    if ((q & 3) != wq) continue;
+                    if (!seen) {
+                        ok = __all_sync(0xffffffffu, wv_wait(&ctl->gate_full[i], par, abort_flag));
+                        if (!ok) break;
+                        ptx::tc_fence_after();
+                        seen = true;
+                    }
+                    ws_gate_tile<G, LN, PEEP>(k, L, s, r, tq + (uint32_t)(i * nr), tq + col_h + (uint32_t)(i * nr), i, quarter, r0, lane);
+                }
+                if (!ok) break;                                // (on to the next meeting point)
             }
             ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&ctl->acc_empty);
             wv_epi_sync();
-            stay = ws_elementwise<G, LN, PEEP>(k, L, s, r, t, last_layer, pt, tid);
+            stay = ws_elementwise<G, LN, PEEP>(k, L, s, r, at, t, last_layer, pt, tid);
             if (!stay || !proj) continue;
             if (ntp > 0 && __all_sync(0xffffffffu, wv_wait(&ctl->p_full, par, abort_flag))) {
                 ptx::tc_fence_after();

@@ -45,6 +45,19 @@ def test_wave_configs(index, kw):
     check(make_workload(index, **kw))
 
 
+# gate sums so small that layer-norm quotients leave the fast range (2^4, 2^9 below the calibrated scale) or that whole rows
+# are zero (sigma = 0): the division out of line
+@pytest.mark.parametrize("B", [5, 70])
+@pytest.mark.parametrize("shift", [4, 9, 15])
+@pytest.mark.parametrize("peephole", [False, True])
+def test_wave_layernorm_of_small_deviations(shift, B, peephole):
+    w = random_layer_stack(840 + B, 3, 48, 112, 64, projection=True, layernorm=True, peephole=peephole, T=5, B=B)
+    for q in w.layers:
+        q.eff_x = [(m, s - shift) for m, s in q.eff_x]
+        q.eff_h = [(m, s - shift) for m, s in q.eff_h]
+    check(w)
+
+
 def test_wave_timeout_is_reported_and_the_handle_recovers():
     import paper_2101_05453_b200 as qlstm
     w = random_layer_stack(9, 3, 48, 112, 64, projection=True, layernorm=True, T=5, B=40)
