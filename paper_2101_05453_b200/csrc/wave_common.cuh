@@ -35,7 +35,7 @@ struct WaveLayer {
     const int16_t *P, *L;
     int x_left[4], h_left[4];      // left shift before the rescale of the input / recurrent term (0 for scales below 1)
     FastScale f_x[4], f_h[4], f_c[4], f_ln[4], f_m, f_proj;      // by gate slot
-    double inv_c;                  // (1 + 2^-46) / C
+    DivMagic div_c;
     uint32_t sigma_min;            // layer norm: from this sigma on every quotient is below 2^16 and q' L + b inside an int32
     int8_t *in_img;                // [T][units][kb_i][ra][128] input activations
     int8_t *out_img;               // [T + 1][units][kb_h][ra][128]: slot t + 1 holds h^t
@@ -146,64 +146,92 @@ __device__ __forceinline__ uint32_t wv_img_off(int row, int col, int ra)
 
 // ---- layer norm and nonlinearities -----------------------------------------------------------------------------------------------
 
-// Layer-norm constants of one (row, gate).  The quotient q' = round(2^10 (2^10 q - mean) / sigma) (ties away from zero) is one
-// fp64 multiply-add: the product of the exact 2^10 q - mean with inv = 2^10 / sigma (1 + 2^-48) is off by a relative 2^-47 at
-// most, always outwards - ties, |q'| >= 1/2, move by more than inv's rounding errors (2^-51) can take back, and other quotients
-// below 2^16 stay on their side, since they are 1 / (2 sigma) >= 2^-27 away from a tie.  The added 1.5 * 2^52 leaves the
-// rounded quotient in the low word.  (An fp32 estimate with an exact remainder test took three times the instructions.)
+// Layer-norm constants of one (row, gate).  The quotient q' = round(2^10 (2^10 q - mean) / sigma), ties away from zero, is
+// floor(d M + 1/2) with d = 2^10 q - mean and M the next multiple of 2^-63 above 2^10 / sigma: strictly above, so that ties go
+// outwards on both sides, and by so little (|d| < 2^26: 2^-37) that no other quotient, 1 / (2 sigma) > 2^-27 away from a tie, is
+// moved across it.  M in two 31-bit limbs makes that two 32 x 32 + 64 multiply-adds whose high word is q': half the
+// instructions of an estimate with a remainder test.  (fp64 would take one: but it shares its unit with the tensor core and
+// took five times as long while MMAs ran.)
 struct alignas(16) WvLnRow {
-    double inv;
-    uint32_t off;                  // 2^31 - mean
+    int32_t m_hi, m_lo;            // 2^32 M = m_hi + 2^-31 m_lo
+    int32_t mean;
     uint32_t sigma;                // top bit: quotients of this row may leave the fast range
 };
 constexpr uint32_t WV_LN_SLOW = 0x80000000u;
 
-// Statistics as ln_stats_fast (qmath.cuh), the divisions by n as fp64 multiplications by inv_n = (1 + 2^-46) / n: sums below
-// 2^43 and n < 2^13 keep every quotient 2^-14 from the next tie or integer, and the bias moves it by less than 2^-16.
-__device__ __forceinline__ WvLnRow wv_make_ln(long long sum, long long sq, int n, double inv_n, uint32_t sigma_min)
+// floor(n / d) for n < 2^57, d < 2^26 and a quotient below 2^31; x: reciprocal estimate of d (relative error 2^-21 at most)
+QL_HD uint32_t wv_div(uint64_t n, uint32_t d, float x)
 {
-    const int32_t mean = __double2loint(__fma_rn(1024.0 * (double)(int32_t)sum, inv_n, 6755399441055744.0));
-    // round(sq 2^20 / n) = floor(sq / n) 2^20 + floor(((sq mod n) 2^20 + n / 2) / n)
-    const uint32_t q1 = (uint32_t)__double2loint(__fma_rd((double)sq, inv_n, 4503599627370496.0));
-    const uint32_t r1 = (uint32_t)sq - q1 * (uint32_t)n;
-    const uint32_t m2 = (uint32_t)__double2loint(__fma_rd((double)(((uint64_t)r1 << 20) + (uint64_t)(n >> 1)), inv_n, 4503599627370496.0));
-    long long var = (long long)(((uint64_t)q1 << 20) + m2) - (long long)mean * mean;
+    uint32_t q = (uint32_t)((float)n * x);                     // within 2^11
+    int64_t r = (int64_t)(n - (uint64_t)q * d);
+    const int32_t c = (int32_t)((float)r * x);                 // then within 1
+    q += (uint32_t)c;
+    r -= (int64_t)c * d;
+    if (r < 0) { --q; r += d; }
+    if (r >= (int64_t)d) ++q;
+    return q;
+}
+
+QL_HD float wv_sqrt_est(float x)
+{
+#if defined(__CUDA_ARCH__)
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return __builtin_sqrtf(x);
+#endif
+}
+
+// Statistics as ln_stats_fast (qmath.cuh) with a shorter chain: one thread per (row, gate) computes them while a group waits.
+QL_HD WvLnRow wv_make_ln(int64_t sum, int64_t sumsq, const DivMagic &dn, uint32_t sigma_min)
+{
+    const uint64_t half = dn.n >> 1;
+    const int32_t am = (int32_t)div_by_magic((uint64_t)(sum < 0 ? -sum : sum) * 1024u + half, dn);
+    const int32_t mean = sum < 0 ? -am : am;
+    const uint64_t q1 = div_by_magic((uint64_t)sumsq, dn);
+    const uint64_t r1 = (uint64_t)sumsq - q1 * dn.n;
+    int64_t var = (int64_t)((q1 << 20) + div_by_magic((r1 << 20) + half, dn)) - (int64_t)mean * mean;
     if (var < 0) var = 0;
-    // integer root: fp32 estimate (within 4), one Newton step in fp64 (within 2^-18), exact correction
-    const double v = (double)var;
-    const float s0 = __fsqrt_rn((float)var);
-    const double e = __fma_rn(-(double)s0, (double)s0, v);
-    const float es = s0 > 0.0f ? __fdividef((float)e, 2.0f * s0) : 0.0f;
-    uint32_t sigma = (uint32_t)((double)s0 + (double)es);
-    if ((long long)sigma * sigma > var) --sigma;
-    else if ((long long)(sigma + 1u) * (sigma + 1u) <= var) ++sigma;
+    // integer root: fp32 estimate (within 2^4), one Newton step, exact correction
+    uint32_t s = (uint32_t)wv_sqrt_est((float)var);
+    const int64_t e = var - (int64_t)s * s;
+    if (s) s += (uint32_t)(int32_t)(0.5f * (float)e * rcp_est((float)s));
+    for (int i = 0; i < 2; ++i)
+        if ((int64_t)s * s > var) --s;
+    for (int i = 0; i < 2; ++i)
+        if ((int64_t)(s + 1u) * (s + 1u) <= var) ++s;
     WvLnRow r;
-    r.off = 0x80000000u - (uint32_t)mean;
-    r.inv = 0.0;                                               // sigma = 0: the quotient is 0
-    if (sigma) {
-        const double d = (double)sigma;
-        double x = (double)rcp_est((float)sigma);              // two Newton steps from 2^-22: 2^-43, then full precision
-        x = __fma_rn(x, __fma_rn(-d, x, 1.0), x);
-        x = __fma_rn(x, __fma_rn(-d, x, 1.0), x);
-        r.inv = x * (1024.0 * (1.0 + 0x1p-48));
-        if (sigma < sigma_min) sigma |= WV_LN_SLOW;
+    r.mean = mean; r.sigma = s; r.m_hi = 0; r.m_lo = 0;        // sigma = 0: the quotient is 0
+    if (s >= sigma_min) {
+        const float x = rcp_est((float)s);
+        const uint32_t hi = wv_div((uint64_t)1 << 42, s, x);
+        const uint32_t lo = wv_div((uint64_t)((1ull << 42) - (uint64_t)hi * s) << 31, s, x) + 1u;
+        r.m_hi = (int32_t)(hi + (lo >> 31)); r.m_lo = (int32_t)(lo & 0x7fffffffu);
+    } else if (s) {
+        r.sigma |= WV_LN_SLOW;
     }
-    r.sigma = sigma;
     return r;
 }
 
-// sat32(q' L + b) where q' and the product are known to be in range
-__device__ __forceinline__ int32_t wv_ln_fast(int32_t q, double inv, uint32_t off, int32_t Lw, int32_t b)
+QL_HD int32_t wv_ln_quotient(int32_t q, int32_t m_hi, int32_t m_lo, int32_t mean)
 {
-    // 2^52 + 2^31 + 2^10 q - mean, whose low word is one integer multiply-add
-    const double d = __dadd_rn(__hiloint2double(0x43300000, (int)((uint32_t)(q * 1024) + off)), -4503601774854144.0);
-    return __double2loint(__fma_rn(d, inv, 6755399441055744.0)) * Lw + b;
+    const int32_t d = 1024 * q - mean;
+    // the added 2^63 makes the low product's high word non-negative and is the 1/2 of the sum
+    const uint64_t lo = (uint64_t)((int64_t)(2 * d) * m_lo) + 0x8000000000000000ull;
+    return (int32_t)(((int64_t)d * m_hi + (int64_t)(lo >> 32)) >> 32);
+}
+
+// sat32(q' L + b) where q' and the sum are known to be in range
+__device__ __forceinline__ int32_t wv_ln_fast(int32_t q, int32_t m_hi, int32_t m_lo, int32_t mean, int32_t Lw, int32_t b)
+{
+    return wv_ln_quotient(q, m_hi, m_lo, mean) * Lw + b;
 }
 
 // the same for any row, by division, out of line
 static __device__ __noinline__ int32_t wv_ln_slow(int32_t q, WvLnRow row, int32_t Lw, int32_t b)
 {
-    const int32_t d = 1024 * q - (int32_t)(0x80000000u - row.off);
+    const int32_t d = 1024 * q - row.mean;
     const uint32_t ad = (uint32_t)(d < 0 ? -d : d), sg = row.sigma & ~WV_LN_SLOW;
     const uint64_t quo = sg == 0u ? 0u : ((uint64_t)ad * 1024u + (sg >> 1)) / sg;
     const int64_t qp = d < 0 ? -(int64_t)quo : (int64_t)quo;

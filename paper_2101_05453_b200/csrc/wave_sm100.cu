@@ -214,7 +214,7 @@ __device__ __forceinline__ void wv_proj_tile(const WaveCall &k, const WaveLayer 
 // ---- elementwise phase -----------------------------------------------------------------------------------------------
 
 // Layer-norm constants of a thread's row in registers: those that the fast form needs.
-struct WvLnRegs { double inv[4]; uint32_t off[4]; bool slow; };
+struct WvLnRegs { int32_t m_hi[4], m_lo[4], mean[4]; bool slow; };
 
 template <int G>
 __device__ __forceinline__ void wv_load_ln(const WaveSmem &s, int row, unsigned mask, WvLnRegs &r)
@@ -224,7 +224,7 @@ __device__ __forceinline__ void wv_load_ln(const WaveSmem &s, int row, unsigned 
     for (int g = 0; g < G; ++g)
         if ((mask >> g) & 1u) {
             const WvLnRow v = s.ln[g * 128 + row];
-            r.inv[g] = v.inv; r.off[g] = v.off; any |= v.sigma;
+            r.m_hi[g] = v.m_hi; r.m_lo[g] = v.m_lo; r.mean[g] = v.mean; any |= v.sigma;
         }
     r.slow = (any & WV_LN_SLOW) != 0u;
 }
@@ -242,7 +242,7 @@ __device__ __forceinline__ void wv_ln_pair(const WaveLayer &L, const WaveSmem &s
     for (int g = 0; g < G; ++g)
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if ((mask >> g) & 1u) v[g][k] = wv_ln_fast(a[g][k], r.inv[g], r.off[g], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k]);
+            if ((mask >> g) & 1u) v[g][k] = wv_ln_fast(a[g][k], r.m_hi[g], r.m_lo[g], r.mean[g], k ? wv_hi(lws[g]) : wv_lo(lws[g]), bb[2 * g + k]);
     if (r.slow) {
 #pragma unroll
         for (int g = 0; g < G; ++g)
@@ -309,7 +309,7 @@ __device__ __forceinline__ void wv_pull_stats(const WaveLayer &L, const WaveSmem
         const int g = i / rows, row = i - g * rows;
         if (!((mask >> g) & 1u)) continue;
         const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(totals + (size_t)(row * 4 + g) * 2));
-        s.ln[g * 128 + row] = wv_make_ln(v.x, v.y, L.C, L.inv_c, L.sigma_min);
+        s.ln[g * 128 + row] = wv_make_ln(v.x, v.y, L.div_c, L.sigma_min);
     }
 }
 // Everything between the gate sums and m for one unit.  Tasks are (pair, row) with the row fastest, so that the gate
@@ -344,10 +344,15 @@ __device__ __forceinline__ bool wv_elementwise(const WaveCall &k, const WaveLaye
     WvLnRegs lr = {};
     if (LN && p0 < per) wv_load_ln<G>(s, row, PEEP ? ALL & ~(1u << SO) : ALL, lr);
     if (p0 < per) {
+        // the next pair's inputs are requested before the present one is worked on (the buffers may lie in L2)
+        uint4 g_next = make_uint4(0, 0, 0, 0);
+        uint32_t c_next = 0;
+        if (p0 < r.pairs) { g_next = g_s[p0 * rows + row]; c_next = c_s[p0 * rows + row]; }
 #pragma unroll 1
         for (int pr = p0; pr < r.pairs; pr += per) {
-            const uint4 g4 = g_s[pr * rows + row];
-            const uint32_t cw = c_s[pr * rows + row];
+            const uint4 g4 = g_next;
+            const uint32_t cw = c_next;
+            if (pr + per < r.pairs) { g_next = g_s[(pr + per) * rows + row]; c_next = c_s[(pr + per) * rows + row]; }
             const uint32_t gw[4] = {g4.x, g4.y, g4.z, g4.w};
             int32_t a[4][2];
 #pragma unroll
@@ -877,11 +882,29 @@ void wave_units(int B, int rg, int &units, int &nu, int &ra)
     ra = wv_round((B + nu - 1) / nu, 8);
 }
 
-// How many groups the rows of a batch are split into.  (Deep stacks: the layers already share out the SMs.)
-int wave_row_groups(int mode, int n_layers, int max_B, int sm_count)
+// How many groups the rows of a batch are split into.  Fewer blocks per group make every exchange cheaper (two 512-cell layers,
+// 16 rows: 9.0 us per step with one group, 8.5 with four; one 2048-cell layer with layer norm and peephole, 32 rows: 26 and 17),
+// but a block then streams more weights per step: below 16 blocks, or beyond 320 KB, the groups cost more than they save (the
+// same layers with eight groups: 9.2 and 18; five 1024-cell layers, 4 rows: 7.5 with one group, 10.3 with two).  Where a split
+// brings the rows of a group down to the 32 that wave_small_sm100.cu takes, it pays down to 12 blocks and up to 512 KB (five
+// 1024-cell CIFG layers, 64 rows: 14.1 us per step as one group here, 12.0 as two there).
+int wave_row_groups(int mode, const std::vector<const LayerParams *> &lp, int max_B, int sm_count)
 {
+    const int n = (int)lp.size();
+    size_t bytes = 0;
+    for (const LayerParams *p : lp)
+        bytes = std::max(bytes, (size_t)p->N * (p->I + p->O) + ((p->flags & F_PROJECTION) ? (size_t)p->O * p->C : 0));
     int rg = 1;
-    while (rg > 1 && (rg > max_B || sm_count / (n_layers * rg) < 2)) rg >>= 1;
+    // [0]: more than 64 rows per group and at least 32 blocks left (one 2048-cell layer with layer norm, 256 rows: 40 us per step as
+    // one group of two units, 32 as four groups; two 1024-cell layers: 32 and 25)
+    while (mode == 0 && (max_B + rg - 1) / rg > 64 && sm_count / (2 * rg * n) >= 32) rg *= 2;
+    while (mode == 1 && 2 * rg <= max_B) {
+        const int blocks = sm_count / (2 * rg * n);
+        const bool fits_now = (max_B + rg - 1) / rg <= WV_SMALL_ROWS, fits_then = (max_B + 2 * rg - 1) / (2 * rg) <= WV_SMALL_ROWS;
+        const bool entry = !fits_now && fits_then;
+        if (blocks < (entry ? 12 : 16) || bytes / blocks > (size_t)(entry ? 512 : 320) * 1024) break;
+        rg *= 2;
+    }
     return rg;
 }
 
@@ -942,6 +965,8 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
 
 }  // namespace
 
+static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool tables, WaveCall &k, size_t &smem);
+
 // Plans the wavefront kernels for a handle; *out stays null when the stack does not qualify: layers of different variants,
 // a scale with a left shift where none is expected, or sums that could leave int32.
 int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B, int sm_count, WaveStack **out)
@@ -976,16 +1001,14 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
     auto fail = [&](int rc) { wave_destroy(s); return rc; };
     int nu_max = 1;
     for (int mode = 0; mode < 2; ++mode) {
-        WavePlan &pl = s->plan[mode];
-        pl.rg = wave_row_groups(mode, n, s->max_B, sm_count);
-        nu_max = std::max(nu_max, (mode == 0 ? 2 : 1) * pl.rg);
+        s->plan[mode].rg = wave_row_groups(mode, lp, s->max_B, sm_count);
+        nu_max = std::max(nu_max, (mode == 0 ? 2 : 1) * s->plan[mode].rg);
     }
-    s->plan[1].ok = true;                                            // [0] only where [1] does not cover every batch
-    s->plan[0].ok = (s->max_B + s->plan[1].rg - 1) / s->plan[1].rg > WV_SMALL_ROWS;
+    s->plan[1].ok = true;
     const size_t rows_alloc = (size_t)s->max_B + 8 * nu_max;         // rows of all units, each rounded up to 8
     long long h_off = 0, c_off = 0;
     int8_t *prev_img = nullptr;
-    int prev_n[2] = {0, 0};
+    std::vector<WaveLayer> base;
     s->tabs = true;
     std::vector<std::pair<int, std::pair<uint8_t *, ActLineLayout>>> blobs;
     for (int l = 0; l < n; ++l) {
@@ -1006,7 +1029,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
             L.f_c[g] = make_fast_scale(p.eff_c[g]); L.f_ln[g] = make_fast_scale(p.eff_ln[g]);
         }
         L.f_m = make_fast_scale(p.eff_m); L.f_proj = make_fast_scale(p.eff_proj);
-        L.inv_c = (1.0 + 0x1p-46) / p.C;
+        L.div_c = make_div_magic((uint32_t)p.C);
         {
             // q' L + b stays inside an int32 for |q'| <= room, and |2^10 (2^10 q - mean)| <= 2^36
             const long long room = std::min(65535ll, (0x7fffffffll - p.max_bln) / (p.max_L > 0 ? p.max_L : 1)) - 1;
@@ -1033,21 +1056,32 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
         if (!blob) s->tabs = false;
         L.tab = blob; L.tab_lay = lay;
         s->max_tab = std::max(s->max_tab, (int)lay.bytes);
-        for (int mode = 0; mode < 2; ++mode) {
-            WavePlan &pl = s->plan[mode];
-            if (!pl.ok) continue;
-            WaveLayer M = L;
+        base.push_back(L);
+    }
+    if (cudaFuncSetAttribute(wave_small_kernel(s->G, s->ln, s->peep), cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess)
+        s->plan[1].ok = false;
+    for (int mode = 1; mode >= 0; --mode) {
+        WavePlan &pl = s->plan[mode];
+        if (mode == 0) {
+            WaveCall k;
+            size_t smem;
+            pl.ok = !wave_describe(s, 1, max_T, s->max_B, true, k, smem);       // only where [1] does not cover every batch
+        }
+        int prev_n = 0;
+        for (int l = 0; l < n && pl.ok; ++l) {
+            const LayerParams &p = *lp[l];
+            WaveLayer M = base[l];
             const int rc = wave_share_layer(s, mode, p, sm_count / (n * pl.rg), M);
             if (rc != QLSTM_OK) return fail(rc);
-            if (M.n == 0) { pl.ok = false; continue; }
+            if (M.n == 0) { pl.ok = false; break; }
             M.cta0 = pl.grid;
             pl.grid += M.n * pl.rg;
-            M.below = l > 0 ? prev_n[mode] : 0;
-            prev_n[mode] = M.n;
+            M.below = l > 0 ? prev_n : 0;
+            prev_n = M.n;
             pl.max_ppc = std::max(pl.max_ppc, M.ppc);
             pl.max_cpc = std::max(pl.max_cpc, wv_round(M.cpc, 2));
             pl.max_opc = std::max(pl.max_opc, wv_round(M.opc, 4));
-            pl.b_slot = mode == 1 ? WS_SLOT_ROWS * 128 : std::max(pl.b_slot, std::max(M.npad, proj ? M.npadp : 0) * 128);
+            pl.b_slot = mode == 1 ? WS_SLOT_ROWS * 128 : std::max(pl.b_slot, std::max(M.npad, (p.flags & F_PROJECTION) ? M.npadp : 0) * 128);
             pl.layer.push_back(M);
         }
     }
@@ -1076,8 +1110,6 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
             if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) big.ok = false;
         }
     }
-    if (small.ok && cudaFuncSetAttribute(wave_small_kernel(s->G, s->ln, s->peep), cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess)
-        small.ok = false;
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(QLSTM_ERR_CUDA);
     if (!big.ok && !small.ok) return fail(QLSTM_OK);
     *out = s;
@@ -1103,7 +1135,7 @@ static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool table
         for (const WaveLayer &L : pl.layer)
             if ((2 * L.nt + L.ntp) * k.ra > 512) return false;
         k.nb = 8;
-        while (k.nb > 3 && wave_small_smem(k, k.nb, s->peep) > room) --k.nb;
+        while (k.nb > 2 && wave_small_smem(k, k.nb, s->peep) > room) --k.nb;
         smem = wave_small_smem(k, k.nb, s->peep);
         return smem <= room;
     }
@@ -1139,10 +1171,19 @@ bool wave_supported(const WaveStack *s, int T, int B)
     return wave_mode(s, T, B, true, k, smem) >= 0;
 }
 
+// Where the wavefront kernels are the faster path (measured, us per call, against the whole-stack kernel or layer after layer):
+// one step of one or two rows stays with the whole-stack kernel (eight 2048-cell layers 138 against 170, one 512-cell layer 10
+// against 15; two steps 266 against 186); calls of a few steps of many rows, in which a wavefront has little to overlap, run
+// layer after layer (eight layers, 256 rows: one step 452 against 1057, four 1152 against 1404, sixteen 4050 against 2757; 64
+// rows: one step 377 against 451, two 538 against 478; five layers, 256 rows: four steps 324 against 340, sixteen 926 against
+// 628; two layers always).
 bool wave_preferred(const WaveStack *s, int T, int B)
 {
     if (!wave_supported(s, T, B)) return false;
-    return s->ragged || (B > 4 && (s->n_layers >= 3 || (s->n_layers == 2 && B <= WV_SMALL_ROWS)));
+    if (s->ragged) return true;
+    if (T == 1 && B <= 2) return false;
+    if (s->n_layers == 1 && s->ln && B > 64) return false;
+    return T * 256 > s->n_layers * (B - 32);
 }
 
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns)

@@ -146,7 +146,7 @@ __device__ __forceinline__ void ws_pull_stats(const WaveLayer &L, const WsSmem &
     const int g = tid >> 5, row = tid & 31;
     if (g < G && row < rows && ((mask >> g) & 1u)) {
         const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(totals + (size_t)(row * 4 + g) * 2));
-        s.ln[g * WS_ROWS + row] = wv_make_ln(v.x, v.y, L.C, L.inv_c, L.sigma_min);
+        s.ln[g * WS_ROWS + row] = wv_make_ln(v.x, v.y, L.div_c, L.sigma_min);
     }
 }
 
@@ -161,7 +161,7 @@ __device__ __forceinline__ void ws_ln_cell(const WaveLayer &L, const WsSmem &s, 
         if ((mask >> g) & 1u) {
             const WvLnRow r = s.ln[g * WS_ROWS + row];
             any |= r.sigma;
-            v[g] = wv_ln_fast(a[g], r.inv, r.off, s.L[g * L.cpc + ul], s.bln[g * L.cpc + ul]);
+            v[g] = wv_ln_fast(a[g], r.m_hi, r.m_lo, r.mean, s.L[g * L.cpc + ul], s.bln[g * L.cpc + ul]);
         }
     if (any & WV_LN_SLOW) {
 #pragma unroll
