@@ -110,6 +110,29 @@ __device__ __forceinline__ bool wv_wait_count(const WaveCall &k, const unsigned 
     }
     return *abort_flag == 0;
 }
+// The same for a warp that stays together: one lane looks, all decide.  (A single thread that polls while its warp waits at the
+// next barrier leaves the warp split, and everything after it then runs twice: 2 us per step.)
+__device__ __forceinline__ void wv_wait_count_warp(const WaveCall &k, const unsigned *cnt, unsigned target, volatile int *abort_flag)
+{
+    const bool look = (threadIdx.x & 31) == 0;
+    target += k.missing;
+    const unsigned long long t0 = wv_timer();
+    for (unsigned spins = 1;; ++spins) {
+        unsigned v = 0;
+        if (look) v = wv_ld_acquire(cnt);
+        v = __shfl_sync(0xffffffffu, v, 0);
+        if (v >= target) return;
+        if ((spins & 31u) == 0u) {
+            unsigned stop = 0;
+            if (look) {
+                if (*abort_flag) stop = 1;
+                else if (wv_ld_acquire(k.abort_word) != 0u) { *abort_flag = 1; stop = 1; }
+                else if (wv_timer() - t0 > k.limit_ns) { atomicExch(k.abort_word, 1u); *abort_flag = 1; stop = 1; }
+            }
+            if (__shfl_sync(0xffffffffu, stop, 0)) return;
+        }
+    }
+}
 __device__ __forceinline__ void wv_epi_sync() { asm volatile("barrier.sync 1, 512;" ::: "memory"); }
 
 // The same for a whole warp that stays together.
@@ -283,7 +306,7 @@ __device__ __forceinline__ bool wv_publish(unsigned *cnt, bool operands, WvPoint
 // all epilogue threads: wait for the group; false: leave
 __device__ __forceinline__ bool wv_meet(const WaveCall &k, const unsigned *cnt, unsigned target, WvPoint &pt, int tid)
 {
-    if (tid == 0) wv_wait_count(k, cnt, target, pt.abort_flag);
+    if (tid < 32) wv_wait_count_warp(k, cnt, target, pt.abort_flag);
     return wv_point(pt, tid);
 }
 
