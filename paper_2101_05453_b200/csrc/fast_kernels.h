@@ -6,6 +6,7 @@
 
 #include <vector>
 
+#include "../../include/qlstm.h"
 #include "act_table.cuh"
 #include "qlstm_internal.h"
 
@@ -91,13 +92,21 @@ int stack_small_groups(const StackSmall *s, int *blocks_per_layer);     // layer
 // ---- wavefront kernel (wave_sm100.cu): all layers and steps in one cooperative launch, tensor-core products, batches up to
 // 256 rows, any dimensions.
 struct WaveStack;
-int wave_create(const std::vector<const LayerParams *> &layers, int max_T, int max_B, int sm_count, WaveStack **out);
+// The first n_fwd layers are one stack; any that follow are a second one over the same x, backwards in time (bidirectional).
+int wave_create(const std::vector<const LayerParams *> &layers, int n_fwd, int max_T, int max_B, int sm_count, WaveStack **out);
 void wave_destroy(WaveStack *s);
 bool wave_supported(const WaveStack *s, int T, int B);
 bool wave_preferred(const WaveStack *s, int T, int B);             // supported and, by measurement, the faster path
-// tables: memoised nonlinearities where they pay.  The launch clears the status word itself.
-int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *h, int16_t *c, int8_t *y, int *status, bool tables, cudaStream_t st,
-                int *launches);
+// h, c: state of the one or two stacks; y: rows of the stacks' outputs side by side; status2: another status word to clear, or
+// null.  tables: memoised nonlinearities.  The launch clears the status word itself.
+int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
+                bool tables, cudaStream_t st, int *launches);
+// The two handles of a bidirectional stack and, where both directions fit one plan, the wavefront kernels that run them side by
+// side (else *wave stays null and each handle has its own); qlstm_api.cu.
+int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b,
+                      WaveStack **wave);
+int bidir_wave_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
+                   cudaStream_t st);
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns);
 
 int debug_ring_plan(int stages, int n_own, int contig, int per, int n_total, int *out);

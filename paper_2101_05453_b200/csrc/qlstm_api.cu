@@ -258,9 +258,7 @@ int run_projection(qlstm *q, LayerHost &L, const int8_t *x, int rows, int16_t *X
 
 }  // namespace
 
-extern "C" {
-
-int qlstm_create(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B, int device, qlstm_t **out)
+static int create_handle(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B, int device, bool with_wave, qlstm_t **out)
 {
     if (!out) return QLSTM_ERR_ARG;
     *out = nullptr;
@@ -322,12 +320,52 @@ int qlstm_create(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B
         std::vector<const LayerParams *> lp;
         for (auto &L : q->layers) lp.push_back(&L.p);
         int src = stack_small_create(lp, max_T, max_B, q->sm_count, &q->stack);
-        if (src == QLSTM_OK) src = wave_create(lp, max_T, max_B, q->sm_count, &q->wave);
+        if (src == QLSTM_OK && with_wave) src = wave_create(lp, n_layers, max_T, max_B, q->sm_count, &q->wave);
         if (src != QLSTM_OK) { ok = false; rc = src; }
     }
     if (!ok) { qlstm_destroy(q); return rc; }
     *out = q;
     return QLSTM_OK;
+}
+
+namespace ql {
+
+int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b,
+                      WaveStack **wave)
+{
+    *f = *b = nullptr;
+    *wave = nullptr;
+    int rc = create_handle(fwd, n_layers, max_T, max_B, device, false, f);
+    if (rc == QLSTM_OK) rc = create_handle(bwd, n_layers, max_T, max_B, device, false, b);
+    if (rc != QLSTM_OK) return rc;
+    std::vector<const LayerParams *> lp;
+    for (auto &L : (*f)->layers) lp.push_back(&L.p);
+    for (auto &L : (*b)->layers) lp.push_back(&L.p);
+    rc = wave_create(lp, n_layers, max_T, max_B, (*f)->sm_count, wave);
+    // the directions do not go together: each has its own kernels
+    for (qlstm_t *q : {*f, *b}) {
+        if (rc != QLSTM_OK || *wave) break;
+        lp.clear();
+        for (auto &L : q->layers) lp.push_back(&L.p);
+        rc = wave_create(lp, n_layers, max_T, max_B, q->sm_count, &q->wave);
+    }
+    return rc;
+}
+
+int bidir_wave_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
+                   cudaStream_t st)
+{
+    f->last_stream = b->last_stream = st;
+    return launch_wave(wave, x, T, B, h, c, y, f->status, b->status, true, st, nullptr);
+}
+
+}  // namespace ql
+
+extern "C" {
+
+int qlstm_create(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B, int device, qlstm_t **out)
+{
+    return create_handle(layers, n_layers, max_T, max_B, device, true, out);
 }
 
 void qlstm_destroy(qlstm_t *q)
@@ -382,7 +420,7 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
         if (q->impl_rec == 0 ? wave_preferred(q->wave, T, B) : wave_supported(q->wave, T, B)) {
             SpanGuard g(q, st, 1);
             int launches = 0;
-            const int rc = launch_wave(q->wave, x_dev, T, B, h_dev, c_dev, y_dev, q->status, q->tables, st, &launches);
+            const int rc = launch_wave(q->wave, x_dev, T, B, {h_dev, nullptr}, {c_dev, nullptr}, y_dev, q->status, nullptr, q->tables, st, &launches);
             g.done(launches);
             return rc;
         }

@@ -43,7 +43,11 @@ struct WaveLayer {
     long long *totals;             // [2][units][ra][4][2] layer-norm sums of the group
     unsigned *cnt;                 // [units][WC_PER_UNIT][WC_WORDS]
     int below;                     // blocks of the layer below, 0: none
-    long long h_off, c_off;        // of this layer in the caller's state, in units of one batch row
+    long long h_off, c_off;        // of this layer in its stack's state, in units of one batch row
+    int8_t *h; int16_t *c;         // the caller's state of this layer (set per call)
+    int first, last;               // of its stack
+    int dir;                       // 1: the stack reads x from the last step backwards
+    int y_off;                     // last layer: its columns within a row of y
     const uint8_t *tab;
     ActLineLayout tab_lay;
 };
@@ -59,15 +63,22 @@ struct WaveCall {
     int gx_s;                      // gate buffers in shared memory
     int nbuf;                      // gate buffers per unit: [gate sums | X ...]
     int max_ppc, max_opc, max_tab;
-    int8_t *h; int16_t *c; int8_t *y;
+    int8_t *y;
+    int y_stride;                  // bytes of a row of y
     uint4 *gbuf;                   // [blocks][units][nbuf][max_ppc][max rows] gate buffers in global memory
     uint32_t *cbuf;                // [blocks][units][max_ppc][max rows] cell states
     unsigned *abort_word;
-    int *status;
+    int *status, *status2;         // status2: another word to clear, or null
     unsigned long long limit_ns;
     unsigned missing;
     WaveLayer layer[WV_MAX_LAYERS];
 };
+
+// the row of y that a last layer's step t and batch row b go to
+__device__ __forceinline__ int8_t *wv_y_row(const WaveCall &k, const WaveLayer &L, int t, int b)
+{
+    return k.y + ((size_t)(L.dir ? k.T - 1 - t : t) * k.B + b) * k.y_stride + L.y_off;
+}
 
 // ---- waits ---------------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool wv_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag)

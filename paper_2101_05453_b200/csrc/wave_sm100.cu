@@ -197,8 +197,8 @@ __device__ __forceinline__ void wv_proj_tile(const WaveCall &k, const WaveLayer 
         *reinterpret_cast<uint32_t *>(out_unit + wv_img_off(row, col, k.ra)) = w;
         const bool fin = t == k.T - 1;
         if (last_layer || fin) {
-            int8_t *dst[2] = {last_layer ? k.y + ((size_t)t * k.B + b) * L.O + col : nullptr,
-                              fin ? k.h + L.h_off * k.B + (size_t)b * L.O + col : nullptr};
+            int8_t *dst[2] = {last_layer ? wv_y_row(k, L, t, b) + col : nullptr,
+                              fin ? L.h + (size_t)b * L.O + col : nullptr};
 #pragma unroll
             for (int d = 0; d < 2; ++d) {
                 if (!dst[d]) continue;
@@ -267,12 +267,12 @@ __device__ __forceinline__ void wv_store_m(const WaveCall &k, const WaveLayer &L
     if (L.flags & F_PROJECTION) return;
     const bool both = u + 1 < L.C, fin = t == k.T - 1;
     if (last_layer) {
-        int8_t *y = k.y + ((size_t)t * k.B + b) * L.O + u;
+        int8_t *y = wv_y_row(k, L, t, b) + u;
         if (both && ((uintptr_t)y & 1) == 0) *reinterpret_cast<uint16_t *>(y) = w;
         else { y[0] = (int8_t)m0; if (both) y[1] = (int8_t)m1; }
     }
     if (fin) {
-        int8_t *h = k.h + L.h_off * k.B + (size_t)b * L.O + u;
+        int8_t *h = L.h + (size_t)b * L.O + u;
         h[0] = (int8_t)m0;
         if (both) h[1] = (int8_t)m1;
     }
@@ -280,7 +280,7 @@ __device__ __forceinline__ void wv_store_m(const WaveCall &k, const WaveLayer &L
 
 __device__ __forceinline__ void wv_store_c(const WaveCall &k, const WaveLayer &L, int u, int b, int32_t c0, int32_t c1)
 {
-    int16_t *c = k.c + L.c_off * k.B + (size_t)b * L.C + u;
+    int16_t *c = L.c + (size_t)b * L.C + u;
     if (u < L.C) c[0] = (int16_t)c0;
     if (u + 1 < L.C) c[1] = (int16_t)c1;
 }
@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
         if (cta >= k.layer[l].cta0 && cta < k.layer[l].cta0 + k.layer[l].n * k.rg) r.li = l;
     if (r.li < 0) return;                                      // spare block: takes no part in any counter
     const WaveLayer &L = k.layer[r.li];
-    const bool proj = (L.flags & F_PROJECTION) != 0, last_layer = r.li == k.n_layers - 1;
+    const bool proj = (L.flags & F_PROJECTION) != 0, last_layer = L.last != 0;
     r.rgi = (cta - L.cta0) / L.n;
     r.rank = cta - L.cta0 - r.rgi * L.n;
     r.u0 = r.rank * L.ppc * 2;
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
     for (int u = 0; u < 2; ++u)
         for (int i = threadIdx.x; i < r.pairs * r.rows[u]; i += WV_THREADS) {
             const int pr = i / r.rows[u], b = r.row0[u] + i - pr * r.rows[u], c = r.u0 + 2 * pr;
-            const int16_t *src = k.c + L.c_off * k.B + (size_t)b * L.C + c;
+            const int16_t *src = L.c + (size_t)b * L.C + c;
             const uint32_t lo = c < L.C ? (uint16_t)src[0] : 0u, hi = c + 1 < L.C ? (uint16_t)src[1] : 0u;
             r.c[u][i] = lo | (hi << 16);
         }
@@ -766,14 +766,15 @@ __global__ void k_wave_prepare(const __grid_constant__ WaveCall k, const int8_t 
         const int row = b - (int)((long long)gu * k.B / k.nu);
         *reinterpret_cast<uint4 *>(img + (block * k.nu + gu) * kbs * k.ra * 128 + wv_img_off(row, chunk * 16, k.ra)) = v;
     };
-    {
-        const WaveLayer &L = k.layer[0];
+    for (int l = 0; l < k.n_layers; ++l) {
+        const WaveLayer &L = k.layer[l];
+        if (!L.first) continue;
         const int per = (L.I + 15) >> 4;
         const size_t total = (size_t)k.T * k.B * per;
         for (size_t i = first; i < total; i += step) {
-            const size_t rt = i / per;
+            const size_t rt = i / per, t = rt / k.B;
             const int chunk = (int)(i - rt * per), b = (int)(rt % k.B);
-            put(L.in_img, L.kb_i, rt / k.B, b, chunk, wv_load16(x + rt * L.I + chunk * 16, L.I - chunk * 16));
+            put(L.in_img, L.kb_i, L.dir ? k.T - 1 - t : t, b, chunk, wv_load16(x + rt * L.I + chunk * 16, L.I - chunk * 16));
         }
     }
     for (int l = 0; l < k.n_layers; ++l) {
@@ -781,11 +782,14 @@ __global__ void k_wave_prepare(const __grid_constant__ WaveCall k, const int8_t 
         const int per = (L.O + 15) >> 4;
         for (size_t i = first; i < (size_t)k.B * per; i += step) {
             const int b = (int)(i / per), chunk = (int)(i - (size_t)b * per);
-            put(L.out_img, L.kb_h, 0, b, chunk, wv_load16(k.h + L.h_off * k.B + (size_t)b * L.O + chunk * 16, L.O - chunk * 16));
+            put(L.out_img, L.kb_h, 0, b, chunk, wv_load16(L.h + (size_t)b * L.O + chunk * 16, L.O - chunk * 16));
         }
     }
     for (size_t i = first; i < zero_words; i += step) zero[i] = 0u;
-    if (first == 0) *k.status = 0;
+    if (first == 0) {
+        *k.status = 0;
+        if (k.status2) *k.status2 = 0;
+    }
 }
 
 // A weight matrix into the tiles its blocks stream: [rank][tile][k-block][column][128 bytes], swizzled.  Gate matrices
@@ -841,6 +845,8 @@ struct WavePlan {
 
 struct WaveStack {
     int n_layers = 0, max_T = 0, max_B = 0, max_smem = 0;
+    int depth = 0;                 // layers of one stack (two of them: the directions of a bidirectional one)
+    int y_stride = 0;
     int G = 4;
     bool ln = false, peep = false, tabs = false;
     bool ragged = false;           // some dimension is not a multiple of 16
@@ -882,29 +888,52 @@ void wave_units(int B, int rg, int &units, int &nu, int &ra)
     ra = wv_round((B + nu - 1) / nu, 8);
 }
 
-// How many groups the rows of a batch are split into.  Fewer blocks per group make every exchange cheaper (two 512-cell layers,
-// 16 rows: 9.0 us per step with one group, 8.5 with four; one 2048-cell layer with layer norm and peephole, 32 rows: 26 and 17),
-// but a block then streams more weights per step: below 16 blocks, or beyond 320 KB, the groups cost more than they save (the
-// same layers with eight groups: 9.2 and 18; five 1024-cell layers, 4 rows: 7.5 with one group, 10.3 with two).  Where a split
-// brings the rows of a group down to the 32 that wave_small_sm100.cu takes, it pays down to 12 blocks and up to 512 KB (five
-// 1024-cell CIFG layers, 64 rows: 14.1 us per step as one group here, 12.0 as two there).
-int wave_row_groups(int mode, const std::vector<const LayerParams *> &lp, int max_B, int sm_count)
+// Whether wave_small_sm100.cu can take B rows in rg groups of blocks (shared memory and tensor memory of the widest layer).
+bool wave_small_fits(const WaveStack *s, const std::vector<const LayerParams *> &lp, int rg, int B, int sm_count)
+{
+    const int per = sm_count / ((int)lp.size() * rg), rows = (B + rg - 1) / rg;
+    if (per < 1 || rows > WV_SMALL_ROWS) return false;
+    WaveCall k;
+    memset(&k, 0, sizeof(k));
+    k.B = B; k.nu = rg; k.ra = wv_round(rows, 8); k.b_slot = WS_SLOT_ROWS * 128; k.max_tab = s->max_tab;
+    for (const LayerParams *p : lp) {
+        const int cpc = (p->C + per - 1) / per, n = (p->C + cpc - 1) / cpc, nt = (cpc + 31) / 32;
+        const bool proj = p->flags & F_PROJECTION;
+        const int opc = proj ? (p->O + n - 1) / n : 0, ntp = (opc + 127) / 128;
+        if (nt > 8 || (2 * nt + ntp) * k.ra > 512) return false;
+        k.max_cpc = std::max(k.max_cpc, wv_round(cpc, 2));
+        k.max_opc = std::max(k.max_opc, wv_round(opc, 4));
+        k.max_kb_i = std::max(k.max_kb_i, (p->I + 127) / 128);
+        k.max_kb_h = std::max(k.max_kb_h, (p->O + 127) / 128);
+        if (proj) k.max_kb_c = std::max(k.max_kb_c, (p->C + 127) / 128);
+    }
+    return wave_small_smem(k, 2, s->peep) <= (size_t)s->max_smem;
+}
+
+// How many groups the rows of a batch are split into.  (Deep stacks: the layers already share out the SMs.)
+int wave_row_groups(const WaveStack *s, int mode, const std::vector<const LayerParams *> &lp, int max_B, int sm_count)
 {
     const int n = (int)lp.size();
+    int rg = 1;
+    if (mode == 0) {
+        // more than 64 rows per group and at least 32 blocks left (one 2048-cell layer with layer norm, 256 rows: 40 us per step as
+        // one group of two units, 32 as four groups; two 1024-cell layers: 32 and 25)
+        while ((max_B + rg - 1) / rg > 64 && sm_count / (2 * rg * n) >= 32) rg *= 2;
+        return rg;
+    }
+    // As many as it takes for the few-row kernel to hold a group's rows, down to 9 blocks: it is the faster one even then (us per
+    // step against the many-row kernel as one group: five 1024-cell CIFG layers, 64 rows 12.0 as two groups against 14.1; four
+    // 1024-cell layers, 100 rows 24 as four against 28; eight 2048-cell layers, 32 rows 37 as two against 41).
+    while (!wave_small_fits(s, lp, rg, max_B, sm_count) && 2 * rg <= max_B && sm_count / (2 * rg * n) >= 9) rg *= 2;
+    if (!wave_small_fits(s, lp, rg, max_B, sm_count)) rg = 1;
+    // Then, fewer blocks per group make every exchange cheaper (two 512-cell layers, 16 rows: 9.0 us per step with one group, 8.5
+    // with four; one 2048-cell layer with layer norm and peephole, 32 rows: 26 and 17), but a block streams more weights per step:
+    // below 16 blocks, or beyond 320 KB, the groups cost more than they save (the same layers with eight groups: 9.2 and 18; five
+    // 1024-cell layers, 4 rows: 7.5 with one group, 10.3 with two).
     size_t bytes = 0;
     for (const LayerParams *p : lp)
         bytes = std::max(bytes, (size_t)p->N * (p->I + p->O) + ((p->flags & F_PROJECTION) ? (size_t)p->O * p->C : 0));
-    int rg = 1;
-    // [0]: more than 64 rows per group and at least 32 blocks left (one 2048-cell layer with layer norm, 256 rows: 40 us per step as
-    // one group of two units, 32 as four groups; two 1024-cell layers: 32 and 25)
-    while (mode == 0 && (max_B + rg - 1) / rg > 64 && sm_count / (2 * rg * n) >= 32) rg *= 2;
-    while (mode == 1 && 2 * rg <= max_B) {
-        const int blocks = sm_count / (2 * rg * n);
-        const bool fits_now = (max_B + rg - 1) / rg <= WV_SMALL_ROWS, fits_then = (max_B + 2 * rg - 1) / (2 * rg) <= WV_SMALL_ROWS;
-        const bool entry = !fits_now && fits_then;
-        if (blocks < (entry ? 12 : 16) || bytes / blocks > (size_t)(entry ? 512 : 320) * 1024) break;
-        rg *= 2;
-    }
+    while (2 * rg <= max_B && sm_count / (2 * rg * n) >= 16 && bytes / (sm_count / (2 * rg * n)) <= 320 * 1024) rg *= 2;
     return rg;
 }
 
@@ -967,9 +996,10 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
 
 static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool tables, WaveCall &k, size_t &smem);
 
-// Plans the wavefront kernels for a handle; *out stays null when the stack does not qualify: layers of different variants,
+// Plans the wavefront kernels for a handle - one stack of n_fwd layers, or two that read the same x, the second one backwards in
+// time; *out stays null when the stack does not qualify: layers of different variants,
 // a scale with a left shift where none is expected, or sums that could leave int32.
-int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B, int sm_count, WaveStack **out)
+int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T, int max_B, int sm_count, WaveStack **out)
 {
     *out = nullptr;
     const int n = (int)lp.size();
@@ -989,6 +1019,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
     }
     WaveStack *s = new WaveStack();
     s->n_layers = n;
+    s->depth = n_fwd;
     s->max_T = max_T;
     s->max_B = max_B < 256 ? max_B : 256;
     s->G = lp[0]->G;
@@ -999,9 +1030,26 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&s->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     auto fail = [&](int rc) { wave_destroy(s); return rc; };
+    s->tabs = true;
+    std::vector<std::pair<uint8_t *, ActLineLayout>> tables;
+    for (int l = 0; l < n; ++l) {
+        int same = 0;
+        while (same < l && lp[same]->m_bits != lp[l]->m_bits) ++same;
+        if (same < l) {
+            tables.push_back(tables[same]);
+            continue;
+        }
+        uint8_t *blob = nullptr;
+        ActLineLayout lay;
+        if (!act_lines_build(lp[l]->m_bits, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
+        if (blob) s->owned.push_back(blob);
+        else s->tabs = false;
+        tables.push_back({blob, lay});
+        s->max_tab = std::max(s->max_tab, (int)lay.bytes);
+    }
     int nu_max = 1;
     for (int mode = 0; mode < 2; ++mode) {
-        s->plan[mode].rg = wave_row_groups(mode, lp, s->max_B, sm_count);
+        s->plan[mode].rg = wave_row_groups(s, mode, lp, s->max_B, sm_count);
         nu_max = std::max(nu_max, (mode == 0 ? 2 : 1) * s->plan[mode].rg);
     }
     s->plan[1].ok = true;
@@ -1009,8 +1057,6 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
     long long h_off = 0, c_off = 0;
     int8_t *prev_img = nullptr;
     std::vector<WaveLayer> base;
-    s->tabs = true;
-    std::vector<std::pair<int, std::pair<uint8_t *, ActLineLayout>>> blobs;
     for (int l = 0; l < n; ++l) {
         const LayerParams &p = *lp[l];
         const bool proj = p.flags & F_PROJECTION;
@@ -1035,7 +1081,12 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
             const long long room = std::min(65535ll, (0x7fffffffll - p.max_bln) / (p.max_L > 0 ? p.max_L : 1)) - 1;
             L.sigma_min = room < 64 ? 0x7fffffffu : (uint32_t)((1ll << 36) / room + 1);
         }
-        L.in_img = l > 0 ? prev_img : (int8_t *)wv_alloc(s, (size_t)max_T * rows_alloc * L.kb_i * 128);
+        L.dir = l >= n_fwd ? 1 : 0;
+        L.first = l == 0 || l == n_fwd;
+        L.last = l == n_fwd - 1 || l == n - 1;
+        if (L.first) h_off = c_off = 0;
+        if (L.last) { L.y_off = s->y_stride; s->y_stride += p.O; }
+        L.in_img = !L.first ? prev_img : (int8_t *)wv_alloc(s, (size_t)max_T * rows_alloc * L.kb_i * 128);
         L.out_img = (int8_t *)wv_alloc(s, ((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
         L.m_img = proj ? (int8_t *)wv_alloc(s, rows_alloc * L.kb_c * 128) : nullptr;
         if (!L.in_img || !L.out_img || (proj && !L.m_img)) return fail(QLSTM_ERR_NOMEM);
@@ -1043,19 +1094,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
         prev_img = L.out_img;
         L.h_off = h_off; L.c_off = c_off;
         h_off += p.O; c_off += p.C;
-        uint8_t *blob = nullptr;
-        ActLineLayout lay = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-        bool have = false;
-        for (auto &b : blobs)
-            if (b.first == p.m_bits) { blob = b.second.first; lay = b.second.second; have = true; }
-        if (!have) {
-            if (!act_lines_build(p.m_bits, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
-            if (blob) s->owned.push_back(blob);
-            blobs.push_back({p.m_bits, {blob, lay}});
-        }
-        if (!blob) s->tabs = false;
-        L.tab = blob; L.tab_lay = lay;
-        s->max_tab = std::max(s->max_tab, (int)lay.bytes);
+        L.tab = tables[l].first; L.tab_lay = tables[l].second;
         base.push_back(L);
     }
     if (cudaFuncSetAttribute(wave_small_kernel(s->G, s->ln, s->peep), cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess)
@@ -1076,7 +1115,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int max_T, int max_B
             if (M.n == 0) { pl.ok = false; break; }
             M.cta0 = pl.grid;
             pl.grid += M.n * pl.rg;
-            M.below = l > 0 ? prev_n : 0;
+            M.below = M.first ? 0 : prev_n;
             prev_n = M.n;
             pl.max_ppc = std::max(pl.max_ppc, M.ppc);
             pl.max_cpc = std::max(pl.max_cpc, wv_round(M.cpc, 2));
@@ -1125,7 +1164,7 @@ static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool table
     k.T = T; k.B = B; k.n_layers = s->n_layers; k.rg = pl.rg;
     wave_units(B, pl.rg, k.units, k.nu, k.ra);
     const int rows = (B + k.nu - 1) / k.nu;
-    k.early = T >= 4 * s->n_layers;
+    k.early = T >= 4 * s->depth;
     k.max_ppc = pl.max_ppc; k.max_cpc = pl.max_cpc; k.max_opc = pl.max_opc; k.b_slot = pl.b_slot;
     k.max_kb_i = s->max_kb_i; k.max_kb_h = s->max_kb_h; k.max_kb_c = s->max_kb_c;
     const size_t room = (size_t)s->max_smem;
@@ -1183,8 +1222,8 @@ bool wave_preferred(const WaveStack *s, int T, int B)
     if (!wave_supported(s, T, B)) return false;
     if (s->ragged) return true;
     if (T == 1 && B <= 2) return false;
-    if (s->n_layers == 1 && s->ln && B > 64) return false;
-    return T * 256 > s->n_layers * (B - 32);
+    if (s->depth == 1 && s->ln && B > 64) return false;
+    return T * 256 > s->depth * (B - 32);
 }
 
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns)
@@ -1194,21 +1233,26 @@ void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long l
     s->dbg_limit_ns = missing_arrivals ? limit_ns : 0;
 }
 
-int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *h, int16_t *c, int8_t *y, int *status, bool tables, cudaStream_t st,
-                int *launches)
+int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
+                bool tables, cudaStream_t st, int *launches)
 {
     WaveCall k;
     size_t smem = 0;
     const int mode = wave_mode(s, T, B, tables, k, smem);
     if (mode < 0) return QLSTM_ERR_DIM;
     const WavePlan &pl = s->plan[mode];
-    k.h = h; k.c = c; k.y = y;
+    k.y = y; k.y_stride = s->y_stride;
     k.gbuf = s->gbuf; k.cbuf = s->cbuf;
     k.abort_word = s->zero + s->cnt_words - WC_WORDS;
-    k.status = status;
+    k.status = status; k.status2 = status2;
     k.limit_ns = s->dbg_limit_ns ? s->dbg_limit_ns : WV_WAIT_LIMIT_NS;
     k.missing = s->dbg_missing;
-    for (int l = 0; l < s->n_layers; ++l) k.layer[l] = pl.layer[l];
+    for (int l = 0; l < s->n_layers; ++l) {
+        WaveLayer &L = k.layer[l];
+        L = pl.layer[l];
+        L.h = h[L.dir] + L.h_off * B;
+        L.c = c[L.dir] + L.c_off * B;
+    }
     const size_t items = (size_t)T * B * ((pl.layer[0].I + 15) / 16);
     const int blocks = (int)std::min<size_t>(1184, (items + 255) / 256 + 32);
     k_wave_prepare<<<blocks, 256, 0, st>>>(k, x, s->zero, s->cnt_words + s->tot_words);

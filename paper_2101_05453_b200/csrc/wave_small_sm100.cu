@@ -178,8 +178,8 @@ __device__ __forceinline__ void ws_store_m(const WaveCall &k, const WaveLayer &L
 {
     img_unit[wv_img_off(row, u, k.ra)] = (int8_t)m;
     if (L.flags & F_PROJECTION) return;
-    if (last_layer) k.y[((size_t)t * k.B + b) * L.O + u] = (int8_t)m;
-    if (t == k.T - 1) k.h[L.h_off * k.B + (size_t)b * L.O + u] = (int8_t)m;
+    if (last_layer) wv_y_row(k, L, t, b)[u] = (int8_t)m;
+    if (t == k.T - 1) L.h[(size_t)b * L.O + u] = (int8_t)m;
 }
 
 // Everything between the gate sums and m, one cell per task, consecutive threads on consecutive cells of a row.
@@ -219,7 +219,7 @@ __device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLaye
         else { ig = 32768 - f; if (ig > 32767) ig = 32767; }               // coupled input gate, Section 3.2.9
         const int32_t c_new = cell_update_fast(ig, z, f, s.c[row * cpc + ul], L.m_bits);
         s.c[row * cpc + ul] = (int16_t)c_new;
-        if (fin) k.c[L.c_off * k.B + (size_t)b * L.C + u] = (int16_t)c_new;
+        if (fin) L.c[(size_t)b * L.C + u] = (int16_t)c_new;
         int32_t ao = a[SO];
         if (PEEP) {
             ao = sat16((int32_t)s.g[(4 * rows + row) * cpc + ul] + a[SO] + sat16(fast_rescale((int32_t)s.P[SO * cpc + ul] * c_new, L.f_c[SO])));   // Eq. 5
@@ -275,8 +275,8 @@ __device__ __forceinline__ void ws_proj_tile(const WaveCall &k, const WaveLayer 
             const int8_t h = (int8_t)sat8(fast_rescale((int32_t)a[e] + bias, L.f_proj) + L.zp_h);
             if (in && row < r.rows) {
                 out_unit[wv_img_off(row, col, k.ra)] = h;
-                if (last_layer) k.y[((size_t)t * k.B + b) * L.O + col] = h;
-                if (fin) k.h[L.h_off * k.B + (size_t)b * L.O + col] = h;
+                if (last_layer) wv_y_row(k, L, t, b)[col] = h;
+                if (fin) L.h[(size_t)b * L.O + col] = h;
             }
         }
     }
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         if (cta >= k.layer[l].cta0 && cta < k.layer[l].cta0 + k.layer[l].n * k.rg) r.li = l;
     if (r.li < 0) return;
     const WaveLayer &L = k.layer[r.li];
-    const bool proj = (L.flags & F_PROJECTION) != 0, last_layer = r.li == k.n_layers - 1;
+    const bool proj = (L.flags & F_PROJECTION) != 0, last_layer = L.last != 0;
     r.gu = (cta - L.cta0) / L.n;
     r.rank = cta - L.cta0 - r.gu * L.n;
     r.u0 = r.rank * L.cpc;
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     for (int i = threadIdx.x; i < 12 * WS_ROWS; i += WV_THREADS) s.st[i] = 0u;
     for (int i = threadIdx.x; i < r.rows * r.cells; i += WV_THREADS) {
         const int row = i / r.cells, ul = i - row * r.cells;
-        s.c[row * L.cpc + ul] = k.c[L.c_off * k.B + (size_t)(r.row0 + row) * L.C + r.u0 + ul];
+        s.c[row * L.cpc + ul] = L.c[(size_t)(r.row0 + row) * L.C + r.u0 + ul];
     }
     ptx::tc_fence_before();
     ptx::cta_sync();

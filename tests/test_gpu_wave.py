@@ -58,6 +58,14 @@ def test_wave_layernorm_of_small_deviations(shift, B, peephole):
     check(w)
 
 
+# both directions in one launch: few and many rows, one and two units
+@pytest.mark.parametrize("B", [3, 70, 140])
+@pytest.mark.parametrize("kw", [dict(), dict(projection=True, layernorm=True)], ids=lambda k: "+".join(sorted(k)) or "basic")
+def test_wave_bidirectional(kw, B):
+    from tests.test_gpu_bidirectional import test_bidirectional_matches_two_oracle_runs
+    test_bidirectional_matches_two_oracle_runs(kw, B, 9)
+
+
 def test_wave_timeout_is_reported_and_the_handle_recovers():
     import paper_2101_05453_b200 as qlstm
     w = random_layer_stack(9, 3, 48, 112, 64, projection=True, layernorm=True, T=5, B=40)
