@@ -83,7 +83,8 @@ struct WaveRole {
 // (the sums acc + b fit 32 bits: checked on the host).
 template <int G, bool LN, bool PEEP, bool IS_H>
 __device__ __forceinline__ void wv_gate_tile(const WaveLayer &L, const WaveSmem &s, uint32_t taddr, int pair0, int np, int part, int nparts,
-                                             int row, int rows, bool valid, const uint4 *xbuf, uint4 *gbuf, const uint32_t *cbuf)
+                                             int row, int rows, bool valid, const uint4 *xbuf, uint4 *gbuf, const uint32_t *cbuf,
+                                             uint64_t *full, uint32_t parity, volatile int *abort_flag)
 {
     constexpr int SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
     int32_t sum[4] = {0, 0, 0, 0};
@@ -129,6 +130,15 @@ __device__ __forceinline__ void wv_gate_tile(const WaveLayer &L, const WaveSmem 
         }
         gbuf[pr * rows + row] = make_uint4(w[0], w[1], w[2], w[3]);
     };
+    // X(t) may lie in L2: the first trip's is requested before the accumulators are waited for, a later one's a trip ahead
+    uint4 xa = make_uint4(0, 0, 0, 0), xb = xa;
+    if (IS_H && valid) {
+        const int p = G == 4 ? part : 2 * part, pb = G == 4 ? p + nparts : p + 1;
+        if (p < np) xa = xbuf[(pair0 + p) * rows + row];
+        if (pb < np) xb = xbuf[(pair0 + pb) * rows + row];
+    }
+    if (!__all_sync(0xffffffffu, wv_wait(full, parity, abort_flag))) return;
+    ptx::tc_fence_after();
     // four gates: two pairs nparts apart, eight columns each; three gates: two adjacent pairs, twelve columns in pieces of
     // four (np is then even)
 #pragma unroll 1
@@ -149,15 +159,16 @@ __device__ __forceinline__ void wv_gate_tile(const WaveLayer &L, const WaveSmem 
             for (int i = 0; i < 12; ++i) acc[i / 6][i % 6] = q[i >> 2][i & 3];
             acc[0][6] = acc[0][7] = acc[1][6] = acc[1][7] = 0;
         }
-        uint4 xa = make_uint4(0, 0, 0, 0), xb = xa;
-        if (IS_H && valid) {
-            xa = xbuf[(pair0 + p) * rows + row];
-            if (two) xb = xbuf[(pair0 + pb) * rows + row];
+        const uint4 x0 = xa, x1 = xb;
+        if (IS_H && valid) {                               // the next trip's X
+            const int pn = p + 2 * nparts, pbn = pb + 2 * nparts;
+            if (pn < np) xa = xbuf[(pair0 + pn) * rows + row];
+            if (pbn < np) xb = xbuf[(pair0 + pbn) * rows + row];
         }
         if (G == 4) ptx::tmem_ld_wait();
         if (valid) {
-            one(acc[0], p, xa);
-            if (two) one(acc[1], pb, xb);
+            one(acc[0], p, x0);
+            if (two) one(acc[1], pb, x1);
         }
     }
     if (IS_H && LN && valid) {
@@ -705,27 +716,30 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
         wv_walk(ctl, k.T, [&](const WaveOp &op, int t) -> bool {
             const int u = op.u, rows = r.rows[u], gu = r.gu[u];
             if (op.kind <= OP_P) {
-                const bool ok = wv_wait(&ctl->t_full[job & 1], (uint32_t)(job >> 1) & 1u, abort_flag);
-                if (__all_sync(0xffffffffu, ok)) {
+                // (after an abort the tile is skipped: on to the next meeting point)
+                uint64_t *full = &ctl->t_full[job & 1];
+                const uint32_t parity = (uint32_t)(job >> 1) & 1u;
+                const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(job & 1) * WV_ACC_COLS;
+                const bool valid = row < rows;
+                uint4 *gb = r.g[u];
+                uint4 *xb = gb + (size_t)(k.units == 1 ? 1 + (PEEP ? (t & 1) : 0) : (PEEP ? 1 : 0)) * r.pairs * rows;
+                const int pair0 = op.tile * L.ppt;
+                if (op.kind == OP_X) {
+                    wv_gate_tile<G, LN, PEEP, false>(L, s, ta, pair0, gate_tile_pairs(op.tile), part, nparts, row, rows, valid, nullptr, xb, nullptr, full, parity,
+                                                     abort_flag);
+                } else if (op.kind == OP_H) {
+                    wv_gate_tile<G, LN, PEEP, true>(L, s, ta, pair0, gate_tile_pairs(op.tile), part, nparts, row, rows, valid, xb, gb, r.c[u], full, parity,
+                                                    abort_flag);
+                } else if (__all_sync(0xffffffffu, wv_wait(full, parity, abort_flag))) {
                     ptx::tc_fence_after();
-                    const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(job & 1) * WV_ACC_COLS;
-                    const bool valid = row < rows;
-                    uint4 *gb = r.g[u];
-                    uint4 *xb = gb + (size_t)(k.units == 1 ? 1 + (PEEP ? (t & 1) : 0) : (PEEP ? 1 : 0)) * r.pairs * rows;
-                    const int pair0 = op.tile * L.ppt;
-                    if (op.kind == OP_X)
-                        wv_gate_tile<G, LN, PEEP, false>(L, s, ta, pair0, gate_tile_pairs(op.tile), part, nparts, row, rows, valid, nullptr, xb, nullptr);
-                    else if (op.kind == OP_H)
-                        wv_gate_tile<G, LN, PEEP, true>(L, s, ta, pair0, gate_tile_pairs(op.tile), part, nparts, row, rows, valid, xb, gb, r.c[u]);
-                    else
-                        wv_proj_tile(k, L, s, r, ta, op.tile * L.opt, r.outs - op.tile * L.opt < L.opt ? r.outs - op.tile * L.opt : L.opt, part, nparts,
-                                     row, valid, L.out_img + ((size_t)(t + 1) * k.nu + gu) * L.kb_h * k.ra * 128, r.row0[u] + row, t, last_layer);
-                    ptx::tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(&ctl->t_empty[job & 1]);
+                    wv_proj_tile(k, L, s, r, ta, op.tile * L.opt, r.outs - op.tile * L.opt < L.opt ? r.outs - op.tile * L.opt : L.opt, part, nparts, row, valid,
+                                 L.out_img + ((size_t)(t + 1) * k.nu + gu) * L.kb_h * k.ra * 128, r.row0[u] + row, t, last_layer);
                 }
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&ctl->t_empty[job & 1]);
                 ++job;
-                return true;                                   // (after an abort: on to the next meeting point)
+                return true;
             }
             unsigned *cnt = cnt0 + (size_t)gu * WC_PER_UNIT * WC_WORDS;
             if (op.kind == OP_S) {
@@ -1188,8 +1202,10 @@ static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool table
     k.gx_s = total(3, 3, k.tab, true) <= room;
     k.na = 2; k.nb = 2;
     while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
-    while (k.nb < WV_MAX_SLOTS && total(k.na, k.nb + 1, k.tab, k.gx_s) <= room) ++k.nb;
-    while (k.na < WV_MAX_SLOTS && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
+    // (two units keep their gate buffers in global memory and read them back through L1, which a third slot of weights would take
+    // away: eight 2048-cell layers, 256 rows 110 us per step with three, 106 with two)
+    while (k.nb < (k.units == 2 ? 2 : WV_MAX_SLOTS) && total(k.na, k.nb + 1, k.tab, k.gx_s) <= room) ++k.nb;
+    while (k.units == 1 && k.na < WV_MAX_SLOTS && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
     k.max_tab = k.tab ? s->max_tab : 0;
     smem = total(k.na, k.nb, k.tab, k.gx_s);
     return true;
