@@ -334,6 +334,9 @@ def main():
     n_l = len(w.layers)
     proj_ms = prof["projection_ms"] / max(args.steps, 1)
     rec_ms = prof["recurrent_ms"] / max(args.steps, 1)
+    wave = prof["projection_launches"] == 0              # the wavefront kernels: input term inside the step, one launch for all layers
+    if wave:
+        rec_ops += gemm_ops
     proj_tops = gemm_ops / (proj_ms * 1e-3) / 1e12 if proj_ms > 0 else 0.0
     rec_tops = rec_ops / (rec_ms * 1e-3) / 1e12 if rec_ms > 0 else 0.0
     sm_mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 1965.0
@@ -365,7 +368,12 @@ def main():
     alu_peak = 148 * INT_LANES_PER_SM * sm_ghz / 1e3                     # T int-op/s at the clock seen during the run
     rec_alu = int_ops / (rec_ms * 1e-3) / 1e12 if rec_ms > 0 else 0.0
     rec_bytes = T * B * (q0.n_cell * G0 * 2 + q0.n_output) + 2 * B * (q0.n_output + 2 * q0.n_cell)
-    roof_rec = {"kernel": "recurrent", "bound": "alu", "achieved": rec_alu, "peak": alu_peak, "unit": "Tint-op/s",
+    rec_launches = n_l
+    if wave:                                              # weights, x, y and the state once
+        rec_launches = 1
+        rec_bytes = (B * T * (q0.n_input + O) + 2 * B * sum(q.n_output + 2 * q.n_cell for q in w.layers)
+                     + sum(q.n_cell * G0 * (q.n_input + q.n_output) + (q.n_cell * q.n_output if q.flags & 1 else 0) for q in w.layers))
+    roof_rec = {"kernel": "wavefront (all layers and steps)" if wave else "recurrent", "bound": "alu", "achieved": rec_alu, "peak": alu_peak, "unit": "Tint-op/s",
                 "frac": rec_alu / alu_peak, "traffic": None,
                 "peak_source": f"148 SMs x {INT_LANES_PER_SM} int32 lanes x {sm_ghz:.3f} GHz (SM clock sampled during the run); "
                                "a derived model: the per-unit operation counts are this library's own leanest forms",
@@ -375,17 +383,17 @@ def main():
                 "activation_note": "achieved / frac count a sigmoid or tanh as the arithmetic of its fixed-point definition "
                                    f"({OPS_ACTIVATION} operations: the unit of work of the method); the kernel reads memoised "
                                    f"values instead ({OPS_ACTIVATION_LOOKUP} operations), which the second fraction counts",
-                "algorithmic_int_ops_per_launch": int_ops / n_l,
+                "algorithmic_int_ops_per_launch": int_ops / rec_launches,
                 "matmul_tops": rec_tops, "matmul_frac_of_int8_peak": rec_tops / int8_sustained,
                 "matmul_frac_of_2x_bf16_burst": rec_tops / int8_burst,
-                "hbm_frac": rec_bytes / (rec_ms / n_l * 1e-3) / 1e9 / peaks["hbm_gbs"] if rec_ms > 0 else None,
-                "ms_per_launch": rec_ms / n_l,
+                "hbm_frac": rec_bytes / (rec_ms / rec_launches * 1e-3) / 1e9 / peaks["hbm_gbs"] if rec_ms > 0 else None,
+                "ms_per_launch": rec_ms / rec_launches,
                 "us_per_layer_step": 1e3 * rec_ms / (n_l * T),
-                "phase_us_per_layer_step": {k: 1e3 * prof_phase[k] / (n_l * T) for k in
+                "phase_us_per_layer_step": None if wave else {k: 1e3 * prof_phase[k] / (n_l * T) for k in
                                             ("phase_a_ms", "matmul_a_ms", "wait_a_ms", "phase_b_ms", "wait_b_ms", "phase_c_ms", "wait_c_ms")},
-                "phase_note": "separate pass with the device phase timers on (they slow the kernel: "
+                "phase_note": None if wave else "separate pass with the device phase timers on (they slow the kernel: "
                               f"{1e3 * prof_phase['recurrent_ms'] / (n_l * T):.2f} us per layer-step in that pass)"}
-    if (args.config == NCU_RECURRENT["config"] and B == NCU_RECURRENT["batch"] and T == NCU_RECURRENT["steps"]
+    if (not wave and args.config == NCU_RECURRENT["config"] and B == NCU_RECURRENT["batch"] and T == NCU_RECURRENT["steps"]
             and recurrent_source_sha() == NCU_RECURRENT["source_sha"]):
         roof_rec["traffic"] = NCU_RECURRENT["bytes"]                                     # bytes per launch (one layer)
     # algorithmic HBM bytes of the recurrent kernel per launch: X read once, y written once, state in and out
@@ -397,8 +405,7 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": "int8", "data": "synthetic",
             "config": {"workload": f"config{args.config}-{w.config.name} batch {B} T {T}",
                        "layers": n_l, "n_input": w.layers[0].n_input, "n_cell": w.layers[0].n_cell,
-                       "n_output": O, "l2": "256 MiB buffer written between timed passes; X workspace "
-                       f"{T * B * w.layers[0].n_cell * 8 / 1e6:.0f} MB per layer exceeds L2"},
+                       "n_output": O, "l2": "256 MiB buffer written between timed passes"},
             "clocks": clocks, "e2e": e2e, "e2e_matches_device_run": e2e_matches,
             "gpu_launches": prof["projection_launches"] + prof["recurrent_launches"] + prof["other_launches"],
             "roofline": dominant, "roofline_projection": roof_proj, "roofline_recurrent": roof_rec}
@@ -462,7 +469,7 @@ def main():
                        projection_frac_of_2x_bf16_burst=tops / int8_burst,
                        recurrent_us_per_layer_step=1e3 * pr["recurrent_ms"] / (n * nl * wl.T))
         else:
-            ent.update(path="whole-stack kernel (layers as a wavefront, input projection inside the step)",
+            ent.update(path="one launch for all layers and steps (wavefront kernels; whole-stack kernel for one step of one or two rows)",
                        us_per_layer_step=1e3 * ms / (nl * wl.T))
         if wl.B <= 4:
             ent["streaming_us_per_call_T1"] = streaming_us(qh, wl)
@@ -486,7 +493,7 @@ def main():
             ms_layers, pr_l, n = time_passes(q1, w1, impl=(0, 2), profile=True)
             q1.set_impl(0, 0)
             line["latency_batch1"] = {"us_per_timestep_whole_stack": 1e3 * ms / T, "us_per_layer_step": 1e3 * ms / (T * n_l),
-                                      "ms_per_pass": ms, "kernel": "whole-stack kernel, one launch for all layers and steps",
+                                      "ms_per_pass": ms, "kernel": "one launch for all layers and steps",
                                       "layer_after_layer_us_per_timestep": 1e3 * ms_layers / T,
                                       "layer_after_layer_recurrent_us_per_layer_step": 1e3 * pr_l["recurrent_ms"] / (n * n_l * T),
                                       "streaming_us_per_call_T1": streaming_us(q1, w1)}
