@@ -366,12 +366,12 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     // accumulators: X tiles, H tiles, projection tiles
     const uint32_t col_h = (uint32_t)(nt * nr), col_p = (uint32_t)(2 * nt * nr);
     unsigned *cnt0 = L.cnt + (size_t)r.gu * WC_PER_UNIT * WC_WORDS;
-    // the order of a step's products, which the three service warps share: X of step 0, then per step
-    // H(t), X(t + 1), P(t) - or P before X in calls too short to be ahead of the layer below
+    // the order of a step's products, which the service warps share: H(t), X(t + 1), P(t) - or P before X in calls too short to be
+    // ahead of the layer below.  At the start H comes first: it does not wait for the layer below.
     auto walk = [&](auto f) -> bool {
-        if (!f(0, 0)) return false;
+        if (!f(1, 0) || !f(0, 0)) return false;
         for (int t = 0; t < T; ++t) {
-            if (!f(1, t)) return false;
+            if (t > 0 && !f(1, t)) return false;
             if (k.early && t + 1 < T && !f(0, t + 1)) return false;
             if (ntp > 0 && !f(2, t)) return false;
             if (!k.early && t + 1 < T && !f(0, t + 1)) return false;
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                     if (!tile((i & 1) == me, tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u, WS_CHUNKS,
                               G * 4096u))
                         return false;
-                    if (op == 1 && (i & 1) == me) wv_commit(&ctl->gate_full[i]);      // (X of this step was issued before)
+                    if (op == (t > 0 ? 1 : 0) && (i & 1) == me) wv_commit(&ctl->gate_full[i]);      // the step's last product
                 }
             }
             wv_commit(&ctl->op_empty[op]);
