@@ -30,6 +30,7 @@ struct WaveLayer {
     int cpc, ct, ctp, kpg;         // wave_small_sm100.cu: cells per block; cells of a tile, rounded up; k-blocks per chunk
     int opp, kpp;                  // ... outputs of a projection tile rounded up to 8, k-blocks per ring slot
     int kb_i, kb_h, kb_c;          // 128-byte k-blocks of the three products
+    size_t w_bytes;                // of the images (wave_sm100.cu)
     const int8_t *img_w, *img_r, *img_p;       // weights in the order and image in which the blocks stream them
     const int32_t *bx, *bh, *bln, *bp;
     const int16_t *P, *L;
@@ -61,6 +62,7 @@ struct WaveCall {
     int na, nb, b_slot;            // ring depths, bytes of a weight slot
     int max_cpc, max_kb_i, max_kb_h, max_kb_c;
     int gx_s;                      // gate buffers in shared memory
+    int w_evict;                   // weights with an evict-first hint
     int nbuf;                      // gate buffers per unit: [gate sums | X ...]
     int max_ppc, max_opc, max_tab;
     int8_t *y;
@@ -166,6 +168,22 @@ __device__ __forceinline__ void wv_commit(uint64_t *bar)
 {
     if (ptx::elect_one()) ptx::mma_commit(bar);
     __syncwarp();
+}
+
+// Where a stack's weights and the buffers between its phases together exceed L2 (WaveCall::w_evict), the weights pass through with
+// an evict-first hint: of the two it is the buffers, read again within a step, that should stay (eight 2048-cell layers: 64 rows
+// 46 -> 43 us per step, 256 rows 105 -> 100).  Weights that fit must not have it (five 1024-cell layers, 64 rows: 12.0 -> 16.3).
+__device__ __forceinline__ uint64_t wv_weights_policy()
+{
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ void wv_load_weights(void *dst, const void *src, uint32_t bytes, uint64_t *bar, uint64_t policy)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(ptx::smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(ptx::smem_u32(bar)), "l"(policy)
+                 : "memory");
 }
 
 // ---- fixed-point pieces ----------------------------------------------------------------------------------------------

@@ -652,6 +652,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
     } else if (warp == 1) {
         // ---------------- weights ----------------
         if (lane == 0) {
+            const uint64_t policy = wv_weights_policy();
             int slot = 0; uint32_t phase = 0;
             wv_walk(ctl, k.T, [&](const WaveOp &op, int) -> bool {
                 if (op.kind > OP_P) return true;
@@ -668,7 +669,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
                 for (int kb = 0; kb < nkb; ++kb) {
                     if (!wv_wait(&ctl->b_empty[slot], phase ^ 1u, abort_flag)) return false;
                     ptx::mbar_arrive_expect_tx(&ctl->b_full[slot], bytes);
-                    ptx::bulk_load_1d(b_ring + (size_t)slot * k.b_slot, src + (size_t)kb * bytes, bytes, &ctl->b_full[slot]);
+                    if (k.w_evict) wv_load_weights(b_ring + (size_t)slot * k.b_slot, src + (size_t)kb * bytes, bytes, &ctl->b_full[slot], policy);
+                    else ptx::bulk_load_1d(b_ring + (size_t)slot * k.b_slot, src + (size_t)kb * bytes, bytes, &ctl->b_full[slot]);
                     if (++slot == k.nb) { slot = 0; phase ^= 1u; }
                 }
                 return true;
@@ -1003,6 +1005,7 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
     }
     if (cudaGetLastError() != cudaSuccess) return QLSTM_ERR_CUDA;
     L.img_w = iw; L.img_r = ir; L.img_p = ip;
+    L.w_bytes = row_bytes * (L.kb_i + L.kb_h) + (proj ? (size_t)L.n * L.ntp * L.npadp * 128 * L.kb_c : 0);
     return QLSTM_OK;
 }
 
@@ -1200,6 +1203,12 @@ static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool table
     };
     k.tab = tables && s->tabs && total(2, 2, true, false) <= room;
     k.gx_s = total(3, 3, k.tab, true) <= room;
+    {
+        // 100 MB of the 126: the rest goes to activations
+        size_t used = k.gx_s ? 0 : gates * (size_t)pl.grid;
+        for (const WaveLayer &L : pl.layer) used += L.w_bytes;
+        k.w_evict = used > (size_t)100 << 20;
+    }
     k.na = 2; k.nb = 2;
     while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
     // (two units keep their gate buffers in global memory and read them back through L1, which a third slot of weights would take
