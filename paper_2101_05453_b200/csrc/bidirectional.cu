@@ -90,7 +90,7 @@ int qlstm_bidir_run(qlstm_bidir_t *q, const int8_t *x_dev, int T, int B, int8_t 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     // both directions side by side, each step's outputs written where they belong: two 512-cell layers each way, 16 rows, T = 150: 1290 us
     // one after the other, 672 like this
-    if (q->wave && wave_preferred(q->wave, T, B)) {
+    if (q->wave && wave_preferred(q->wave, T, B, true)) {
         if ((((uintptr_t)c_fwd_dev | (uintptr_t)c_bwd_dev) & 15) != 0) return QLSTM_ERR_ARG;       // as qlstm_run
         return bidir_wave_run(q->fwd, q->bwd, q->wave, x_dev, T, B, {h_fwd_dev, h_bwd_dev}, {c_fwd_dev, c_bwd_dev}, y_dev, st);
     }

@@ -95,10 +95,11 @@ struct WaveStack;
 // The first n_fwd layers are one stack; any that follow are a second one over the same x, backwards in time (bidirectional).
 int wave_create(const std::vector<const LayerParams *> &layers, int n_fwd, int max_T, int max_B, int sm_count, WaveStack **out);
 void wave_destroy(WaveStack *s);
-bool wave_supported(const WaveStack *s, int T, int B);
-bool wave_preferred(const WaveStack *s, int T, int B);             // supported and, by measurement, the faster path
+// tables: memoised nonlinearities, without which only the many-row form runs
+bool wave_supported(const WaveStack *s, int T, int B, bool tables);
+bool wave_preferred(const WaveStack *s, int T, int B, bool tables);      // supported and, by measurement, the faster path
 // h, c: state of the one or two stacks; y: rows of the stacks' outputs side by side; status2: another status word to clear, or
-// null.  tables: memoised nonlinearities.  The launch clears the status word itself.
+// null.  The launch clears the status word itself.
 int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
                 bool tables, cudaStream_t st, int *launches);
 // The two handles of a bidirectional stack and, where both directions fit one plan, the wavefront kernels that run them side by

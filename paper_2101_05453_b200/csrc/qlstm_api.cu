@@ -417,7 +417,7 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
     const int nl = (int)q->layers.size();
     // small batches: the whole stack in one launch (layers as a wavefront, input projection inside the step)
     if (!trace && (q->impl_rec == 0 || q->impl_rec == 8) && q->impl_proj != 1) {
-        if (q->impl_rec == 0 ? wave_preferred(q->wave, T, B) : wave_supported(q->wave, T, B)) {
+        if (q->impl_rec == 0 ? wave_preferred(q->wave, T, B, q->tables) : wave_supported(q->wave, T, B, q->tables)) {
             SpanGuard g(q, st, 1);
             int launches = 0;
             const int rc = launch_wave(q->wave, x_dev, T, B, {h_dev, nullptr}, {c_dev, nullptr}, y_dev, q->status, nullptr, q->tables, st, &launches);
@@ -559,7 +559,7 @@ int qlstm_debug_activation_tables(qlstm_t *q, int enable)
 {
     if (!q || enable < 0 || enable > 2) return QLSTM_ERR_ARG;
     int n = 0;
-    q->tables = enable == 1;
+    q->tables = enable != 0;
     for (auto &L : q->layers) {
         L.fast.dbg_no_tables = enable == 0;
         L.fast.dbg_general_kernel = enable == 2;

@@ -1228,11 +1228,11 @@ static int wave_mode(const WaveStack *s, int T, int B, bool tables, WaveCall &k,
     return -1;
 }
 
-bool wave_supported(const WaveStack *s, int T, int B)
+bool wave_supported(const WaveStack *s, int T, int B, bool tables)
 {
     WaveCall k;
     size_t smem;
-    return wave_mode(s, T, B, true, k, smem) >= 0;
+    return wave_mode(s, T, B, tables, k, smem) >= 0;
 }
 
 // Where the wavefront kernels are the faster path (measured, us per call, against the whole-stack kernel or layer after layer):
@@ -1242,9 +1242,9 @@ bool wave_supported(const WaveStack *s, int T, int B)
 // rows: one step 377 against 451, two 538 against 478; five layers, 256 rows: four steps 324 against 340, sixteen 926 against
 // 628; two layers always).  A single layer with layer norm beyond 64 rows, with nothing to overlap, does so too (2048 cells, 128
 // rows: 24.6 us per step against 28.2; 64 rows 20.9 against 17.7).
-bool wave_preferred(const WaveStack *s, int T, int B)
+bool wave_preferred(const WaveStack *s, int T, int B, bool tables)
 {
-    if (!wave_supported(s, T, B)) return false;
+    if (!wave_supported(s, T, B, tables)) return false;
     if (s->ragged) return true;
     if (T == 1 && B <= 2) return false;
     if (s->depth == 1 && s->ln && B > 64) return false;

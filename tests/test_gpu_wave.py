@@ -66,6 +66,26 @@ def test_wave_bidirectional(kw, B):
     test_bidirectional_matches_two_oracle_runs(kw, B, 9)
 
 
+# memoised nonlinearities off (0: the definition, which only the many-row form evaluates) or the per-layer kernels' general form
+# (2): whatever form the handle has, an ordinary call still runs, by the older kernels where it has to
+@pytest.mark.parametrize("enable", [0, 2])
+@pytest.mark.parametrize("dims,layers,B", [((48, 112, 64), 3, 5), ((19, 37, 23), 2, 5), ((48, 112, 64), 9, 40)])
+def test_wave_without_tables(dims, layers, B, enable):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(850 + B, layers, *dims, projection=True, layernorm=True, T=6, B=B)
+    h0, c0 = w.initial_state()
+    want = R.run(w.layers, w.x, h0, c0)
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        q.activation_tables(enable)
+        got = run_gpu(w, handle=q)
+        for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+            assert np.array_equal(g, r), name
+        if layers > 3:                                          # the many-row form without tables
+            got = run_gpu(w, handle=q, impl=(0, WAVE))
+            for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+                assert np.array_equal(g, r), name
+
+
 def test_wave_timeout_is_reported_and_the_handle_recovers():
     import paper_2101_05453_b200 as qlstm
     w = random_layer_stack(9, 3, 48, 112, 64, projection=True, layernorm=True, T=5, B=40)
