@@ -102,10 +102,10 @@ bool wave_preferred(const WaveStack *s, int T, int B, bool tables);      // supp
 // null.  The launch clears the status word itself.
 int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
                 bool tables, cudaStream_t st, int *launches);
-// The two handles of a bidirectional stack and, where both directions fit one plan, the wavefront kernels that run them side by
-// side (else *wave stays null and each handle has its own); qlstm_api.cu.
-int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b,
-                      WaveStack **wave);
+// The two handles of a bidirectional stack; then, once its workspaces are allocated, the wavefront kernels: where both directions
+// fit one plan those that run them side by side, else (*wave stays null) each handle's own; qlstm_api.cu.
+int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b);
+int bidir_wave_create(qlstm_t *f, qlstm_t *b, WaveStack **wave);
 int bidir_wave_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
                    cudaStream_t st);
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns);

@@ -330,24 +330,26 @@ static int create_handle(const qlstm_layer_t *layers, int n_layers, int max_T, i
 
 namespace ql {
 
-int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b,
-                      WaveStack **wave)
+int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b)
 {
     *f = *b = nullptr;
+    const int rc = create_handle(fwd, n_layers, max_T, max_B, device, false, f);
+    return rc != QLSTM_OK ? rc : create_handle(bwd, n_layers, max_T, max_B, device, false, b);
+}
+
+int bidir_wave_create(qlstm_t *f, qlstm_t *b, WaveStack **wave)
+{
     *wave = nullptr;
-    int rc = create_handle(fwd, n_layers, max_T, max_B, device, false, f);
-    if (rc == QLSTM_OK) rc = create_handle(bwd, n_layers, max_T, max_B, device, false, b);
-    if (rc != QLSTM_OK) return rc;
     std::vector<const LayerParams *> lp;
-    for (auto &L : (*f)->layers) lp.push_back(&L.p);
-    for (auto &L : (*b)->layers) lp.push_back(&L.p);
-    rc = wave_create(lp, n_layers, max_T, max_B, (*f)->sm_count, wave);
+    for (auto &L : f->layers) lp.push_back(&L.p);
+    for (auto &L : b->layers) lp.push_back(&L.p);
+    int rc = wave_create(lp, (int)f->layers.size(), f->max_T, f->max_B, f->sm_count, wave);
     // the directions do not go together: each has its own kernels
-    for (qlstm_t *q : {*f, *b}) {
+    for (qlstm_t *q : {f, b}) {
         if (rc != QLSTM_OK || *wave) break;
         lp.clear();
         for (auto &L : q->layers) lp.push_back(&L.p);
-        rc = wave_create(lp, n_layers, max_T, max_B, q->sm_count, &q->wave);
+        rc = wave_create(lp, (int)lp.size(), q->max_T, q->max_B, q->sm_count, &q->wave);
     }
     return rc;
 }

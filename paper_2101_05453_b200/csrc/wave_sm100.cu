@@ -1014,8 +1014,8 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
 static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool tables, WaveCall &k, size_t &smem);
 
 // Plans the wavefront kernels for a handle - one stack of n_fwd layers, or two that read the same x, the second one backwards in
-// time; *out stays null when the stack does not qualify: layers of different variants,
-// a scale with a left shift where none is expected, or sums that could leave int32.
+// time; *out stays null when the stack does not qualify (layers of different variants,
+// a scale with a left shift where none is expected, sums that could leave int32) or device memory does not suffice.
 int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T, int max_B, int sm_count, WaveStack **out)
 {
     *out = nullptr;
@@ -1046,7 +1046,13 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&s->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    auto fail = [&](int rc) { wave_destroy(s); return rc; };
+    // no memory left for a path that a handle can go without is no failure of the handle
+    auto fail = [&](int rc) {
+        const bool mem = rc == QLSTM_ERR_NOMEM || cudaPeekAtLastError() == cudaErrorMemoryAllocation;
+        if (mem) cudaGetLastError();
+        wave_destroy(s);
+        return mem ? QLSTM_OK : rc;
+    };
     s->tabs = true;
     std::vector<std::pair<uint8_t *, ActLineLayout>> tables;
     for (int l = 0; l < n; ++l) {

@@ -86,6 +86,42 @@ def test_wave_without_tables(dims, layers, B, enable):
                 assert np.array_equal(g, r), name
 
 
+# device memory for the handle but not for the wavefront plan (its weight images alone are 21 MB a stack): the handle goes without
+@pytest.mark.parametrize("directions", [1, 2])
+def test_wave_plan_that_does_not_fit_in_memory_is_left_out(directions):
+    import torch
+    import paper_2101_05453_b200 as qlstm
+    from tests.test_gpu_bidirectional import two_directions
+    f, b = two_directions(77, 1, 512, 2048, 2048, 2, 2)
+    make = lambda: qlstm.QLSTM(f.layers, 2, 2) if directions == 1 else qlstm.BiQLSTM(f.layers, b.layers, 2, 2)
+    h0, c0 = f.initial_state()
+    want = R.run(f.layers, f.x, h0, c0)
+    with qlstm.QLSTM(f.layers, 2, 2) as q:                      # (loads the kernels)
+        run_gpu(f, handle=q)
+        run_gpu(f, handle=q, impl=(0, WAVE))
+        run_gpu(f, handle=q, impl=(0, 2))
+    make().close()
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    q = make()
+    size = before - torch.cuda.mem_get_info()[0]
+    q.close()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - size + (14 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        q = make()
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    if directions == 1:
+        got = run_gpu(f, handle=q)
+        for g, r in zip(got[:3], want[:3]):
+            assert np.array_equal(g, r)
+        with pytest.raises(qlstm.QlstmError):
+            run_gpu(f, handle=q, impl=(0, WAVE))
+    q.close()
+
+
 def test_wave_timeout_is_reported_and_the_handle_recovers():
     import paper_2101_05453_b200 as qlstm
     w = random_layer_stack(9, 3, 48, 112, 64, projection=True, layernorm=True, T=5, B=40)
