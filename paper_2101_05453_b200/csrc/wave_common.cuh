@@ -93,6 +93,18 @@ __device__ __forceinline__ bool wv_wait(uint64_t *bar, uint32_t parity, volatile
     *abort_flag = 1;
     return false;
 }
+// The end of a copy or an MMA that has been issued, whatever the abort flag says: none may be in flight when a block leaves, in the
+// normal course (they have all been waited for, so this passes at once) or after an abort.  Bounded like the other waits.
+__device__ __forceinline__ void wv_drain(uint64_t *bar, uint32_t parity)
+{
+    for (uint32_t i = 0; i < 100000u; ++i)
+        if (ptx::mbar_try_wait_parked(bar, parity, 20000u)) return;
+}
+// the copies of a ring whose next one would go to `slot` with parity `phase` (before a slot's first copy: passes at once)
+__device__ __forceinline__ void wv_drain_ring(uint64_t *full, int n, int slot, uint32_t phase)
+{
+    for (int i = 0; i < n; ++i) wv_drain(&full[i], i < slot ? phase : phase ^ 1u);
+}
 __device__ __forceinline__ unsigned wv_ld_acquire(const unsigned *p)
 {
     unsigned v;
@@ -147,6 +159,14 @@ __device__ __forceinline__ void wv_wait_count_warp(const WaveCall &k, const unsi
     }
 }
 __device__ __forceinline__ void wv_epi_sync() { asm volatile("barrier.sync 1, 512;" ::: "memory"); }
+
+// all MMAs that this warp has issued, through a barrier of its own
+__device__ __forceinline__ void wv_drain_mmas(uint64_t *bar)
+{
+    if (ptx::elect_one()) ptx::mma_commit(bar);
+    __syncwarp();
+    wv_drain(bar, 0);
+}
 
 // The same for a whole warp that stays together.
 __device__ __forceinline__ bool wv_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag)

@@ -48,7 +48,7 @@ struct WaveOp { uint8_t kind, u, tile, pad; };
 
 struct WaveCtl {
     uint64_t a_full[WV_MAX_SLOTS], a_empty[WV_MAX_SLOTS], b_full[WV_MAX_SLOTS], b_empty[WV_MAX_SLOTS];
-    uint64_t t_full[2], t_empty[2], tab_full;
+    uint64_t t_full[2], t_empty[2], tab_full, mma_done;
     uint32_t tmem_base;
     int abort_flag;
     int exit_at;                   // meeting point of the epilogue threads at which they all leave
@@ -563,6 +563,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
         }
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&ctl->t_full[i], 1); ptx::mbar_init(&ctl->t_empty[i], WV_EPI / 32); }
         ptx::mbar_init(&ctl->tab_full, 1);
+        ptx::mbar_init(&ctl->mma_done, 1);
         ctl->abort_flag = 0;
         ctl->exit_at = 0x7fffffff;
         ptx::fence_barrier_init();
@@ -649,6 +650,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
             }
             return true;
         });
+        wv_drain_ring(ctl->a_full, k.na, slot, phase);
+        if (TAB) wv_drain(&ctl->tab_full, 0);
     } else if (warp == 1) {
         // ---------------- weights ----------------
         if (lane == 0) {
@@ -675,6 +678,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
                 }
                 return true;
             });
+            wv_drain_ring(ctl->b_full, k.nb, slot, phase);
         }
         __syncwarp();
     } else if (warp == 2) {
@@ -706,6 +710,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
             ++job;
             return true;
         });
+        wv_drain_mmas(&ctl->mma_done);
     } else if (warp >= WV_EPI_WARP0) {
         // ---------------- epilogues and elementwise work ----------------
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0;
@@ -759,9 +764,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
     // ---------------- teardown ----------------
     ptx::cta_sync();
     if (*abort_flag) {
-        // a wait ran out: give copies and MMAs in flight time to finish, then report
+        // a wait ran out (the service warps have waited for their copies and MMAs in flight): report
         if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
-        for (int i = 0; i < 200; ++i) __nanosleep(500);
     }
     ptx::cta_sync();
     if (warp == 2) {

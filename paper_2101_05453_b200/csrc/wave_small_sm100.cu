@@ -25,7 +25,7 @@ constexpr int WS_ROWS = 32;
 struct WsCtl {
     uint64_t w_full[WS_SLOTS], w_empty[WS_SLOTS];
     uint64_t op_full[3], op_empty[3];          // operands x, h, m
-    uint64_t gate_full[WS_MAX_TILES], acc_empty, p_full, p_empty, tab_full;
+    uint64_t gate_full[WS_MAX_TILES], acc_empty, p_full, p_empty, tab_full, mma_done[2];
     uint32_t tmem_base;
     int abort_flag, exit_at;
 };
@@ -332,6 +332,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         ptx::mbar_init(&ctl->p_full, 2);
         ptx::mbar_init(&ctl->p_empty, WV_EPI / 32);
         ptx::mbar_init(&ctl->tab_full, 1);
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(&ctl->mma_done[i], 1);
         ctl->abort_flag = 0;
         ctl->exit_at = 0x7fffffff;
         ptx::fence_barrier_init();
@@ -382,6 +383,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     if (warp == 0) {
         // ---------------- operands: x, h, m of a unit, each one contiguous copy ----------------
         if (lane == 0) {
+            int issued[3] = {0, 0, 0};                         // copies of each operand
             walk([&](int op, int t) -> bool {
                 const unsigned *cnt = nullptr;
                 unsigned target = 0;
@@ -405,8 +407,12 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                 wv_fence_async_global();
                 ptx::mbar_arrive_expect_tx(&ctl->op_full[op], bytes);
                 ptx::bulk_load_1d(smem + lay.act[op], src, bytes, &ctl->op_full[op]);
+                issued[op] = t + 1;
                 return true;
             });
+            for (int op = 0; op < 3; ++op)
+                if (issued[op]) wv_drain(&ctl->op_full[op], (uint32_t)(issued[op] - 1) & 1u);
+            wv_drain(&ctl->tab_full, 0);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -436,6 +442,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                     if (!put((op == 0 ? L.img_w : L.img_r) + (size_t)(r.rank * L.nt + i) * total, total, WS_CHUNKS * G * 4096u)) return false;
                 return true;
             });
+            wv_drain_ring(ctl->w_full, k.nb, slot, phase);
         }
         __syncwarp();
     } else if (warp < WV_EPI_WARP0) {
@@ -495,6 +502,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
             wv_commit(&ctl->op_empty[op]);
             return true;
         });
+        wv_drain_mmas(&ctl->mma_done[me]);
     } else if (warp >= WV_EPI_WARP0) {
         // ---------------- epilogues and elementwise work ----------------
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0, quarter = warp & 3, wq = (warp - WV_EPI_WARP0) >> 2;
@@ -544,9 +552,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     // ---------------- teardown ----------------
     ptx::cta_sync();
     if (*abort_flag) {
-        // a wait ran out: give copies and MMAs in flight time to finish, then report
+        // a wait ran out (the service warps have waited for their copies and MMAs in flight): report
         if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
-        for (int i = 0; i < 200; ++i) __nanosleep(500);
     }
     ptx::cta_sync();
     if (warp == 2) {

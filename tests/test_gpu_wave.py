@@ -136,3 +136,23 @@ def test_wave_timeout_is_reported_and_the_handle_recovers():
         got = run_gpu(w, handle=q, impl=(0, WAVE))
     for g, r in zip(got[:3], want[:3]):
         assert np.array_equal(g, r)
+
+
+# both forms, copies and MMAs in flight when the wait runs out: later calls on the same handle are not disturbed
+@pytest.mark.parametrize("layers,B", [(9, 40), (9, 128), (9, 20), (2, 150)])
+def test_wave_abort_leaves_nothing_in_flight(layers, B):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(860 + B, layers, 48, 112, 64, projection=True, layernorm=True, T=12, B=B)
+    h0, c0 = w.initial_state()
+    want = R.run(w.layers, w.x, h0, c0)
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        for limit in (300_000, 3_000_000):
+            q.debug_barrier_timeout(1, limit)
+            with pytest.raises(qlstm.QlstmError) as e:
+                run_gpu(w, handle=q, impl=(0, WAVE))
+            assert e.value.code == qlstm.binding.ERR_TIMEOUT
+            q.debug_barrier_timeout(0)
+            for _ in range(2):
+                got = run_gpu(w, handle=q, impl=(0, WAVE))
+                for g, r in zip(got[:3], want[:3]):
+                    assert np.array_equal(g, r)
