@@ -34,6 +34,12 @@ int qlstm_set_impl(qlstm_t *q, int projection_impl, int recurrent_impl);
  * reports QLSTM_ERR_TIMEOUT.  Nothing faults or hangs and the handle stays usable; 0 restores normal operation. */
 int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long long limit_ns);
 
+/* The wavefront kernels' plan for a call of T steps and B rows on this handle: out4 (host) receives the kernel's form (1 few rows:
+ * gate rows as the M side of the products; 0 many rows: batch rows as the M side; -1 none takes the call), the row groups that the
+ * batch is split into, the units of at most 128 rows of a group, and whether an ordinary call of these sizes takes this path. */
+int qlstm_debug_wave_plan(qlstm_t *q, int T, int B, int *out4);
+int qlstm_bidir_debug_wave_plan(qlstm_bidir_t *q, int T, int B, int *out4);
+
 /* Host logic of the persistent kernel's operand ring, exposed for tests (no device is touched).  The matmuls of
  * Section 3.2.4 / 3.2.8 stream their batch operand through `stages` ring stages that one producer fills and
  * `n_owners` MMA issuers drain; within a phase owner o uses the stages o, o + n_owners, ... only, so that no

@@ -24,7 +24,7 @@ EXPORTS = ["qlstm_create", "qlstm_run", "qlstm_run_host", "qlstm_input_projectio
            "qlstm_get_profile", "qlstm_device_info", "qlstm_eval_activations", "qlstm_eval_layernorm_row",
            "qlstm_eval_activation_tables", "qlstm_debug_activation_tables",
            "qlstm_layernorm_rows_static", "qlstm_debug_barrier_timeout", "qlstm_debug_ring_plan",
-           "qlstm_debug_projection_plan", "qlstm_debug_mma_i8_peak", "qlstm_debug_barrier_latency",
+           "qlstm_debug_wave_plan", "qlstm_bidir_debug_wave_plan", "qlstm_debug_projection_plan", "qlstm_debug_mma_i8_peak", "qlstm_debug_barrier_latency",
            "qlstm_bidir_create", "qlstm_bidir_run", "qlstm_bidir_last_status", "qlstm_bidir_destroy",
            "qlstm_calibrate", "qlstm_quantize_model", "qlstm_quantized_layers", "qlstm_quantized_scales",
            "qlstm_quantized_destroy"]
@@ -123,6 +123,9 @@ def lib():
         L.qlstm_eval_layernorm_row.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, Scale, C.c_void_p, C.c_void_p]
         L.qlstm_debug_barrier_timeout.restype = C.c_int
         L.qlstm_debug_barrier_timeout.argtypes = [C.c_void_p, C.c_int, C.c_ulonglong]
+        for f in (L.qlstm_debug_wave_plan, L.qlstm_bidir_debug_wave_plan):
+            f.restype = C.c_int
+            f.argtypes = [C.c_void_p, C.c_int, C.c_int, C.POINTER(C.c_int)]
         L.qlstm_debug_ring_plan.restype = C.c_int
         L.qlstm_debug_ring_plan.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int)]
         L.qlstm_debug_projection_plan.restype = C.c_int
@@ -291,6 +294,12 @@ class QLSTM:
     def debug_barrier_timeout(self, missing_arrivals: int, limit_ns: int = 0):
         _check(lib().qlstm_debug_barrier_timeout(self._h, missing_arrivals, limit_ns), "qlstm_debug_barrier_timeout")
 
+    def debug_wave_plan(self, T: int, B: int):
+        """(form, row groups, units, taken) of the wavefront kernels for a call; see qlstm_debug.h."""
+        out = (C.c_int * 4)()
+        _check(lib().qlstm_debug_wave_plan(self._h, T, B, out), "qlstm_debug_wave_plan")
+        return tuple(out)
+
     def device_info(self):
         a, b = C.c_int(), C.c_int()
         _check(lib().qlstm_device_info(self._h, C.byref(a), C.byref(b)), "qlstm_device_info")
@@ -312,6 +321,11 @@ class BiQLSTM:
     def run(self, x, T: int, B: int, h_fwd, c_fwd, h_bwd, c_bwd, y, stream: int = 0):
         _check(lib().qlstm_bidir_run(self._h, _dev_ptr(x), T, B, _dev_ptr(h_fwd), _dev_ptr(c_fwd), _dev_ptr(h_bwd),
                                      _dev_ptr(c_bwd), _dev_ptr(y), stream), "qlstm_bidir_run")
+
+    def debug_wave_plan(self, T: int, B: int):
+        out = (C.c_int * 4)()
+        _check(lib().qlstm_bidir_debug_wave_plan(self._h, T, B, out), "qlstm_bidir_debug_wave_plan")
+        return tuple(out)
 
     def last_status(self):
         _check(lib().qlstm_bidir_last_status(self._h), "qlstm_bidir_last_status")

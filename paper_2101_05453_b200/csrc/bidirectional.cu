@@ -10,6 +10,7 @@
 #include <new>
 
 #include "../../include/qlstm.h"
+#include "../../include/qlstm_debug.h"
 #include "fast_kernels.h"
 
 using namespace ql;
@@ -115,6 +116,8 @@ int qlstm_bidir_last_status(qlstm_bidir_t *q)
     const int a = qlstm_last_status(q->fwd), b = qlstm_last_status(q->bwd);
     return a != QLSTM_OK ? a : b;
 }
+
+int qlstm_bidir_debug_wave_plan(qlstm_bidir_t *q, int T, int B, int *out4) { return q ? wave_debug_plan(q->wave, T, B, true, out4) : QLSTM_ERR_ARG; }
 
 void qlstm_bidir_destroy(qlstm_bidir_t *q)
 {

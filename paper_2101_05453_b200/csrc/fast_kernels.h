@@ -97,6 +97,7 @@ int wave_create(const std::vector<const LayerParams *> &layers, int n_fwd, int m
 void wave_destroy(WaveStack *s);
 // tables: memoised nonlinearities, without which only the many-row form runs
 bool wave_supported(const WaveStack *s, int T, int B, bool tables);
+int wave_debug_plan(const WaveStack *s, int T, int B, bool tables, int *out4);       // include/qlstm_debug.h
 bool wave_preferred(const WaveStack *s, int T, int B, bool tables);      // supported and, by measurement, the faster path
 // h, c: state of the one or two stacks; y: rows of the stacks' outputs side by side; status2: another status word to clear, or
 // null.  The launch clears the status word itself.

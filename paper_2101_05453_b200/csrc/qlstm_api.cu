@@ -557,6 +557,8 @@ int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long 
     return QLSTM_OK;
 }
 
+int qlstm_debug_wave_plan(qlstm_t *q, int T, int B, int *out4) { return q ? wave_debug_plan(q->wave, T, B, q->tables, out4) : QLSTM_ERR_ARG; }
+
 int qlstm_debug_activation_tables(qlstm_t *q, int enable)
 {
     if (!q || enable < 0 || enable > 2) return QLSTM_ERR_ARG;

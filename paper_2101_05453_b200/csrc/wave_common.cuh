@@ -30,7 +30,7 @@ struct WaveLayer {
     int cpc, ct, ctp, kpg;         // wave_small_sm100.cu: cells per block; cells of a tile, rounded up; k-blocks per chunk
     int opp, kpp;                  // ... outputs of a projection tile rounded up to 8, k-blocks per ring slot
     int kb_i, kb_h, kb_c;          // 128-byte k-blocks of the three products
-    size_t w_bytes;                // of the images (wave_sm100.cu)
+    size_t w_size[3];              // bytes of the three images
     const int8_t *img_w, *img_r, *img_p;       // weights in the order and image in which the blocks stream them
     const int32_t *bx, *bh, *bln, *bp;
     const int16_t *P, *L;

@@ -28,6 +28,7 @@
 // Every wait is bounded; on expiry the block sets the abort word, all blocks see it at their next wait and leave, and the
 // host reports QLSTM_ERR_TIMEOUT.
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 #include <utility>
 #include <vector>
@@ -854,26 +855,28 @@ const void *wave_kernel_of(int G, bool ln, bool peep)
 
 }  // namespace
 
-// One way of sharing a stack out over the SMs: [0] batch as the M side (this file), [1] gate rows as the M side, for up to 32
-// rows per row group (wave_small_sm100.cu).
+constexpr int WV_MAX_ROWS = 256;
+
+// One way of sharing a stack out over the SMs: mode 0 batch as the M side (this file), mode 1 gate rows as the M side, for up to
+// 32 rows per row group (wave_small_sm100.cu).
 struct WavePlan {
-    bool ok = false;
-    int rg = 1, grid = 0;
+    int mode = 0, rg = 1, grid = 0;
+    bool ok = true, used = false;
     int max_ppc = 0, max_cpc = 0, max_opc = 0, b_slot = 0;
     std::vector<WaveLayer> layer;
 };
 
 struct WaveStack {
-    int n_layers = 0, max_T = 0, max_B = 0, max_smem = 0;
+    int n_layers = 0, max_T = 0, max_B = 0, max_smem = 0, sm_count = 0;
     int depth = 0;                 // layers of one stack (two of them: the directions of a bidirectional one)
     int y_stride = 0;
     int G = 4;
     bool ln = false, peep = false, tabs = false;
     bool ragged = false;           // some dimension is not a multiple of 16
-    WavePlan plan[2];
+    std::vector<WavePlan> plan;
+    int8_t by_rows[2][WV_MAX_ROWS + 1];        // plan of a call by its rows, [0] without and [1] with memoised nonlinearities; -1: none
     int max_tab = 0, max_kb_i = 0, max_kb_h = 0, max_kb_c = 0;
-    unsigned *zero = nullptr;      // counters, abort word, totals: cleared before every call
-    size_t cnt_words = 0, tot_words = 0;
+    unsigned *zero = nullptr;      // abort word, counters, totals: cleared before every call
     uint4 *gbuf = nullptr;
     uint32_t *cbuf = nullptr;
     std::vector<void *> owned;
@@ -930,35 +933,36 @@ bool wave_small_fits(const WaveStack *s, const std::vector<const LayerParams *> 
     return wave_small_smem(k, 2, s->peep) <= (size_t)s->max_smem;
 }
 
-// How many groups the rows of a batch are split into.  (Deep stacks: the layers already share out the SMs.)
-int wave_row_groups(const WaveStack *s, int mode, const std::vector<const LayerParams *> &lp, int max_B, int sm_count)
+// How many groups the B rows of a call are split into.  (Deep stacks: the layers already share out the SMs.)
+int wave_row_groups(const WaveStack *s, int mode, const std::vector<const LayerParams *> &lp, int B)
 {
-    const int n = (int)lp.size();
+    const int n = (int)lp.size(), sm_count = s->sm_count;
     int rg = 1;
     if (mode == 0) {
-        // more than 64 rows per group and at least 32 blocks left (one 2048-cell layer with layer norm, 256 rows: 40 us per step as
-        // one group of two units, 32 as four groups; two 1024-cell layers: 32 and 25)
-        while ((max_B + rg - 1) / rg > 64 && sm_count / (2 * rg * n) >= 32) rg *= 2;
+        // more than 64 rows per group and at least 32 blocks left (two 1024-cell layers, 256 rows: 32 us per step as one group of two
+        // units, 25 as two groups)
+        while ((B + rg - 1) / rg > 64 && sm_count / (2 * rg * n) >= 32) rg *= 2;
         return rg;
     }
     // As many as it takes for the few-row kernel to hold a group's rows, down to 9 blocks: it is the faster one even then (us per
     // step against the many-row kernel as one group: five 1024-cell CIFG layers, 64 rows 12.0 as two groups against 14.1; four
     // 1024-cell layers, 100 rows 24 as four against 28; eight 2048-cell layers, 32 rows 37 as two against 41).
-    while (!wave_small_fits(s, lp, rg, max_B, sm_count) && 2 * rg <= max_B && sm_count / (2 * rg * n) >= 9) rg *= 2;
-    if (!wave_small_fits(s, lp, rg, max_B, sm_count)) rg = 1;
+    while (!wave_small_fits(s, lp, rg, B, sm_count) && 2 * rg <= B && sm_count / (2 * rg * n) >= 9) rg *= 2;
+    if (!wave_small_fits(s, lp, rg, B, sm_count)) rg = 1;
     // Then, fewer blocks per group make every exchange cheaper (two 512-cell layers, 16 rows: 9.0 us per step with one group, 8.5
     // with four; one 2048-cell layer with layer norm and peephole, 32 rows: 26 and 17), but a block streams more weights per step:
     // below 16 blocks, or beyond 320 KB, the groups cost more than they save (the same layers with eight groups: 9.2 and 18; five
-    // 1024-cell layers, 4 rows: 7.5 with one group, 10.3 with two).
+    // 1024-cell layers, 4 rows: 7.5 with one group, 10.3 with two), unless a block has little to stream: up to 64 KB, groups go down
+    // to 9 blocks (us per call of 100 steps, 16 blocks and 9: three 256-cell layers, 64 rows 493 and 446; two, 32 rows 404 and 385).
     size_t bytes = 0;
     for (const LayerParams *p : lp)
         bytes = std::max(bytes, (size_t)p->N * (p->I + p->O) + ((p->flags & F_PROJECTION) ? (size_t)p->O * p->C : 0));
-    while (2 * rg <= max_B && sm_count / (2 * rg * n) >= 16 && bytes / (sm_count / (2 * rg * n)) <= 320 * 1024) rg *= 2;
+    for (int per; 2 * rg <= B && (per = sm_count / (2 * rg * n)) >= 9 && bytes / per <= (per >= 16 ? 320 : 64) * 1024;) rg *= 2;
     return rg;
 }
 
-// Shares of the blocks and weight images of one layer under plan `mode`; a qlstm_error.  L.n = 0: the plan does not work.
-int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, WaveLayer &L)
+// Shares of the blocks of one layer under `mode`, `per` blocks at most; false: the plan does not work.
+bool wave_share_layer(int mode, const LayerParams &p, int per, WaveLayer &L)
 {
     const bool proj = p.flags & F_PROJECTION;
     L.opc = 0; L.ntp = 0; L.opt = 4; L.npadp = 16; L.opp = 8; L.kpp = 1;
@@ -976,7 +980,7 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
             L.opt = wv_round((L.opc + L.ntp - 1) / L.ntp, 4);
             L.npadp = wv_round(L.opt, 16);
         }
-        if (L.npad > WV_ACC_COLS || L.npadp > WV_ACC_COLS || 2 * (4 * L.nt + L.ntp + 4) > WV_MAX_OPS) { L.n = 0; return QLSTM_OK; }
+        if (L.npad > WV_ACC_COLS || L.npadp > WV_ACC_COLS || 2 * (4 * L.nt + L.ntp + 4) > WV_MAX_OPS) return false;
     } else {
         L.cpc = (p.C + per - 1) / per;
         L.n = (p.C + L.cpc - 1) / L.cpc;
@@ -991,12 +995,46 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
             L.opp = wv_round(L.opt, 8);
             L.kpp = WS_SLOT_ROWS / L.opp;
         }
-        if (L.nt > 8 || (2 * L.nt + L.ntp) * 8 > 512) { L.n = 0; return QLSTM_OK; }
+        if (L.nt > 8 || (2 * L.nt + L.ntp) * 8 > 512) return false;
     }
     const size_t row_bytes = mode == 0 ? (size_t)L.n * L.nt * L.npad * 128 : (size_t)L.n * L.nt * p.G * L.ctp * 128;
-    auto kbs = [&](int kb) { return mode == 0 ? kb : wv_round(kb, L.kpg); };
-    int8_t *iw = (int8_t *)wv_alloc(s, row_bytes * kbs(L.kb_i)), *ir = (int8_t *)wv_alloc(s, row_bytes * kbs(L.kb_h)), *ip = nullptr;
-    if (proj) ip = (int8_t *)wv_alloc(s, (size_t)L.n * L.ntp * (mode == 0 ? L.npadp : L.opp) * 128 * L.kb_c);
+    auto kbs = [&](int kb) { return (size_t)(mode == 0 ? kb : wv_round(kb, L.kpg)); };
+    L.w_size[0] = row_bytes * kbs(L.kb_i);
+    L.w_size[1] = row_bytes * kbs(L.kb_h);
+    L.w_size[2] = proj ? (size_t)L.n * L.ntp * (mode == 0 ? L.npadp : L.opp) * 128 * L.kb_c : 0;
+    return true;
+}
+
+// The plan of `mode` with rg row groups, made on first request; its number in s->plan.
+int wave_plan(WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, int mode, int rg)
+{
+    for (size_t i = 0; i < s->plan.size(); ++i)
+        if (s->plan[i].mode == mode && s->plan[i].rg == rg) return (int)i;
+    WavePlan pl;
+    pl.mode = mode; pl.rg = rg;
+    int prev_n = 0;
+    for (size_t l = 0; l < lp.size() && pl.ok; ++l) {
+        WaveLayer M = base[l];
+        if (!wave_share_layer(mode, *lp[l], s->sm_count / ((int)lp.size() * rg), M)) { pl.ok = false; break; }
+        M.cta0 = pl.grid;
+        pl.grid += M.n * rg;
+        M.below = M.first ? 0 : prev_n;
+        prev_n = M.n;
+        pl.max_ppc = std::max(pl.max_ppc, M.ppc);
+        pl.max_cpc = std::max(pl.max_cpc, wv_round(M.cpc, 2));
+        pl.max_opc = std::max(pl.max_opc, wv_round(M.opc, 4));
+        pl.b_slot = mode == 1 ? WS_SLOT_ROWS * 128 : std::max(pl.b_slot, std::max(M.npad, (M.flags & F_PROJECTION) ? M.npadp : 0) * 128);
+        pl.layer.push_back(M);
+    }
+    s->plan.push_back(pl);
+    return (int)s->plan.size() - 1;
+}
+
+// The weight images of one layer of a plan.
+int wave_fill_images(WaveStack *s, int mode, const LayerParams &p, WaveLayer &L)
+{
+    const bool proj = p.flags & F_PROJECTION;
+    int8_t *iw = (int8_t *)wv_alloc(s, L.w_size[0]), *ir = (int8_t *)wv_alloc(s, L.w_size[1]), *ip = proj ? (int8_t *)wv_alloc(s, L.w_size[2]) : nullptr;
     if (!iw || !ir || (proj && !ip)) return QLSTM_ERR_NOMEM;
     if (mode == 0) {
         k_wave_tile_weights<<<2048, 256>>>(p.W, iw, p.G, p.N, p.I, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_i);
@@ -1007,15 +1045,65 @@ int wave_share_layer(WaveStack *s, int mode, const LayerParams &p, int per, Wave
         wave_small_tile_weights(p.R, ir, p.G, p.N, p.O, L.n, L.cpc, L.nt, L.ct, L.ctp, L.kb_h, L.kpg);
         if (proj) wave_small_tile_weights(p.Wproj, ip, 0, p.O, p.C, L.n, L.opc, L.ntp, L.opt, L.opp, L.kb_c, L.kpp);
     }
-    if (cudaGetLastError() != cudaSuccess) return QLSTM_ERR_CUDA;
     L.img_w = iw; L.img_r = ir; L.img_p = ip;
-    L.w_bytes = row_bytes * (L.kb_i + L.kb_h) + (proj ? (size_t)L.n * L.ntp * L.npadp * 128 * L.kb_c : 0);
-    return QLSTM_OK;
+    return cudaGetLastError() == cudaSuccess ? QLSTM_OK : QLSTM_ERR_CUDA;
+}
+
+// The description of a call of B rows under a plan; false if the plan cannot take it.
+bool wave_describe(const WaveStack *s, const WavePlan &pl, int T, int B, bool tables, WaveCall &k, size_t &smem)
+{
+    if (!pl.ok) return false;
+    memset(&k, 0, offsetof(WaveCall, layer));
+    k.T = T; k.B = B; k.n_layers = s->n_layers; k.rg = pl.rg;
+    wave_units(B, pl.rg, k.units, k.nu, k.ra);
+    const int rows = (B + k.nu - 1) / k.nu;
+    k.early = T >= 4 * s->depth;
+    k.max_ppc = pl.max_ppc; k.max_cpc = pl.max_cpc; k.max_opc = pl.max_opc; k.b_slot = pl.b_slot;
+    k.max_kb_i = s->max_kb_i; k.max_kb_h = s->max_kb_h; k.max_kb_c = s->max_kb_c;
+    const size_t room = (size_t)s->max_smem;
+    if (pl.mode == 1) {
+        if (rows > WV_SMALL_ROWS || !tables || !s->tabs) return false;
+        k.max_tab = s->max_tab;
+        for (const WaveLayer &L : pl.layer)
+            if ((2 * L.nt + L.ntp) * k.ra > 512) return false;
+        k.nb = 8;
+        while (k.nb > 2 && wave_small_smem(k, k.nb, s->peep) > room) --k.nb;
+        smem = wave_small_smem(k, k.nb, s->peep);
+        return smem <= room;
+    }
+    k.nrep = rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
+    k.nbuf = k.units == 1 ? (s->peep ? 3 : 2) : (s->peep ? 2 : 1);
+    const size_t gates = (size_t)k.units * pl.max_ppc * rows * (k.nbuf * 16 + 4);
+    auto total = [&](int na, int nb, bool tab, bool in_smem) {
+        return wv_layout(na, nb, pl.b_slot, pl.max_ppc, pl.max_opc, tab ? s->max_tab : 0, in_smem ? gates : 0).total;
+    };
+    if (total(2, 2, false, false) > room) return false;
+    k.tab = tables && s->tabs && total(2, 2, true, false) <= room;
+    k.gx_s = total(3, 3, k.tab, true) <= room;
+    {
+        // 100 MB of the 126: the rest goes to activations
+        size_t used = k.gx_s ? 0 : gates * (size_t)pl.grid;
+        for (const WaveLayer &L : pl.layer) used += L.w_size[0] + L.w_size[1] + L.w_size[2];
+        k.w_evict = used > (size_t)100 << 20;
+    }
+    k.na = 2; k.nb = 2;
+    while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
+    // (two units keep their gate buffers in global memory and read them back through L1, which a third slot of weights would take
+    // away: eight 2048-cell layers, 256 rows 110 us per step with three, 106 with two)
+    while (k.nb < (k.units == 2 ? 2 : WV_MAX_SLOTS) && total(k.na, k.nb + 1, k.tab, k.gx_s) <= room) ++k.nb;
+    while (k.units == 1 && k.na < WV_MAX_SLOTS && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
+    k.max_tab = k.tab ? s->max_tab : 0;
+    smem = total(k.na, k.nb, k.tab, k.gx_s);
+    return true;
+}
+
+// words of WaveStack::zero that a call of nu units of ra rows uses: abort word, counters, layer-norm totals
+size_t wave_zero_words(const WaveStack *s, int nu, int ra)
+{
+    return WC_WORDS + (size_t)s->n_layers * nu * (WC_PER_UNIT * WC_WORDS + (s->ln ? 2 * ra * 8 * 2 : 0));
 }
 
 }  // namespace
-
-static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool tables, WaveCall &k, size_t &smem);
 
 // Plans the wavefront kernels for a handle - one stack of n_fwd layers, or two that read the same x, the second one backwards in
 // time; *out stays null when the stack does not qualify (layers of different variants,
@@ -1042,10 +1130,12 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     s->n_layers = n;
     s->depth = n_fwd;
     s->max_T = max_T;
-    s->max_B = max_B < 256 ? max_B : 256;
+    s->max_B = max_B < WV_MAX_ROWS ? max_B : WV_MAX_ROWS;
+    s->sm_count = sm_count;
     s->G = lp[0]->G;
     s->ln = lp[0]->flags & F_LAYERNORM;
     s->peep = lp[0]->flags & F_PEEPHOLE;
+    memset(s->by_rows, -1, sizeof(s->by_rows));
     for (const LayerParams *p : lp) s->ragged = s->ragged || p->I % 16 || p->C % 16 || p->O % 16;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -1074,15 +1164,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
         tables.push_back({blob, lay});
         s->max_tab = std::max(s->max_tab, (int)lay.bytes);
     }
-    int nu_max = 1;
-    for (int mode = 0; mode < 2; ++mode) {
-        s->plan[mode].rg = wave_row_groups(s, mode, lp, s->max_B, sm_count);
-        nu_max = std::max(nu_max, (mode == 0 ? 2 : 1) * s->plan[mode].rg);
-    }
-    s->plan[1].ok = true;
-    const size_t rows_alloc = (size_t)s->max_B + 8 * nu_max;         // rows of all units, each rounded up to 8
     long long h_off = 0, c_off = 0;
-    int8_t *prev_img = nullptr;
     std::vector<WaveLayer> base;
     for (int l = 0; l < n; ++l) {
         const LayerParams &p = *lp[l];
@@ -1113,137 +1195,80 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
         L.last = l == n_fwd - 1 || l == n - 1;
         if (L.first) h_off = c_off = 0;
         if (L.last) { L.y_off = s->y_stride; s->y_stride += p.O; }
-        L.in_img = !L.first ? prev_img : (int8_t *)wv_alloc(s, (size_t)max_T * rows_alloc * L.kb_i * 128);
-        L.out_img = (int8_t *)wv_alloc(s, ((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
-        L.m_img = proj ? (int8_t *)wv_alloc(s, rows_alloc * L.kb_c * 128) : nullptr;
-        if (!L.in_img || !L.out_img || (proj && !L.m_img)) return fail(QLSTM_ERR_NOMEM);
-        if (proj && cudaMemset(L.m_img, 0, rows_alloc * L.kb_c * 128) != cudaSuccess) return fail(QLSTM_ERR_CUDA);
-        prev_img = L.out_img;
         L.h_off = h_off; L.c_off = c_off;
         h_off += p.O; c_off += p.C;
         L.tab = tables[l].first; L.tab_lay = tables[l].second;
         base.push_back(L);
     }
-    if (cudaFuncSetAttribute(wave_small_kernel(s->G, s->ln, s->peep), cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess)
-        s->plan[1].ok = false;
-    for (int mode = 1; mode >= 0; --mode) {
-        WavePlan &pl = s->plan[mode];
-        if (mode == 0) {
-            WaveCall k;
-            size_t smem;
-            pl.ok = !wave_describe(s, 1, max_T, s->max_B, true, k, smem);       // only where [1] does not cover every batch
-        }
-        int prev_n = 0;
-        for (int l = 0; l < n && pl.ok; ++l) {
-            const LayerParams &p = *lp[l];
-            WaveLayer M = base[l];
-            const int rc = wave_share_layer(s, mode, p, sm_count / (n * pl.rg), M);
+    // the kernels that exist for this stack's variants
+    bool form[2] = {true, cudaFuncSetAttribute(wave_small_kernel(s->G, s->ln, s->peep), cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) == cudaSuccess};
+    for (int tab = 0; tab < 2; ++tab) {
+        const void *f = tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
+        form[0] = form[0] && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) == cudaSuccess;
+    }
+    // A plan for every number of rows that a call may have: the few-row form where it can hold them, else the many-row one.  Calls
+    // of fewer rows than the handle was made for get the shares that a handle of their own would have (us per call of 100 steps, all
+    // calls with the shares of the handle's rows and like this: five 1024-cell CIFG layers made for 64 rows, one row 968 and 641; two
+    // 768-cell layers made for 256 rows, two rows 725 and 469, 64 rows 803 and 651).  The form that evaluates the nonlinearities by
+    // definition is the many-row one; it has the plans that other calls need.
+    WaveCall k;
+    size_t smem, rows_alloc = 0, zero_words = 0, g_bytes = 0, c_bytes = 0;
+    for (int tab = 1; tab >= 0; --tab)
+        for (int B = 1; B <= s->max_B; ++B)
+            for (int mode = tab; mode >= 0 && s->by_rows[tab][B] < 0; --mode) {
+                if (!form[mode]) continue;
+                const int rg = wave_row_groups(s, mode, lp, B);
+                bool made = false;
+                for (const WavePlan &pl : s->plan) made = made || (pl.mode == mode && pl.rg == rg && pl.used);
+                if (tab == 0 && !made) continue;
+                const int i = wave_plan(s, lp, base, mode, rg);
+                WavePlan &pl = s->plan[i];
+                if (!wave_describe(s, pl, max_T, B, tab, k, smem)) continue;
+                pl.used = true;
+                s->by_rows[tab][B] = (int8_t)i;
+                rows_alloc = std::max(rows_alloc, (size_t)k.nu * k.ra);
+                zero_words = std::max(zero_words, wave_zero_words(s, k.nu, k.ra));
+                if (mode == 0 && !k.gx_s) {
+                    // gate buffers and cell states in global memory, for batches whose buffers do not fit in shared memory
+                    const size_t cells = (size_t)pl.grid * k.units * pl.max_ppc * ((B + k.nu - 1) / k.nu);
+                    g_bytes = std::max(g_bytes, cells * k.nbuf * sizeof(uint4));
+                    c_bytes = std::max(c_bytes, cells * sizeof(uint32_t));
+                }
+            }
+    if (rows_alloc == 0) return fail(QLSTM_OK);
+    s->zero = (unsigned *)wv_alloc(s, zero_words * sizeof(unsigned));
+    s->gbuf = (uint4 *)wv_alloc(s, g_bytes);
+    s->cbuf = (uint32_t *)wv_alloc(s, c_bytes);
+    if (!s->zero || !s->gbuf || !s->cbuf) return fail(QLSTM_ERR_NOMEM);
+    int8_t *prev_img = nullptr;
+    for (int l = 0; l < n; ++l) {
+        WaveLayer &L = base[l];
+        const bool proj = L.flags & F_PROJECTION;
+        L.in_img = !L.first ? prev_img : (int8_t *)wv_alloc(s, (size_t)max_T * rows_alloc * L.kb_i * 128);
+        L.out_img = (int8_t *)wv_alloc(s, ((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
+        L.m_img = proj ? (int8_t *)wv_alloc(s, rows_alloc * L.kb_c * 128) : nullptr;
+        if (!L.in_img || !L.out_img || (proj && !L.m_img)) return fail(QLSTM_ERR_NOMEM);
+        prev_img = L.out_img;
+        for (WavePlan &pl : s->plan) {
+            if (!pl.used) continue;
+            WaveLayer &M = pl.layer[l];
+            M.in_img = L.in_img; M.out_img = L.out_img; M.m_img = L.m_img;
+            const int rc = wave_fill_images(s, pl.mode, *lp[l], M);
             if (rc != QLSTM_OK) return fail(rc);
-            if (M.n == 0) { pl.ok = false; break; }
-            M.cta0 = pl.grid;
-            pl.grid += M.n * pl.rg;
-            M.below = M.first ? 0 : prev_n;
-            prev_n = M.n;
-            pl.max_ppc = std::max(pl.max_ppc, M.ppc);
-            pl.max_cpc = std::max(pl.max_cpc, wv_round(M.cpc, 2));
-            pl.max_opc = std::max(pl.max_opc, wv_round(M.opc, 4));
-            pl.b_slot = mode == 1 ? WS_SLOT_ROWS * 128 : std::max(pl.b_slot, std::max(M.npad, (p.flags & F_PROJECTION) ? M.npadp : 0) * 128);
-            pl.layer.push_back(M);
-        }
-    }
-    s->cnt_words = (size_t)n * nu_max * WC_PER_UNIT * WC_WORDS + WC_WORDS;      // + abort word
-    s->tot_words = s->ln ? (size_t)n * 2 * rows_alloc * 8 * 2 : 0;
-    s->zero = (unsigned *)wv_alloc(s, (s->cnt_words + s->tot_words) * sizeof(unsigned));
-    if (!s->zero) return fail(QLSTM_ERR_NOMEM);
-    for (WavePlan &pl : s->plan) {
-        unsigned *c = s->zero;
-        long long *t = (long long *)(s->zero + s->cnt_words);
-        for (WaveLayer &L : pl.layer) {
-            L.cnt = c; c += (size_t)nu_max * WC_PER_UNIT * WC_WORDS;
-            if (s->ln) { L.totals = t; t += (size_t)2 * rows_alloc * 8; }
-        }
-    }
-    WavePlan &big = s->plan[0], &small = s->plan[1];
-    if (big.ok && wv_layout(2, 2, big.b_slot, big.max_ppc, big.max_opc, 0, 0).total > (size_t)s->max_smem) big.ok = false;
-    if (big.ok) {
-        // gate buffers and cell states in global memory, for batches whose buffers do not fit in shared memory
-        const size_t cells = (size_t)big.grid * big.max_ppc * (((size_t)s->max_B + big.rg - 1) / big.rg + 2);
-        s->gbuf = (uint4 *)wv_alloc(s, cells * 3 * sizeof(uint4));
-        s->cbuf = (uint32_t *)wv_alloc(s, cells * sizeof(uint32_t));
-        if (!s->gbuf || !s->cbuf) return fail(QLSTM_ERR_NOMEM);
-        for (int tab = 0; tab < 2; ++tab) {
-            const void *f = tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
-            if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) big.ok = false;
         }
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(QLSTM_ERR_CUDA);
-    if (!big.ok && !small.ok) return fail(QLSTM_OK);
     *out = s;
     return QLSTM_OK;
 }
 
-// The description of a call under plan `mode`; false if the plan cannot take it.
-static bool wave_describe(const WaveStack *s, int mode, int T, int B, bool tables, WaveCall &k, size_t &smem)
+static const WavePlan *wave_plan_of(const WaveStack *s, int T, int B, bool tables)
 {
-    const WavePlan &pl = s->plan[mode];
-    if (!pl.ok) return false;
-    memset(&k, 0, sizeof(k));
-    k.T = T; k.B = B; k.n_layers = s->n_layers; k.rg = pl.rg;
-    wave_units(B, pl.rg, k.units, k.nu, k.ra);
-    const int rows = (B + k.nu - 1) / k.nu;
-    k.early = T >= 4 * s->depth;
-    k.max_ppc = pl.max_ppc; k.max_cpc = pl.max_cpc; k.max_opc = pl.max_opc; k.b_slot = pl.b_slot;
-    k.max_kb_i = s->max_kb_i; k.max_kb_h = s->max_kb_h; k.max_kb_c = s->max_kb_c;
-    const size_t room = (size_t)s->max_smem;
-    if (mode == 1) {
-        if (rows > WV_SMALL_ROWS || !tables || !s->tabs) return false;
-        k.max_tab = s->max_tab;
-        for (const WaveLayer &L : pl.layer)
-            if ((2 * L.nt + L.ntp) * k.ra > 512) return false;
-        k.nb = 8;
-        while (k.nb > 2 && wave_small_smem(k, k.nb, s->peep) > room) --k.nb;
-        smem = wave_small_smem(k, k.nb, s->peep);
-        return smem <= room;
-    }
-    k.nrep = rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
-    k.nbuf = k.units == 1 ? (s->peep ? 3 : 2) : (s->peep ? 2 : 1);
-    const size_t gates = (size_t)k.units * pl.max_ppc * rows * (k.nbuf * 16 + 4);
-    auto total = [&](int na, int nb, bool tab, bool in_smem) {
-        return wv_layout(na, nb, pl.b_slot, pl.max_ppc, pl.max_opc, tab ? s->max_tab : 0, in_smem ? gates : 0).total;
-    };
-    k.tab = tables && s->tabs && total(2, 2, true, false) <= room;
-    k.gx_s = total(3, 3, k.tab, true) <= room;
-    {
-        // 100 MB of the 126: the rest goes to activations
-        size_t used = k.gx_s ? 0 : gates * (size_t)pl.grid;
-        for (const WaveLayer &L : pl.layer) used += L.w_bytes;
-        k.w_evict = used > (size_t)100 << 20;
-    }
-    k.na = 2; k.nb = 2;
-    while (k.na < 3 && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
-    // (two units keep their gate buffers in global memory and read them back through L1, which a third slot of weights would take
-    // away: eight 2048-cell layers, 256 rows 110 us per step with three, 106 with two)
-    while (k.nb < (k.units == 2 ? 2 : WV_MAX_SLOTS) && total(k.na, k.nb + 1, k.tab, k.gx_s) <= room) ++k.nb;
-    while (k.units == 1 && k.na < WV_MAX_SLOTS && total(k.na + 1, k.nb, k.tab, k.gx_s) <= room) ++k.na;
-    k.max_tab = k.tab ? s->max_tab : 0;
-    smem = total(k.na, k.nb, k.tab, k.gx_s);
-    return true;
+    if (!s || B < 1 || B > s->max_B || T < 1 || T > s->max_T || s->by_rows[tables][B] < 0) return nullptr;
+    return &s->plan[s->by_rows[tables][B]];
 }
 
-static int wave_mode(const WaveStack *s, int T, int B, bool tables, WaveCall &k, size_t &smem)
-{
-    if (!s || B < 1 || B > s->max_B || T < 1 || T > s->max_T) return -1;
-    for (int mode = 1; mode >= 0; --mode)
-        if (wave_describe(s, mode, T, B, tables, k, smem)) return mode;
-    return -1;
-}
-
-bool wave_supported(const WaveStack *s, int T, int B, bool tables)
-{
-    WaveCall k;
-    size_t smem;
-    return wave_mode(s, T, B, tables, k, smem) >= 0;
-}
+bool wave_supported(const WaveStack *s, int T, int B, bool tables) { return wave_plan_of(s, T, B, tables) != nullptr; }
 
 // Where the wavefront kernels are the faster path (measured, us per call, against the whole-stack kernel or layer after layer):
 // one step of one or two rows stays with the whole-stack kernel (eight 2048-cell layers 138 against 170, one 512-cell layer 10
@@ -1261,6 +1286,19 @@ bool wave_preferred(const WaveStack *s, int T, int B, bool tables)
     return T * 256 > s->depth * (B - 32);
 }
 
+int wave_debug_plan(const WaveStack *s, int T, int B, bool tables, int *out4)
+{
+    if (!out4) return QLSTM_ERR_ARG;
+    const WavePlan *pl = wave_plan_of(s, T, B, tables);
+    int units = 0, nu = 0, ra = 0;
+    if (pl) wave_units(B, pl->rg, units, nu, ra);
+    out4[0] = pl ? pl->mode : -1;
+    out4[1] = pl ? pl->rg : 0;
+    out4[2] = units;
+    out4[3] = wave_preferred(s, T, B, tables) ? 1 : 0;
+    return QLSTM_OK;
+}
+
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns)
 {
     if (!s) return;
@@ -1273,27 +1311,31 @@ int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[
 {
     WaveCall k;
     size_t smem = 0;
-    const int mode = wave_mode(s, T, B, tables, k, smem);
-    if (mode < 0) return QLSTM_ERR_DIM;
-    const WavePlan &pl = s->plan[mode];
+    const WavePlan *plan = wave_plan_of(s, T, B, tables);
+    if (!plan || !wave_describe(s, *plan, T, B, tables, k, smem)) return QLSTM_ERR_DIM;
+    const WavePlan &pl = *plan;
     k.y = y; k.y_stride = s->y_stride;
     k.gbuf = s->gbuf; k.cbuf = s->cbuf;
-    k.abort_word = s->zero + s->cnt_words - WC_WORDS;
+    k.abort_word = s->zero;
     k.status = status; k.status2 = status2;
     k.limit_ns = s->dbg_limit_ns ? s->dbg_limit_ns : WV_WAIT_LIMIT_NS;
     k.missing = s->dbg_missing;
+    unsigned *cnt = s->zero + WC_WORDS;
+    long long *totals = (long long *)(cnt + (size_t)s->n_layers * k.nu * WC_PER_UNIT * WC_WORDS);
     for (int l = 0; l < s->n_layers; ++l) {
         WaveLayer &L = k.layer[l];
         L = pl.layer[l];
+        L.cnt = cnt + (size_t)l * k.nu * WC_PER_UNIT * WC_WORDS;
+        L.totals = s->ln ? totals + (size_t)l * 2 * k.nu * k.ra * 8 : nullptr;
         L.h = h[L.dir] + L.h_off * B;
         L.c = c[L.dir] + L.c_off * B;
     }
     const size_t items = (size_t)T * B * ((pl.layer[0].I + 15) / 16);
     const int blocks = (int)std::min<size_t>(1184, (items + 255) / 256 + 32);
-    k_wave_prepare<<<blocks, 256, 0, st>>>(k, x, s->zero, s->cnt_words + s->tot_words);
+    k_wave_prepare<<<blocks, 256, 0, st>>>(k, x, s->zero, wave_zero_words(s, k.nu, k.ra));
     if (cudaGetLastError() != cudaSuccess) return QLSTM_ERR_CUDA;
     void *args[] = {(void *)&k};
-    const void *f = mode == 1 ? wave_small_kernel(s->G, s->ln, s->peep)
+    const void *f = pl.mode == 1 ? wave_small_kernel(s->G, s->ln, s->peep)
                               : (k.tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep));
     cudaError_t e = cudaLaunchCooperativeKernel(f, dim3(pl.grid), dim3(WV_THREADS), args, smem, st);
     if (e != cudaSuccess) {

@@ -86,6 +86,30 @@ def test_wave_without_tables(dims, layers, B, enable):
                 assert np.array_equal(g, r), name
 
 
+# a handle made for many rows, called with fewer: each call has the plan of a handle of its own size, whole row groups working
+@pytest.mark.parametrize("dims,layers,kw,max_B", [((48, 112, 64), 2, dict(), 256), ((48, 112, 64), 3, dict(projection=True, layernorm=True), 200),
+                                                  ((48, 112, 64), 9, dict(projection=True, layernorm=True, peephole=True), 140),
+                                                  ((19, 37, 23), 1, dict(projection=True, layernorm=True, cifg=True), 600)])
+def test_wave_calls_of_fewer_rows_than_the_handle(dims, layers, kw, max_B):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(870 + max_B, layers, *dims, T=6, B=300, **kw)
+    with qlstm.QLSTM(w.layers, 6, max_B) as q:
+        for T, B in ((6, 1), (5, 3), (6, 33), (2, 64), (6, 130), (6, 7), (6, 300)):
+            if B > max_B:
+                continue
+            with qlstm.QLSTM(w.layers, 6, B) as own:
+                assert q.debug_wave_plan(T, B) == own.debug_wave_plan(T, B)
+            form, groups, _, _ = q.debug_wave_plan(T, B)
+            assert form == (-1 if B > 256 else form) and groups <= B
+            x = np.ascontiguousarray(w.x[:T, :B])
+            h0, c0 = (np.concatenate([v.reshape(300, -1)[:B].ravel() for v in np.split(s, np.cumsum([300 * n for n in per])[:-1])])
+                      for s, per in zip(w.initial_state(), ([p.n_output for p in w.layers], [p.n_cell for p in w.layers])))
+            want = R.run(w.layers, x, h0, c0)
+            got = run_gpu(w, handle=q, x=x, h0=h0, c0=c0, impl=(0, WAVE if form >= 0 else 0))
+            for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+                assert np.array_equal(g, r), (name, T, B)
+
+
 # device memory for the handle but not for the wavefront plan (its weight images alone are 21 MB a stack): the handle goes without
 @pytest.mark.parametrize("directions", [1, 2])
 def test_wave_plan_that_does_not_fit_in_memory_is_left_out(directions):
