@@ -93,8 +93,8 @@ __device__ __forceinline__ bool wv_wait(uint64_t *bar, uint32_t parity, volatile
     *abort_flag = 1;
     return false;
 }
-// The end of a copy or an MMA that has been issued, whatever the abort flag says: none may be in flight when a block leaves, in the
-// normal course (they have all been waited for, so this passes at once) or after an abort.  Bounded like the other waits.
+// The end of a copy or an MMA that has been issued, for a block that leaves early: none may be in flight then.  Bounded like the
+// other waits.  (In the normal course all have been waited for.)
 __device__ __forceinline__ void wv_drain(uint64_t *bar, uint32_t parity)
 {
     for (uint32_t i = 0; i < 100000u; ++i)

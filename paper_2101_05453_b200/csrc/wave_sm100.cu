@@ -52,6 +52,8 @@ struct WaveCtl {
     uint64_t t_full[2], t_empty[2], tab_full, mma_done;
     uint32_t tmem_base;
     int abort_flag;
+    int end_slot[2];               // where the two copying warps stopped in their rings
+    uint32_t end_phase[2];
     int exit_at;                   // meeting point of the epilogue threads at which they all leave
     int n_ops, n_pro;              // operations of a step; of the prologue (X of step 0)
     WaveOp ops[WV_MAX_OPS];
@@ -501,6 +503,16 @@ __host__ __device__ inline WvLayout wv_layout(int na, int nb, int b_slot, int ma
     return l;
 }
 
+// A block that leaves early: its copies and MMAs in flight end (whole warps; `warp` 0 to 3 are the service warps).  Out of line, so
+// that the kernel's loops keep their shape.
+__device__ __noinline__ void wv_drain_block(WaveCtl *ctl, int na, int nb, bool tab, int warp)
+{
+    if (warp == 0) wv_drain_ring(ctl->a_full, na, ctl->end_slot[0], ctl->end_phase[0]);
+    else if (warp == 1) wv_drain_ring(ctl->b_full, nb, ctl->end_slot[1], ctl->end_phase[1]);
+    else if (warp == 2) wv_drain_mmas(&ctl->mma_done);
+    else if (warp == 3 && tab) wv_drain(&ctl->tab_full, 0);
+}
+
 template <int G, bool LN, bool PEEP, bool TAB>
 __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_constant__ WaveCall k)
 {
@@ -651,8 +663,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
             }
             return true;
         });
-        wv_drain_ring(ctl->a_full, k.na, slot, phase);
-        if (TAB) wv_drain(&ctl->tab_full, 0);
+        if (lane == 0) { ctl->end_slot[0] = slot; ctl->end_phase[0] = phase; }
     } else if (warp == 1) {
         // ---------------- weights ----------------
         if (lane == 0) {
@@ -679,7 +690,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
                 }
                 return true;
             });
-            wv_drain_ring(ctl->b_full, k.nb, slot, phase);
+            ctl->end_slot[1] = slot; ctl->end_phase[1] = phase;
         }
         __syncwarp();
     } else if (warp == 2) {
@@ -711,7 +722,6 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
             ++job;
             return true;
         });
-        wv_drain_mmas(&ctl->mma_done);
     } else if (warp >= WV_EPI_WARP0) {
         // ---------------- epilogues and elementwise work ----------------
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0;
@@ -765,7 +775,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_sm100(const __grid_const
     // ---------------- teardown ----------------
     ptx::cta_sync();
     if (*abort_flag) {
-        // a wait ran out (the service warps have waited for their copies and MMAs in flight): report
+        // a wait ran out: copies and MMAs in flight end, then report
+        wv_drain_block(ctl, k.na, k.nb, TAB, warp);
         if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
     }
     ptx::cta_sync();

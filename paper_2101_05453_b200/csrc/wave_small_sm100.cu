@@ -28,6 +28,9 @@ struct WsCtl {
     uint64_t gate_full[WS_MAX_TILES], acc_empty, p_full, p_empty, tab_full, mma_done[2];
     uint32_t tmem_base;
     int abort_flag, exit_at;
+    int op_copies[3];              // copies of each operand that have been requested
+    int end_slot;                  // where the weights' warp stopped in its ring
+    uint32_t end_phase;
 };
 
 // [weight ring][x][h][m][control][constants][statistics][tables][gates][cell states]
@@ -282,6 +285,22 @@ __device__ __forceinline__ void ws_proj_tile(const WaveCall &k, const WaveLayer 
     }
 }
 
+// A block that leaves early: its copies and MMAs in flight end (whole warps; `warp` 0 to 3 are the service warps).  Out of line, so
+// that the kernel's loops keep their shape (us per call of 100 steps, five 1024-cell CIFG layers, 4 rows: 660 without, 665 like this,
+// 678 inline at the end of each role).
+__device__ __noinline__ void ws_drain(WsCtl *ctl, int nb, int warp)
+{
+    if (warp == 0) {
+        for (int op = 0; op < 3; ++op)
+            if (ctl->op_copies[op]) wv_drain(&ctl->op_full[op], (uint32_t)(ctl->op_copies[op] - 1) & 1u);
+        wv_drain(&ctl->tab_full, 0);
+    } else if (warp == 1) {
+        wv_drain_ring(ctl->w_full, nb, ctl->end_slot, ctl->end_phase);
+    } else if (warp < WV_EPI_WARP0) {
+        wv_drain_mmas(&ctl->mma_done[warp - 2]);
+    }
+}
+
 template <int G, bool LN, bool PEEP>
 __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid_constant__ WaveCall k)
 {
@@ -335,6 +354,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         for (int i = 0; i < 2; ++i) ptx::mbar_init(&ctl->mma_done[i], 1);
         ctl->abort_flag = 0;
         ctl->exit_at = 0x7fffffff;
+        for (int i = 0; i < 3; ++i) ctl->op_copies[i] = 0;
         ptx::fence_barrier_init();
         ptx::mbar_arrive_expect_tx(&ctl->tab_full, L.tab_lay.bytes);
         ptx::bulk_load_1d(smem + lay.tab, L.tab, L.tab_lay.bytes, &ctl->tab_full);
@@ -383,7 +403,6 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     if (warp == 0) {
         // ---------------- operands: x, h, m of a unit, each one contiguous copy ----------------
         if (lane == 0) {
-            int issued[3] = {0, 0, 0};                         // copies of each operand
             walk([&](int op, int t) -> bool {
                 const unsigned *cnt = nullptr;
                 unsigned target = 0;
@@ -407,12 +426,9 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                 wv_fence_async_global();
                 ptx::mbar_arrive_expect_tx(&ctl->op_full[op], bytes);
                 ptx::bulk_load_1d(smem + lay.act[op], src, bytes, &ctl->op_full[op]);
-                issued[op] = t + 1;
+                ctl->op_copies[op] = t + 1;
                 return true;
             });
-            for (int op = 0; op < 3; ++op)
-                if (issued[op]) wv_drain(&ctl->op_full[op], (uint32_t)(issued[op] - 1) & 1u);
-            wv_drain(&ctl->tab_full, 0);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -442,7 +458,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                     if (!put((op == 0 ? L.img_w : L.img_r) + (size_t)(r.rank * L.nt + i) * total, total, WS_CHUNKS * G * 4096u)) return false;
                 return true;
             });
-            wv_drain_ring(ctl->w_full, k.nb, slot, phase);
+            ctl->end_slot = slot; ctl->end_phase = phase;
         }
         __syncwarp();
     } else if (warp < WV_EPI_WARP0) {
@@ -502,7 +518,6 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
             wv_commit(&ctl->op_empty[op]);
             return true;
         });
-        wv_drain_mmas(&ctl->mma_done[me]);
     } else if (warp >= WV_EPI_WARP0) {
         // ---------------- epilogues and elementwise work ----------------
         const int tid = threadIdx.x - 32 * WV_EPI_WARP0, quarter = warp & 3, wq = (warp - WV_EPI_WARP0) >> 2;
@@ -552,7 +567,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     // ---------------- teardown ----------------
     ptx::cta_sync();
     if (*abort_flag) {
-        // a wait ran out (the service warps have waited for their copies and MMAs in flight): report
+        // a wait ran out: copies and MMAs in flight end, then report
+        ws_drain(ctl, k.nb, warp);
         if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
     }
     ptx::cta_sync();
