@@ -63,33 +63,35 @@ bool pack_quads(const int32_t *v, int amax, std::vector<uint32_t> &out)
     return true;
 }
 
-// quotients of the definition for |x| = 0 .. 32768: sigmoid, gate tanh, cell tanh; bad: they are not symmetric
-bool act_domain(int m_cell, std::vector<int32_t> &v, bool &bad_out)
+// quotients of the definition for |x| = 0 .. 32768: sigmoid, gate tanh, cell tanh; one more word: they are not symmetric
+bool act_domain(ActDomains &dom, int m_cell)
 {
+    std::vector<int32_t> &v = dom.of[m_cell];
+    if (!v.empty()) return true;
     int32_t *v_dev = nullptr;
-    if (cudaMalloc(&v_dev, (3 * ACT_DOMAIN + 1) * sizeof(int32_t)) != cudaSuccess) return false;
+    const size_t n = 3 * ACT_DOMAIN + 1;
+    if (cudaMalloc(&v_dev, n * sizeof(int32_t)) != cudaSuccess) return false;
     int *bad_dev = v_dev + 3 * ACT_DOMAIN;
-    v.resize((size_t)3 * ACT_DOMAIN + 1);
     bool ok = cudaMemset(bad_dev, 0, sizeof(int)) == cudaSuccess;
     if (ok) {
+        v.resize(n);
         k_act_domain<<<(ACT_DOMAIN + 255) / 256, 256>>>(m_cell, v_dev, bad_dev);
-        ok = cudaGetLastError() == cudaSuccess && cudaMemcpy(v.data(), v_dev, v.size() * sizeof(int32_t), cudaMemcpyDeviceToHost) == cudaSuccess;
+        ok = cudaGetLastError() == cudaSuccess && cudaMemcpy(v.data(), v_dev, n * sizeof(int32_t), cudaMemcpyDeviceToHost) == cudaSuccess;
     }
     cudaFree(v_dev);
-    bad_out = v.back() != 0;
+    if (!ok) v.clear();
     return ok;
 }
 
 }  // namespace
 
-bool act_tables_build(int m_cell, size_t max_bytes, uint8_t **blob_dev, ActTabLayout *lay)
+bool act_tables_build(ActDomains &dom, int m_cell, size_t max_bytes, uint8_t **blob_dev, ActTabLayout *lay)
 {
     *blob_dev = nullptr;
     *lay = ActTabLayout{0, 0, 0, 0, 0, 0, 0};
-    std::vector<int32_t> v;
-    bool bad = false;
-    if (!act_domain(m_cell, v, bad)) return false;
-    if (bad) return true;
+    if (!act_domain(dom, m_cell)) return false;
+    const std::vector<int32_t> &v = dom.of[m_cell];
+    if (v.back() != 0) return true;
     const int32_t *sg = v.data(), *tz = sg + ACT_DOMAIN, *tc = tz + ACT_DOMAIN;
     for (int a = 0; a < ACT_DOMAIN; ++a)
         if (sg[a] < 0 || sg[a] > 32768 || tc[a] < 0 || tc[a] > 32768) return true;
@@ -181,14 +183,13 @@ bool build_lines(const std::vector<int32_t> &f, int lo, int hi, int sh, int k, s
 
 }  // namespace
 
-bool act_lines_build(int m_cell, uint8_t **blob_dev, ActLineLayout *lay)
+bool act_lines_build(ActDomains &dom, int m_cell, std::vector<uint8_t> &blob, ActLineLayout *lay)
 {
-    *blob_dev = nullptr;
+    blob.clear();
     *lay = ActLineLayout{0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    std::vector<int32_t> v;
-    bool bad = false;
-    if (!act_domain(m_cell, v, bad)) return false;
-    if (bad) return true;
+    if (!act_domain(dom, m_cell)) return false;
+    const std::vector<int32_t> &v = dom.of[m_cell];
+    if (v.back() != 0) return true;
     // values over the signed domain, as the definition's last step forms them
     std::vector<int32_t> f[3];
     for (int t = 0; t < 3; ++t) {
@@ -219,14 +220,10 @@ bool act_lines_build(int m_cell, uint8_t **blob_dev, ActLineLayout *lay)
     lay->sig_at = 4u * (32768u >> ACT_SIG_SH);
     lay->tz_at = tz_off - 4u * (uint32_t)(lay->tz_lo >> ACT_TZ_SH);
     lay->tc_at = tc_off - 4u * (uint32_t)(lay->tc_lo >> lay->tc_sh);
-    std::vector<uint8_t> blob(bytes, 0);
+    blob.assign(bytes, 0);
     memcpy(blob.data(), sig.data(), sig.size() * 4);
     memcpy(blob.data() + tz_off, tz.data(), tz.size() * 4);
     if (m_cell != 3) memcpy(blob.data() + tc_off, tc.data(), tc.size() * 4);
-    uint8_t *d = nullptr;
-    if (cudaMalloc(&d, bytes) != cudaSuccess) return false;
-    if (cudaMemcpy(d, blob.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(d); return false; }
-    *blob_dev = d;
     lay->bytes = bytes;
     return true;
 }

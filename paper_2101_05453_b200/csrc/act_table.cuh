@@ -21,6 +21,7 @@
 #pragma once
 
 #include <cstdint>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -103,10 +104,13 @@ __device__ __forceinline__ int32_t tab_tanh_cell(const ActTabs &t, int32_t x)
     return t.tc_mode == 2 ? tab_plain_odd(t.tc, t.tc_amax, x) : tab_packed(t.tc, t.tc_amax, x);
 }
 
+// The definition over the whole domain, per cell format: evaluated once while a handle is created, for all tables of all its layers.
+struct ActDomains { std::vector<int32_t> of[16]; };
+
 // Builds the blob of a layer whose cell state has m_cell integer bits (act_table.cu).  *blob_dev = nullptr and
 // lay->bytes = 0 when a check fails or the blob would exceed max_bytes (the caller then keeps the arithmetic path);
 // false only on a CUDA error.
-bool act_tables_build(int m_cell, size_t max_bytes, uint8_t **blob_dev, ActTabLayout *lay);
+bool act_tables_build(ActDomains &dom, int m_cell, size_t max_bytes, uint8_t **blob_dev, ActTabLayout *lay);
 
 // ---- piecewise-linear form, for the wavefront kernels ----------------------------------------------------------------
 //
@@ -153,8 +157,8 @@ __device__ __forceinline__ int32_t line_tanh_cell(const ActLines &t, int32_t x)
     return act_line_value((int32_t)lds_u32(t.tc + (uint32_t)((x >> t.tc_sh) << 2)), x, t.tc_sh, t.tc_k);
 }
 
-// Builds the blob for a cell format; *blob_dev = nullptr and lay->bytes = 0 when some input has no entry that yields its value
+// Builds the blob (host memory) for a cell format; empty and lay->bytes = 0 when some input has no entry that yields its value
 // (the caller then evaluates the definition); false only on a CUDA error.
-bool act_lines_build(int m_cell, uint8_t **blob_dev, ActLineLayout *lay);
+bool act_lines_build(ActDomains &dom, int m_cell, std::vector<uint8_t> &blob, ActLineLayout *lay);
 
 }  // namespace ql

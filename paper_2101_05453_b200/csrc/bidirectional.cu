@@ -67,14 +67,15 @@ int qlstm_bidir_create(const qlstm_layer_t *fwd_layers, const qlstm_layer_t *bwd
     q->n_input = fwd_layers[0].n_input;
     q->o_fwd = fwd_layers[n_layers - 1].n_output;
     q->o_bwd = bwd_layers[n_layers - 1].n_output;
-    int rc = bidir_pair_create(fwd_layers, bwd_layers, n_layers, max_T, max_B, device, &q->fwd, &q->bwd);
+    ActDomains dom;
+    int rc = bidir_pair_create(fwd_layers, bwd_layers, n_layers, max_T, max_B, device, dom, &q->fwd, &q->bwd);
     if (rc == QLSTM_OK) {
         const size_t rows = (size_t)max_T * max_B;
         if (cudaMalloc(&q->x_rev, rows * q->n_input) != cudaSuccess || cudaMalloc(&q->y_fwd, rows * q->o_fwd) != cudaSuccess ||
             cudaMalloc(&q->y_bwd, rows * q->o_bwd) != cudaSuccess)
             rc = QLSTM_ERR_NOMEM;
     }
-    if (rc == QLSTM_OK) rc = bidir_wave_create(q->fwd, q->bwd, &q->wave);        // last: a handle can go without
+    if (rc == QLSTM_OK) rc = bidir_wave_create(q->fwd, q->bwd, dom, &q->wave);        // last: a handle can go without
     if (rc != QLSTM_OK) { qlstm_bidir_destroy(q); return rc; }
     *out = q;
     return QLSTM_OK;

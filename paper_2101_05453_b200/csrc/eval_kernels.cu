@@ -68,7 +68,8 @@ int qlstm_eval_activation_tables(int cell_int_bits, int max_bytes, int16_t *sigm
     int *layout_out6 = layout_out7;
     uint8_t *blob = nullptr;
     ql::ActTabLayout lay;
-    if (!ql::act_tables_build(cell_int_bits, (size_t)max_bytes, &blob, &lay)) return QLSTM_ERR_CUDA;
+    ql::ActDomains dom;
+    if (!ql::act_tables_build(dom, cell_int_bits, (size_t)max_bytes, &blob, &lay)) return QLSTM_ERR_CUDA;
     layout_out6[0] = (int)lay.bytes; layout_out6[1] = (int)lay.tz_off; layout_out6[2] = (int)lay.tc_off;
     layout_out6[3] = lay.tz_amax; layout_out6[4] = lay.tc_amax; layout_out6[5] = lay.tc_mode; layout_out7[6] = lay.sig_packed;
     if (!blob) return QLSTM_OK;

@@ -56,10 +56,10 @@ struct FastLayer {
 int fast_scratch_init(FastScratch &s, int max_B, int maxC, int maxO, int maxN, int sm_count);
 void fast_scratch_destroy(FastScratch &s);
 
-int fast_layer_init(FastLayer &f, const LayerParams &p, const FastScratch &s, int max_T, int max_B);
+int fast_layer_init(FastLayer &f, const LayerParams &p, const FastScratch &s, ActDomains &dom, int max_T, int max_B);
 void fast_layer_destroy(FastLayer &f);
 int fast_projection_init(FastLayer &f, const LayerParams &p);
-int fast_recurrent_init(FastLayer &f, const LayerParams &p, const FastScratch &s, int max_B);
+int fast_recurrent_init(FastLayer &f, const LayerParams &p, const FastScratch &s, ActDomains &dom, int max_B);
 
 bool fast_projection_supported(const FastLayer &f, const LayerParams &p);
 cudaError_t launch_projection_fast(const FastLayer &f, const LayerParams &p, const int8_t *x, int rows, int16_t *X,
@@ -93,7 +93,9 @@ int stack_small_groups(const StackSmall *s, int *blocks_per_layer);     // layer
 // 256 rows, any dimensions.
 struct WaveStack;
 // The first n_fwd layers are one stack; any that follow are a second one over the same x, backwards in time (bidirectional).
-int wave_create(const std::vector<const LayerParams *> &layers, int n_fwd, int max_T, int max_B, int sm_count, WaveStack **out);
+// scratch: memory of the caller's that nothing else uses while these kernels run; they keep a call's activations there if they fit.
+int wave_create(const std::vector<const LayerParams *> &layers, int n_fwd, int max_T, int max_B, int sm_count, ActDomains &dom, void *scratch,
+                size_t scratch_bytes, WaveStack **out);
 void wave_destroy(WaveStack *s);
 // tables: memoised nonlinearities, without which only the many-row form runs
 bool wave_supported(const WaveStack *s, int T, int B, bool tables);
@@ -105,8 +107,9 @@ int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[
                 bool tables, cudaStream_t st, int *launches);
 // The two handles of a bidirectional stack; then, once its workspaces are allocated, the wavefront kernels: where both directions
 // fit one plan those that run them side by side, else (*wave stays null) each handle's own; qlstm_api.cu.
-int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b);
-int bidir_wave_create(qlstm_t *f, qlstm_t *b, WaveStack **wave);
+int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, ActDomains &dom, qlstm_t **f,
+                      qlstm_t **b);
+int bidir_wave_create(qlstm_t *f, qlstm_t *b, ActDomains &dom, WaveStack **wave);
 int bidir_wave_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
                    cudaStream_t st);
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns);

@@ -258,7 +258,16 @@ int run_projection(qlstm *q, LayerHost &L, const int8_t *x, int rows, int16_t *X
 
 }  // namespace
 
-static int create_handle(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B, int device, bool with_wave, qlstm_t **out)
+// The wavefront kernels of the layers lp, the first of which are q's own.  X belongs to the per-layer path: a call takes one or the
+// other.
+static int wave_of_handle(qlstm *q, const std::vector<const LayerParams *> &lp, ActDomains &dom, WaveStack **wave)
+{
+    size_t maxN = 0;
+    for (auto &L : q->layers) maxN = (size_t)L.p.N > maxN ? (size_t)L.p.N : maxN;
+    return wave_create(lp, (int)q->layers.size(), q->max_T, q->max_B, q->sm_count, dom, q->X, (size_t)q->max_T * q->max_B * maxN * sizeof(int16_t), wave);
+}
+
+static int create_handle(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B, int device, bool with_wave, ActDomains &dom, qlstm_t **out)
 {
     if (!out) return QLSTM_ERR_ARG;
     *out = nullptr;
@@ -313,14 +322,14 @@ static int create_handle(const qlstm_layer_t *layers, int n_layers, int max_T, i
     }
     for (int l = 0; l < n_layers && ok; ++l) {
         q->layers[l].fast.proj_rows_hint = (long long)max_T * max_B;
-        int frc = fast_layer_init(q->layers[l].fast, q->layers[l].p, q->fscratch, max_T, max_B);
+        int frc = fast_layer_init(q->layers[l].fast, q->layers[l].p, q->fscratch, dom, max_T, max_B);
         if (frc != QLSTM_OK) { ok = false; rc = frc; }
     }
     if (ok) {
         std::vector<const LayerParams *> lp;
         for (auto &L : q->layers) lp.push_back(&L.p);
         int src = stack_small_create(lp, max_T, max_B, q->sm_count, &q->stack);
-        if (src == QLSTM_OK && with_wave) src = wave_create(lp, n_layers, max_T, max_B, q->sm_count, &q->wave);
+        if (src == QLSTM_OK && with_wave) src = wave_of_handle(q, lp, dom, &q->wave);
         if (src != QLSTM_OK) { ok = false; rc = src; }
     }
     if (!ok) { qlstm_destroy(q); return rc; }
@@ -330,26 +339,27 @@ static int create_handle(const qlstm_layer_t *layers, int n_layers, int max_T, i
 
 namespace ql {
 
-int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, qlstm_t **f, qlstm_t **b)
+int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, ActDomains &dom, qlstm_t **f,
+                      qlstm_t **b)
 {
     *f = *b = nullptr;
-    const int rc = create_handle(fwd, n_layers, max_T, max_B, device, false, f);
-    return rc != QLSTM_OK ? rc : create_handle(bwd, n_layers, max_T, max_B, device, false, b);
+    const int rc = create_handle(fwd, n_layers, max_T, max_B, device, false, dom, f);
+    return rc != QLSTM_OK ? rc : create_handle(bwd, n_layers, max_T, max_B, device, false, dom, b);
 }
 
-int bidir_wave_create(qlstm_t *f, qlstm_t *b, WaveStack **wave)
+int bidir_wave_create(qlstm_t *f, qlstm_t *b, ActDomains &dom, WaveStack **wave)
 {
     *wave = nullptr;
     std::vector<const LayerParams *> lp;
     for (auto &L : f->layers) lp.push_back(&L.p);
     for (auto &L : b->layers) lp.push_back(&L.p);
-    int rc = wave_create(lp, (int)f->layers.size(), f->max_T, f->max_B, f->sm_count, wave);
+    int rc = wave_of_handle(f, lp, dom, wave);
     // the directions do not go together: each has its own kernels
     for (qlstm_t *q : {f, b}) {
         if (rc != QLSTM_OK || *wave) break;
         lp.clear();
         for (auto &L : q->layers) lp.push_back(&L.p);
-        rc = wave_create(lp, (int)lp.size(), q->max_T, q->max_B, q->sm_count, &q->wave);
+        rc = wave_of_handle(q, lp, dom, &q->wave);
     }
     return rc;
 }
@@ -367,7 +377,8 @@ extern "C" {
 
 int qlstm_create(const qlstm_layer_t *layers, int n_layers, int max_T, int max_B, int device, qlstm_t **out)
 {
-    return create_handle(layers, n_layers, max_T, max_B, device, true, out);
+    ActDomains dom;
+    return create_handle(layers, n_layers, max_T, max_B, device, true, dom, out);
 }
 
 void qlstm_destroy(qlstm_t *q)

@@ -1327,7 +1327,7 @@ void fast_scratch_destroy(FastScratch &s)
     s = FastScratch();
 }
 
-int fast_recurrent_init(FastLayer &f, const LayerParams &p, const FastScratch &s, int max_B)
+int fast_recurrent_init(FastLayer &f, const LayerParams &p, const FastScratch &s, ActDomains &dom, int max_B)
 {
     f.rec_ok = false;
     const bool proj = (p.flags & F_PROJECTION) != 0;
@@ -1379,17 +1379,17 @@ int fast_recurrent_init(FastLayer &f, const LayerParams &p, const FastScratch &s
             return QLSTM_OK;
     }
     // memoised nonlinearities, if their tables fit into the ring (they live there between the matmul phases)
-    if (!act_tables_build(p.m_bits, (size_t)f.stages * STAGE_BYTES, &f.act_tab, &f.act_lay)) return QLSTM_ERR_CUDA;
+    if (!act_tables_build(dom, p.m_bits, (size_t)f.stages * STAGE_BYTES, &f.act_tab, &f.act_lay)) return QLSTM_ERR_CUDA;
     f.rec_ok = true;
     return QLSTM_OK;
 }
 
-int fast_layer_init(FastLayer &f, const LayerParams &p, const FastScratch &s, int max_T, int max_B)
+int fast_layer_init(FastLayer &f, const LayerParams &p, const FastScratch &s, ActDomains &dom, int max_T, int max_B)
 {
     (void)max_T;
     int rc = fast_projection_init(f, p);
     if (rc != QLSTM_OK) return rc;
-    return fast_recurrent_init(f, p, s, max_B);
+    return fast_recurrent_init(f, p, s, dom, max_B);
 }
 
 void fast_layer_destroy(FastLayer &f)

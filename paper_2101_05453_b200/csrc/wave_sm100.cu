@@ -890,7 +890,7 @@ struct WaveStack {
     unsigned *zero = nullptr;      // abort word, counters, totals: cleared before every call
     uint4 *gbuf = nullptr;
     uint32_t *cbuf = nullptr;
-    std::vector<void *> owned;
+    void *block[2] = {nullptr, nullptr};       // plans and tables; a call's activations, unless they lie in the caller's scratch
     unsigned dbg_missing = 0;
     unsigned long long dbg_limit_ns = 0;
 };
@@ -898,7 +898,7 @@ struct WaveStack {
 void wave_destroy(WaveStack *s)
 {
     if (!s) return;
-    for (void *p : s->owned) cudaFree(p);
+    for (void *p : s->block) cudaFree(p);
     delete s;
 }
 
@@ -906,13 +906,19 @@ namespace {
 
 constexpr int WV_SMALL_ROWS = 32;
 
-void *wv_alloc(WaveStack *s, size_t bytes)
-{
-    void *d = nullptr;
-    if (cudaMalloc(&d, bytes ? bytes : 16) != cudaSuccess) return nullptr;
-    s->owned.push_back(d);
-    return d;
-}
+// Memory handed out front to back; without a base it is only counted.  Pieces start 64 KB apart: packed at 256 bytes, what a step's
+// exchanges touch lay closer together and took longer (us per call of 100 steps, median of eight handles: four 1024-cell layers with
+// layer norm and projection, 16 rows 1345 and 1300; three of 1000 cells, 37 rows 1568 and 1545).
+struct WaveArena {
+    uint8_t *base = nullptr;
+    size_t used = 0;
+    template <class T>
+    void take(T *&p, size_t bytes)
+    {
+        p = base ? (T *)(base + used) : nullptr;
+        used += wv_up(bytes, 65536);
+    }
+};
 
 // Rows a call of B rows is cut into: `rg` row groups times one or two units of at most 128 rows each.
 void wave_units(int B, int rg, int &units, int &nu, int &ra)
@@ -1042,11 +1048,9 @@ int wave_plan(WaveStack *s, const std::vector<const LayerParams *> &lp, const st
 }
 
 // The weight images of one layer of a plan.
-int wave_fill_images(WaveStack *s, int mode, const LayerParams &p, WaveLayer &L)
+int wave_fill_images(int mode, const LayerParams &p, const WaveLayer &L, int8_t *iw, int8_t *ir, int8_t *ip)
 {
     const bool proj = p.flags & F_PROJECTION;
-    int8_t *iw = (int8_t *)wv_alloc(s, L.w_size[0]), *ir = (int8_t *)wv_alloc(s, L.w_size[1]), *ip = proj ? (int8_t *)wv_alloc(s, L.w_size[2]) : nullptr;
-    if (!iw || !ir || (proj && !ip)) return QLSTM_ERR_NOMEM;
     if (mode == 0) {
         k_wave_tile_weights<<<2048, 256>>>(p.W, iw, p.G, p.N, p.I, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_i);
         k_wave_tile_weights<<<2048, 256>>>(p.R, ir, p.G, p.N, p.O, L.n, L.ppc, L.nt, L.ppt, L.npad, L.kb_h);
@@ -1056,7 +1060,6 @@ int wave_fill_images(WaveStack *s, int mode, const LayerParams &p, WaveLayer &L)
         wave_small_tile_weights(p.R, ir, p.G, p.N, p.O, L.n, L.cpc, L.nt, L.ct, L.ctp, L.kb_h, L.kpg);
         if (proj) wave_small_tile_weights(p.Wproj, ip, 0, p.O, p.C, L.n, L.opc, L.ntp, L.opt, L.opp, L.kb_c, L.kpp);
     }
-    L.img_w = iw; L.img_r = ir; L.img_p = ip;
     return cudaGetLastError() == cudaSuccess ? QLSTM_OK : QLSTM_ERR_CUDA;
 }
 
@@ -1119,7 +1122,8 @@ size_t wave_zero_words(const WaveStack *s, int nu, int ra)
 // Plans the wavefront kernels for a handle - one stack of n_fwd layers, or two that read the same x, the second one backwards in
 // time; *out stays null when the stack does not qualify (layers of different variants,
 // a scale with a left shift where none is expected, sums that could leave int32) or device memory does not suffice.
-int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T, int max_B, int sm_count, WaveStack **out)
+int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T, int max_B, int sm_count, ActDomains &dom, void *scratch,
+                size_t scratch_bytes, WaveStack **out)
 {
     *out = nullptr;
     const int n = (int)lp.size();
@@ -1159,21 +1163,22 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
         return mem ? QLSTM_OK : rc;
     };
     s->tabs = true;
-    std::vector<std::pair<uint8_t *, ActLineLayout>> tables;
+    // one table per cell format
+    std::vector<int> tab_of(n);
+    std::vector<std::vector<uint8_t>> blobs;
+    std::vector<ActLineLayout> tab_lays;
     for (int l = 0; l < n; ++l) {
         int same = 0;
         while (same < l && lp[same]->m_bits != lp[l]->m_bits) ++same;
-        if (same < l) {
-            tables.push_back(tables[same]);
-            continue;
+        if (same == l) {
+            tab_of[l] = (int)blobs.size();
+            blobs.emplace_back();
+            tab_lays.emplace_back();
+            if (!act_lines_build(dom, lp[l]->m_bits, blobs.back(), &tab_lays.back())) return fail(QLSTM_ERR_CUDA);
+            if (blobs.back().empty()) s->tabs = false;
+            s->max_tab = std::max(s->max_tab, (int)tab_lays.back().bytes);
         }
-        uint8_t *blob = nullptr;
-        ActLineLayout lay;
-        if (!act_lines_build(lp[l]->m_bits, &blob, &lay)) return fail(QLSTM_ERR_CUDA);
-        if (blob) s->owned.push_back(blob);
-        else s->tabs = false;
-        tables.push_back({blob, lay});
-        s->max_tab = std::max(s->max_tab, (int)lay.bytes);
+        tab_of[l] = tab_of[same];
     }
     long long h_off = 0, c_off = 0;
     std::vector<WaveLayer> base;
@@ -1208,7 +1213,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
         if (L.last) { L.y_off = s->y_stride; s->y_stride += p.O; }
         L.h_off = h_off; L.c_off = c_off;
         h_off += p.O; c_off += p.C;
-        L.tab = tables[l].first; L.tab_lay = tables[l].second;
+        L.tab_lay = tab_lays[tab_of[l]];
         base.push_back(L);
     }
     // the kernels that exist for this stack's variants
@@ -1247,25 +1252,47 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
                 }
             }
     if (rows_alloc == 0) return fail(QLSTM_OK);
-    s->zero = (unsigned *)wv_alloc(s, zero_words * sizeof(unsigned));
-    s->gbuf = (uint4 *)wv_alloc(s, g_bytes);
-    s->cbuf = (uint32_t *)wv_alloc(s, c_bytes);
-    if (!s->zero || !s->gbuf || !s->cbuf) return fail(QLSTM_ERR_NOMEM);
-    int8_t *prev_img = nullptr;
-    for (int l = 0; l < n; ++l) {
-        WaveLayer &L = base[l];
-        const bool proj = L.flags & F_PROJECTION;
-        L.in_img = !L.first ? prev_img : (int8_t *)wv_alloc(s, (size_t)max_T * rows_alloc * L.kb_i * 128);
-        L.out_img = (int8_t *)wv_alloc(s, ((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
-        L.m_img = proj ? (int8_t *)wv_alloc(s, rows_alloc * L.kb_c * 128) : nullptr;
-        if (!L.in_img || !L.out_img || (proj && !L.m_img)) return fail(QLSTM_ERR_NOMEM);
-        prev_img = L.out_img;
-        for (WavePlan &pl : s->plan) {
-            if (!pl.used) continue;
-            WaveLayer &M = pl.layer[l];
-            M.in_img = L.in_img; M.out_img = L.out_img; M.m_img = L.m_img;
-            const int rc = wave_fill_images(s, pl.mode, *lp[l], M);
-            if (rc != QLSTM_OK) return fail(rc);
+    // everything in at most two allocations (a handle's creation is mostly allocations): counted first, then filled
+    WaveArena keep, work;
+    for (int pass = 0; pass < 2; ++pass) {
+        keep.used = work.used = 0;
+        std::vector<uint8_t *> tab(blobs.size());
+        for (size_t i = 0; i < blobs.size(); ++i) {
+            keep.take(tab[i], blobs[i].size());
+            if (pass && !blobs[i].empty() && cudaMemcpy(tab[i], blobs[i].data(), blobs[i].size(), cudaMemcpyHostToDevice) != cudaSuccess)
+                return fail(QLSTM_ERR_CUDA);
+        }
+        keep.take(s->zero, zero_words * sizeof(unsigned));
+        work.take(s->gbuf, g_bytes);
+        work.take(s->cbuf, c_bytes);
+        int8_t *prev_img = nullptr;
+        for (int l = 0; l < n; ++l) {
+            WaveLayer &L = base[l];
+            L.tab = tab[tab_of[l]];
+            if (L.first) work.take(L.in_img, (size_t)max_T * rows_alloc * L.kb_i * 128);
+            else L.in_img = prev_img;
+            work.take(L.out_img, ((size_t)max_T + 1) * rows_alloc * L.kb_h * 128);
+            if (L.flags & F_PROJECTION) work.take(L.m_img, rows_alloc * L.kb_c * 128);
+            prev_img = L.out_img;
+            for (WavePlan &pl : s->plan) {
+                if (!pl.used) continue;
+                WaveLayer &M = pl.layer[l];
+                M.in_img = L.in_img; M.out_img = L.out_img; M.m_img = L.m_img; M.tab = L.tab;
+                int8_t *img[3];
+                for (int i = 0; i < 3; ++i) keep.take(img[i], M.w_size[i]);
+                M.img_w = img[0]; M.img_r = img[1]; M.img_p = img[2];
+                if (!pass) continue;
+                const int rc = wave_fill_images(pl.mode, *lp[l], M, img[0], img[1], img[2]);
+                if (rc != QLSTM_OK) return fail(rc);
+            }
+        }
+        if (pass) break;
+        if (cudaMalloc(&s->block[0], keep.used) != cudaSuccess) return fail(QLSTM_ERR_NOMEM);
+        keep.base = (uint8_t *)s->block[0];
+        work.base = (uint8_t *)scratch;
+        if (work.used > scratch_bytes) {
+            if (cudaMalloc(&s->block[1], work.used) != cudaSuccess) return fail(QLSTM_ERR_NOMEM);
+            work.base = (uint8_t *)s->block[1];
         }
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(QLSTM_ERR_CUDA);

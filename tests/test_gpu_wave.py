@@ -146,6 +146,29 @@ def test_wave_plan_that_does_not_fit_in_memory_is_left_out(directions):
     q.close()
 
 
+# the wavefront kernels' images of a long call lie in the per-layer path's workspace, and the two paths take turns on one handle
+def test_wave_images_add_no_memory_and_paths_take_turns():
+    import torch
+    import paper_2101_05453_b200 as qlstm
+    T, B = 1200, 64
+    w = random_layer_stack(880, 3, 48, 256, 256, T=20, B=B)
+    torch.cuda.empty_cache()
+    qlstm.QLSTM(w.layers, 1, 1).close()
+    before = torch.cuda.mem_get_info()[0]
+    q = qlstm.QLSTM(w.layers, T, B)
+    used = before - torch.cuda.mem_get_info()[0]
+    rows = T * B
+    per_layer_path = rows * (1024 * 2 + 2 * 256 + 48 + 256)     # X, the two sequences between layers, staged x and y
+    assert used < per_layer_path + (48 << 20), used
+    h0, c0 = w.initial_state()
+    want = R.run(w.layers, w.x, h0, c0)
+    for impl in ((0, WAVE), (0, 2), (0, WAVE), (1, 1), (0, 0)):
+        got = run_gpu(w, handle=q, impl=impl)
+        for g, r in zip(got[:3], want[:3]):
+            assert np.array_equal(g, r), impl
+    q.close()
+
+
 def test_wave_timeout_is_reported_and_the_handle_recovers():
     import paper_2101_05453_b200 as qlstm
     w = random_layer_stack(9, 3, 48, 112, 64, projection=True, layernorm=True, T=5, B=40)
