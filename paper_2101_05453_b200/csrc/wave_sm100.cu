@@ -883,7 +883,12 @@ struct WaveStack {
     int y_stride = 0;
     int G = 4;
     bool ln = false, peep = false, tabs = false;
+    bool proj = false;             // some layer has a projection
     bool ragged = false;           // some dimension is not a multiple of 16
+    int max_C = 0;
+    size_t weights = 0;            // bytes of all layers' weights
+    size_t resident = 0;           // ... of the first layer's R and W_proj, which the per-layer kernel keeps in shared memory
+    uint16_t fit_groups[WV_MAX_ROWS + 1];      // groups in which the few-row form could hold a call's rows, 0: none
     std::vector<WavePlan> plan;
     int8_t by_rows[2][WV_MAX_ROWS + 1];        // plan of a call by its rows, [0] without and [1] with memoised nonlinearities; -1: none
     int max_tab = 0, max_kb_i = 0, max_kb_h = 0, max_kb_c = 0;
@@ -950,6 +955,15 @@ bool wave_small_fits(const WaveStack *s, const std::vector<const LayerParams *> 
     return wave_small_smem(k, 2, s->peep) <= (size_t)s->max_smem;
 }
 
+// The fewest groups of at least 9 blocks in which the few-row kernel can hold the B rows of a call; 0: none.
+int wave_fit_groups(const WaveStack *s, const std::vector<const LayerParams *> &lp, int B)
+{
+    for (int rg = 1;; rg *= 2) {
+        if (wave_small_fits(s, lp, rg, B, s->sm_count)) return rg;
+        if (2 * rg > B || s->sm_count / (2 * rg * (int)lp.size()) < 9) return 0;
+    }
+}
+
 // How many groups the B rows of a call are split into.  (Deep stacks: the layers already share out the SMs.)
 int wave_row_groups(const WaveStack *s, int mode, const std::vector<const LayerParams *> &lp, int B)
 {
@@ -964,17 +978,23 @@ int wave_row_groups(const WaveStack *s, int mode, const std::vector<const LayerP
     // As many as it takes for the few-row kernel to hold a group's rows, down to 9 blocks: it is the faster one even then (us per
     // step against the many-row kernel as one group: five 1024-cell CIFG layers, 64 rows 12.0 as two groups against 14.1; four
     // 1024-cell layers, 100 rows 24 as four against 28; eight 2048-cell layers, 32 rows 37 as two against 41).
-    while (!wave_small_fits(s, lp, rg, B, sm_count) && 2 * rg <= B && sm_count / (2 * rg * n) >= 9) rg *= 2;
-    if (!wave_small_fits(s, lp, rg, B, sm_count)) rg = 1;
+    // Every group streams all weights, though: above 128 MB per step (200 with layer norm, whose exchanges the few-row form has
+    // cheaper) the many-row form, with its one group, is ahead of it (us per call, few-row, many-row and layer by layer: three 2048-cell
+    // layers, 64 rows, 16 steps, four groups of 88 MB 951, 455 and 691; two 2048-cell layers, 33 rows, 218 MB 493, 352 and 417; below the
+    // line four 1024-cell layers, 96 rows, 126 MB 4 % ahead).
+    rg = wave_fit_groups(s, lp, B);
+    if (rg == 0 || (rg > 1 && rg * s->weights > (size_t)(s->ln ? 200 : 128) * 1000000)) return 1;
     // Then, fewer blocks per group make every exchange cheaper (two 512-cell layers, 16 rows: 9.0 us per step with one group, 8.5
     // with four; one 2048-cell layer with layer norm and peephole, 32 rows: 26 and 17), but a block streams more weights per step:
     // below 16 blocks, or beyond 320 KB, the groups cost more than they save (the same layers with eight groups: 9.2 and 18; five
-    // 1024-cell layers, 4 rows: 7.5 with one group, 10.3 with two), unless a block has little to stream: up to 64 KB, groups go down
-    // to 9 blocks (us per call of 100 steps, 16 blocks and 9: three 256-cell layers, 64 rows 493 and 446; two, 32 rows 404 and 385).
+    // 1024-cell layers, 4 rows: 7.5 with one group, 10.3 with two), unless a block has little to do: up to 64 KB and 32 cells, groups go
+    // down to 9 blocks (us per call of 100 steps, 16 blocks and 9: three 256-cell layers, 64 rows 493 and 446; two, 32 rows 404 and 385;
+    // 107 cells per block, eight layers, 5 rows, 12 steps 180 and 191).
     size_t bytes = 0;
     for (const LayerParams *p : lp)
         bytes = std::max(bytes, (size_t)p->N * (p->I + p->O) + ((p->flags & F_PROJECTION) ? (size_t)p->O * p->C : 0));
-    for (int per; 2 * rg <= B && (per = sm_count / (2 * rg * n)) >= 9 && bytes / per <= (per >= 16 ? 320 : 64) * 1024;) rg *= 2;
+    auto worth = [&](int per) { return per >= 16 ? bytes / per <= 320 * 1024 : per >= 9 && bytes / per <= 64 * 1024 && s->max_C <= 32 * per; };
+    while (2 * rg <= B && worth(sm_count / (2 * rg * n))) rg *= 2;
     return rg;
 }
 
@@ -1151,7 +1171,14 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     s->ln = lp[0]->flags & F_LAYERNORM;
     s->peep = lp[0]->flags & F_PEEPHOLE;
     memset(s->by_rows, -1, sizeof(s->by_rows));
-    for (const LayerParams *p : lp) s->ragged = s->ragged || p->I % 16 || p->C % 16 || p->O % 16;
+    for (const LayerParams *p : lp) {
+        const size_t wp = (p->flags & F_PROJECTION) ? (size_t)p->O * p->C : 0;
+        s->ragged = s->ragged || p->I % 16 || p->C % 16 || p->O % 16;
+        s->proj = s->proj || wp;
+        s->max_C = std::max(s->max_C, p->C);
+        s->weights += (size_t)p->N * (p->I + p->O) + wp;
+        if (p == lp[0]) s->resident = (size_t)p->N * p->O + wp;
+    }
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&s->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -1229,6 +1256,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     // definition is the many-row one; it has the plans that other calls need.
     WaveCall k;
     size_t smem, rows_alloc = 0, zero_words = 0, g_bytes = 0, c_bytes = 0;
+    for (int B = 1; B <= s->max_B; ++B) s->fit_groups[B] = (uint16_t)wave_fit_groups(s, lp, B);
     for (int tab = 1; tab >= 0; --tab)
         for (int B = 1; B <= s->max_B; ++B)
             for (int mode = tab; mode >= 0 && s->by_rows[tab][B] < 0; --mode) {
@@ -1308,19 +1336,44 @@ static const WavePlan *wave_plan_of(const WaveStack *s, int T, int B, bool table
 
 bool wave_supported(const WaveStack *s, int T, int B, bool tables) { return wave_plan_of(s, T, B, tables) != nullptr; }
 
+// Calls of one or two rows that are over before a wavefront's fill and launch have paid for themselves, on the whole-stack kernel (us
+// per call of that kernel over this one's): two or three steps of narrow stacks without layer norm or projection (one 256-cell layer 16
+// and 19, two 21 and 23); with a projection, whose exchange of m costs more here, up to 16 steps (four 256-cell layers, 8 steps: 8 % ahead;
+// with layer norm and at most two layers only up to three); one step of up to four rows or two of two rows of a narrow layer (128 cells
+// 17 % and 16 %); two steps of stacks whose weights come from memory either way (eight 2048-cell layers without projection 205 and 260).
+static bool wave_short_call(const WaveStack *s, int T, int B)
+{
+    if (T == 1 && B <= 2) return true;
+    if (s->n_layers != s->depth || B > 4) return false;
+    const int depth = s->depth, cells = depth * s->max_C;
+    if (T == 2 && B <= 2 && s->weights > (size_t)200 * 1000000) return true;
+    if (depth == 1 && !s->ln && ((T == 1 && s->max_C <= 512) || (T == 2 && B == 2 && s->max_C <= 1024))) return true;
+    if (B > 1 || T < depth) return false;                          // (shorter than deep: its layers run one after the other)
+    if (s->proj) return T <= (s->ln && depth <= 2 ? 3 : 16) && ((s->max_C <= 512 && cells <= 2048) || (cells <= 1024 && T <= 8));
+    return !s->ln && T <= 3 && cells * (T - 1) <= 1024;
+}
+
 // Where the wavefront kernels are the faster path (measured, us per call, against the whole-stack kernel or layer after layer):
-// one step of one or two rows stays with the whole-stack kernel (eight 2048-cell layers 138 against 170, one 512-cell layer 10
-// against 15; two steps 266 against 186); calls of a few steps of many rows, in which a wavefront has little to overlap, run
+// one step of one or two rows stays with the whole-stack kernel (eight 2048-cell layers 137 against 151, one 512-cell layer 10
+// against 15; two steps 266 against 186), and so do a few other short calls (above); calls of a few steps of many rows, in which a
+// wavefront has little to overlap, run
 // layer after layer (eight layers, 256 rows: one step 452 against 1057, four 1152 against 1404, sixteen 4050 against 2757; 64
 // rows: one step 377 against 451, two 538 against 478; five layers, 256 rows: four steps 324 against 340, sixteen 926 against
 // 628; two layers always).  A single layer with layer norm beyond 64 rows, with nothing to overlap, does so too (2048 cells, 128
-// rows: 24.6 us per step against 28.2; 64 rows 20.9 against 17.7).
+// rows: 24.6 us per step against 28.2; 64 rows 20.9 against 17.7), and a single one without layer norm and peephole beyond 128 rows
+// where the groups that hold them would stream more than 66 MB per step (100 with a projection) and the per-layer kernel keeps its
+// weights in shared memory (16 steps, 192 rows: 2048 cells with projection 311 against 365, 1536 cells 222 against 243, 1536 with CIFG
+// 218 against 231; under the lines, 1024 cells at 256 rows 191 against 168, 2048 cells with projection at 160 rows, 40 steps 679 against
+// 620; 2048 cells without projection, 113 KB per SM, 256 rows 429 against 360).
 bool wave_preferred(const WaveStack *s, int T, int B, bool tables)
 {
     if (!wave_supported(s, T, B, tables)) return false;
     if (s->ragged) return true;
-    if (T == 1 && B <= 2) return false;
+    if (wave_short_call(s, T, B)) return false;
     if (s->depth == 1 && s->ln && B > 64) return false;
+    if (s->n_layers == 1 && !s->ln && !s->peep && B > 128 && s->fit_groups[B] * s->weights > (size_t)(s->proj ? 100 : 66) * 1000000 &&
+        s->resident <= (size_t)s->sm_count * 96 * 1024)
+        return false;
     return T * 256 > s->depth * (B - 32);
 }
 

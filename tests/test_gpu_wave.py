@@ -169,6 +169,27 @@ def test_wave_images_add_no_memory_and_paths_take_turns():
     q.close()
 
 
+# which path a call takes where the wavefront kernels were measured slower (lines in wave_preferred and wave_row_groups): few steps of one
+# row, wide single layers of many rows; and where the few-row form's groups would stream too much, the many-row form
+@pytest.mark.parametrize("dims,layers,kw,T,B,taken,form", [
+    ((64, 256, 256), 1, dict(), 2, 1, 0, 1), ((64, 256, 256), 1, dict(), 5, 1, 1, 1), ((64, 256, 128), 4, dict(projection=True), 8, 1, 0, 1),
+    ((64, 256, 128), 4, dict(projection=True), 3, 1, 1, 1), ((64, 128, 128), 1, dict(), 1, 3, 0, 1), ((64, 256, 256), 2, dict(), 2, 2, 1, 1),
+    ((512, 1536, 1536), 1, dict(), 4, 192, 0, 1), ((512, 1536, 1536), 1, dict(), 4, 128, 1, 1), ((512, 2048, 2048), 1, dict(cifg=True), 2, 200, 0, 0),
+    ((512, 2048, 2048), 2, dict(), 2, 33, 1, 0), ((512, 2048, 2048), 2, dict(), 2, 200, 1, 0)])
+def test_wave_selection(dims, layers, kw, T, B, taken, form):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(890 + T, layers, *dims, T=T, B=B, **kw)
+    h0, c0 = w.initial_state()
+    want = R.run(w.layers, w.x, h0, c0)
+    with qlstm.QLSTM(w.layers, T, B) as q:
+        plan = q.debug_wave_plan(T, B)
+        assert (plan[3], plan[0]) == (taken, form), plan
+        for impl in ((0, 0), (0, WAVE)):
+            got = run_gpu(w, handle=q, impl=impl)
+            for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+                assert np.array_equal(g, r), (name, impl)
+
+
 def test_wave_timeout_is_reported_and_the_handle_recovers():
     import paper_2101_05453_b200 as qlstm
     w = random_layer_stack(9, 3, 48, 112, 64, projection=True, layernorm=True, T=5, B=40)
