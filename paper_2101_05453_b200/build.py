@@ -60,8 +60,8 @@ HOST_CHECK_LIB = os.path.join(HERE, "libqmath_host.so")
 
 
 def build_host_check(force: bool = False) -> str:
-    """g++ build of the kernels' integer arithmetic (qmath.cuh) for CPU-side sweeps in the tests."""
-    deps = [HOST_CHECK_SRC, os.path.join(CSRC, "qmath.cuh")]
+    """g++ build of the kernels' integer arithmetic (qmath.cuh, wave_math.cuh) for CPU-side sweeps in the tests."""
+    deps = [HOST_CHECK_SRC, os.path.join(CSRC, "qmath.cuh"), os.path.join(CSRC, "wave_math.cuh")]
     if force or not os.path.exists(HOST_CHECK_LIB) or any(os.path.getmtime(f) > os.path.getmtime(HOST_CHECK_LIB) for f in deps):
         tmp = HOST_CHECK_LIB + f".{os.getpid()}.tmp"
         subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-o", tmp, HOST_CHECK_SRC])

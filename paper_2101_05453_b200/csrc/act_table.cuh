@@ -25,6 +25,8 @@
 
 #include <cuda_runtime.h>
 
+#include "wave_math.cuh"
+
 namespace ql {
 
 struct ActTabLayout {
@@ -138,10 +140,6 @@ __device__ __forceinline__ ActLines make_act_lines(uint32_t blob_smem_addr, cons
     return ActLines{blob_smem_addr + l.sig_at, blob_smem_addr + l.tz_at, blob_smem_addr + l.tc_at, l.tz_lo, l.tz_hi, l.tc_lo, l.tc_hi, l.tc_sh, l.tc_k};
 }
 
-__host__ __device__ __forceinline__ int32_t act_line_value(int32_t e, int32_t x, int sh, int k)
-{
-    return (e + (((e & 1023) * (x & ((1 << sh) - 1))) << k)) >> 16;
-}
 __device__ __forceinline__ int32_t line_sigmoid(const ActLines &t, int32_t x)
 {
     return act_line_value((int32_t)lds_u32(t.sig + (uint32_t)((x >> ACT_SIG_SH) << 2)), x, ACT_SIG_SH, ACT_SIG_K);

@@ -1,6 +1,7 @@
-// Host build of the kernels' fixed-point arithmetic (qmath.cuh) so that CPU-only tests can sweep it
+// Host build of the kernels' fixed-point arithmetic (qmath.cuh, wave_math.cuh) so that CPU-only tests can sweep it
 // exhaustively.  Not part of libqlstm.so and not used by any product path.
 #include "../qmath.cuh"
+#include "../wave_math.cuh"
 
 extern "C" {
 int32_t qmh_mbqm(int32_t x, int32_t mult, int32_t shift) { return ql::mbqm(x, ql::Scale{mult, shift}); }
@@ -44,4 +45,20 @@ void qmh_ln_stats(int64_t sum, int64_t sumsq, int n, int fast, int64_t *mean_sig
     ql::LnStats s = fast ? ql::ln_stats_fast(sum, sumsq, ql::make_div_magic((uint32_t)n)) : ql::ln_stats(sum, sumsq, n);
     mean_sigma[0] = s.mean; mean_sigma[1] = s.sigma;
 }
+// statistics of a row as the wavefront kernels form them: mean, sigma, whether the quotients need the division, and the limbs
+void qmh_wave_ln(int64_t sum, int64_t sumsq, int n, uint32_t sigma_min, int64_t *out5)
+{
+    const ql::WvLnRow r = ql::wv_make_ln(sum, sumsq, ql::make_div_magic((uint32_t)n), sigma_min);
+    out5[0] = r.mean; out5[1] = r.sigma & ~ql::WV_LN_SLOW; out5[2] = (r.sigma & ql::WV_LN_SLOW) != 0; out5[3] = r.m_hi; out5[4] = r.m_lo;
+}
+// quotients of many inputs with the limbs that wv_make_ln forms for a given sigma
+void qmh_wave_quotients(const int32_t *q, int count, int32_t mean, uint32_t sigma, int32_t *out)
+{
+    const float x = ql::rcp_est((float)sigma);
+    const uint32_t hi = ql::wv_div((uint64_t)1 << 42, sigma, x);
+    const uint32_t lo = ql::wv_div((uint64_t)((1ull << 42) - (uint64_t)hi * sigma) << 31, sigma, x) + 1u;
+    for (int i = 0; i < count; ++i) out[i] = ql::wv_ln_quotient(q[i], (int32_t)(hi + (lo >> 31)), (int32_t)(lo & 0x7fffffffu), mean);
+}
+uint32_t qmh_wave_div(uint64_t n, uint32_t d) { return ql::wv_div(n, d, ql::rcp_est((float)d)); }
+int32_t qmh_line_value(int32_t e, int32_t x, int sh, int k) { return ql::act_line_value(e, x, sh, k); }
 }

@@ -1,4 +1,4 @@
-"""The kernels' integer arithmetic (csrc/qmath.cuh), compiled for the host and swept on the CPU.
+"""The kernels' integer arithmetic (csrc/qmath.cuh, csrc/wave_math.cuh), compiled for the host and swept on the CPU.
 
 This runs the very source the CUDA kernels compile, so that a wrong shift or rounding in the device
 code shows up without a GPU.  Two kinds of check: against the oracle (the reference; nothing here feeds
@@ -262,3 +262,96 @@ def test_fast_statistics_equal_the_plain_ones_and_the_definition(H):
         sigma = math.isqrt(max(var, 0))
         assert (out_f[0], out_f[1]) == (mean, sigma), (s, s2, n)
         assert (out_p[0], out_p[1]) == (mean, sigma), (s, s2, n)
+
+
+# ---------------------------------------------------------------- the wavefront kernels' forms
+
+def _quotient(d, sigma):
+    """round(2^10 d / sigma), ties away from zero"""
+    n = (2 * 1024 * abs(d) + sigma) // (2 * sigma)
+    return -n if d < 0 else n
+
+
+def test_wave_statistics_against_python_integers(H):
+    """wv_make_ln: the statistics of the definition (Section 3.2.6) and the reciprocal's limbs, 2^32 M = m_hi + 2^-31 m_lo."""
+    H.qmh_wave_ln.restype = None
+    H.qmh_wave_ln.argtypes = [C.c_int64, C.c_int64, C.c_int, C.c_uint32, C.POINTER(C.c_int64)]
+    rng = np.random.default_rng(51)
+    out = (C.c_int64 * 5)()
+    sigma_min = (1 << 36) // 65534 + 1
+    for n in [1, 2, 16, 48, 640, 1024, 2048, 3000, 8191]:
+        for kind in range(60):
+            if kind < 5:
+                q = [np.full(n, 32767), np.full(n, -32768), np.where(np.arange(n) % 2 == 0, 32767, -32768), np.eye(1, n, 0, dtype=np.int64)[0] * -32768,
+                     np.full(n, 123)][kind]
+            else:
+                q = rng.integers(-32768, 32768, n) // int(rng.integers(1, 3000))
+            q = q.astype(np.int64)
+            s, s2 = int(q.sum()), int((q * q).sum())
+            mean = (abs(s) * 1024 + n // 2) // n * (-1 if s < 0 else 1)
+            sigma = math.isqrt(max((s2 * 1048576 + n // 2) // n - mean * mean, 0))
+            H.qmh_wave_ln(s, s2, n, sigma_min, out)
+            assert (out[0], out[1]) == (mean, sigma), (s, s2, n)
+            assert out[2] == (0 < sigma < sigma_min)
+            if sigma >= sigma_min:
+                assert (out[3] << 31) + out[4] == (1 << 73) // sigma + 1
+            else:
+                assert (out[3], out[4]) == (0, 0)
+
+
+def test_wave_division(H):
+    """wv_div over the range it is used for: n < 2^57, d < 2^26, quotient below 2^31."""
+    H.qmh_wave_div.restype = C.c_uint32
+    H.qmh_wave_div.argtypes = [C.c_uint64, C.c_uint32]
+    rng = np.random.default_rng(52)
+    for _ in range(20000):
+        d = int(rng.integers(1 << 12, 1 << 26))
+        for n in (1 << 42, int(rng.integers(0, min(d << 31, 1 << 57))), int(rng.integers(0, 1 << 30)) * d, max(int(rng.integers(1, 1 << 30)) * d - 1, 0)):
+            if n < min(d << 31, 1 << 57):
+                assert H.qmh_wave_div(n, d) == n // d, (n, d)
+
+
+def test_wave_quotients_with_exact_ties(H):
+    """wv_ln_quotient from the smallest sigma of the fast form on: round(2^10 (2^10 q - mean) / sigma) for random rows, and for means that put
+    the quotient exactly on a tie (the error of M is below 2^-37 of a quotient step, the nearest non-tie 1 / (2 sigma) > 2^-27 away)."""
+    H.qmh_wave_quotients.restype = None
+    rng = np.random.default_rng(53)
+    sigma_min = (1 << 36) // 65534 + 1
+    sigmas = [sigma_min, sigma_min + 1, 1 << 21, (1 << 21) + 1, 3 << 20, (1 << 26) - 1, 33554431, 1 << 25] + [int(v) for v in rng.integers(sigma_min, 1 << 26, 300)]
+    out = np.empty(2048, np.int32)
+    for sigma in sigmas:
+        q = np.concatenate([rng.integers(-32768, 32768, 2040), [0, 1, -1, 32767, -32768, 2, -2, 77]]).astype(np.int32)
+        mean = int(rng.integers(-(1 << 24), 1 << 24))
+        H.qmh_wave_quotients(q.ctypes.data_as(C.c_void_p), len(q), mean, C.c_uint32(sigma), out.ctypes.data_as(C.c_void_p))
+        for a, o in zip(q[::13].tolist() + q[-8:].tolist(), out[::13].tolist() + out[-8:].tolist()):
+            assert o == _quotient(1024 * a - mean, sigma), (a, mean, sigma)
+    # ties: 2 * 1024 d = (2 j + 1) sigma needs sigma a multiple of 2^11
+    for sigma in [1 << 21, 3 << 20, 5 << 20, (1 << 25) + (1 << 11), 1021 << 11, 1235 << 12]:
+        if sigma < sigma_min:
+            continue
+        for j in [0, 1, 2, 5, 100, 4095, 30000]:
+            d = (2 * j + 1) * (sigma >> 11)
+            if d >= 1 << 26:
+                continue
+            for sign in (1, -1):
+                for off in (-1, 0, 1):
+                    q = max(-32768, min(32767, (sign * d) // 1024))
+                    mean = 1024 * q - (sign * d + off)
+                    if abs(mean) > 1 << 25:
+                        continue
+                    qa = np.array([q], np.int32)
+                    H.qmh_wave_quotients(qa.ctypes.data_as(C.c_void_p), 1, mean, C.c_uint32(sigma), out.ctypes.data_as(C.c_void_p))
+                    assert out[0] == _quotient(sign * d + off, sigma), (sigma, j, sign, off)
+
+
+def test_line_value(H):
+    """act_line_value against its formula in Python integers: (e + ((e mod 2^10) << k) (x mod 2^sh)) >> 16."""
+    H.qmh_line_value.restype = C.c_int32
+    H.qmh_line_value.argtypes = [C.c_int32] * 4
+    rng = np.random.default_rng(54)
+    for _ in range(20000):
+        sh, k = [(4, 8), (3, 10), (3, 9), (2, 11), (1, 12), (0, 8)][int(rng.integers(6))]
+        e, x = int(rng.integers(-(1 << 31), 1 << 30)), int(rng.integers(-32768, 32768))
+        rise = ((e % 1024) << k) * (x % (1 << sh))
+        if e + rise < 1 << 31:
+            assert H.qmh_line_value(e, x, sh, k) == (e + rise) >> 16
