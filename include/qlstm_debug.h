@@ -17,18 +17,20 @@ extern "C" {
 /* Kernel selection, for tests and measurements.  0 = automatic (default), 1 = simple kernels
  * (one thread per output, one launch per phase), 2 = fast kernels (tensor-core projection,
  * persistent recurrent kernel); 2 fails with QLSTM_ERR_DIM at run time if a shape is unsupported.
- * recurrent_impl 2 always runs layer after layer (projection launch + persistent kernel per layer), where 0 takes the
- * wavefront kernel for stacks of three or more layers beyond 4 rows and for dimensions that are no multiples of 16, and
- * the whole-stack kernel at small batches; 3 = like 2 but with the tensor-core matmuls even at batch <= 4, where 2 uses dp4a
+ * recurrent_impl 2 always runs layer after layer (projection launch + persistent kernel per layer), where 0 takes the wavefront kernels
+ * for every call that they support (up to 256 rows, layers of one kind) but these: one step of one or two rows and a few other short
+ * calls of up to four rows (whole-stack kernel), calls of few steps of many rows - T * 256 <= layers * (B - 32) - and single layers
+ * of many rows (layer after layer).  Dimensions that are no multiples of 16 always take the wavefront kernels.
+ * 3 = like 2 but with the tensor-core matmuls even at batch <= 4, where 2 uses dp4a
  * mat-vecs; 4 = like 2 but with the dp4a mat-vecs up to batch 16 (the crossover is a measured default, not a limit);
  * 5 = the whole-stack kernel or QLSTM_ERR_DIM (batch > 16, or a dimension that is not a multiple of 16), with its
  * schedule chosen from the call's length; 6 = the same with the wavefront schedule (one group of blocks per layer)
- * forced, 7 = with the sequential schedule (every layer on all blocks) forced; 8 = the wavefront kernel (every layer at
+ * forced, 7 = with the sequential schedule (every layer on all blocks) forced; 8 = the wavefront kernels (every layer at
  * once on its own group of SMs, tensor-core products, up to 256 rows, any dimensions) or QLSTM_ERR_DIM. */
 int qlstm_set_impl(qlstm_t *q, int projection_impl, int recurrent_impl);
 
 /* Failure-path check: with missing_arrivals > 0 every grid barrier of the persistent recurrent kernel (and every
- * counter wait of the whole-stack kernel) waits for
+ * counter wait of the whole-stack and wavefront kernels) waits for
  * that many arrivals that never come, for at most limit_ns (<= 1 s); the wait then runs out, the kernel sets its
  * status word, every block leaves the time loop, frees its tensor memory and returns, and qlstm_last_status
  * reports QLSTM_ERR_TIMEOUT.  Nothing faults or hangs and the handle stays usable; 0 restores normal operation. */
@@ -101,13 +103,18 @@ int qlstm_eval_activations(int cell_int_bits, int16_t *sigmoid_dev, int16_t *tan
  *     (0 shared with the gate's, 1 packed, 2 plain), format of the sigmoid (0 plain, 1 packed) }; bytes = 0 means that
  *     the tables do not fit or that the definition failed a check the formats rely on (the outputs are then untouched;
  *     such a layer keeps the arithmetic).  Synchronises the stream.
- *   qlstm_debug_activation_tables(q, 0) makes the kernel evaluate the definition instead (1 restores the default); 2
- *     selects the kernel's general instantiation, the one a layer gets when one of its scales has a left shift
+ *   qlstm_eval_activation_lines does the same for the wavefront kernels' tables (one 32-bit word per 2^s consecutive inputs, whose
+ *     low bits are the slope between them), with those kernels' lookup code; bytes_out (HOST) = bytes of the tables, 0: some
+ *     input has no word that yields its value (the outputs are then untouched; the kernels evaluate the definition).
+ *   qlstm_debug_activation_tables(q, 0) makes the kernels evaluate the definition instead (of the wavefront kernels the many-row form;
+ *     1 restores the default); 2 selects the persistent kernel's general instantiation, the one a layer gets when one of its scales has a left shift
  *     (shift > 0), which otherwise only such layers reach.  Returns the number of layers that hold tables, or a
  *     negative qlstm_error.
  */
 int qlstm_eval_activation_tables(int cell_int_bits, int max_bytes, int16_t *sigmoid_dev, int16_t *tanh_gate_dev,
                                  int16_t *tanh_cell_dev, int *layout_out7, void *cuda_stream);
+int qlstm_eval_activation_lines(int cell_int_bits, int16_t *sigmoid_dev, int16_t *tanh_gate_dev, int16_t *tanh_cell_dev, int *bytes_out,
+                                void *cuda_stream);
 int qlstm_debug_activation_tables(qlstm_t *q, int enable);
 int qlstm_eval_layernorm_row(const int16_t *q_dev, int n, const int16_t *L_dev, const int32_t *b_dev,
                              qlstm_scale_t eff_ln, int16_t *out_dev, void *cuda_stream);

@@ -22,7 +22,7 @@ IMPL_AUTO, IMPL_SIMPLE, IMPL_FAST = 0, 1, 2
 EXPORTS = ["qlstm_create", "qlstm_run", "qlstm_run_host", "qlstm_input_projection", "qlstm_last_status",
            "qlstm_destroy", "qlstm_strerror", "qlstm_trace_bytes", "qlstm_set_impl", "qlstm_set_profiling",
            "qlstm_get_profile", "qlstm_device_info", "qlstm_eval_activations", "qlstm_eval_layernorm_row",
-           "qlstm_eval_activation_tables", "qlstm_debug_activation_tables",
+           "qlstm_eval_activation_tables", "qlstm_eval_activation_lines", "qlstm_debug_activation_tables",
            "qlstm_layernorm_rows_static", "qlstm_debug_barrier_timeout", "qlstm_debug_ring_plan",
            "qlstm_debug_wave_plan", "qlstm_bidir_debug_wave_plan", "qlstm_debug_projection_plan", "qlstm_debug_mma_i8_peak", "qlstm_debug_barrier_latency",
            "qlstm_bidir_create", "qlstm_bidir_run", "qlstm_bidir_last_status", "qlstm_bidir_destroy",
@@ -117,6 +117,8 @@ def lib():
         L.qlstm_eval_activation_tables.restype = C.c_int
         L.qlstm_eval_activation_tables.argtypes = [C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(C.c_int),
                                                    C.c_void_p]
+        L.qlstm_eval_activation_lines.restype = C.c_int
+        L.qlstm_eval_activation_lines.argtypes = [C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(C.c_int), C.c_void_p]
         L.qlstm_debug_activation_tables.restype = C.c_int
         L.qlstm_debug_activation_tables.argtypes = [C.c_void_p, C.c_int]
         L.qlstm_eval_layernorm_row.restype = C.c_int
@@ -352,6 +354,14 @@ def eval_activations(cell_int_bits: int, sigmoid_out, tanh_out, stream: int = 0)
     """qlstm_eval_activations on two device int16 [65536] tensors."""
     _check(lib().qlstm_eval_activations(cell_int_bits, _dev_ptr(sigmoid_out), _dev_ptr(tanh_out), stream),
            "qlstm_eval_activations")
+
+
+def eval_activation_lines(cell_int_bits: int, sigmoid_out, tanh_gate_out, tanh_cell_out, stream: int = 0) -> int:
+    """qlstm_eval_activation_lines on three device int16 [65536] tensors; returns the tables' bytes."""
+    n = C.c_int()
+    _check(lib().qlstm_eval_activation_lines(cell_int_bits, _dev_ptr(sigmoid_out), _dev_ptr(tanh_gate_out), _dev_ptr(tanh_cell_out),
+                                             C.byref(n), stream), "qlstm_eval_activation_lines")
+    return n.value
 
 
 def eval_activation_tables(cell_int_bits: int, max_bytes: int, sigmoid_out, tanh_gate_out, tanh_cell_out, stream: int = 0):

@@ -55,9 +55,50 @@ __global__ void k_eval_activation_tables(const uint8_t *blob, ActTabLayout lay, 
     }
 }
 
+// The same for the wavefront kernels' piecewise-linear tables.
+__global__ void k_eval_activation_lines(const uint8_t *blob, ActLineLayout lay, int16_t *sig, int16_t *tz, int16_t *tc)
+{
+    extern __shared__ __align__(16) uint8_t tab_s[];
+    for (uint32_t i = threadIdx.x; i < lay.bytes / 16; i += blockDim.x)
+        reinterpret_cast<uint4 *>(tab_s)[i] = reinterpret_cast<const uint4 *>(blob)[i];
+    __syncthreads();
+    const ActLines at = make_act_lines((uint32_t)__cvta_generic_to_shared(tab_s), lay);
+    for (int i = threadIdx.x; i < 65536; i += blockDim.x) {
+        const int32_t x = i - 32768;
+        sig[i] = (int16_t)line_sigmoid(at, x);
+        tz[i] = (int16_t)line_tanh_gate(at, x);
+        tc[i] = (int16_t)line_tanh_cell(at, x);
+    }
+}
+
 }  // namespace ql
 
 extern "C" {
+
+int qlstm_eval_activation_lines(int cell_int_bits, int16_t *sigmoid_dev, int16_t *tanh_gate_dev, int16_t *tanh_cell_dev, int *bytes_out, void *cuda_stream)
+{
+    if (cell_int_bits < 0 || cell_int_bits > 15 || !sigmoid_dev || !tanh_gate_dev || !tanh_cell_dev || !bytes_out) return QLSTM_ERR_ARG;
+    ql::ActDomains dom;
+    ql::ActLineLayout lay;
+    std::vector<uint8_t> blob;
+    if (!ql::act_lines_build(dom, cell_int_bits, blob, &lay)) return QLSTM_ERR_CUDA;
+    *bytes_out = (int)lay.bytes;
+    if (blob.empty()) return QLSTM_OK;
+    cudaStream_t st = (cudaStream_t)cuda_stream;
+    uint8_t *d = nullptr;
+    if (cudaMalloc(&d, blob.size()) != cudaSuccess) return QLSTM_ERR_NOMEM;
+    int rc = QLSTM_OK;
+    if (cudaMemcpy(d, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaFuncSetAttribute(ql::k_eval_activation_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes) != cudaSuccess)
+        rc = QLSTM_ERR_CUDA;
+    if (rc == QLSTM_OK) {
+        ql::k_eval_activation_lines<<<1, 1024, lay.bytes, st>>>(d, lay, sigmoid_dev, tanh_gate_dev, tanh_cell_dev);
+        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) rc = QLSTM_ERR_CUDA;
+    }
+    cudaFree(d);
+    return rc;
+}
+
 
 int qlstm_eval_activation_tables(int cell_int_bits, int max_bytes, int16_t *sigmoid_dev, int16_t *tanh_gate_dev,
                                  int16_t *tanh_cell_dev, int *layout_out7, void *cuda_stream)

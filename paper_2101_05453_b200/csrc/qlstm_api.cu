@@ -428,7 +428,7 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
     uint8_t *trace = (uint8_t *)trace_dev;
     if (trace && cudaMemsetAsync(trace, 0, qlstm_trace_bytes(q, T, B), st) != cudaSuccess) return QLSTM_ERR_CUDA;
     const int nl = (int)q->layers.size();
-    // small batches: the whole stack in one launch (layers as a wavefront, input projection inside the step)
+    // the whole stack in one launch, every layer at once on its own SMs (wave_sm100.cu)
     if (!trace && (q->impl_rec == 0 || q->impl_rec == 8) && q->impl_proj != 1) {
         if (q->impl_rec == 0 ? wave_preferred(q->wave, T, B, q->tables) : wave_supported(q->wave, T, B, q->tables)) {
             SpanGuard g(q, st, 1);
@@ -439,6 +439,7 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
         }
         if (q->impl_rec == 8) return QLSTM_ERR_DIM;
     }
+    // short calls of few rows, and stacks of few rows that the wavefront kernels do not take: mat-vecs (stack_small_sm100.cu)
     if (!trace && (q->impl_rec == 0 || q->impl_rec >= 5) && q->impl_proj != 1) {
         if (q->impl_rec == 0 ? stack_small_preferred(q->stack, T, B) : stack_small_supported(q->stack, T, B)) {
             SpanGuard g(q, st, 1);

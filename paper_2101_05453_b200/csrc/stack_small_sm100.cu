@@ -918,8 +918,8 @@ int stack_small_create(const std::vector<const LayerParams *> &lp, int max_T, in
 
 bool stack_small_supported(const StackSmall *s, int T, int B) { return s && s->ok && B >= 1 && B <= s->max_B && T >= 1 && T <= s->max_T; }
 
-// Where the whole-stack kernel is the faster path (measured, us per time step of the whole stack, this kernel against
-// layer after layer): the wavefront's step costs one layer-step whatever the depth, the per-layer kernels' cost grows
+// Where the whole-stack kernel is the faster path against layer after layer, for calls that the wavefront kernels leave (wave_preferred in
+// wave_sm100.cu is asked first; measured, us per time step of the whole stack, this kernel against layer after layer): the wavefront's step costs one layer-step whatever the depth, the per-layer kernels' cost grows
 // with it.  Eight 2048-cell layers: 26 / 127 at batch 1, 59 / 157 at 8, 107 / 158 at 16; five 1024-cell layers: 17 / 32
 // at batch 4, 23 / 39 at 8, 33 / 39 at 16; two 256-cell layers: 6 / 10 at batch 2, 8.5 / 11 at 8; a single 2048-cell
 // layer (nothing to overlap): 27 / 28 at batch 4, 39 / 27 at 8, 54 / 27 at 16.

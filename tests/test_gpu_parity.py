@@ -495,6 +495,22 @@ def test_device_activation_tables_exhaustive(m, room):
     assert np.array_equal(tc, R.tanh_all(m))
 
 
+@pytest.mark.parametrize("m", range(16))
+def test_device_activation_lines_exhaustive(m):
+    """The wavefront kernels' piecewise-linear tables (built as at create time, the kernels' own lookup code: biased offsets, clamps, the
+    gate's table shared at m = 3) on every int16 input against the oracle."""
+    import torch
+    from paper_2101_05453_b200 import binding
+    out = [torch.full((65536,), 12345, dtype=torch.int16, device="cuda") for _ in range(3)]
+    nbytes = binding.eval_activation_lines(m, *out, stream=torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert 0 < nbytes <= 56 * 1024 and nbytes % 16 == 0
+    sig, tz, tc = (o.cpu().numpy().astype(np.int32) for o in out)
+    assert np.array_equal(sig, R.sigmoid_all(3))
+    assert np.array_equal(tz, R.tanh_all(3))
+    assert np.array_equal(tc, R.tanh_all(m))
+
+
 def test_device_activation_tables_that_do_not_fit():
     import torch
     from paper_2101_05453_b200 import binding

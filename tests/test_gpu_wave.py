@@ -1,4 +1,4 @@
-"""The wavefront kernel against the CPU oracle, bit for bit, at the edges of its tiles (needs a B200)."""
+"""The wavefront kernels against the CPU oracle, bit for bit, at the edges of their tiles (needs a B200)."""
 import numpy as np
 import pytest
 
@@ -15,19 +15,41 @@ VARIANTS = [dict(), dict(projection=True), dict(cifg=True), dict(peephole=True, 
             dict(peephole=True, layernorm=True, cifg=True)]
 
 
-def check(w):
+FEW, MANY = 1, 0     # the kernels' forms, as qlstm_debug_wave_plan names them
+
+
+def check(w, form=None, units=None):
+    import paper_2101_05453_b200 as qlstm
     h0, c0 = w.initial_state()
     want = R.run(w.layers, w.x, h0, c0)
-    got = run_gpu(w, impl=(0, WAVE))
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        plan = q.debug_wave_plan(w.T, w.B)
+        assert form is None or plan[0] == form, plan
+        assert units is None or plan[2] == units, plan
+        got = run_gpu(w, handle=q, impl=(0, WAVE))
     for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
         assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
 
 
-# one row; MMA columns of eight and 32 rows; copies of the rows in the lanes end at 64; one unit ends at 128; two full units
+# few rows: one row; MMA columns of eight and 32 rows; two and four row groups of up to 32 rows.  Many rows: two units, odd and full
 @pytest.mark.parametrize("B", [1, 8, 9, 32, 33, 64, 65, 128, 129, 256])
 @pytest.mark.parametrize("kw", VARIANTS, ids=lambda k: "+".join(sorted(k)) or "basic")
 def test_wave_variants(kw, B):
     check(random_layer_stack(810 + B, 3, 48, 112, 64, T=6, B=B, **kw))
+
+
+# many rows in one unit (nine layers leave no room for row groups of the few-row form): rows twice in the lanes up to 64, once up to
+# 128; then two units.  Fewer than four steps per layer and more order X differently
+@pytest.mark.parametrize("B,T", [(33, 5), (64, 5), (65, 5), (128, 5), (129, 5), (33, 37), (100, 37)])
+@pytest.mark.parametrize("kw", VARIANTS, ids=lambda k: "+".join(sorted(k)) or "basic")
+def test_wave_many_rows(kw, B, T):
+    check(random_layer_stack(815 + B, 9, 48, 112, 64, T=T, B=B, **kw), MANY, 1 if B <= 128 else 2)
+
+
+# many rows with each row four times in the lanes: layers too wide for the few-row form's shared memory at 32 rows
+@pytest.mark.parametrize("kw", [dict(projection=True, layernorm=True), dict(projection=True, peephole=True, cifg=True)], ids=lambda k: "+".join(sorted(k)))
+def test_wave_many_rows_repeated_four_times(kw):
+    check(random_layer_stack(817, 9, 64, 1600, 512, T=3, B=29, **kw), MANY, 1)
 
 
 # dimensions that no tile, vector or pair of cells divides
@@ -56,6 +78,17 @@ def test_wave_layernorm_of_small_deviations(shift, B, peephole):
         q.eff_x = [(m, s - shift) for m, s in q.eff_x]
         q.eff_h = [(m, s - shift) for m, s in q.eff_h]
     check(w)
+
+
+# the same out-of-line division in the many-row form
+@pytest.mark.parametrize("shift", [4, 9, 15])
+@pytest.mark.parametrize("kw", [dict(projection=True), dict(peephole=True), dict(peephole=True, cifg=True)], ids=lambda k: "+".join(sorted(k)))
+def test_wave_many_rows_layernorm_of_small_deviations(shift, kw):
+    w = random_layer_stack(845, 9, 48, 112, 64, layernorm=True, T=5, B=70, **kw)
+    for q in w.layers:
+        q.eff_x = [(m, s - shift) for m, s in q.eff_x]
+        q.eff_h = [(m, s - shift) for m, s in q.eff_h]
+    check(w, MANY, 1)
 
 
 # both directions in one launch: few and many rows, one and two units
@@ -169,6 +202,30 @@ def test_wave_images_add_no_memory_and_paths_take_turns():
     q.close()
 
 
+# both directions in one launch of the many-row form, one and two units
+@pytest.mark.parametrize("B,units", [(40, 1), (140, 2)])
+def test_wave_bidirectional_many_rows(B, units):
+    import torch
+    import paper_2101_05453_b200 as qlstm
+    from tests.test_gpu_bidirectional import two_directions
+    T = 9
+    f, b = two_directions(72, 8, 32, 96, 48, T, B, projection=True, layernorm=True)
+    states = [a for w in (f, b) for a in w.initial_state()]
+    yf, hf, cf, _ = R.run(f.layers, f.x, *f.initial_state())
+    yb, hb, cb, _ = R.run(b.layers, f.x[::-1], *b.initial_state())
+    with qlstm.BiQLSTM(f.layers, b.layers, T, B) as q:
+        plan = q.debug_wave_plan(T, B)
+        assert plan[0] == MANY and plan[2:] == (units, 1), plan
+        dev = torch.device("cuda:0")
+        st = [torch.from_numpy(a.copy()).to(dev) for a in states]
+        y = torch.zeros((T, B, q.n_output), dtype=torch.int8, device=dev)
+        q.run(torch.from_numpy(np.ascontiguousarray(f.x)).to(dev), T, B, *st, y, stream=torch.cuda.current_stream().cuda_stream)
+        q.last_status()
+        assert np.array_equal(y.cpu().numpy(), np.concatenate([yf, yb[::-1]], axis=2))
+        for got, ref in zip(st, (hf, cf, hb, cb)):
+            assert np.array_equal(got.cpu().numpy(), ref)
+
+
 # which path a call takes where the wavefront kernels were measured slower (lines in wave_preferred and wave_row_groups): few steps of one
 # row, wide single layers of many rows; and where the few-row form's groups would stream too much, the many-row form
 @pytest.mark.parametrize("dims,layers,kw,T,B,taken,form", [
@@ -207,13 +264,14 @@ def test_wave_timeout_is_reported_and_the_handle_recovers():
 
 
 # both forms, copies and MMAs in flight when the wait runs out: later calls on the same handle are not disturbed
-@pytest.mark.parametrize("layers,B", [(9, 40), (9, 128), (9, 20), (2, 150)])
-def test_wave_abort_leaves_nothing_in_flight(layers, B):
+@pytest.mark.parametrize("layers,B,form", [(9, 40, MANY), (9, 128, MANY), (9, 20, FEW), (9, 150, MANY), (2, 150, FEW)])
+def test_wave_abort_leaves_nothing_in_flight(layers, B, form):
     import paper_2101_05453_b200 as qlstm
     w = random_layer_stack(860 + B, layers, 48, 112, 64, projection=True, layernorm=True, T=12, B=B)
     h0, c0 = w.initial_state()
     want = R.run(w.layers, w.x, h0, c0)
     with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        assert q.debug_wave_plan(w.T, w.B)[0] == form
         for limit in (300_000, 3_000_000):
             q.debug_barrier_timeout(1, limit)
             with pytest.raises(qlstm.QlstmError) as e:
