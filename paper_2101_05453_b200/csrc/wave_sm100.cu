@@ -1243,12 +1243,6 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
         L.tab_lay = tab_lays[tab_of[l]];
         base.push_back(L);
     }
-    // the kernels that exist for this stack's variants
-    bool form[2] = {true, cudaFuncSetAttribute(wave_small_kernel(s->G, s->ln, s->peep), cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) == cudaSuccess};
-    for (int tab = 0; tab < 2; ++tab) {
-        const void *f = tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep);
-        form[0] = form[0] && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) == cudaSuccess;
-    }
     // A plan for every number of rows that a call may have: the few-row form where it can hold them, else the many-row one.  Calls
     // of fewer rows than the handle was made for get the shares that a handle of their own would have (us per call of 100 steps, all
     // calls with the shares of the handle's rows and like this: five 1024-cell CIFG layers made for 64 rows, one row 968 and 641; two
@@ -1260,7 +1254,6 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     for (int tab = 1; tab >= 0; --tab)
         for (int B = 1; B <= s->max_B; ++B)
             for (int mode = tab; mode >= 0 && s->by_rows[tab][B] < 0; --mode) {
-                if (!form[mode]) continue;
                 const int rg = wave_row_groups(s, mode, lp, B);
                 bool made = false;
                 for (const WavePlan &pl : s->plan) made = made || (pl.mode == mode && pl.rg == rg && pl.used);
@@ -1280,6 +1273,14 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
                 }
             }
     if (rows_alloc == 0) return fail(QLSTM_OK);
+    // (only of the forms that some call takes: setting an attribute loads a kernel, some milliseconds the first time in a process)
+    for (const WavePlan &pl : s->plan) {
+        if (!pl.used) continue;
+        const void *f[2] = {wave_small_kernel(s->G, s->ln, s->peep), nullptr};
+        if (pl.mode == 0) { f[0] = wave_kernel_of<true>(s->G, s->ln, s->peep); f[1] = wave_kernel_of<false>(s->G, s->ln, s->peep); }
+        for (const void *kernel : f)
+            if (kernel && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) return fail(QLSTM_ERR_CUDA);
+    }
     // everything in at most two allocations (a handle's creation is mostly allocations): counted first, then filled
     WaveArena keep, work;
     for (int pass = 0; pass < 2; ++pass) {
