@@ -42,6 +42,15 @@ int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long 
 int qlstm_debug_wave_plan(qlstm_t *q, int T, int B, int *out4);
 int qlstm_bidir_debug_wave_plan(qlstm_bidir_t *q, int T, int B, int *out4);
 
+/* The wavefront kernel with resident weights (thread-block clusters; it comes before all others for the calls that it takes, with
+ * automatic selection).  Its plan: out4 (host) receives the blocks of a cluster (0: does not take such calls), the row groups, the
+ * tiles of eight rows of a group, and the groups of eight cells per warp.  Mode 0: automatic, 1: never taken; returns whether the
+ * handle has such a plan, or QLSTM_ERR_ARG. */
+int qlstm_debug_resident_plan(qlstm_t *q, int T, int B, int *out4);
+int qlstm_bidir_debug_resident_plan(qlstm_bidir_t *q, int T, int B, int *out4);
+int qlstm_debug_resident(qlstm_t *q, int mode);
+int qlstm_bidir_debug_resident(qlstm_bidir_t *q, int mode);
+
 /* Host logic of the persistent kernel's operand ring, exposed for tests (no device is touched).  The matmuls of
  * Section 3.2.4 / 3.2.8 stream their batch operand through `stages` ring stages that one producer fills and
  * `n_owners` MMA issuers drain; within a phase owner o uses the stages o, o + n_owners, ... only, so that no

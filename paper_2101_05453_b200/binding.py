@@ -24,7 +24,8 @@ EXPORTS = ["qlstm_create", "qlstm_run", "qlstm_run_host", "qlstm_input_projectio
            "qlstm_get_profile", "qlstm_device_info", "qlstm_eval_activations", "qlstm_eval_layernorm_row",
            "qlstm_eval_activation_tables", "qlstm_eval_activation_lines", "qlstm_debug_activation_tables",
            "qlstm_layernorm_rows_static", "qlstm_debug_barrier_timeout", "qlstm_debug_ring_plan",
-           "qlstm_debug_wave_plan", "qlstm_bidir_debug_wave_plan", "qlstm_debug_projection_plan", "qlstm_debug_mma_i8_peak", "qlstm_debug_barrier_latency",
+           "qlstm_debug_wave_plan", "qlstm_bidir_debug_wave_plan", "qlstm_debug_resident_plan", "qlstm_bidir_debug_resident_plan",
+           "qlstm_debug_resident", "qlstm_bidir_debug_resident", "qlstm_debug_projection_plan", "qlstm_debug_mma_i8_peak", "qlstm_debug_barrier_latency",
            "qlstm_bidir_create", "qlstm_bidir_run", "qlstm_bidir_last_status", "qlstm_bidir_destroy",
            "qlstm_calibrate", "qlstm_quantize_model", "qlstm_quantized_layers", "qlstm_quantized_scales",
            "qlstm_quantized_destroy"]
@@ -125,7 +126,10 @@ def lib():
         L.qlstm_eval_layernorm_row.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, Scale, C.c_void_p, C.c_void_p]
         L.qlstm_debug_barrier_timeout.restype = C.c_int
         L.qlstm_debug_barrier_timeout.argtypes = [C.c_void_p, C.c_int, C.c_ulonglong]
-        for f in (L.qlstm_debug_wave_plan, L.qlstm_bidir_debug_wave_plan):
+        for f in (L.qlstm_debug_resident, L.qlstm_bidir_debug_resident):
+            f.restype = C.c_int
+            f.argtypes = [C.c_void_p, C.c_int]
+        for f in (L.qlstm_debug_wave_plan, L.qlstm_bidir_debug_wave_plan, L.qlstm_debug_resident_plan, L.qlstm_bidir_debug_resident_plan):
             f.restype = C.c_int
             f.argtypes = [C.c_void_p, C.c_int, C.c_int, C.POINTER(C.c_int)]
         L.qlstm_debug_ring_plan.restype = C.c_int
@@ -302,6 +306,18 @@ class QLSTM:
         _check(lib().qlstm_debug_wave_plan(self._h, T, B, out), "qlstm_debug_wave_plan")
         return tuple(out)
 
+    def debug_resident_plan(self, T: int, B: int):
+        """(blocks of a cluster, row groups, tiles of rows, cell groups per warp) of the kernel with resident weights; see qlstm_debug.h."""
+        out = (C.c_int * 4)()
+        _check(lib().qlstm_debug_resident_plan(self._h, T, B, out), "qlstm_debug_resident_plan")
+        return tuple(out)
+
+    def debug_resident(self, mode: int):
+        """0: taken where it fits, 1: never."""
+        n = lib().qlstm_debug_resident(self._h, mode)
+        _check(n if n < 0 else 0, "qlstm_debug_resident")
+        return n
+
     def device_info(self):
         a, b = C.c_int(), C.c_int()
         _check(lib().qlstm_device_info(self._h, C.byref(a), C.byref(b)), "qlstm_device_info")
@@ -328,6 +344,16 @@ class BiQLSTM:
         out = (C.c_int * 4)()
         _check(lib().qlstm_bidir_debug_wave_plan(self._h, T, B, out), "qlstm_bidir_debug_wave_plan")
         return tuple(out)
+
+    def debug_resident_plan(self, T: int, B: int):
+        out = (C.c_int * 4)()
+        _check(lib().qlstm_bidir_debug_resident_plan(self._h, T, B, out), "qlstm_bidir_debug_resident_plan")
+        return tuple(out)
+
+    def debug_resident(self, mode: int):
+        n = lib().qlstm_bidir_debug_resident(self._h, mode)
+        _check(n if n < 0 else 0, "qlstm_bidir_debug_resident")
+        return n
 
     def last_status(self):
         _check(lib().qlstm_bidir_last_status(self._h), "qlstm_bidir_last_status")

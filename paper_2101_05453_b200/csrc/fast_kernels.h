@@ -105,6 +105,12 @@ bool wave_preferred(const WaveStack *s, int T, int B, bool tables);      // supp
 // null.  The launch clears the status word itself.
 int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
                 bool tables, cudaStream_t st, int *launches);
+// The form with resident weights (wave_resident_sm100.cu), for stacks that fit it: whether a call takes it; the launch.
+bool wave_resident_taken(const WaveStack *s, int T, int B, bool tables);
+int launch_wave_resident(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
+                         cudaStream_t st);
+int wave_resident_mode(WaveStack *s, int mode);                          // include/qlstm_debug.h
+int wave_resident_debug_plan(const WaveStack *s, int T, int B, int *out4);
 // The two handles of a bidirectional stack; then, once its workspaces are allocated, the wavefront kernels: where both directions
 // fit one plan those that run them side by side, else (*wave stays null) each handle's own; qlstm_api.cu.
 int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_layers, int max_T, int max_B, int device, ActDomains &dom, qlstm_t **f,
@@ -112,6 +118,8 @@ int bidir_pair_create(const qlstm_layer_t *fwd, const qlstm_layer_t *bwd, int n_
 int bidir_wave_create(qlstm_t *f, qlstm_t *b, ActDomains &dom, WaveStack **wave);
 int bidir_wave_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
                    cudaStream_t st);
+int bidir_resident_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
+                       cudaStream_t st);
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns);
 
 int debug_ring_plan(int stages, int n_own, int contig, int per, int n_total, int *out);

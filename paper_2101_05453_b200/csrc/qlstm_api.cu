@@ -371,6 +371,13 @@ int bidir_wave_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int
     return launch_wave(wave, x, T, B, h, c, y, f->status, b->status, true, st, nullptr);
 }
 
+int bidir_resident_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
+                       cudaStream_t st)
+{
+    f->last_stream = b->last_stream = st;
+    return launch_wave_resident(wave, x, T, B, h, c, y, f->status, b->status, st);
+}
+
 }  // namespace ql
 
 extern "C" {
@@ -428,6 +435,13 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
     uint8_t *trace = (uint8_t *)trace_dev;
     if (trace && cudaMemsetAsync(trace, 0, qlstm_trace_bytes(q, T, B), st) != cudaSuccess) return QLSTM_ERR_CUDA;
     const int nl = (int)q->layers.size();
+    // the whole stack in one launch, weights resident in the shared memory of thread-block clusters (wave_resident_sm100.cu)
+    if (!trace && q->impl_rec == 0 && q->impl_proj != 1 && wave_resident_taken(q->wave, T, B, q->tables)) {
+        SpanGuard g(q, st, 1);
+        const int rc = launch_wave_resident(q->wave, x_dev, T, B, {h_dev, nullptr}, {c_dev, nullptr}, y_dev, q->status, nullptr, st);
+        g.done(1);
+        return rc;
+    }
     // the whole stack in one launch, every layer at once on its own SMs (wave_sm100.cu)
     if (!trace && (q->impl_rec == 0 || q->impl_rec == 8) && q->impl_proj != 1) {
         if (q->impl_rec == 0 ? wave_preferred(q->wave, T, B, q->tables) : wave_supported(q->wave, T, B, q->tables)) {
@@ -570,6 +584,10 @@ int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long 
 }
 
 int qlstm_debug_wave_plan(qlstm_t *q, int T, int B, int *out4) { return q ? wave_debug_plan(q->wave, T, B, q->tables, out4) : QLSTM_ERR_ARG; }
+
+int qlstm_debug_resident_plan(qlstm_t *q, int T, int B, int *out4) { return q ? wave_resident_debug_plan(q->wave, T, B, out4) : QLSTM_ERR_ARG; }
+
+int qlstm_debug_resident(qlstm_t *q, int mode) { return q && mode >= 0 && mode <= 1 ? wave_resident_mode(q->wave, mode) : QLSTM_ERR_ARG; }
 
 int qlstm_debug_activation_tables(qlstm_t *q, int enable)
 {

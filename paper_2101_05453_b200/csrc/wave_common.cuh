@@ -293,6 +293,20 @@ __device__ __forceinline__ uint4 wv_load16(const int8_t *src, int valid)      //
 
 __host__ __device__ inline size_t wv_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Memory handed out front to back; without a base it is only counted.  Pieces start 64 KB apart: packed at 256 bytes, what a step's
+// exchanges touch lay closer together and took longer (us per call of 100 steps, median of eight handles: four 1024-cell layers with
+// layer norm and projection, 16 rows 1345 and 1300; three of 1000 cells, 37 rows 1568 and 1545).
+struct WaveArena {
+    uint8_t *base = nullptr;
+    size_t used = 0;
+    template <class T>
+    void take(T *&p, size_t bytes)
+    {
+        p = base ? (T *)(base + used) : nullptr;
+        used += wv_up(bytes, 65536);
+    }
+};
+
 // wave_small_sm100.cu
 const void *wave_small_kernel(int G, bool ln, bool peep);
 size_t wave_small_smem(const WaveCall &k, int ns, bool peep);

@@ -33,19 +33,18 @@ QL_HD int32_t floor_s32(float v)
 #endif
 }
 
-// floor(n / d) for n < 2^57, d < 2^26 and a quotient below 2^31; x: reciprocal estimate of d (relative error 2^-21 at most)
-QL_HD uint32_t wv_div(uint64_t n, uint32_t d, float x)
+// Estimates of the hardware.  On a CPU they are exact and are made as wrong as the hardware's may be (skew, relative).
+#if !defined(__CUDA_ARCH__)
+inline float &wv_skew() { static float v = 0.0f; return v; }
+#endif
+QL_HD float wv_rcp_est(float x)
 {
-    uint32_t q = (uint32_t)((float)n * x);                     // within 2^11
-    int64_t r = (int64_t)(n - (uint64_t)q * d);
-    const int32_t c = floor_s32((float)r * x);                 // then within 1 (rounded towards zero, a negative one could be 2 off)
-    q += (uint32_t)c;
-    r -= (int64_t)c * d;
-    if (r < 0) { --q; r += d; }
-    if (r >= (int64_t)d) ++q;
-    return q;
+#if defined(__CUDA_ARCH__)
+    return rcp_est(x);
+#else
+    return 1.0f / x * (1.0f + wv_skew());
+#endif
 }
-
 QL_HD float wv_sqrt_est(float x)
 {
 #if defined(__CUDA_ARCH__)
@@ -53,11 +52,41 @@ QL_HD float wv_sqrt_est(float x)
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 #else
-    return __builtin_sqrtf(x);
+    return __builtin_sqrtf(x) * (1.0f + wv_skew());
 #endif
 }
 
-// Statistics as ln_stats_fast (qmath.cuh) with a shorter chain: one thread per (row, gate) computes them while a group waits.
+QL_HD float wv_to_float(uint64_t v)                 // relative error 2^-23: two 32-bit conversions side by side, where one of 64 bits is several
+{
+    return fma_rn((float)(uint32_t)(v >> 32), 4294967296.0f, (float)(uint32_t)v);
+}
+
+// M for a sigma s >= 2^20 (see sigma_min), in two limbs: 2^42 / s and 2^31 times its remainder / s, plus one.
+QL_HD void wv_limbs(uint32_t s, int32_t &m_hi, int32_t &m_lo)
+{
+    // x is the reciprocal within 2^-22: the first quotient is within 2, its remainder fits 32 bits (2^42 = 0 modulo 2^32)
+    const float x = wv_rcp_est((float)s);
+    uint32_t hi = (uint32_t)(4398046511104.0f * x);
+    int32_t rem = (int32_t)(0u - hi * s);
+    for (int i = 0; i < 2; ++i)
+        if (rem < 0) { --hi; rem += (int32_t)s; }
+    for (int i = 0; i < 2; ++i)
+        if (rem >= (int32_t)s) { ++hi; rem -= (int32_t)s; }
+    // the second within 2^10 at first; what is left is below 2^37 in magnitude, and 2^-8 of it within 32 bits
+    uint32_t lo = (uint32_t)((float)rem * 2147483648.0f * x);
+    const int64_t left = ((int64_t)rem << 31) - (int64_t)lo * s;
+    const int32_t c = floor_s32((float)(int32_t)(left >> 8) * 256.0f * x);
+    lo += (uint32_t)c;
+    const int32_t last = (int32_t)((uint32_t)left - (uint32_t)c * s);
+    if (last < 0) --lo;
+    else if (last >= (int32_t)s) ++lo;
+    ++lo;
+    m_hi = (int32_t)(hi + (lo >> 31));
+    m_lo = (int32_t)(lo & 0x7fffffffu);
+}
+
+// Statistics as ln_stats_fast (qmath.cuh) with a shorter chain: one thread per (row, gate) computes them while a group waits (alone in a
+// warp 1350 cycles with 64-bit conversions and divisions throughout, 850 like this).
 QL_HD WvLnRow wv_make_ln(int64_t sum, int64_t sumsq, const DivMagic &dn, uint32_t sigma_min)
 {
     const uint64_t half = dn.n >> 1;
@@ -67,21 +96,19 @@ QL_HD WvLnRow wv_make_ln(int64_t sum, int64_t sumsq, const DivMagic &dn, uint32_
     const uint64_t r1 = (uint64_t)sumsq - q1 * dn.n;
     int64_t var = (int64_t)((q1 << 20) + div_by_magic((r1 << 20) + half, dn)) - (int64_t)mean * mean;
     if (var < 0) var = 0;
-    // integer root: fp32 estimate (within 2^4), one Newton step, exact correction
-    uint32_t s = (uint32_t)wv_sqrt_est((float)var);
-    const int64_t e = var - (int64_t)s * s;
-    if (s) s += (uint32_t)(int32_t)(0.5f * (float)e * rcp_est((float)s));
-    for (int i = 0; i < 2; ++i)
-        if ((int64_t)s * s > var) --s;
-    for (int i = 0; i < 2; ++i)
-        if ((int64_t)(s + 1u) * (s + 1u) <= var) ++s;
+    // integer root of var < 2^50: fp32 estimate s (relative error 2^-21: within 2^4), one Newton step s + floor(e / 2 s) with the exact
+    // e = var - s^2 (|e| < 2^31).  The root is s + e / 2 s - k with 0 <= k < 1 (k < 2^7 / s; below s = 2^7 the estimate is within 1),
+    // so that the step is within 1 of it.
+    uint32_t s = (uint32_t)wv_sqrt_est(wv_to_float((uint64_t)var));
+    const int32_t e = (int32_t)(var - (int64_t)s * s);
+    if (s) s += (uint32_t)floor_s32(0.5f * (float)e * wv_rcp_est((float)s));
+    const int64_t rest = var - (int64_t)s * s;
+    if (rest < 0) --s;
+    else if (rest > 2 * (int64_t)s) ++s;
     WvLnRow r;
     r.mean = mean; r.sigma = s; r.m_hi = 0; r.m_lo = 0;        // sigma = 0: the quotient is 0
     if (s >= sigma_min) {
-        const float x = rcp_est((float)s);
-        const uint32_t hi = wv_div((uint64_t)1 << 42, s, x);
-        const uint32_t lo = wv_div((uint64_t)((1ull << 42) - (uint64_t)hi * s) << 31, s, x) + 1u;
-        r.m_hi = (int32_t)(hi + (lo >> 31)); r.m_lo = (int32_t)(lo & 0x7fffffffu);
+        wv_limbs(s, r.m_hi, r.m_lo);
     } else if (s) {
         r.sigma |= WV_LN_SLOW;
     }

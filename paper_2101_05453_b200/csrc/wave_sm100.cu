@@ -33,7 +33,7 @@
 #include <utility>
 #include <vector>
 
-#include "wave_common.cuh"
+#include "wave_resident.h"
 
 namespace ql {
 
@@ -896,6 +896,8 @@ struct WaveStack {
     uint4 *gbuf = nullptr;
     uint32_t *cbuf = nullptr;
     void *block[2] = {nullptr, nullptr};       // plans and tables; a call's activations, unless they lie in the caller's scratch
+    ResidentStack *res = nullptr;  // wave_resident_sm100.cu; null: no call of this stack fits it
+    int res_mode = 0;              // 0 where it is the faster path, 1 never, 2 always
     unsigned dbg_missing = 0;
     unsigned long long dbg_limit_ns = 0;
 };
@@ -904,26 +906,13 @@ void wave_destroy(WaveStack *s)
 {
     if (!s) return;
     for (void *p : s->block) cudaFree(p);
+    resident_destroy(s->res);
     delete s;
 }
 
 namespace {
 
 constexpr int WV_SMALL_ROWS = 32;
-
-// Memory handed out front to back; without a base it is only counted.  Pieces start 64 KB apart: packed at 256 bytes, what a step's
-// exchanges touch lay closer together and took longer (us per call of 100 steps, median of eight handles: four 1024-cell layers with
-// layer norm and projection, 16 rows 1345 and 1300; three of 1000 cells, 37 rows 1568 and 1545).
-struct WaveArena {
-    uint8_t *base = nullptr;
-    size_t used = 0;
-    template <class T>
-    void take(T *&p, size_t bytes)
-    {
-        p = base ? (T *)(base + used) : nullptr;
-        used += wv_up(bytes, 65536);
-    }
-};
 
 // Rows a call of B rows is cut into: `rg` row groups times one or two units of at most 128 rows each.
 void wave_units(int B, int rg, int &units, int &nu, int &ra)
@@ -1281,10 +1270,11 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
         for (const void *kernel : f)
             if (kernel && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) return fail(QLSTM_ERR_CUDA);
     }
+    if (s->tabs) s->res = resident_plan(lp, base, max_T, s->max_B, s->max_smem, s->y_stride);
     // everything in at most two allocations (a handle's creation is mostly allocations): counted first, then filled
-    WaveArena keep, work;
+    WaveArena keep, work, rwork;                               // (a call takes one path: their activations share memory)
     for (int pass = 0; pass < 2; ++pass) {
-        keep.used = work.used = 0;
+        keep.used = work.used = rwork.used = 0;
         std::vector<uint8_t *> tab(blobs.size());
         for (size_t i = 0; i < blobs.size(); ++i) {
             keep.take(tab[i], blobs[i].size());
@@ -1315,14 +1305,24 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
                 if (rc != QLSTM_OK) return fail(rc);
             }
         }
-        if (pass) break;
-        if (cudaMalloc(&s->block[0], keep.used) != cudaSuccess) return fail(QLSTM_ERR_NOMEM);
-        keep.base = (uint8_t *)s->block[0];
-        work.base = (uint8_t *)scratch;
-        if (work.used > scratch_bytes) {
-            if (cudaMalloc(&s->block[1], work.used) != cudaSuccess) return fail(QLSTM_ERR_NOMEM);
-            work.base = (uint8_t *)s->block[1];
+        if (s->res) {
+            const int rc = resident_place(s->res, lp, base, keep, rwork, pass);
+            if (rc != QLSTM_OK) return fail(rc);
         }
+        if (pass) break;
+        const size_t activations = std::max(work.used, rwork.used);
+        if (cudaMalloc(&s->block[0], keep.used) != cudaSuccess || (activations > scratch_bytes && cudaMalloc(&s->block[1], activations) != cudaSuccess)) {
+            if (!s->res) return fail(QLSTM_ERR_NOMEM);
+            // without the resident form, then
+            cudaGetLastError();
+            for (void *&b : s->block) { cudaFree(b); b = nullptr; }
+            resident_destroy(s->res);
+            s->res = nullptr;
+            --pass;
+            continue;
+        }
+        keep.base = (uint8_t *)s->block[0];
+        work.base = rwork.base = activations > scratch_bytes ? (uint8_t *)s->block[1] : (uint8_t *)scratch;
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(QLSTM_ERR_CUDA);
     *out = s;
@@ -1376,6 +1376,31 @@ bool wave_preferred(const WaveStack *s, int T, int B, bool tables)
         s->resident <= (size_t)s->sm_count * 96 * 1024)
         return false;
     return T * 256 > s->depth * (B - 32);
+}
+
+bool wave_resident_taken(const WaveStack *s, int T, int B, bool tables)
+{
+    return s && s->res_mode != 1 && tables && resident_supported(s->res, T, B);
+}
+
+int wave_resident_mode(WaveStack *s, int mode)
+{
+    if (s) s->res_mode = mode;
+    return s && s->res ? 1 : 0;
+}
+
+int wave_resident_debug_plan(const WaveStack *s, int T, int B, int *out4)
+{
+    if (!out4) return QLSTM_ERR_ARG;
+    if (s) resident_debug_plan(s->res, T, B, out4);
+    else out4[0] = out4[1] = out4[2] = out4[3] = 0;
+    return QLSTM_OK;
+}
+
+int launch_wave_resident(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
+                         cudaStream_t st)
+{
+    return launch_resident(s->res, x, T, B, h, c, y, status, status2, s->dbg_missing, s->dbg_limit_ns ? s->dbg_limit_ns : WV_WAIT_LIMIT_NS, st);
 }
 
 int wave_debug_plan(const WaveStack *s, int T, int B, bool tables, int *out4)

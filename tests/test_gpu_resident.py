@@ -1,0 +1,69 @@
+"""The wavefront kernel with resident weights against the CPU oracle, bit for bit, at the edges of its tiles and clusters (needs a B200)."""
+import numpy as np
+import pytest
+
+from oracle import qlstm_ref as R
+from tests.gpu_util import run_gpu
+from tests.test_gpu_wave import VARIANTS
+from workloads import random_layer_stack
+
+pytestmark = pytest.mark.gpu
+
+IDS = lambda k: "+".join(sorted(k)) or "basic"
+
+
+def check(w, **plan):
+    """One call through the kernel; `plan` pins what its plan must be (cluster: 1 or "many", tiles, groups)."""
+    import paper_2101_05453_b200 as qlstm
+    want = R.run(w.layers, w.x, *w.initial_state())
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        cluster, groups, tiles, units = q.debug_resident_plan(w.T, w.B)
+        assert cluster >= 1, "not taken"
+        if "cluster" in plan:
+            assert (cluster == 1) == (plan["cluster"] == 1), cluster
+        if "tiles" in plan:
+            assert tiles == plan["tiles"], tiles
+        for _ in range(2):                                     # (a second call: what the first one left behind)
+            got = run_gpu(w, handle=q)
+            for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+                assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}, plan {(cluster, groups, tiles, units)}"
+
+
+# one block per layer and row group, and clusters of several; one row to several tiles of eight; partial groups of eight cells
+@pytest.mark.parametrize("B", [1, 7, 8, 40])
+@pytest.mark.parametrize("kw", VARIANTS, ids=IDS)
+def test_resident_one_block(kw, B):
+    check(random_layer_stack(910 + B, 2, 32, 40, 24, T=7, B=B, **kw), cluster=1)
+
+
+@pytest.mark.parametrize("B", [1, 9, 30, 60])
+@pytest.mark.parametrize("kw", VARIANTS, ids=IDS)
+def test_resident_clusters(kw, B):
+    check(random_layer_stack(920 + B, 3, 80, 304, 208, T=7, B=B, **kw), cluster="many")
+
+
+# dimensions that nothing divides (x and y in bytes), more blocks than outputs, calls of one and two steps
+@pytest.mark.parametrize("T", [1, 2, 9])
+@pytest.mark.parametrize("kw", VARIANTS, ids=IDS)
+def test_resident_odd_dimensions(kw, T):
+    check(random_layer_stack(930 + T, 2, 19, 37, 23, T=T, B=5, **kw))
+    check(random_layer_stack(940 + T, 3, 83, 501, 9, T=T, B=13, **dict(kw, projection=True)))
+
+
+# two and four tiles of eight rows, some groups with one tile fewer than others
+@pytest.mark.parametrize("B,tiles", [(100, 2), (200, 4)])
+@pytest.mark.parametrize("kw", VARIANTS, ids=IDS)
+def test_resident_tiles_of_rows(kw, B, tiles):
+    check(random_layer_stack(950 + B, 16, 32, 48, 32, T=3, B=B, **kw), tiles=tiles)
+
+
+# gate sums so small that layer-norm quotients leave the fast range, or that whole rows are zero
+@pytest.mark.parametrize("shift", [4, 9, 15])
+@pytest.mark.parametrize("peephole", [False, True])
+def test_resident_layernorm_of_small_deviations(shift, peephole):
+    for dims in ((48, 112, 64), (64, 400, 160)):
+        w = random_layer_stack(960, 3, *dims, projection=True, layernorm=True, peephole=peephole, T=5, B=5)
+        for q in w.layers:
+            q.eff_x = [(m, s - shift) for m, s in q.eff_x]
+            q.eff_h = [(m, s - shift) for m, s in q.eff_h]
+        check(w)

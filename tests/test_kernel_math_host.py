@@ -299,6 +299,18 @@ def test_wave_statistics_against_python_integers(H):
                 assert (out[3], out[4]) == (0, 0)
 
 
+@pytest.mark.parametrize("skew", [2.0 ** -22, -2.0 ** -22])
+def test_wave_statistics_with_estimates_as_wrong_as_the_hardwares(H, skew):
+    """The same with square root and reciprocal estimates off by more than the instructions' documented 2^-23."""
+    H.qmh_wave_skew.argtypes = [C.c_float]
+    H.qmh_wave_skew(skew)
+    try:
+        test_wave_statistics_against_python_integers(H)
+        test_wave_quotients_with_exact_ties(H)
+    finally:
+        H.qmh_wave_skew(0.0)
+
+
 def test_wave_division(H):
     """wv_div over the range it is used for: n < 2^57, d < 2^26, quotient below 2^31."""
     H.qmh_wave_div.restype = C.c_uint32
