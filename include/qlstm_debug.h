@@ -42,6 +42,10 @@ int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long 
 int qlstm_debug_wave_plan(qlstm_t *q, int T, int B, int *out4);
 int qlstm_bidir_debug_wave_plan(qlstm_bidir_t *q, int T, int B, int *out4);
 
+/* Blocks of the thread-block clusters in which the few-row wavefront kernel takes such calls (with memoised nonlinearities); 0: without
+ * clusters, or not taken by that kernel.  Negative: error code. */
+int qlstm_debug_wave_cluster(qlstm_t *q, int T, int B);
+
 /* The wavefront kernel with resident weights (thread-block clusters; it comes before all others for the calls that it takes, with
  * automatic selection).  Its plan: out4 (host) receives the blocks of a cluster (0: does not take such calls), the row groups, the
  * tiles of eight rows of a group, and the groups of eight cells per warp.  Mode 0: automatic, 1: never taken; returns whether the

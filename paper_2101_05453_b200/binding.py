@@ -24,7 +24,7 @@ EXPORTS = ["qlstm_create", "qlstm_run", "qlstm_run_host", "qlstm_input_projectio
            "qlstm_get_profile", "qlstm_device_info", "qlstm_eval_activations", "qlstm_eval_layernorm_row",
            "qlstm_eval_activation_tables", "qlstm_eval_activation_lines", "qlstm_debug_activation_tables",
            "qlstm_layernorm_rows_static", "qlstm_debug_barrier_timeout", "qlstm_debug_ring_plan",
-           "qlstm_debug_wave_plan", "qlstm_bidir_debug_wave_plan", "qlstm_debug_resident_plan", "qlstm_bidir_debug_resident_plan",
+           "qlstm_debug_wave_plan", "qlstm_bidir_debug_wave_plan", "qlstm_debug_wave_cluster", "qlstm_debug_resident_plan", "qlstm_bidir_debug_resident_plan",
            "qlstm_debug_resident", "qlstm_bidir_debug_resident", "qlstm_debug_projection_plan", "qlstm_debug_mma_i8_peak", "qlstm_debug_barrier_latency",
            "qlstm_bidir_create", "qlstm_bidir_run", "qlstm_bidir_last_status", "qlstm_bidir_destroy",
            "qlstm_calibrate", "qlstm_quantize_model", "qlstm_quantized_layers", "qlstm_quantized_scales",
@@ -126,6 +126,8 @@ def lib():
         L.qlstm_eval_layernorm_row.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, Scale, C.c_void_p, C.c_void_p]
         L.qlstm_debug_barrier_timeout.restype = C.c_int
         L.qlstm_debug_barrier_timeout.argtypes = [C.c_void_p, C.c_int, C.c_ulonglong]
+        L.qlstm_debug_wave_cluster.restype = C.c_int
+        L.qlstm_debug_wave_cluster.argtypes = [C.c_void_p, C.c_int, C.c_int]
         for f in (L.qlstm_debug_resident, L.qlstm_bidir_debug_resident):
             f.restype = C.c_int
             f.argtypes = [C.c_void_p, C.c_int]
@@ -305,6 +307,12 @@ class QLSTM:
         out = (C.c_int * 4)()
         _check(lib().qlstm_debug_wave_plan(self._h, T, B, out), "qlstm_debug_wave_plan")
         return tuple(out)
+
+    def debug_wave_cluster(self, T: int, B: int) -> int:
+        """Blocks of a cluster of the few-row wavefront kernel, 0: none; see qlstm_debug.h."""
+        n = lib().qlstm_debug_wave_cluster(self._h, T, B)
+        _check(n if n < 0 else 0, "qlstm_debug_wave_cluster")
+        return n
 
     def debug_resident_plan(self, T: int, B: int):
         """(blocks of a cluster, row groups, tiles of rows, cell groups per warp) of the kernel with resident weights; see qlstm_debug.h."""

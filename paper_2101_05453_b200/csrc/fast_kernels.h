@@ -120,6 +120,7 @@ int bidir_wave_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int
                    cudaStream_t st);
 int bidir_resident_run(qlstm_t *f, qlstm_t *b, WaveStack *wave, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y,
                        cudaStream_t st);
+int wave_debug_cluster(const WaveStack *s, int T, int B);                // include/qlstm_debug.h
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns);
 
 int debug_ring_plan(int stages, int n_own, int contig, int per, int n_total, int *out);

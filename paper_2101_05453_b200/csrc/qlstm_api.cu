@@ -585,6 +585,8 @@ int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long 
 
 int qlstm_debug_wave_plan(qlstm_t *q, int T, int B, int *out4) { return q ? wave_debug_plan(q->wave, T, B, q->tables, out4) : QLSTM_ERR_ARG; }
 
+int qlstm_debug_wave_cluster(qlstm_t *q, int T, int B) { return q ? wave_debug_cluster(q->wave, T, B) : QLSTM_ERR_ARG; }
+
 int qlstm_debug_resident_plan(qlstm_t *q, int T, int B, int *out4) { return q ? wave_resident_debug_plan(q->wave, T, B, out4) : QLSTM_ERR_ARG; }
 
 int qlstm_debug_resident(qlstm_t *q, int mode) { return q && mode >= 0 && mode <= 1 ? wave_resident_mode(q->wave, mode) : QLSTM_ERR_ARG; }

@@ -66,6 +66,7 @@ struct WaveCall {
     int w_evict;                   // weights with an evict-first hint
     int nbuf;                      // gate buffers per unit: [gate sums | X ...]
     int max_ppc, max_opc, max_tab;
+    int cl, cl_slots;              // wave_small_sm100.cu: blocks of a cluster (0: exchanges through global memory), its slots of layer-norm sums
     int8_t *y;
     int y_stride;                  // bytes of a row of y
     uint4 *gbuf;                   // [blocks][units][nbuf][max_ppc][max rows] gate buffers in global memory
@@ -207,6 +208,64 @@ __device__ __forceinline__ void wv_load_weights(void *dst, const void *src, uint
                  : "memory");
 }
 
+// ---- thread-block clusters: stores into the shared memory of peers, counted in bytes on an mbarrier there ----------------------
+__device__ __forceinline__ uint32_t wv_peer(uint32_t addr, int rank)
+{
+    uint32_t d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+    return d;
+}
+__device__ __forceinline__ void wv_cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void wv_send8(uint32_t dst, uint2 v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void wv_send16(uint32_t dst, uint4 v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z),
+                 "r"(v.w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ bool wv_try_cluster(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, P;\n\t}"
+        : "=r"(ok)
+        : "r"(ptx::smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// The rest of a wait (whole warp) whose first attempt has not seen its phase complete: until it does, another block has given up or
+// the limit is over.
+static __device__ __noinline__ bool wv_wait_cluster_slow(uint64_t *bar, uint32_t parity, unsigned *abort_word, unsigned long long limit_ns, volatile int *abort_flag)
+{
+    const unsigned long long t0 = wv_timer();
+    for (unsigned n = 1;; ++n) {
+        if (__all_sync(0xffffffffu, wv_try_cluster(bar, parity))) return true;
+        unsigned stop = 0;
+        if ((threadIdx.x & 31) == 0) {
+            if (*abort_flag) stop = 1;
+            else if ((n & 7u) == 0u) {
+                if (wv_ld_acquire(abort_word) != 0u) { *abort_flag = 1; stop = 1; }
+                else if (wv_timer() - t0 > limit_ns) { atomicExch(abort_word, 1u); *abort_flag = 1; stop = 1; }
+            }
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+    }
+}
+// whole warp; what peers stored and counted on `bar` (wv_send8, wv_send16) has arrived; false once an abort is seen
+__device__ __forceinline__ bool wv_wait_cluster(uint64_t *bar, uint32_t parity, unsigned *abort_word, unsigned long long limit_ns, volatile int *abort_flag)
+{
+    if (__all_sync(0xffffffffu, wv_try_cluster(bar, parity))) return true;
+    return wv_wait_cluster_slow(bar, parity, abort_word, limit_ns, abort_flag);
+}
+
 // ---- fixed-point pieces ----------------------------------------------------------------------------------------------
 __device__ __forceinline__ int32_t wv_lo(uint32_t w) { return (int32_t)(w << 16) >> 16; }
 __device__ __forceinline__ int32_t wv_hi(uint32_t w) { return (int32_t)w >> 16; }
@@ -308,7 +367,7 @@ struct WaveArena {
 };
 
 // wave_small_sm100.cu
-const void *wave_small_kernel(int G, bool ln, bool peep);
+const void *wave_small_kernel(int G, bool ln, bool peep, bool cluster);
 size_t wave_small_smem(const WaveCall &k, int ns, bool peep);
 void wave_small_tile_weights(const int8_t *src, int8_t *dst, int G, int rows, int K, int n, int per_rank, int nt, int per_tile, int padded, int nkb, int kps);
 

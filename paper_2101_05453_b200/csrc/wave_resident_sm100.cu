@@ -22,7 +22,7 @@
 // h^t for the layer above or y; neither is on the chain.  Buffers of h alternate between two; a peer's h^t is complete only after
 // every block has read h^{t-2}, so that writing it needs no permission.
 //
-// Every wait is bounded: see rs_wait_slow.
+// Every wait is bounded: see wv_wait_cluster_slow.
 #include <algorithm>
 #include <cstring>
 
@@ -110,39 +110,7 @@ __host__ __device__ inline RsLayout rs_layout(const ResLayer &L, int cl, int nt,
     return l;
 }
 
-// ---- cluster and mma.sync primitives -------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t rs_peer(uint32_t addr, int rank)
-{
-    uint32_t d;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
-    return d;
-}
-__device__ __forceinline__ void rs_cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ void rs_send8(uint32_t dst, uint2 v, uint32_t bar)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void rs_send16(uint32_t dst, uint4 v, uint32_t bar)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z),
-                 "r"(v.w), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ bool rs_try(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred P;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, P;\n\t}"
-        : "=r"(ok)
-        : "r"(ptx::smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
+// ---- waits and mma.sync -------------------------------------------------------------------------------------
 // without waiting
 __device__ __forceinline__ bool rs_test(uint64_t *bar, uint32_t parity)
 {
@@ -156,28 +124,9 @@ __device__ __forceinline__ bool rs_test(uint64_t *bar, uint32_t parity)
         : "memory");
     return __all_sync(0xffffffffu, ok != 0);
 }
-// The rest of a wait (whole warp) whose first attempt has not seen its phase complete: until it does, another block has given up or
-// the limit is over.
-__device__ __noinline__ bool rs_wait_slow(uint64_t *bar, uint32_t parity, unsigned *abort_word, unsigned long long limit_ns, volatile int *abort_flag)
-{
-    const unsigned long long t0 = wv_timer();
-    for (unsigned n = 1;; ++n) {
-        if (__all_sync(0xffffffffu, rs_try(bar, parity))) return true;
-        unsigned stop = 0;
-        if ((threadIdx.x & 31) == 0) {
-            if (*abort_flag) stop = 1;
-            else if ((n & 7u) == 0u) {
-                if (wv_ld_acquire(abort_word) != 0u) { *abort_flag = 1; stop = 1; }
-                else if (wv_timer() - t0 > limit_ns) { atomicExch(abort_word, 1u); *abort_flag = 1; stop = 1; }
-            }
-        }
-        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
-    }
-}
 __device__ __forceinline__ bool rs_wait(const ResCall &k, uint64_t *bar, uint32_t parity, volatile int *abort_flag)
 {
-    if (__all_sync(0xffffffffu, rs_try(bar, parity))) return true;
-    return rs_wait_slow(bar, parity, k.abort_word, k.limit_ns, abort_flag);
+    return wv_wait_cluster(bar, parity, k.abort_word, k.limit_ns, abort_flag);
 }
 // until *cnt has reached target (whole warp)
 __device__ __forceinline__ bool rs_wait_count(const ResCall &k, const unsigned *cnt, unsigned target, volatile int *abort_flag)
@@ -272,7 +221,7 @@ __device__ __forceinline__ void rs_send_tile(uint8_t *stage, int32_t v0, int32_t
     for (int j = 0; j < 4; ++j) {
         const int p = (lane >> 3) + 4 * j;
         if (4 * j >= n) break;                                 // warp-uniform
-        if (p < n && p != rank && valid) rs_send8(a + peer[j], v, bar + peer[j]);
+        if (p < n && p != rank && valid) wv_send8(a + peer[j], v, bar + peer[j]);
     }
     if (lane < 8 && valid) *reinterpret_cast<uint2 *>(at) = v;
 }
@@ -416,7 +365,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
             const int r = i / L.O;
             smem[lay.h + (size_t)r * L.ph + (i - r * L.O)] = (uint8_t)L.h[(size_t)row0 * L.O + i];
         }
-    rs_cluster_sync();
+    wv_cluster_sync();
 
     if (warp == 0) {
         // ---------------- x ----------------
@@ -522,7 +471,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int p = (lane >> 3) + 4 * j;
-            peer[j] = (uint32_t)rs_keep((int)(rs_peer(ptx::smem_u32(smem), p < cl ? p : 0) - ptx::smem_u32(smem)));
+            peer[j] = (uint32_t)rs_keep((int)(wv_peer(ptx::smem_u32(smem), p < cl ? p : 0) - ptx::smem_u32(smem)));
         }
         const ActLines at = make_act_lines(ptx::smem_u32(smem + lay.tab), L.tab_lay);
         uint8_t *stage = smem + lay.stage + (size_t)cw * 64;
@@ -636,7 +585,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
                                 if (r >= rows) continue;
                                 const uint32_t *v = st + (z0 + e) * 3 * r8 + r;
                                 uint4 *dst = sx + ((size_t)rank * sx_slots + e) * r8 + r;
-                                rs_send16(rs_peer(ptx::smem_u32(dst), p), make_uint4(v[0], v[r8], v[2 * r8], 0u), rs_peer(ptx::smem_u32(bar), p));
+                                wv_send16(wv_peer(ptx::smem_u32(dst), p), make_uint4(v[0], v[r8], v[2 * r8], 0u), wv_peer(ptx::smem_u32(bar), p));
                             }
                     for (int i0 = uidx * 32; i0 < nc; i0 += uw * 32) {
                         if (ncb > 1 && !rs_wait(k, bar, par, abort_flag)) return false;
@@ -789,7 +738,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int p = (lane >> 3) + 4 * j;
-            peer[j] = (uint32_t)rs_keep((int)(rs_peer(ptx::smem_u32(smem), p < cl ? p : 0) - ptx::smem_u32(smem)));
+            peer[j] = (uint32_t)rs_keep((int)(wv_peer(ptx::smem_u32(smem), p < cl ? p : 0) - ptx::smem_u32(smem)));
         }
         uint8_t *stage = smem + lay.stage + (size_t)(hw + pi) * 64;
         uint8_t *const hbuf = smem + lay.h, *const mbuf = smem + lay.m;
@@ -857,7 +806,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
             if (n > 0) wv_drain(&ctl->x_full[i], (uint32_t)(n - 1) & 1u);
         }
     }
-    rs_cluster_sync();
+    wv_cluster_sync();
     if (threadIdx.x == 0) {
         if (aborted) {
             // what peers sent before they came here arrives within microseconds; this block does not end before

@@ -872,6 +872,7 @@ constexpr int WV_MAX_ROWS = 256;
 // 32 rows per row group (wave_small_sm100.cu).
 struct WavePlan {
     int mode = 0, rg = 1, grid = 0;
+    int cl = 0;                    // mode 1: blocks of a cluster that is a (layer, row group); 0: no clusters
     bool ok = true, used = false;
     int max_ppc = 0, max_cpc = 0, max_opc = 0, b_slot = 0;
     std::vector<WaveLayer> layer;
@@ -897,7 +898,7 @@ struct WaveStack {
     uint32_t *cbuf = nullptr;
     void *block[2] = {nullptr, nullptr};       // plans and tables; a call's activations, unless they lie in the caller's scratch
     ResidentStack *res = nullptr;  // wave_resident_sm100.cu; null: no call of this stack fits it
-    int res_mode = 0;              // 0 where it is the faster path, 1 never, 2 always
+    int res_mode = 0;              // 1: never taken
     unsigned dbg_missing = 0;
     unsigned long long dbg_limit_ns = 0;
 };
@@ -988,7 +989,7 @@ int wave_row_groups(const WaveStack *s, int mode, const std::vector<const LayerP
 }
 
 // Shares of the blocks of one layer under `mode`, `per` blocks at most; false: the plan does not work.
-bool wave_share_layer(int mode, const LayerParams &p, int per, WaveLayer &L)
+bool wave_share_layer(int mode, const LayerParams &p, int per, bool cluster, WaveLayer &L)
 {
     const bool proj = p.flags & F_PROJECTION;
     L.opc = 0; L.ntp = 0; L.opt = 4; L.npadp = 16; L.opp = 8; L.kpp = 1;
@@ -1009,6 +1010,7 @@ bool wave_share_layer(int mode, const LayerParams &p, int per, WaveLayer &L)
         if (L.npad > WV_ACC_COLS || L.npadp > WV_ACC_COLS || 2 * (4 * L.nt + L.ntp + 4) > WV_MAX_OPS) return false;
     } else {
         L.cpc = (p.C + per - 1) / per;
+        if (cluster) L.cpc = wv_round(L.cpc, 8);               // (m and h cross the cluster in pieces of at least 8 bytes)
         L.n = (p.C + L.cpc - 1) / L.cpc;
         L.nt = (L.cpc + 31) / 32;
         L.ct = (L.cpc + L.nt - 1) / L.nt;
@@ -1016,6 +1018,7 @@ bool wave_share_layer(int mode, const LayerParams &p, int per, WaveLayer &L)
         L.kpg = 32 / L.ctp;
         if (proj) {
             L.opc = (p.O + L.n - 1) / L.n;
+            if (cluster) L.opc = wv_round(L.opc, 8);
             L.ntp = (L.opc + 127) / 128;
             L.opt = (L.opc + L.ntp - 1) / L.ntp;
             L.opp = wv_round(L.opt, 8);
@@ -1032,18 +1035,18 @@ bool wave_share_layer(int mode, const LayerParams &p, int per, WaveLayer &L)
 }
 
 // The plan of `mode` with rg row groups, made on first request; its number in s->plan.
-int wave_plan(WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, int mode, int rg)
+int wave_plan(WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, int mode, int rg, int cl = 0)
 {
     for (size_t i = 0; i < s->plan.size(); ++i)
-        if (s->plan[i].mode == mode && s->plan[i].rg == rg) return (int)i;
+        if (s->plan[i].mode == mode && s->plan[i].rg == rg && s->plan[i].cl == cl) return (int)i;
     WavePlan pl;
-    pl.mode = mode; pl.rg = rg;
+    pl.mode = mode; pl.rg = rg; pl.cl = cl;
     int prev_n = 0;
     for (size_t l = 0; l < lp.size() && pl.ok; ++l) {
         WaveLayer M = base[l];
-        if (!wave_share_layer(mode, *lp[l], s->sm_count / ((int)lp.size() * rg), M)) { pl.ok = false; break; }
+        if (!wave_share_layer(mode, *lp[l], cl ? cl : s->sm_count / ((int)lp.size() * rg), cl > 0, M)) { pl.ok = false; break; }
         M.cta0 = pl.grid;
-        pl.grid += M.n * rg;
+        pl.grid += (cl ? cl : M.n) * rg;
         M.below = M.first ? 0 : prev_n;
         prev_n = M.n;
         pl.max_ppc = std::max(pl.max_ppc, M.ppc);
@@ -1087,6 +1090,8 @@ bool wave_describe(const WaveStack *s, const WavePlan &pl, int T, int B, bool ta
     if (pl.mode == 1) {
         if (rows > WV_SMALL_ROWS || !tables || !s->tabs) return false;
         k.max_tab = s->max_tab;
+        k.cl = pl.cl;
+        k.cl_slots = s->ln ? (s->peep ? 5 : 4) : 0;
         for (const WaveLayer &L : pl.layer)
             if ((2 * L.nt + L.ntp) * k.ra > 512) return false;
         k.nb = 8;
@@ -1118,6 +1123,54 @@ bool wave_describe(const WaveStack *s, const WavePlan &pl, int T, int B, bool ta
     k.max_tab = k.tab ? s->max_tab : 0;
     smem = total(k.na, k.nb, k.tab, k.gx_s);
     return true;
+}
+
+// Clusters of cl blocks of the few-row kernel that fit on the device at once (a block per SM).
+int wave_max_clusters(const WaveStack *s, int cl)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(cl); c.blockDim = dim3(WV_THREADS); c.dynamicSmemBytes = (size_t)s->max_smem;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeClusterDimension;
+    a[0].val.clusterDim.x = (unsigned)cl; a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+    c.attrs = a; c.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, wave_small_kernel(s->G, s->ln, s->peep, true), &c) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return n;
+}
+
+// An estimate of a step of the few-row kernel in us: the weights of a block at 125 KB/us, its exchanges, and what grows with its cells.
+double wave_step_estimate(const WaveStack *s, const std::vector<const LayerParams *> &lp, int per, bool cluster, int rows)
+{
+    double worst = 0;
+    for (const LayerParams *p : lp) {
+        int cpc = (p->C + per - 1) / per;
+        if (cluster) cpc = wv_round(cpc, 8);
+        const int n = (p->C + cpc - 1) / cpc;
+        const bool proj = p->flags & F_PROJECTION;
+        const double bytes = (double)cpc * p->G * (p->I + p->O) + (proj ? (double)((p->O + n - 1) / n) * p->C : 0.0);
+        const int exchanges = 1 + (s->ln ? 1 : 0) + (proj ? 1 : 0) + (s->ln && s->peep ? 1 : 0);
+        worst = std::max(worst, bytes / 125e3 + exchanges * (cluster ? 1.0 : 2.1) + 0.5 * rows * cpc / 512);
+    }
+    return worst;
+}
+
+// Whether calls of B rows go to clusters, and to how many groups of clusters of which size.  `clusters`: [cl] that fit at once.
+bool wave_cluster_plan(const WaveStack *s, const std::vector<const LayerParams *> &lp, const int *clusters, int B, int rg_other, int &rg, int &cl)
+{
+    const int n = (int)lp.size();
+    double best = 0.97 * wave_step_estimate(s, lp, s->sm_count / (n * rg_other), false, (B + rg_other - 1) / rg_other);
+    cl = 0;
+    for (int size = 8; size <= 16; ++size)
+        for (int groups = 1; groups <= B && groups * n <= clusters[size]; groups *= 2) {
+            const int rows = (B + groups - 1) / groups;
+            if (rows > WV_SMALL_ROWS || (groups > 1 && groups * s->weights > (size_t)(s->ln ? 200 : 128) * 1000000)) continue;
+            const double e = wave_step_estimate(s, lp, size, true, rows);
+            if (e >= best) continue;
+            best = e;
+            rg = groups; cl = size;
+        }
+    return cl > 0;
 }
 
 // words of WaveStack::zero that a call of nu units of ra rows uses: abort word, counters, layer-norm totals
@@ -1240,6 +1293,27 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     WaveCall k;
     size_t smem, rows_alloc = 0, zero_words = 0, g_bytes = 0, c_bytes = 0;
     for (int B = 1; B <= s->max_B; ++B) s->fit_groups[B] = (uint16_t)wave_fit_groups(s, lp, B);
+    int clusters[17] = {};
+    if (s->tabs) {
+        const void *f = wave_small_kernel(s->G, s->ln, s->peep, true);
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) == cudaSuccess &&
+            cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+            for (int size = 8; size <= 16; ++size) clusters[size] = wave_max_clusters(s, size);
+        else
+            cudaGetLastError();
+    }
+    for (int B = 1; B <= s->max_B; ++B) {
+        int rg, cl;
+        const int other = wave_row_groups(s, 1, lp, B);
+        if (!wave_small_fits(s, lp, other, B, s->sm_count) || !wave_cluster_plan(s, lp, clusters, B, other, rg, cl)) continue;
+        const int i = wave_plan(s, lp, base, 1, rg, cl);
+        WavePlan &pl = s->plan[i];
+        if (!wave_describe(s, pl, max_T, B, true, k, smem)) continue;
+        pl.used = true;
+        s->by_rows[1][B] = (int8_t)i;
+        rows_alloc = std::max(rows_alloc, (size_t)k.nu * k.ra);
+        zero_words = std::max(zero_words, wave_zero_words(s, k.nu, k.ra));
+    }
     for (int tab = 1; tab >= 0; --tab)
         for (int B = 1; B <= s->max_B; ++B)
             for (int mode = tab; mode >= 0 && s->by_rows[tab][B] < 0; --mode) {
@@ -1265,7 +1339,8 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     // (only of the forms that some call takes: setting an attribute loads a kernel, some milliseconds the first time in a process)
     for (const WavePlan &pl : s->plan) {
         if (!pl.used) continue;
-        const void *f[2] = {wave_small_kernel(s->G, s->ln, s->peep), nullptr};
+        if (pl.cl) continue;                                   // (set above)
+        const void *f[2] = {wave_small_kernel(s->G, s->ln, s->peep, false), nullptr};
         if (pl.mode == 0) { f[0] = wave_kernel_of<true>(s->G, s->ln, s->peep); f[1] = wave_kernel_of<false>(s->G, s->ln, s->peep); }
         for (const void *kernel : f)
             if (kernel && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess) return fail(QLSTM_ERR_CUDA);
@@ -1416,6 +1491,12 @@ int wave_debug_plan(const WaveStack *s, int T, int B, bool tables, int *out4)
     return QLSTM_OK;
 }
 
+int wave_debug_cluster(const WaveStack *s, int T, int B)
+{
+    const WavePlan *pl = wave_plan_of(s, T, B, true);
+    return pl ? pl->cl : 0;
+}
+
 void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long long limit_ns)
 {
     if (!s) return;
@@ -1452,9 +1533,17 @@ int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[
     k_wave_prepare<<<blocks, 256, 0, st>>>(k, x, s->zero, wave_zero_words(s, k.nu, k.ra));
     if (cudaGetLastError() != cudaSuccess) return QLSTM_ERR_CUDA;
     void *args[] = {(void *)&k};
-    const void *f = pl.mode == 1 ? wave_small_kernel(s->G, s->ln, s->peep)
+    const void *f = pl.mode == 1 ? wave_small_kernel(s->G, s->ln, s->peep, pl.cl > 0)
                               : (k.tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep));
-    cudaError_t e = cudaLaunchCooperativeKernel(f, dim3(pl.grid), dim3(WV_THREADS), args, smem, st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(pl.grid); cfg.blockDim = dim3(WV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)pl.cl; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = pl.cl ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, f, args);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e == cudaErrorCooperativeLaunchTooLarge ? QLSTM_ERR_LAUNCH : QLSTM_ERR_CUDA;

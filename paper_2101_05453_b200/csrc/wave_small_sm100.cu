@@ -8,6 +8,11 @@
 //     step t have been read, and is only rescaled together with H(t + 1).
 // A gate tile holds up to 32 cells, gate slot g in the lanes 32 g .. 32 g + 31: a warp's lanes share a gate and its scales,
 // and a row's layer-norm sums over a tile are warp-wide reductions.
+//
+// Two forms.  With CL a (layer, row group) is one thread-block cluster of up to 16 blocks, and what its own chain needs - layer-norm sums,
+// m, h - goes from shared memory into the shared memory of the peers (16 or 8 bytes at a time, counted on an mbarrier there) instead of
+// through L2 with a counter to poll and a copy back; only what the layer above reads is still written and published there, off the chain.
+// Without, groups may have any number of blocks.  The plan takes the cheaper one (wave_cluster_plan).
 #include <cstring>
 
 #include "wave_common.cuh"
@@ -26,6 +31,7 @@ struct WsCtl {
     uint64_t w_full[WS_SLOTS], w_empty[WS_SLOTS];
     uint64_t op_full[3], op_empty[3];          // operands x, h, m
     uint64_t gate_full[WS_MAX_TILES], acc_empty, p_full, p_empty, tab_full, mma_done[2];
+    uint64_t hx_full[2], mx_full, s_full[2];   // CL: what the cluster has sent to this block
     uint32_t tmem_base;
     int abort_flag, exit_at;
     int op_copies[3];              // copies of each operand that have been requested
@@ -33,8 +39,8 @@ struct WsCtl {
     uint32_t end_phase;
 };
 
-// [weight ring][x][h][m][control][constants][statistics][tables][gates][cell states]
-struct WsLayout { size_t act[3], ctl, consts, st, ln, tab, gates, c, total; };
+// [weight ring][x][h][m][control][constants][statistics][tables][gates][cell states][peers' sums][m and h on their way out]
+struct WsLayout { size_t act[3], ctl, consts, st, ln, tab, gates, c, sx, stage_m, stage_h, total; };
 
 __host__ __device__ inline WsLayout ws_layout(const WaveCall &k, int ns, int rows, bool peep)
 {
@@ -42,6 +48,7 @@ __host__ __device__ inline WsLayout ws_layout(const WaveCall &k, int ns, int row
     l.act[0] = (size_t)ns * k.b_slot;
     l.act[1] = l.act[0] + (size_t)k.max_kb_i * k.ra * 128;
     l.act[2] = l.act[1] + (size_t)k.max_kb_h * k.ra * 128;
+    if (k.cl) l.act[2] += (size_t)k.max_kb_h * k.ra * 128;     // (h in two buffers: peers may be a step ahead)
     l.ctl = l.act[2] + (size_t)k.max_kb_c * k.ra * 128;
     l.consts = l.ctl + wv_up(sizeof(WsCtl), 16);
     l.st = l.consts + wv_up((size_t)k.max_cpc * 4 * (3 * 4 + 2 * 2) + (size_t)k.max_opc * 4, 16);
@@ -49,7 +56,10 @@ __host__ __device__ inline WsLayout ws_layout(const WaveCall &k, int ns, int row
     l.tab = l.ln + 4 * WS_ROWS * 16;
     l.gates = l.tab + wv_up((size_t)k.max_tab, 16);
     l.c = l.gates + wv_up((size_t)(peep ? 5 : 4) * rows * k.max_cpc * 2, 16);
-    l.total = l.c + wv_up((size_t)rows * k.max_cpc * 2, 16);
+    l.sx = l.c + wv_up((size_t)rows * k.max_cpc * 2, 16);
+    l.stage_m = l.sx + (size_t)k.cl * k.cl_slots * k.ra * 16;
+    l.stage_h = l.stage_m + (k.cl ? wv_up((size_t)rows * k.max_cpc, 16) : 0);
+    l.total = l.stage_h + (k.cl ? wv_up((size_t)rows * k.max_opc, 16) : 0);
     // an MMA reads 128 rows of 128 bytes from where its k-block starts, whatever the tile holds
     if (l.total < l.act[0] + 128 * 128) l.total = l.act[0] + 128 * 128;
     l.total += 1024;                           // alignment of the ring
@@ -64,6 +74,9 @@ struct WsSmem {
     WvLnRow *ln;                   // [4][32]
     int16_t *g;                    // [slot][row][cpc] gate sums; slot 4: X of the output gate (peephole)
     int16_t *c;                    // [row][cpc]
+    uint4 *sx, *sx2;               // CL: [block][4][ra] the cluster's sums of the first exchange, [block][ra] of the second
+    uint8_t *stage_m, *stage_h;    // CL: [row][cpc], [row][opc]
+    uint8_t *h_buf, *m_buf;        // CL: operands
 };
 
 struct WsRole {
@@ -153,6 +166,77 @@ __device__ __forceinline__ void ws_pull_stats(const WaveLayer &L, const WsSmem &
     }
 }
 
+// ---- exchanges within a cluster ----
+// The block's sums of the gate slots in `mask` to every block; slots: of a block in sx, slot 0 of which is gate g0.
+template <int G>
+__device__ __forceinline__ void ws_send_stats(const WaveCall &k, const WsSmem &s, const WsRole &r, int n, uint4 *sx, int slots, int g0, unsigned mask, uint64_t *bar,
+                                              int tid)
+{
+    const int g = (tid >> 5) & 3, row = tid & 31;
+    if (g < G && row < r.rows && ((mask >> g) & 1u)) {
+        const uint32_t *st = s.st + g * 3 * WS_ROWS + row;
+        const uint4 v = make_uint4(st[0], st[WS_ROWS], st[2 * WS_ROWS], 0u);
+        const uint32_t dst = ptx::smem_u32(sx + ((size_t)r.rank * slots + g - g0) * k.ra + row), b = ptx::smem_u32(bar);
+        for (int p = tid >> 7; p < n; p += 4) wv_send16(wv_peer(dst, p), v, wv_peer(b, p));
+    }
+}
+// The constants of those slots from what has come; false: leave.
+template <int G>
+__device__ __forceinline__ bool ws_merge_stats(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, const uint4 *sx, int slots, int g0,
+                                               unsigned mask, uint64_t *bar, uint32_t par, WvPoint &pt, int tid)
+{
+    const int g = tid >> 5, row = tid & 31;
+    const bool mine = g < G && ((mask >> g) & 1u);             // warp-uniform
+    if (mine && wv_wait_cluster(bar, par, k.abort_word, k.limit_ns, pt.abort_flag)) {
+        // (the first warp of them arms the barrier again; nobody sends to it before this block has sent m or h)
+        if (row == 0 && (mask & ((1u << g) - 1u)) == 0u) ptx::mbar_arrive_expect_tx(bar, (uint32_t)(L.n * __popc(mask) * r.rows * 16));
+        if (row < r.rows) {
+            int32_t sum = 0;
+            uint32_t lo = 0, hi = 0;
+            const uint4 *src = sx + (size_t)(g - g0) * k.ra + row;
+#pragma unroll 4
+            for (int p = 0; p < L.n; ++p) {
+                const uint4 o = src[(size_t)p * slots * k.ra];
+                sum += (int32_t)o.x; lo += o.y; hi += o.z;
+            }
+            s.ln[g * WS_ROWS + row] = wv_make_ln(sum, ((int64_t)hi << 20) + lo, L.div_c, L.sigma_min);
+        }
+    }
+    const bool stay = wv_point(pt, tid);
+    // (every thread that sends them has read the block's sums)
+    if (mine && row < r.rows) {
+        uint32_t *st = s.st + g * 3 * WS_ROWS + row;
+        st[0] = st[WS_ROWS] = st[2 * WS_ROWS] = 0u;
+    }
+    return stay;
+}
+// PIECE bytes at a time, rows of `n` values from column `col0` on into the image `buf` of the blocks [0, peers).
+template <int PIECE>
+__device__ __forceinline__ void ws_send_rows(const WaveCall &k, const uint8_t *stage, int pitch, int rows, int n, int col0, uint8_t *buf, uint64_t *bar, int peers,
+                                             int tid)
+{
+    const int np = (n + PIECE - 1) / PIECE, tasks = rows * np;
+    const uint32_t base = ptx::smem_u32(buf), b = ptx::smem_u32(bar);
+    for (int i = tid & 127; i < tasks; i += 128) {
+        const int row = i / np, j = (i - row * np) * PIECE;
+        const uint32_t dst = base + wv_img_off(row, col0 + j, k.ra);
+        if (PIECE == 16) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(stage + row * pitch + j);
+            for (int p = tid >> 7; p < peers; p += 4) wv_send16(wv_peer(dst, p), v, wv_peer(b, p));
+        } else {
+            const uint2 v = *reinterpret_cast<const uint2 *>(stage + row * pitch + j);
+            for (int p = tid >> 7; p < peers; p += 4) wv_send8(wv_peer(dst, p), v, wv_peer(b, p));
+        }
+    }
+}
+// Bytes of a piece of m.
+__device__ __forceinline__ int ws_piece(const WaveLayer &L) { return (L.cpc & 15) == 0 ? 16 : 8; }
+// h^t of this block is in global memory for the layer above (after a barrier of the epilogue threads; by a warp that is not the first to wait)
+__device__ __forceinline__ void ws_signal(unsigned *cnt, int tid)
+{
+    if (tid == WV_EPI - 32) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+}
+
 // layer norm of the gate slots in `mask` of one cell, in place
 template <int G>
 __device__ __forceinline__ void ws_ln_cell(const WaveLayer &L, const WsSmem &s, int row, int ul, unsigned mask, int32_t (&a)[4])
@@ -177,25 +261,32 @@ __device__ __forceinline__ void ws_ln_cell(const WaveLayer &L, const WsSmem &s, 
 }
 
 // m of one cell (h of a layer without a projection)
-__device__ __forceinline__ void ws_store_m(const WaveCall &k, const WaveLayer &L, int8_t *img_unit, int row, int u, int b, int t, int32_t m, bool last_layer)
+template <bool CL>
+__device__ __forceinline__ void ws_store_m(const WaveCall &k, const WaveLayer &L, const WsSmem &s, int8_t *img_unit, int row, int ul, int u, int b, int t, int32_t m,
+                                           bool last_layer)
 {
-    img_unit[wv_img_off(row, u, k.ra)] = (int8_t)m;
+    if (CL) s.stage_m[row * L.cpc + ul] = (uint8_t)m;
+    if (!CL || (!(L.flags & F_PROJECTION) && !last_layer)) img_unit[wv_img_off(row, u, k.ra)] = (int8_t)m;
     if (L.flags & F_PROJECTION) return;
     if (last_layer) wv_y_row(k, L, t, b)[u] = (int8_t)m;
     if (t == k.T - 1) L.h[(size_t)b * L.O + u] = (int8_t)m;
 }
 
 // Everything between the gate sums and m, one cell per task, consecutive threads on consecutive cells of a row.
-template <int G, bool LN, bool PEEP>
+template <int G, bool LN, bool PEEP, bool CL>
 __device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, const ActLines &at, int t, bool last_layer,
-                                               WvPoint &pt, int tid)
+                                               WvPoint &pt, WsCtl *ctl, int tid)
 {
     constexpr int SI = 0, SF = (G == 4) ? 1 : 0, SZ = SF + 1, SO = SF + 2;
     constexpr unsigned ALL = (1u << G) - 1u;
     const int rows = r.rows, cells = r.cells, cpc = L.cpc, n_tasks = rows * cells;
     unsigned *cnt = L.cnt + (size_t)r.gu * WC_PER_UNIT * WC_WORDS;
     long long *tot = L.totals ? L.totals + ((size_t)(t & 1) * k.nu + r.gu) * k.ra * 8 : nullptr;
-    if (LN) {
+    if (LN && CL) {
+        constexpr unsigned FIRST = PEEP ? ALL & ~(1u << SO) : ALL;
+        ws_send_stats<G>(k, s, r, L.n, s.sx, 4, 0, FIRST, &ctl->s_full[0], tid);
+        if (!ws_merge_stats<G>(k, L, s, r, s.sx, 4, 0, FIRST, &ctl->s_full[0], (uint32_t)t & 1u, pt, tid)) return false;
+    } else if (LN) {
         ws_push_stats<G>(s, tot, rows, PEEP ? ALL & ~(1u << SO) : ALL, tid);
         if (!wv_publish(cnt + WC_STATS * WC_WORDS, false, pt, tid)) return false;
         if (!wv_meet(k, cnt + WC_STATS * WC_WORDS, (unsigned)(t + 1) * L.n, pt, tid)) return false;
@@ -236,28 +327,48 @@ __device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLaye
                 continue;
             }
         }
-        ws_store_m(k, L, img, row, u, b, t, wv_hidden<true>(L, at, line_sigmoid(at, ao), c_new), last_layer);
+        ws_store_m<CL>(k, L, s, img, row, ul, u, b, t, wv_hidden<true>(L, at, line_sigmoid(at, ao), c_new), last_layer);
     }
     if (LN && PEEP) {
         wv_epi_sync();
-        ws_push_stats<G>(s, tot, rows, 1u << SO, tid);
-        if (!wv_publish(cnt + WC_STATS2 * WC_WORDS, false, pt, tid)) return false;
-        if (!wv_meet(k, cnt + WC_STATS2 * WC_WORDS, (unsigned)(t + 1) * L.n, pt, tid)) return false;
-        ws_pull_stats<G>(L, s, tot, rows, 1u << SO, tid);
-        wv_epi_sync();
+        if (CL) {
+            ws_send_stats<G>(k, s, r, L.n, s.sx2, 1, SO, 1u << SO, &ctl->s_full[1], tid);
+            if (!ws_merge_stats<G>(k, L, s, r, s.sx2, 1, SO, 1u << SO, &ctl->s_full[1], (uint32_t)t & 1u, pt, tid)) return false;
+        } else {
+            ws_push_stats<G>(s, tot, rows, 1u << SO, tid);
+            if (!wv_publish(cnt + WC_STATS2 * WC_WORDS, false, pt, tid)) return false;
+            if (!wv_meet(k, cnt + WC_STATS2 * WC_WORDS, (unsigned)(t + 1) * L.n, pt, tid)) return false;
+            ws_pull_stats<G>(L, s, tot, rows, 1u << SO, tid);
+            wv_epi_sync();
+        }
 #pragma unroll 1
         for (int i = tid; i < n_tasks; i += WV_EPI) {
             const int row = (int)(((float)i + 0.5f) * inv_cells), ul = i - row * cells;
             int32_t a[4] = {0, 0, 0, 0};
             a[SO] = s.g[(SO * rows + row) * cpc + ul];
             ws_ln_cell<G>(L, s, row, ul, 1u << SO, a);
-            ws_store_m(k, L, img, row, r.u0 + ul, r.row0 + row, t, wv_hidden<true>(L, at, line_sigmoid(at, a[SO]), s.c[row * cpc + ul]), last_layer);
+            ws_store_m<CL>(k, L, s, img, row, ul, r.u0 + ul, r.row0 + row, t, wv_hidden<true>(L, at, line_sigmoid(at, a[SO]), s.c[row * cpc + ul]), last_layer);
         }
+    }
+    if (CL) {
+        const bool proj = (L.flags & F_PROJECTION) != 0, publish = !proj && !last_layer;
+        if (publish) wv_fence_async_global();
+        if (!wv_point(pt, tid)) return false;
+        if (proj || !fin) {
+            uint8_t *buf = proj ? s.m_buf : s.h_buf + ((t + 1) & 1) * (k.max_kb_h * k.ra * 128);
+            uint64_t *bar = proj ? &ctl->mx_full : &ctl->hx_full[(t + 1) & 1];
+            const int peers = proj ? (L.O + L.opc - 1) / L.opc : L.n;
+            if (ws_piece(L) == 16) ws_send_rows<16>(k, s.stage_m, cpc, rows, cells, r.u0, buf, bar, peers, tid);
+            else ws_send_rows<8>(k, s.stage_m, cpc, rows, cells, r.u0, buf, bar, peers, tid);
+        }
+        if (publish) ws_signal(cnt + WC_H * WC_WORDS, tid);
+        return true;
     }
     return wv_publish(cnt + ((L.flags & F_PROJECTION) ? WC_M : WC_H) * WC_WORDS, true, pt, tid);
 }
 
 // One projection tile: a lane is an output, the four warps of a lane quarter share the rows.
+template <bool CL>
 __device__ __forceinline__ void ws_proj_tile(const WaveCall &k, const WaveLayer &L, const WsSmem &s, const WsRole &r, uint32_t tp, int o_first, int no,
                                              int quarter, int wq, int lane, int8_t *out_unit, int t, bool last_layer)
 {
@@ -277,7 +388,8 @@ __device__ __forceinline__ void ws_proj_tile(const WaveCall &k, const WaveLayer 
             const int row = r0 + e, b = r.row0 + row;
             const int8_t h = (int8_t)sat8(fast_rescale((int32_t)a[e] + bias, L.f_proj) + L.zp_h);
             if (in && row < r.rows) {
-                out_unit[wv_img_off(row, col, k.ra)] = h;
+                if (CL) s.stage_h[row * L.opc + o_first + j] = (uint8_t)h;
+                if (!CL || !last_layer) out_unit[wv_img_off(row, col, k.ra)] = h;
                 if (last_layer) wv_y_row(k, L, t, b)[col] = h;
                 if (fin) L.h[(size_t)b * L.O + col] = h;
             }
@@ -301,7 +413,7 @@ __device__ __noinline__ void ws_drain(WsCtl *ctl, int nb, int warp)
     }
 }
 
-template <int G, bool LN, bool PEEP>
+template <int G, bool LN, bool PEEP, bool CL>
 __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid_constant__ WaveCall k)
 {
     extern __shared__ uint8_t ws_raw[];
@@ -309,13 +421,29 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = blockIdx.x;
     WsRole r;
     r.li = -1;
-    for (int l = 0; l < k.n_layers; ++l)
-        if (cta >= k.layer[l].cta0 && cta < k.layer[l].cta0 + k.layer[l].n * k.rg) r.li = l;
-    if (r.li < 0) return;
+    if (CL) {
+        const int group = cta / k.cl;
+        r.li = group / k.rg;
+    } else {
+        for (int l = 0; l < k.n_layers; ++l)
+            if (cta >= k.layer[l].cta0 && cta < k.layer[l].cta0 + k.layer[l].n * k.rg) r.li = l;
+        if (r.li < 0) return;
+    }
     const WaveLayer &L = k.layer[r.li];
     const bool proj = (L.flags & F_PROJECTION) != 0, last_layer = L.last != 0;
-    r.gu = (cta - L.cta0) / L.n;
-    r.rank = cta - L.cta0 - r.gu * L.n;
+    if (CL) {
+        const int group = cta / k.cl;
+        r.gu = group - r.li * k.rg;
+        r.rank = cta - group * k.cl;
+        if (r.rank >= L.n) {                                   // a block without cells
+            wv_cluster_sync();
+            wv_cluster_sync();
+            return;
+        }
+    } else {
+        r.gu = (cta - L.cta0) / L.n;
+        r.rank = cta - L.cta0 - r.gu * L.n;
+    }
     r.u0 = r.rank * L.cpc;
     r.cells = L.C - r.u0 < L.cpc ? L.C - r.u0 : L.cpc;
     r.o_lo = r.rank * L.opc;
@@ -323,7 +451,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     if (r.outs < 0) r.outs = 0;
     r.row0 = (int)((long long)r.gu * k.B / k.nu);
     r.rows = (int)((long long)(r.gu + 1) * k.B / k.nu) - r.row0;
-    if (r.rows == 0) return;                                   // fewer rows than row groups: this group is idle
+    if (!CL && r.rows == 0) return;                            // fewer rows than row groups: this group is idle
 
     const WsLayout lay = ws_layout(k, k.nb, (k.B + k.nu - 1) / k.nu, PEEP);
     WsCtl *ctl = reinterpret_cast<WsCtl *>(smem + lay.ctl);
@@ -342,7 +470,16 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         s.ln = (WvLnRow *)(smem + lay.ln);
         s.g = (int16_t *)(smem + lay.gates);
         s.c = (int16_t *)(smem + lay.c);
+        s.sx = (uint4 *)(smem + lay.sx);
+        s.sx2 = s.sx + (size_t)k.cl * 4 * k.ra;
+        s.stage_m = smem + lay.stage_m;
+        s.stage_h = smem + lay.stage_h;
+        s.h_buf = smem + lay.act[1];
+        s.m_buf = smem + lay.act[2];
     }
+    // CL: what a step brings
+    const int piece = ws_piece(L);
+    const uint32_t m_bytes = (uint32_t)(r.rows * ((L.C + piece - 1) & -piece)), h_bytes = proj ? (uint32_t)(r.rows * ((L.O + 7) & -8)) : m_bytes;
     if (threadIdx.x == 0) {
         for (int i = 0; i < WS_SLOTS; ++i) { ptx::mbar_init(&ctl->w_full[i], 1); ptx::mbar_init(&ctl->w_empty[i], 2); }
         for (int i = 0; i < 3; ++i) { ptx::mbar_init(&ctl->op_full[i], 1); ptx::mbar_init(&ctl->op_empty[i], 2); }
@@ -352,10 +489,23 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         ptx::mbar_init(&ctl->p_empty, WV_EPI / 32);
         ptx::mbar_init(&ctl->tab_full, 1);
         for (int i = 0; i < 2; ++i) ptx::mbar_init(&ctl->mma_done[i], 1);
+        if (CL) {
+            // two arrivals: each of the issuing warps, when it has seen the phase before (k.missing: arrivals that never come)
+            for (int i = 0; i < 2; ++i) ptx::mbar_init(&ctl->hx_full[i], 2 + k.missing);
+            ptx::mbar_init(&ctl->mx_full, 2 + k.missing);
+            for (int i = 0; i < 2; ++i) ptx::mbar_init(&ctl->s_full[i], 1 + k.missing);
+        }
         ctl->abort_flag = 0;
         ctl->exit_at = 0x7fffffff;
         for (int i = 0; i < 3; ++i) ctl->op_copies[i] = 0;
         ptx::fence_barrier_init();
+        if (CL) {
+            for (int i = 0; i < 2; ++i) { ptx::mbar_arrive_expect_tx(&ctl->hx_full[i], h_bytes); ptx::mbar_arrive(&ctl->hx_full[i]); }
+            ptx::mbar_arrive_expect_tx(&ctl->mx_full, m_bytes);
+            ptx::mbar_arrive(&ctl->mx_full);
+            ptx::mbar_arrive_expect_tx(&ctl->s_full[0], (uint32_t)(L.n * (PEEP ? G - 1 : G) * r.rows * 16));
+            ptx::mbar_arrive_expect_tx(&ctl->s_full[1], (uint32_t)(L.n * r.rows * 16));
+        }
         ptx::mbar_arrive_expect_tx(&ctl->tab_full, L.tab_lay.bytes);
         ptx::bulk_load_1d(smem + lay.tab, L.tab, L.tab_lay.bytes, &ctl->tab_full);
     }
@@ -382,6 +532,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     ptx::tc_fence_before();
     ptx::cta_sync();
     ptx::tc_fence_after();
+    if (CL) wv_cluster_sync();                                 // every block's barriers stand
     const uint32_t tmem_base = ctl->tmem_base;
     const int nt = (r.cells + L.ct - 1) / L.ct, ntp = proj ? (r.outs + L.opt - 1) / L.opt : 0, nr = k.ra, T = k.T;
     // accumulators: X tiles, H tiles, projection tiles
@@ -404,6 +555,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         // ---------------- operands: x, h, m of a unit, each one contiguous copy ----------------
         if (lane == 0) {
             walk([&](int op, int t) -> bool {
+                if (CL && (op == 2 || (op == 1 && t > 0))) return true;        // (sent by the peers)
                 const unsigned *cnt = nullptr;
                 unsigned target = 0;
                 const int8_t *src;
@@ -470,8 +622,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
         const uint64_t w_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem));
         const uint32_t idesc = ptx::idesc_i8(128, nr), b_step = (uint32_t)nr * 128u >> 4;
         // one tile of nkb k-blocks: kpc of them per chunk (kb_bytes apart), the chunks of a ring slot chunk_bytes apart
-        auto tile = [&](bool mine, uint32_t d, int op, int nkb, int kpc, uint32_t kb_bytes, int n_chunks, uint32_t chunk_bytes) -> bool {
-            const uint64_t b_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + lay.act[op]));
+        auto tile = [&](bool mine, uint32_t d, size_t b_at, int nkb, int kpc, uint32_t kb_bytes, int n_chunks, uint32_t chunk_bytes) -> bool {
+            const uint64_t b_desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem + b_at));
             for (int kb0 = 0; kb0 < nkb; kb0 += kpc * n_chunks) {
                 if (!wv_wait_warp(&ctl->w_full[slot], phase, abort_flag)) return false;
                 ptx::tc_fence_after();
@@ -501,21 +653,32 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
             // the gate accumulators of the step before have been read (X(t) waits for step t - 1 as well)
             if (op != 2 && t > 0 && !wv_wait_warp(&ctl->acc_empty, par ^ 1u, abort_flag)) return false;
             if (op == 2 && t > 0 && !wv_wait_warp(&ctl->p_empty, par ^ 1u, abort_flag)) return false;
-            if (!wv_wait_warp(&ctl->op_full[op], par, abort_flag)) return false;
+            size_t b_at = lay.act[op];
+            if (CL && (op == 2 || (op == 1 && t > 0))) {
+                if (op == 1 && par) b_at += (size_t)k.max_kb_h * k.ra * 128;
+                uint64_t *bar = op == 2 ? &ctl->mx_full : &ctl->hx_full[par];
+                if (!wv_wait_cluster(bar, op == 2 ? par : (uint32_t)((t - 1) >> 1) & 1u, k.abort_word, k.limit_ns, abort_flag)) return false;
+                if (lane == 0) {
+                    if (me == 0) ptx::mbar_arrive_expect_tx(bar, op == 2 ? m_bytes : h_bytes);
+                    else ptx::mbar_arrive(bar);
+                }
+                __syncwarp();
+                ptx::fence_proxy_async();                      // (the peers' stores are ordinary ones, an MMA reads as copies do)
+            } else if (!wv_wait_warp(&ctl->op_full[op], par, abort_flag)) return false;
             ptx::tc_fence_after();
             if (op == 2) {
                 for (int j = 0; j < ntp; ++j)
-                    if (!tile((j & 1) != me, tmem_base + col_p + (uint32_t)(j * nr), 2, L.kb_c, L.kpp, (uint32_t)L.opp * 128u, 1, 0u)) return false;
+                    if (!tile((j & 1) != me, tmem_base + col_p + (uint32_t)(j * nr), b_at, L.kb_c, L.kpp, (uint32_t)L.opp * 128u, 1, 0u)) return false;
                 wv_commit(&ctl->p_full);
             } else {
                 for (int i = 0; i < nt; ++i) {
-                    if (!tile((i & 1) == me, tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), op, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u, WS_CHUNKS,
+                    if (!tile((i & 1) == me, tmem_base + (op ? col_h : 0u) + (uint32_t)(i * nr), b_at, op ? L.kb_h : L.kb_i, L.kpg, (uint32_t)L.ctp * 128u, WS_CHUNKS,
                               G * 4096u))
                         return false;
                     if (op == (t > 0 ? 1 : 0) && (i & 1) == me) wv_commit(&ctl->gate_full[i]);      // the step's last product
                 }
             }
-            wv_commit(&ctl->op_empty[op]);
+            if (!CL || op == 0) wv_commit(&ctl->op_empty[op]);
             return true;
         });
     } else if (warp >= WV_EPI_WARP0) {
@@ -547,18 +710,28 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&ctl->acc_empty);
             wv_epi_sync();
-            stay = ws_elementwise<G, LN, PEEP>(k, L, s, r, at, t, last_layer, pt, tid);
+            stay = ws_elementwise<G, LN, PEEP, CL>(k, L, s, r, at, t, last_layer, pt, ctl, tid);
             if (!stay || !proj) continue;
             if (ntp > 0 && __all_sync(0xffffffffu, wv_wait(&ctl->p_full, par, abort_flag))) {
                 ptx::tc_fence_after();
                 for (int j = 0; j < ntp; ++j) {
                     const int left = r.outs - j * L.opt;
-                    ws_proj_tile(k, L, s, r, tq + col_p + (uint32_t)(j * nr), j * L.opt, left < L.opt ? left : L.opt, quarter, wq, lane,
+                    ws_proj_tile<CL>(k, L, s, r, tq + col_p + (uint32_t)(j * nr), j * L.opt, left < L.opt ? left : L.opt, quarter, wq, lane,
                                  L.out_img + ((size_t)(t + 1) * k.nu + r.gu) * L.kb_h * k.ra * 128, t, last_layer);
                 }
                 ptx::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(&ctl->p_empty);
+            }
+            if (CL) {
+                if (!last_layer) wv_fence_async_global();
+                stay = wv_point(pt, tid);
+                if (!stay) continue;
+                if (t + 1 < T)
+                    ws_send_rows<8>(k, s.stage_h, L.opc, r.rows, r.outs, r.o_lo, s.h_buf + ((t + 1) & 1) * (k.max_kb_h * k.ra * 128), &ctl->hx_full[(t + 1) & 1], L.n,
+                                    tid);
+                if (!last_layer) ws_signal(cnt0 + WC_H * WC_WORDS, tid);
+                continue;
             }
             stay = wv_publish(cnt0 + WC_H * WC_WORDS, true, pt, tid);
         }
@@ -569,9 +742,17 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
     if (*abort_flag) {
         // a wait ran out: copies and MMAs in flight end, then report
         ws_drain(ctl, k.nb, warp);
-        if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
+        if (threadIdx.x == 0) {
+            atomicExch(k.abort_word, 1u); atomicExch(k.status, 2);
+            if (CL) {
+                // what peers sent before they left arrives within microseconds; this block does not end before
+                const unsigned long long t0 = wv_timer();
+                while (wv_timer() - t0 < 50000ull) {}
+            }
+        }
     }
     ptx::cta_sync();
+    if (CL) wv_cluster_sync();                                 // no block ends while a peer may still store into it
     if (warp == 2) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, 512);
@@ -615,14 +796,22 @@ void wave_small_tile_weights(const int8_t *src, int8_t *dst, int G, int rows, in
     k_wave_small_tile_weights<<<2048, 256>>>(src, dst, G, rows, K, n, per_rank, nt, per_tile, padded, nkb, kps);
 }
 
-const void *wave_small_kernel(int G, bool ln, bool peep)
+namespace {
+template <bool CL>
+const void *ws_kernel_of(int G, bool ln, bool peep)
 {
     if (G == 4) {
-        if (ln) return peep ? (const void *)k_wave_small_sm100<4, true, true> : (const void *)k_wave_small_sm100<4, true, false>;
-        return peep ? (const void *)k_wave_small_sm100<4, false, true> : (const void *)k_wave_small_sm100<4, false, false>;
+        if (ln) return peep ? (const void *)k_wave_small_sm100<4, true, true, CL> : (const void *)k_wave_small_sm100<4, true, false, CL>;
+        return peep ? (const void *)k_wave_small_sm100<4, false, true, CL> : (const void *)k_wave_small_sm100<4, false, false, CL>;
     }
-    if (ln) return peep ? (const void *)k_wave_small_sm100<3, true, true> : (const void *)k_wave_small_sm100<3, true, false>;
-    return peep ? (const void *)k_wave_small_sm100<3, false, true> : (const void *)k_wave_small_sm100<3, false, false>;
+    if (ln) return peep ? (const void *)k_wave_small_sm100<3, true, true, CL> : (const void *)k_wave_small_sm100<3, true, false, CL>;
+    return peep ? (const void *)k_wave_small_sm100<3, false, true, CL> : (const void *)k_wave_small_sm100<3, false, false, CL>;
+}
+}  // namespace
+
+const void *wave_small_kernel(int G, bool ln, bool peep, bool cluster)
+{
+    return cluster ? ws_kernel_of<true>(G, ln, peep) : ws_kernel_of<false>(G, ln, peep);
 }
 
 // shared memory of a launch with ns ring slots

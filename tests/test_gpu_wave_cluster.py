@@ -1,0 +1,30 @@
+"""The few-row wavefront kernel on thread-block clusters against the CPU oracle, bit for bit, at the edges of its pieces (needs a B200)."""
+import numpy as np
+import pytest
+
+from oracle import qlstm_ref as R
+from tests.gpu_util import run_gpu
+from tests.test_gpu_wave import VARIANTS
+from workloads import random_layer_stack
+
+pytestmark = pytest.mark.gpu
+
+WAVE = 8
+SHAPES = {"blocks without cells": (2, 16, 40, 24), "eights": (5, 32, 280, 48), "blocks without outputs": (2, 48, 272, 20), "several tiles": (2, 80, 640, 176), "odd": (3, 19, 333, 27)}
+
+
+# h and m cross in pieces of 8 and 16 bytes, rows in groups of 8 up to 32; h alternates between two buffers; calls end at either
+@pytest.mark.parametrize("T,B", [(1, 3), (2, 1), (7, 9), (12, 32)])
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("kw", VARIANTS, ids=lambda k: "+".join(sorted(k)) or "basic")
+def test_wave_cluster(kw, shape, T, B):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(970 + B, *SHAPES[shape], T=T, B=B, **kw)
+    want = R.run(w.layers, w.x, *w.initial_state())
+    with qlstm.QLSTM(w.layers, T, B) as q:
+        # (wide layers with a single exchange are left to more blocks)
+        assert q.debug_wave_cluster(T, B) >= 8 or (shape == "several tiles" and not kw.get("layernorm"))
+        for _ in range(2):                                     # (a second call: what the first one left behind)
+            got = run_gpu(w, handle=q, impl=(0, WAVE))
+            for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+                assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
