@@ -37,6 +37,7 @@ constexpr int RS_THREADS = 32 * (RS_MAX_WARPS + 2);
 constexpr int RS_NX = 4;                       // x buffers
 constexpr int RS_MAX_CLUSTER = 16;
 constexpr int RS_MAX_NT = 4;                   // tiles of eight rows
+static_assert(RS_MAX_CLUSTER <= WC_WORDS && WC_WORDS <= 32, "a word per block in a line of counters, a lane per word");
 
 struct ResLayer {
     int I, C, O;
@@ -56,9 +57,9 @@ struct ResLayer {
     const int8_t *in_img;          // [T][B][px] the layer below's outputs; null: x
     int8_t *out_img;               // [T][B][px of the layer above]; null: y
     int out_pitch;
-    const unsigned *cnt_in;        // per row group, WC_WORDS apart
+    const unsigned *cnt_in;        // [row group][WC_WORDS]: by block of the group, the steps that it has written to in_img / out_img
     unsigned *cnt_out;
-    int below;                     // arrivals per step on cnt_in
+    int below;                     // blocks that write in_img
     int8_t *h; int16_t *c;
     int dir, y_off;
     const uint8_t *tab;
@@ -72,8 +73,7 @@ struct ResCall {
     const int8_t *x;
     int8_t *y;
     int y_stride;
-    unsigned *abort_word, *ticket, *cnt;
-    int n_cnt;                                 // words of cnt
+    unsigned *abort_word, *ticket, *cnt;       // cnt: a line of WC_WORDS per (layer, row group)
     int *status, *status2;
     unsigned long long limit_ns;
     unsigned missing;
@@ -128,22 +128,25 @@ __device__ __forceinline__ bool rs_wait(const ResCall &k, uint64_t *bar, uint32_
 {
     return wv_wait_cluster(bar, parity, k.abort_word, k.limit_ns, abort_flag);
 }
-// until *cnt has reached target (whole warp)
-__device__ __forceinline__ bool rs_wait_count(const ResCall &k, const unsigned *cnt, unsigned target, volatile int *abort_flag)
+// until each of the n <= 32 blocks that write to a line has reached target (whole warp, a lane per block).  The blocks do not wait for
+// one another here - what a layer's own recurrence needs goes through shared memory - so that no sum over them says that all have.
+__device__ __forceinline__ bool rs_wait_blocks(const ResCall &k, const unsigned *line, int n, unsigned target, volatile int *abort_flag)
 {
-    const bool look = (threadIdx.x & 31) == 0;
+    const int lane = threadIdx.x & 31;
     const unsigned long long t0 = wv_timer();
     for (unsigned spins = 1;; ++spins) {
-        unsigned v = 0, stop = 0;
-        if (look) v = wv_ld_acquire(cnt);
-        if (__shfl_sync(0xffffffffu, v, 0) >= target) return true;
-        if (look && (spins & 31u) == 0u) {
+        const bool there = lane >= n || wv_ld_acquire(line + lane) >= target;
+        if (__all_sync(0xffffffffu, there)) break;
+        unsigned stop = 0;
+        if (lane == 0 && (spins & 31u) == 0u) {
             if (*abort_flag) stop = 1;
             else if (wv_ld_acquire(k.abort_word) != 0u) { *abort_flag = 1; stop = 1; }
             else if (wv_timer() - t0 > k.limit_ns) { atomicExch(k.abort_word, 1u); *abort_flag = 1; stop = 1; }
         }
         if (__shfl_sync(0xffffffffu, stop, 0)) return false;
     }
+    __syncwarp();                              // (what the lanes acquired, to the lane that copies)
+    return true;
 }
 // one arrival of a warp, for what its lanes wrote
 __device__ __forceinline__ void rs_arrive(uint64_t *bar, int lane)
@@ -375,7 +378,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
                 if (t >= RS_NX && !rs_wait(k, &ctl->x_empty[slot], (uint32_t)(t / RS_NX - 1) & 1u, abort_flag)) break;
                 uint8_t *dst = smem + lay.x + (size_t)slot * r8 * L.px;
                 if (L.in_img) {
-                    if (!rs_wait_count(k, L.cnt_in + gu * WC_WORDS, (unsigned)(t + 1) * (unsigned)L.below + k.missing, abort_flag)) break;
+                    if (!rs_wait_blocks(k, L.cnt_in + gu * WC_WORDS, L.below, (unsigned)(t + 1) + k.missing, abort_flag)) break;
                     if (lane == 0) {
                         wv_fence_async_global();
                         ptx::mbar_arrive_expect_tx(&ctl->x_full[slot], (uint32_t)(rows * L.px));
@@ -451,7 +454,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
             if (!last) {
                 wv_fence_async_global();
                 __syncwarp();
-                if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(L.cnt_out + gu * WC_WORDS), "r"(n) : "memory");
+                if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(L.cnt_out + gu * WC_WORDS + rank), "r"(n) : "memory");
             }
         }
     } else if (warp < 2 + hw) {
@@ -807,22 +810,27 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
         }
     }
     wv_cluster_sync();
-    if (threadIdx.x == 0) {
-        if (aborted) {
+    if (warp == 0) {
+        if (aborted && lane == 0) {
             // what peers sent before they came here arrives within microseconds; this block does not end before
             atomicExch(k.abort_word, 1u);
             const unsigned long long t0 = wv_timer();
             while (wv_timer() - t0 < 50000ull) {}
         }
         // the last block reports, and leaves the counters as the next call wants them
-        __threadfence();
-        if (atomicAdd(k.ticket, 1u) == gridDim.x - 1u) {
+        bool end = false;
+        if (lane == 0) {
             __threadfence();
-            *k.status = atomicExch(k.abort_word, 0u) ? 2 : 0;
-            if (k.status2) *k.status2 = 0;
-            for (int i = 0; i < k.n_cnt; i += WC_WORDS) k.cnt[i] = 0u;
-            *k.ticket = 0u;
+            end = atomicAdd(k.ticket, 1u) == gridDim.x - 1u;
+            if (end) {
+                __threadfence();
+                *k.status = atomicExch(k.abort_word, 0u) ? 2 : 0;
+                if (k.status2) *k.status2 = 0;
+                *k.ticket = 0u;
+            }
         }
+        if (__any_sync(0xffffffffu, end))
+            for (int i = lane; i < k.n_layers * k.rg * WC_WORDS; i += 32) k.cnt[i] = 0u;
     }
 }
 
@@ -1090,7 +1098,6 @@ int launch_resident(const ResidentStack *s, const int8_t *x, int T, int B, int8_
     k.x_bulk = s->x_bulk; k.y_wide = s->y_wide && ((uintptr_t)y & 7) == 0;
     k.x = x; k.y = y; k.y_stride = s->y_stride;
     k.abort_word = s->words; k.ticket = s->words + WC_WORDS; k.cnt = s->words + 2 * WC_WORDS;
-    k.n_cnt = n * p.rg * WC_WORDS;
     k.status = status; k.status2 = status2;
     k.limit_ns = limit_ns; k.missing = missing;
     for (int l = 0; l < n; ++l) {

@@ -67,3 +67,18 @@ def test_resident_layernorm_of_small_deviations(shift, peephole):
             q.eff_x = [(m, s - shift) for m, s in q.eff_x]
             q.eff_h = [(m, s - shift) for m, s in q.eff_h]
         check(w)
+
+
+# long calls of several layers: what a layer reads from the one below is announced by each of its blocks, and nothing holds those
+# blocks together but the exchanges of their own recurrence (one per step without layer norm and projection)
+@pytest.mark.parametrize("kw", [dict(), dict(cifg=True), dict(projection=True), dict(projection=True, layernorm=True)], ids=IDS)
+def test_resident_long_calls_of_several_layers(kw):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(965, 4, 64, 320, 224, T=350, B=3, **kw)
+    want = R.run(w.layers, w.x, *w.initial_state())
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        assert q.debug_resident_plan(w.T, w.B)[0] > 1, "not taken by clusters"
+        for _ in range(20):
+            got = run_gpu(w, handle=q)
+            for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+                assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
