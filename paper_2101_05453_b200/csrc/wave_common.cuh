@@ -160,6 +160,29 @@ __device__ __forceinline__ void wv_wait_count_warp(const WaveCall &k, const unsi
         }
     }
 }
+// For a whole warp, a lane per block: until each of the n <= 32 blocks that write to a line of words has reached target.  For clusters, whose
+// blocks exchange what their own recurrence needs through shared memory and do not wait for one another here: a sum over them would not say
+// that all have.  Call: WaveCall or the like.
+template <class Call>
+__device__ __forceinline__ bool wv_wait_blocks(const Call &k, const unsigned *line, int n, unsigned target, volatile int *abort_flag)
+{
+    const int lane = threadIdx.x & 31;
+    target += k.missing;
+    const unsigned long long t0 = wv_timer();
+    for (unsigned spins = 1;; ++spins) {
+        const bool there = lane >= n || wv_ld_acquire(line + lane) >= target;
+        if (__all_sync(0xffffffffu, there)) break;
+        unsigned stop = 0;
+        if (lane == 0 && (spins & 31u) == 0u) {
+            if (*abort_flag) stop = 1;
+            else if (wv_ld_acquire(k.abort_word) != 0u) { *abort_flag = 1; stop = 1; }
+            else if (wv_timer() - t0 > k.limit_ns) { atomicExch(k.abort_word, 1u); *abort_flag = 1; stop = 1; }
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+    }
+    __syncwarp();                              // (what the lanes acquired, to the lane that copies)
+    return true;
+}
 __device__ __forceinline__ void wv_epi_sync() { asm volatile("barrier.sync 1, 512;" ::: "memory"); }
 
 // all MMAs that this warp has issued, through a barrier of its own

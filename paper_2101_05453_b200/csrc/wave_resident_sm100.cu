@@ -128,26 +128,6 @@ __device__ __forceinline__ bool rs_wait(const ResCall &k, uint64_t *bar, uint32_
 {
     return wv_wait_cluster(bar, parity, k.abort_word, k.limit_ns, abort_flag);
 }
-// until each of the n <= 32 blocks that write to a line has reached target (whole warp, a lane per block).  The blocks do not wait for
-// one another here - what a layer's own recurrence needs goes through shared memory - so that no sum over them says that all have.
-__device__ __forceinline__ bool rs_wait_blocks(const ResCall &k, const unsigned *line, int n, unsigned target, volatile int *abort_flag)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned long long t0 = wv_timer();
-    for (unsigned spins = 1;; ++spins) {
-        const bool there = lane >= n || wv_ld_acquire(line + lane) >= target;
-        if (__all_sync(0xffffffffu, there)) break;
-        unsigned stop = 0;
-        if (lane == 0 && (spins & 31u) == 0u) {
-            if (*abort_flag) stop = 1;
-            else if (wv_ld_acquire(k.abort_word) != 0u) { *abort_flag = 1; stop = 1; }
-            else if (wv_timer() - t0 > k.limit_ns) { atomicExch(k.abort_word, 1u); *abort_flag = 1; stop = 1; }
-        }
-        if (__shfl_sync(0xffffffffu, stop, 0)) return false;
-    }
-    __syncwarp();                              // (what the lanes acquired, to the lane that copies)
-    return true;
-}
 // one arrival of a warp, for what its lanes wrote
 __device__ __forceinline__ void rs_arrive(uint64_t *bar, int lane)
 {
@@ -378,7 +358,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
                 if (t >= RS_NX && !rs_wait(k, &ctl->x_empty[slot], (uint32_t)(t / RS_NX - 1) & 1u, abort_flag)) break;
                 uint8_t *dst = smem + lay.x + (size_t)slot * r8 * L.px;
                 if (L.in_img) {
-                    if (!rs_wait_blocks(k, L.cnt_in + gu * WC_WORDS, L.below, (unsigned)(t + 1) + k.missing, abort_flag)) break;
+                    if (!wv_wait_blocks(k, L.cnt_in + gu * WC_WORDS, L.below, (unsigned)(t + 1), abort_flag)) break;
                     if (lane == 0) {
                         wv_fence_async_global();
                         ptx::mbar_arrive_expect_tx(&ctl->x_full[slot], (uint32_t)(rows * L.px));

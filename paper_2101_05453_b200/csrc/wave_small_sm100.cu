@@ -11,7 +11,8 @@
 //
 // Two forms.  With CL a (layer, row group) is one thread-block cluster of up to 16 blocks, and what its own chain needs - layer-norm sums,
 // m, h - goes from shared memory into the shared memory of the peers (16 or 8 bytes at a time, counted on an mbarrier there) instead of
-// through L2 with a counter to poll and a copy back; only what the layer above reads is still written and published there, off the chain.
+// through L2 with a counter to poll and a copy back; only what the layer above reads is still written and published there, off the chain,
+// each block in a word of its own (wv_wait_blocks).
 // Without, groups may have any number of blocks.  The plan takes the cheaper one (wave_cluster_plan).
 #include <cstring>
 
@@ -231,7 +232,8 @@ __device__ __forceinline__ void ws_send_rows(const WaveCall &k, const uint8_t *s
 }
 // Bytes of a piece of m.
 __device__ __forceinline__ int ws_piece(const WaveLayer &L) { return (L.cpc & 15) == 0 ? 16 : 8; }
-// h^t of this block is in global memory for the layer above (after a barrier of the epilogue threads; by a warp that is not the first to wait)
+// h^t of this block is in global memory for the layer above (after a barrier of the epilogue threads; by a warp that is not the first to
+// wait).  cnt: this block's word.
 __device__ __forceinline__ void ws_signal(unsigned *cnt, int tid)
 {
     if (tid == WV_EPI - 32) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
@@ -361,7 +363,7 @@ __device__ __forceinline__ bool ws_elementwise(const WaveCall &k, const WaveLaye
             if (ws_piece(L) == 16) ws_send_rows<16>(k, s.stage_m, cpc, rows, cells, r.u0, buf, bar, peers, tid);
             else ws_send_rows<8>(k, s.stage_m, cpc, rows, cells, r.u0, buf, bar, peers, tid);
         }
-        if (publish) ws_signal(cnt + WC_H * WC_WORDS, tid);
+        if (publish) ws_signal(cnt + WC_H * WC_WORDS + r.rank, tid);
         return true;
     }
     return wv_publish(cnt + ((L.flags & F_PROJECTION) ? WC_M : WC_H) * WC_WORDS, true, pt, tid);
@@ -553,7 +555,8 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
 
     if (warp == 0) {
         // ---------------- operands: x, h, m of a unit, each one contiguous copy ----------------
-        if (lane == 0) {
+        // (CL: the warp stays together, to look at a word per block of the layer below)
+        if (CL || lane == 0) {
             walk([&](int op, int t) -> bool {
                 if (CL && (op == 2 || (op == 1 && t > 0))) return true;        // (sent by the peers)
                 const unsigned *cnt = nullptr;
@@ -563,7 +566,10 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                 if (op == 0) {
                     bytes *= (uint32_t)L.kb_i;
                     src = L.in_img + ((size_t)(t + (L.below ? 1 : 0)) * k.nu + r.gu) * bytes;
-                    if (L.below) { cnt = k.layer[r.li - 1].cnt + ((size_t)r.gu * WC_PER_UNIT + WC_H) * WC_WORDS; target = (unsigned)(t + 1) * L.below; }
+                    if (L.below) {
+                        cnt = k.layer[r.li - 1].cnt + ((size_t)r.gu * WC_PER_UNIT + WC_H) * WC_WORDS;
+                        target = (unsigned)(t + 1) * (CL ? 1u : (unsigned)L.below);
+                    }
                 } else if (op == 1) {
                     bytes *= (uint32_t)L.kb_h;
                     src = L.out_img + ((size_t)t * k.nu + r.gu) * bytes;
@@ -573,12 +579,20 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                     src = L.m_img + (size_t)r.gu * bytes;
                     cnt = cnt0 + WC_M * WC_WORDS; target = (unsigned)(t + 1) * L.n;
                 }
-                if (cnt && !wv_wait_count(k, cnt, target, abort_flag)) return false;
-                if (!wv_wait(&ctl->op_empty[op], ((uint32_t)t & 1u) ^ 1u, abort_flag)) return false;
-                wv_fence_async_global();
-                ptx::mbar_arrive_expect_tx(&ctl->op_full[op], bytes);
-                ptx::bulk_load_1d(smem + lay.act[op], src, bytes, &ctl->op_full[op]);
-                ctl->op_copies[op] = t + 1;
+                if (CL) {
+                    if (cnt && !wv_wait_blocks(k, cnt, L.below, target, abort_flag)) return false;
+                    if (!wv_wait_warp(&ctl->op_empty[op], ((uint32_t)t & 1u) ^ 1u, abort_flag)) return false;
+                } else {
+                    if (cnt && !wv_wait_count(k, cnt, target, abort_flag)) return false;
+                    if (!wv_wait(&ctl->op_empty[op], ((uint32_t)t & 1u) ^ 1u, abort_flag)) return false;
+                }
+                if (lane == 0) {
+                    wv_fence_async_global();
+                    ptx::mbar_arrive_expect_tx(&ctl->op_full[op], bytes);
+                    ptx::bulk_load_1d(smem + lay.act[op], src, bytes, &ctl->op_full[op]);
+                    ctl->op_copies[op] = t + 1;
+                }
+                if (CL) __syncwarp();
                 return true;
             });
         }
@@ -730,7 +744,7 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
                 if (t + 1 < T)
                     ws_send_rows<8>(k, s.stage_h, L.opc, r.rows, r.outs, r.o_lo, s.h_buf + ((t + 1) & 1) * (k.max_kb_h * k.ra * 128), &ctl->hx_full[(t + 1) & 1], L.n,
                                     tid);
-                if (!last_layer) ws_signal(cnt0 + WC_H * WC_WORDS, tid);
+                if (!last_layer) ws_signal(cnt0 + WC_H * WC_WORDS + r.rank, tid);
                 continue;
             }
             stay = wv_publish(cnt0 + WC_H * WC_WORDS, true, pt, tid);

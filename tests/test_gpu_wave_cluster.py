@@ -28,3 +28,18 @@ def test_wave_cluster(kw, shape, T, B):
             got = run_gpu(w, handle=q, impl=(0, WAVE))
             for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
                 assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
+
+
+# long calls of several layers: what a layer reads from the one below is announced by each of its blocks, and nothing holds those
+# blocks together but the exchanges of their own recurrence (one per step without layer norm and projection)
+@pytest.mark.parametrize("kw", [dict(), dict(cifg=True), dict(projection=True), dict(projection=True, layernorm=True)], ids=lambda k: "+".join(sorted(k)) or "basic")
+def test_wave_cluster_long_calls_of_several_layers(kw):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(985, 4, 64, 320, 224, T=350, B=3, **kw)
+    want = R.run(w.layers, w.x, *w.initial_state())
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        assert q.debug_wave_cluster(w.T, w.B) >= 8
+        for _ in range(20):
+            got = run_gpu(w, handle=q, impl=(0, WAVE))
+            for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
+                assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
