@@ -470,6 +470,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
         }
         bool run = has_units && rs_wait(k, &ctl->w_full, 0, abort_flag);
         uint32_t ln_par = 0;                                   // parity of the next block-wide meeting of the layer norm
+        int done = 0;
         for (int t = 0; run && t < T; ++t) {
             const uint32_t par = (uint32_t)t & 1u, par2 = (uint32_t)(t >> 1) & 1u;
             uint4 xg[U];
@@ -678,10 +679,10 @@ __global__ void __launch_bounds__(RS_THREADS, 1) k_wave_resident(const __grid_co
                 if (cg < ncg) rs_send_tile(stage, mv[i][0], mv[i][1], dst + u0 + cg * 8, row_ok, ptx::smem_u32(bar), peer, rank, proj ? nob : ncb, lane);
             }
             rs_arrive(bar, lane);
+            done = t + 1;
         }
-        // nothing that peers send may be under way when the block ends
-        if (run && cw == 0) rs_wait(k, &ctl->h_full[T & 1], (uint32_t)((T - 1) >> 1) & 1u, abort_flag);
-        if (has_units)
+        // nothing that peers send may be under way when the block ends; a block that did not get this far leaves the state as the caller had it
+        if (done == T && rs_wait(k, &ctl->h_full[T & 1], (uint32_t)((T - 1) >> 1) & 1u, abort_flag))
 #pragma unroll
             for (int i = 0; i < U; ++i) {
                 const int ul = (cg0 + i * cstep) * 8 + g;

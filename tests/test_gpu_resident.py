@@ -82,3 +82,34 @@ def test_resident_long_calls_of_several_layers(kw):
             got = run_gpu(w, handle=q)
             for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
                 assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
+
+
+# a wait that runs out: reported, the caller's state untouched, nothing in flight and no counter left behind for the calls that follow.
+# One block and clusters per layer, x by bulk copies and by bytes, calls that end before the first exchange and after
+@pytest.mark.parametrize("T", [1, 2, 7])
+@pytest.mark.parametrize("dims", [(32, 40, 24), (19, 37, 23), (80, 304, 208), (83, 501, 9)], ids=str)
+@pytest.mark.parametrize("kw", [dict(), dict(projection=True, peephole=True, layernorm=True)], ids=IDS)
+def test_resident_abort_leaves_state_and_handle_as_they_were(kw, dims, T):
+    import torch
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(970 + T, 3, *dims, T=T, B=11, **kw)
+    want = R.run(w.layers, w.x, *w.initial_state())
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(T)
+    with qlstm.QLSTM(w.layers, T, 11) as q:
+        assert q.debug_resident_plan(T, 11)[0] >= 1
+        x = torch.from_numpy(w.x).to(dev)
+        y = torch.zeros((T, 11, w.layers[-1].n_output), dtype=torch.int8, device=dev)
+        h0, c0 = (rng.integers(-100, 100, a.shape).astype(a.dtype) for a in w.initial_state())
+        for limit in (300_000, 3_000_000):
+            h, c = torch.from_numpy(h0).to(dev), torch.from_numpy(c0).to(dev)
+            q.debug_barrier_timeout(1, limit)
+            q.run(x, T, 11, h, c, y, stream=torch.cuda.current_stream().cuda_stream)
+            with pytest.raises(qlstm.QlstmError) as e:
+                q.last_status()
+            assert e.value.code == qlstm.binding.ERR_TIMEOUT
+            assert np.array_equal(h.cpu().numpy(), h0) and np.array_equal(c.cpu().numpy(), c0)
+            q.debug_barrier_timeout(0)
+            for _ in range(2):
+                for name, g, r in zip(("y", "h", "c"), run_gpu(w, handle=q)[:3], want[:3]):
+                    assert np.array_equal(g, r), name
