@@ -48,8 +48,9 @@ int qlstm_debug_wave_cluster(qlstm_t *q, int T, int B);
 
 /* The wavefront kernel with resident weights (thread-block clusters; it comes before all others for the calls that it takes, with
  * automatic selection).  Its plan: out4 (host) receives the blocks of a cluster (0: does not take such calls), the row groups, the
- * tiles of eight rows of a group, and the groups of eight cells per warp.  Mode 0: automatic, 1: never taken; returns whether the
- * handle has such a plan, or QLSTM_ERR_ARG. */
+ * tiles of eight rows of a group, and the groups of eight cells per warp.  Mode 0: automatic, 1: never taken, 2: launches of clusters - this
+ * kernel's and the few-row kernel's - ask for more shared memory than there is, so that the runtime refuses them; returns whether the handle
+ * has such a plan, or QLSTM_ERR_ARG. */
 int qlstm_debug_resident_plan(qlstm_t *q, int T, int B, int *out4);
 int qlstm_bidir_debug_resident_plan(qlstm_bidir_t *q, int T, int B, int *out4);
 int qlstm_debug_resident(qlstm_t *q, int mode);

@@ -321,7 +321,7 @@ class QLSTM:
         return tuple(out)
 
     def debug_resident(self, mode: int):
-        """0: taken where it fits, 1: never."""
+        """0: taken where it fits, 1: never, 2: launches of clusters are refused."""
         n = lib().qlstm_debug_resident(self._h, mode)
         _check(n if n < 0 else 0, "qlstm_debug_resident")
         return n

@@ -91,15 +91,18 @@ int qlstm_bidir_run(qlstm_bidir_t *q, const int8_t *x_dev, int T, int B, int8_t 
     if (((uintptr_t)x_dev & 15) != 0) return QLSTM_ERR_ARG;
     if (cudaSetDevice(q->device) != cudaSuccess) return QLSTM_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    // (a launch that the device has no room for goes on to the next way)
     if (q->wave && wave_resident_taken(q->wave, T, B, true)) {
         if ((((uintptr_t)c_fwd_dev | (uintptr_t)c_bwd_dev) & 15) != 0) return QLSTM_ERR_ARG;       // as qlstm_run
-        return bidir_resident_run(q->fwd, q->bwd, q->wave, x_dev, T, B, {h_fwd_dev, h_bwd_dev}, {c_fwd_dev, c_bwd_dev}, y_dev, st);
+        const int rc = bidir_resident_run(q->fwd, q->bwd, q->wave, x_dev, T, B, {h_fwd_dev, h_bwd_dev}, {c_fwd_dev, c_bwd_dev}, y_dev, st);
+        if (rc != QLSTM_ERR_LAUNCH) return rc;
     }
     // both directions side by side, each step's outputs written where they belong: two 512-cell layers each way, 16 rows, T = 150: 1290 us
     // one after the other, 672 like this
     if (q->wave && wave_preferred(q->wave, T, B, true)) {
         if ((((uintptr_t)c_fwd_dev | (uintptr_t)c_bwd_dev) & 15) != 0) return QLSTM_ERR_ARG;       // as qlstm_run
-        return bidir_wave_run(q->fwd, q->bwd, q->wave, x_dev, T, B, {h_fwd_dev, h_bwd_dev}, {c_fwd_dev, c_bwd_dev}, y_dev, st);
+        const int rc = bidir_wave_run(q->fwd, q->bwd, q->wave, x_dev, T, B, {h_fwd_dev, h_bwd_dev}, {c_fwd_dev, c_bwd_dev}, y_dev, st);
+        if (rc != QLSTM_ERR_LAUNCH) return rc;
     }
     const size_t chunks = (size_t)B * q->n_input / 16;
     const size_t total = (size_t)T * chunks;
@@ -126,7 +129,7 @@ int qlstm_bidir_debug_wave_plan(qlstm_bidir_t *q, int T, int B, int *out4) { ret
 
 int qlstm_bidir_debug_resident_plan(qlstm_bidir_t *q, int T, int B, int *out4) { return q ? wave_resident_debug_plan(q->wave, T, B, out4) : QLSTM_ERR_ARG; }
 
-int qlstm_bidir_debug_resident(qlstm_bidir_t *q, int mode) { return q && mode >= 0 && mode <= 1 ? wave_resident_mode(q->wave, mode) : QLSTM_ERR_ARG; }
+int qlstm_bidir_debug_resident(qlstm_bidir_t *q, int mode) { return q && mode >= 0 && mode <= 2 ? wave_resident_mode(q->wave, mode) : QLSTM_ERR_ARG; }
 
 void qlstm_bidir_destroy(qlstm_bidir_t *q)
 {

@@ -102,7 +102,8 @@ bool wave_supported(const WaveStack *s, int T, int B, bool tables);
 int wave_debug_plan(const WaveStack *s, int T, int B, bool tables, int *out4);       // include/qlstm_debug.h
 bool wave_preferred(const WaveStack *s, int T, int B, bool tables);      // supported and, by measurement, the faster path
 // h, c: state of the one or two stacks; y: rows of the stacks' outputs side by side; status2: another status word to clear, or
-// null.  The launch clears the status word itself.
+// null.  The launch clears the status word itself.  QLSTM_ERR_LAUNCH: the runtime refused it, nothing of it runs; another kernel may take the
+// call.
 int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
                 bool tables, cudaStream_t st, int *launches);
 // The form with resident weights (wave_resident_sm100.cu), for stacks that fit it: whether a call takes it; the launch.

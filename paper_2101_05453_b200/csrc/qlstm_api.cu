@@ -439,8 +439,8 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
     if (!trace && q->impl_rec == 0 && q->impl_proj != 1 && wave_resident_taken(q->wave, T, B, q->tables)) {
         SpanGuard g(q, st, 1);
         const int rc = launch_wave_resident(q->wave, x_dev, T, B, {h_dev, nullptr}, {c_dev, nullptr}, y_dev, q->status, nullptr, st);
-        g.done(1);
-        return rc;
+        g.done(rc == QLSTM_OK ? 1 : 0);
+        if (rc != QLSTM_ERR_LAUNCH) return rc;                 // refused: the device has no room for the clusters, the other kernels may still run
     }
     // the whole stack in one launch, every layer at once on its own SMs (wave_sm100.cu)
     if (!trace && (q->impl_rec == 0 || q->impl_rec == 8) && q->impl_proj != 1) {
@@ -449,7 +449,7 @@ int qlstm_run(qlstm_t *q, const int8_t *x_dev, int T, int B, int8_t *h_dev, int1
             int launches = 0;
             const int rc = launch_wave(q->wave, x_dev, T, B, {h_dev, nullptr}, {c_dev, nullptr}, y_dev, q->status, nullptr, q->tables, st, &launches);
             g.done(launches);
-            return rc;
+            if (rc != QLSTM_ERR_LAUNCH || q->impl_rec == 8) return rc;
         }
         if (q->impl_rec == 8) return QLSTM_ERR_DIM;
     }
@@ -589,7 +589,7 @@ int qlstm_debug_wave_cluster(qlstm_t *q, int T, int B) { return q ? wave_debug_c
 
 int qlstm_debug_resident_plan(qlstm_t *q, int T, int B, int *out4) { return q ? wave_resident_debug_plan(q->wave, T, B, out4) : QLSTM_ERR_ARG; }
 
-int qlstm_debug_resident(qlstm_t *q, int mode) { return q && mode >= 0 && mode <= 1 ? wave_resident_mode(q->wave, mode) : QLSTM_ERR_ARG; }
+int qlstm_debug_resident(qlstm_t *q, int mode) { return q && mode >= 0 && mode <= 2 ? wave_resident_mode(q->wave, mode) : QLSTM_ERR_ARG; }
 
 int qlstm_debug_activation_tables(qlstm_t *q, int enable)
 {

@@ -373,6 +373,24 @@ __device__ __forceinline__ uint4 wv_load16(const int8_t *src, int valid)      //
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// A launch that the runtime has refused: QLSTM_ERR_LAUNCH where a smaller or another one may still go through.
+inline int wv_refused(cudaError_t e)
+{
+    cudaGetLastError();
+    switch (e) {
+        case cudaErrorCooperativeLaunchTooLarge:
+        case cudaErrorLaunchOutOfResources:
+        case cudaErrorInvalidClusterSize:
+        case cudaErrorInvalidConfiguration:
+        case cudaErrorInvalidValue:
+        case cudaErrorNotSupported:
+            return QLSTM_ERR_LAUNCH;
+        default:
+            return QLSTM_ERR_CUDA;
+    }
+}
+constexpr size_t WV_REFUSED_SMEM = (size_t)1 << 20;            // more shared memory than a block can have (qlstm_debug_resident, mode 2)
+
 __host__ __device__ inline size_t wv_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Memory handed out front to back; without a base it is only counted.  Pieces start 64 KB apart: packed at 256 bytes, what a step's

@@ -14,7 +14,7 @@ void resident_destroy(ResidentStack *s);
 int resident_place(ResidentStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, WaveArena &keep, WaveArena &work, bool fill);
 bool resident_supported(const ResidentStack *s, int T, int B);
 int launch_resident(const ResidentStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status,
-                    int *status2, unsigned missing, unsigned long long limit_ns, cudaStream_t st);
+                    int *status2, unsigned missing, unsigned long long limit_ns, bool refuse, cudaStream_t st);
 void resident_debug_plan(const ResidentStack *s, int T, int B, int *out4);
 
 }  // namespace ql

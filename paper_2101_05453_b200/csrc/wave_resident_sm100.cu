@@ -1068,7 +1068,7 @@ void resident_debug_plan(const ResidentStack *s, int T, int B, int *out4)
 }
 
 int launch_resident(const ResidentStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status,
-                    int *status2, unsigned missing, unsigned long long limit_ns, cudaStream_t st)
+                    int *status2, unsigned missing, unsigned long long limit_ns, bool refuse, cudaStream_t st)
 {
     if (!resident_supported(s, T, B)) return QLSTM_ERR_DIM;
     const ResPlan &p = s->by_rows[B];
@@ -1095,7 +1095,7 @@ int launch_resident(const ResidentStack *s, const int8_t *x, int T, int B, int8_
         L.c = c[L.dir] + s->base[l].c_off * B;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n * p.rg * sh.cl)); cfg.blockDim = dim3((unsigned)(32 * (2 + p.hw + p.xw + p.pw))); cfg.dynamicSmemBytes = p.smem; cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)(n * p.rg * sh.cl)); cfg.blockDim = dim3((unsigned)(32 * (2 + p.hw + p.xw + p.pw))); cfg.dynamicSmemBytes = refuse ? WV_REFUSED_SMEM : p.smem; cfg.stream = st;
     cudaLaunchAttribute a[2];
     a[0].id = cudaLaunchAttributeClusterDimension;
     a[0].val.clusterDim.x = (unsigned)sh.cl; a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
@@ -1104,11 +1104,7 @@ int launch_resident(const ResidentStack *s, const int8_t *x, int T, int B, int8_
     cfg.attrs = a; cfg.numAttrs = 2;
     void *args[] = {(void *)&k};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, rs_kernel(s->G, s->ln, s->peep, p.u), args);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e == cudaErrorCooperativeLaunchTooLarge ? QLSTM_ERR_LAUNCH : QLSTM_ERR_CUDA;
-    }
-    return QLSTM_OK;
+    return e == cudaSuccess ? QLSTM_OK : wv_refused(e);
 }
 
 }  // namespace ql

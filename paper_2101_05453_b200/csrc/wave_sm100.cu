@@ -898,7 +898,7 @@ struct WaveStack {
     uint32_t *cbuf = nullptr;
     void *block[2] = {nullptr, nullptr};       // plans and tables; a call's activations, unless they lie in the caller's scratch
     ResidentStack *res = nullptr;  // wave_resident_sm100.cu; null: no call of this stack fits it
-    int res_mode = 0;              // 1: never taken
+    int res_mode = 0;              // 1: never taken, 2: launches of clusters are refused
     unsigned dbg_missing = 0;
     unsigned long long dbg_limit_ns = 0;
 };
@@ -1475,7 +1475,8 @@ int wave_resident_debug_plan(const WaveStack *s, int T, int B, int *out4)
 int launch_wave_resident(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
                          cudaStream_t st)
 {
-    return launch_resident(s->res, x, T, B, h, c, y, status, status2, s->dbg_missing, s->dbg_limit_ns ? s->dbg_limit_ns : WV_WAIT_LIMIT_NS, st);
+    return launch_resident(s->res, x, T, B, h, c, y, status, status2, s->dbg_missing, s->dbg_limit_ns ? s->dbg_limit_ns : WV_WAIT_LIMIT_NS, s->res_mode == 2,
+                           st);
 }
 
 int wave_debug_plan(const WaveStack *s, int T, int B, bool tables, int *out4)
@@ -1507,6 +1508,7 @@ void wave_debug_timeout(WaveStack *s, unsigned missing_arrivals, unsigned long l
 int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[2], int16_t *const (&c)[2], int8_t *y, int *status, int *status2,
                 bool tables, cudaStream_t st, int *launches)
 {
+    if (launches) *launches = 0;
     WaveCall k;
     size_t smem = 0;
     const WavePlan *plan = wave_plan_of(s, T, B, tables);
@@ -1536,7 +1538,8 @@ int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[
     const void *f = pl.mode == 1 ? wave_small_kernel(s->G, s->ln, s->peep, pl.cl > 0)
                               : (k.tab ? wave_kernel_of<true>(s->G, s->ln, s->peep) : wave_kernel_of<false>(s->G, s->ln, s->peep));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pl.grid); cfg.blockDim = dim3(WV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.gridDim = dim3(pl.grid); cfg.blockDim = dim3(WV_THREADS); cfg.stream = st;
+    cfg.dynamicSmemBytes = s->res_mode == 2 && pl.cl ? WV_REFUSED_SMEM : smem;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
@@ -1544,10 +1547,7 @@ int launch_wave(WaveStack *s, const int8_t *x, int T, int B, int8_t *const (&h)[
     attr[1].val.clusterDim.x = (unsigned)pl.cl; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = pl.cl ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelExC(&cfg, f, args);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e == cudaErrorCooperativeLaunchTooLarge ? QLSTM_ERR_LAUNCH : QLSTM_ERR_CUDA;
-    }
+    if (e != cudaSuccess) return wv_refused(e);
     if (launches) *launches = 2;
     return QLSTM_OK;
 }

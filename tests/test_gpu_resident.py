@@ -113,3 +113,43 @@ def test_resident_abort_leaves_state_and_handle_as_they_were(kw, dims, T):
             for _ in range(2):
                 for name, g, r in zip(("y", "h", "c"), run_gpu(w, handle=q)[:3], want[:3]):
                     assert np.array_equal(g, r), name
+
+
+# clusters that the device has no room for (here: launches that the runtime refuses): the other kernels take the call
+@pytest.mark.parametrize("dims,layers,B", [((80, 304, 208), 3, 9), ((83, 301, 131), 2, 5), ((48, 2048, 640), 1, 30), ((32, 40, 24), 2, 1)], ids=str)
+def test_refused_cluster_launch(dims, layers, B):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(980 + B, layers, *dims, T=5, B=B, projection=True, peephole=True, layernorm=True)
+    want = R.run(w.layers, w.x, *w.initial_state())
+    with qlstm.QLSTM(w.layers, w.T, w.B) as q:
+        for mode in (2, 0):
+            q.debug_resident(mode)
+            for name, g, r in zip(("y", "h", "c"), run_gpu(w, handle=q)[:3], want[:3]):
+                assert np.array_equal(g, r), (mode, name)
+        q.debug_resident(2)
+        if q.debug_wave_cluster(w.T, w.B):                     # (forced: no other kernel may stand in)
+            with pytest.raises(qlstm.QlstmError) as e:
+                run_gpu(w, handle=q, impl=(0, 8))
+            assert e.value.code == qlstm.binding.ERR_LAUNCH
+
+
+@pytest.mark.parametrize("dims,layers", [((32, 96, 48), 2), ((64, 512, 512), 2)], ids=str)
+def test_refused_cluster_launch_bidirectional(dims, layers):
+    import torch
+    import paper_2101_05453_b200 as qlstm
+    from tests.test_gpu_bidirectional import two_directions
+    T, B = 6, 7
+    f, b = two_directions(985, layers, *dims, T, B)
+    yf, hf, cf, _ = R.run(f.layers, f.x, *f.initial_state())
+    yb, hb, cb, _ = R.run(b.layers, f.x[::-1], *b.initial_state())
+    dev = torch.device("cuda:0")
+    with qlstm.BiQLSTM(f.layers, b.layers, T, B) as q:
+        for mode in (2, 0):
+            q.debug_resident(mode)
+            st = [torch.from_numpy(a.copy()).to(dev) for w in (f, b) for a in w.initial_state()]
+            y = torch.zeros((T, B, q.n_output), dtype=torch.int8, device=dev)
+            q.run(torch.from_numpy(np.ascontiguousarray(f.x)).to(dev), T, B, *st, y, stream=torch.cuda.current_stream().cuda_stream)
+            q.last_status()
+            assert np.array_equal(y.cpu().numpy(), np.concatenate([yf, yb[::-1]], axis=2)), mode
+            for got, ref in zip(st, (hf, cf, hb, cb)):
+                assert np.array_equal(got.cpu().numpy(), ref), mode
