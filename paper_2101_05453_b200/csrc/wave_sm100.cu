@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
+#include <cmath>
 #include <utility>
 #include <vector>
 
@@ -1139,33 +1140,46 @@ int wave_max_clusters(const WaveStack *s, int cl)
     return n;
 }
 
-// An estimate of a step of the few-row kernel in us: the weights of a block at 125 KB/us, its exchanges, and what grows with its cells.
-double wave_step_estimate(const WaveStack *s, const std::vector<const LayerParams *> &lp, int per, bool cluster, int rows)
+// An estimate of a step of the few-row kernel in us: rg groups of `per` blocks, each a cluster or not.  Least squares over 2500 calls of 64
+// steps, all cluster sizes and group counts that fit, of 300 random stacks (one to eight layers of 128 to 2048 cells with all variants, 1 to 100
+// rows): 5 % standard error without clusters, 9 % with them.  A cluster's exchanges cost less, but its 16 blocks at most have the more weights
+// to stream and the more cells to finish, and leave more of the SMs idle.
+double wave_step_estimate(const WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, int rg, int per, bool cluster, int B)
 {
+    const double ln = s->ln, peep = s->peep, rows = (B + rg - 1) / rg, ra8 = wv_round((B + rg - 1) / rg, 8) / 8;
     double worst = 0;
-    for (const LayerParams *p : lp) {
-        int cpc = (p->C + per - 1) / per;
-        if (cluster) cpc = wv_round(cpc, 8);
-        const int n = (p->C + cpc - 1) / cpc;
-        const bool proj = p->flags & F_PROJECTION;
-        const double bytes = (double)cpc * p->G * (p->I + p->O) + (proj ? (double)((p->O + n - 1) / n) * p->C : 0.0);
-        const int exchanges = 1 + (s->ln ? 1 : 0) + (proj ? 1 : 0) + (s->ln && s->peep ? 1 : 0);
-        worst = std::max(worst, bytes / 125e3 + exchanges * (cluster ? 1.0 : 2.1) + 0.5 * rows * cpc / 512);
+    for (size_t l = 0; l < lp.size(); ++l) {
+        WaveLayer L = base[l];
+        if (!wave_share_layer(1, *lp[l], per, cluster, L)) return 1e9;
+        const double proj = (L.flags & F_PROJECTION) ? 1 : 0, kb = 1.0 / 1024 / L.n;       // KB per block: all weights, those of the recurrent product
+        const double stream = kb * (L.w_size[0] + L.w_size[1] + L.w_size[2]), rec = kb * L.w_size[1];
+        const double ew = rows * L.cpc / 512, pieces = std::ceil(L.nt * ra8 / 4);          // cells, and pieces of gate tiles, per thread and warp
+        const double proj_rows = proj * ra8 * std::max(1, L.ntp);
+        const double e = cluster ? 1.2 + 0.0073 * stream + 0.0022 * rec + 0.78 * pieces + (0.67 + 0.73 * peep) * ew + 0.065 * rows * L.C / 1024 +
+                                       ln * (0.72 + 0.053 * L.n + 0.094 * rows + 1.5 * peep) + proj * (1.7 + 0.03 * L.n) + 0.26 * proj_rows
+                                 : 3.3 + 0.0028 * stream + 0.0056 * rec + (0.74 + 0.54 * peep) * ew + 0.059 * 8 * ra8 * L.C / 1024 +
+                                       ln * (2.3 + 0.11 * pieces + 0.048 * rows + 2.3 * peep) + proj * 3.3 + 0.22 * proj_rows;
+        worst = std::max(worst, e);
     }
-    return worst;
+    // the weights of all groups pass through L2 in every step
+    return worst + (cluster ? 0.082 : 0.11) * std::max(0.0, 1e-6 * rg * s->weights - 60);
 }
 
-// Whether calls of B rows go to clusters, and to how many groups of clusters of which size.  `clusters`: [cl] that fit at once.
-bool wave_cluster_plan(const WaveStack *s, const std::vector<const LayerParams *> &lp, const int *clusters, int B, int rg_other, int &rg, int &cl)
+// Whether calls of B rows go to clusters, and to how many groups of clusters of which size.  `clusters`: [cl] that fit at once.  Where the
+// estimates are close the form without clusters has it (us per call of 64 steps, without clusters and with the best ones: one 2048-cell layer with
+// layer norm, peephole and projection, 32 rows 1116 and 1202; four 1120-cell layers with projection, 20 rows 700 and 756; three of 1000 cells with
+// layer norm and projection, 37 rows 1011 and 898; one of 880 cells with projection, 15 rows 493 and 387; with the factor below none of 290 stacks
+// was more than 4 % slower than without clusters, and the choice 1 % slower in the mean than the best of all, 20 % at most).
+bool wave_cluster_plan(const WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, const int *clusters, int B, int rg_other,
+                       int &rg, int &cl)
 {
     const int n = (int)lp.size();
-    double best = 0.97 * wave_step_estimate(s, lp, s->sm_count / (n * rg_other), false, (B + rg_other - 1) / rg_other);
+    double best = 0.93 * wave_step_estimate(s, lp, base, rg_other, s->sm_count / (n * rg_other), false, B);
     cl = 0;
     for (int size = 8; size <= 16; ++size)
         for (int groups = 1; groups <= B && groups * n <= clusters[size]; groups *= 2) {
-            const int rows = (B + groups - 1) / groups;
-            if (rows > WV_SMALL_ROWS || (groups > 1 && groups * s->weights > (size_t)(s->ln ? 200 : 128) * 1000000)) continue;
-            const double e = wave_step_estimate(s, lp, size, true, rows);
+            if ((B + groups - 1) / groups > WV_SMALL_ROWS) continue;
+            const double e = wave_step_estimate(s, lp, base, groups, size, true, B);
             if (e >= best) continue;
             best = e;
             rg = groups; cl = size;
@@ -1305,7 +1319,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     for (int B = 1; B <= s->max_B; ++B) {
         int rg, cl;
         const int other = wave_row_groups(s, 1, lp, B);
-        if (!wave_small_fits(s, lp, other, B, s->sm_count) || !wave_cluster_plan(s, lp, clusters, B, other, rg, cl)) continue;
+        if (!wave_small_fits(s, lp, other, B, s->sm_count) || !wave_cluster_plan(s, lp, base, clusters, B, other, rg, cl)) continue;
         const int i = wave_plan(s, lp, base, 1, rg, cl);
         WavePlan &pl = s->plan[i];
         if (!wave_describe(s, pl, max_T, B, true, k, smem)) continue;

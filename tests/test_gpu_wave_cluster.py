@@ -43,3 +43,13 @@ def test_wave_cluster_long_calls_of_several_layers(kw):
             got = run_gpu(w, handle=q, impl=(0, WAVE))
             for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
                 assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}"
+
+
+# stacks measured slower in clusters, whose few blocks stream more and finish more cells than the exchanges save
+@pytest.mark.parametrize("layers,dims,B,kw", [(1, (512, 2048, 640), 32, dict(projection=True, peephole=True, layernorm=True)), (4, (128, 1120, 416), 20, dict(projection=True)),
+                                              (2, (576, 1872, 352), 24, dict(projection=True, layernorm=True, cifg=True)), (6, (80, 704, 704), 1, dict())], ids=str)
+def test_wave_cluster_is_left_alone_where_it_is_slower(layers, dims, B, kw):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(990 + B, layers, *dims, T=2, B=B, **kw)
+    with qlstm.QLSTM(w.layers, 2, B) as q:
+        assert q.debug_wave_cluster(2, B) == 0 and q.debug_wave_plan(2, B)[0] == 1
