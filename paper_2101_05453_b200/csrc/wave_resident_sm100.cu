@@ -895,8 +895,15 @@ void rs_share_layer(ResLayer &L, int cl)
     L.img_stride = (size_t)(L.cpc / 8) * (L.ki + L.kh) * G * 512 + (proj ? (size_t)(L.opc / 8) * L.kc * 512 : 0);
 }
 
-// The plan of calls of B rows under a shape, and an estimate of a step in cycles; false: does not fit.
-bool rs_try_plan(const ResidentStack *s, const ResShape &sh, int B, int max_smem, ResPlan &p, double &cycles)
+// The plan of calls of B rows under a shape, and an estimate of a step in us; false: does not fit.
+// The estimate: least squares over 1900 calls of 64 steps, all cluster sizes, of 160 random stacks (one to eight layers of 32 to 900 cells with all
+// variants, 1 to 256 rows), 9 % standard error.  What a warp does for its groups of eight cells one after the other costs more than an
+// exchange saves, and with two or more groups per warp the layer norm's registers spill on top: many blocks of one group per warp are nearly
+// always ahead (us per call of 64 steps in clusters of 1, 2, 4 and 8: two 208-cell layers with layer norm and projection, 4 rows 882, 353, 229 and
+// 211; three 104-cell CIFG layers, 11 rows 187, 107, 83 and 76).  Over 130 other stacks the shape chosen was 2 % slower in the mean than the best
+// one, 19 % at most, and no call was slower than on the kernels that take it otherwise (0.46 of their time in the mean, 0.96 at most; calls of 1, 4
+// and 128 steps 1.01 to 5.5, 1.14 to 3.8 and 1.08 to 7.7 times as fast), so that a call that fits always comes here.
+bool rs_try_plan(const ResidentStack *s, const ResShape &sh, int B, int max_smem, ResPlan &p, double &us)
 {
     const int n = (int)sh.layer.size();
     int rg = std::min(B, sh.clusters / n);
@@ -913,28 +920,27 @@ bool rs_try_plan(const ResidentStack *s, const ResShape &sh, int B, int max_smem
         proj = proj || (L.flags & F_PROJECTION);
     }
     p.hw = std::min(units, 8);
-    p.u = (units + p.hw - 1) / p.hw;
-    if (p.u > 4) return false;
-    if (p.u == 3) p.u = 4;
+    const int u = (units + p.hw - 1) / p.hw;
+    if (u > 4) return false;
+    p.u = u == 3 ? 4 : u;
     p.xw = std::min(units, proj ? 4 : 8);
     p.pw = proj ? 4 : 0;
     p.smem = 0;
-    cycles = 0;
+    us = 0;
     const int ntr = (rows + 7) / 8;
+    const double ln = s->ln, ln_peep = s->ln && s->peep;
     for (const ResLayer &L : sh.layer) {
         p.smem = std::max(p.smem, rs_layout(L, sh.cl, p.nt, p.hw, p.pw, s->ln, s->peep).total);
-        const double per = 4.0 * (s->G + 1) * (L.cpc / 8) * ntr;         // cycles per 64 bytes of K: shared memory reads
-        const double h = std::max(per * L.kh, 45.0 * L.kh), x = std::max(per * L.ki, 45.0 * L.ki);
-        const bool one = L.cpc >= L.C;
-        double e = 450 + h;
-        auto exchange = [&](int width) { return one ? 80.0 : 650.0 + 1.3 * rows * ((width + 7) / 8) * (sh.cl > 12 ? 2 : 1); };
-        e += exchange(L.O);
-        if (s->ln) e += (one ? 500 : 1200) + (s->peep ? (one ? 400 : 1100) : 0);
+        const double tiles = L.cpc / 8 * ntr, many = L.cpc < L.C;              // tiles of eight cells and rows; several blocks
+        double e = 0.46 + 0.07 * L.kh * u + 0.088 * s->G * u + 0.07 * tiles + 0.0015 * tiles * L.ki * (s->G + 1) + many * 0.0001 * rows * L.O;
+        if (p.u == 2) e += 0.06 + 0.99 * ln;
+        if (p.u == 4) e += u * (0.13 + 0.83 * ln);
+        e += ln * (1.16 + 0.144 * u + many * (0.0012 * rows * s->G + 0.058 * sh.cl)) + ln_peep * (1.16 + 0.07 * u + many * 0.33);
         if (L.flags & F_PROJECTION) {
-            e += 200 + exchange(L.C) + std::max(12.0 * ((L.opc / 8 + 1) / 2) * ntr * L.kc, 25.0 * L.kc / std::max(1, p.pw / (((L.opc / 8 + 1) / 2) * ntr)));
+            const int tasks = ((L.opc / 8 + 1) / 2) * ntr;
+            e += 0.33 + 0.025 * L.kc * std::max(1.0, tasks / 4.0) + 0.067 * L.kc / std::max(1, p.pw / tasks);
         }
-        e = std::max(e, x + 200);
-        cycles = std::max(cycles, e);
+        us = std::max(us, e);
     }
     return p.smem <= (size_t)max_smem;
 }
@@ -1004,10 +1010,10 @@ ResidentStack *resident_plan(const std::vector<const LayerParams *> &lp, const s
         double best = 0;
         for (size_t i = 0; i < s->shape.size(); ++i) {
             ResPlan p;
-            double cycles;
-            if (!rs_try_plan(s, s->shape[i], B, max_smem, p, cycles)) continue;
-            if (s->by_rows[B].shape >= 0 && cycles >= best) continue;
-            best = cycles;
+            double us;
+            if (!rs_try_plan(s, s->shape[i], B, max_smem, p, us)) continue;
+            if (s->by_rows[B].shape >= 0 && us >= best) continue;
+            best = us;
             p.shape = (int)i;
             s->by_rows[B] = p;
         }

@@ -1168,8 +1168,8 @@ double wave_step_estimate(const WaveStack *s, const std::vector<const LayerParam
 // Whether calls of B rows go to clusters, and to how many groups of clusters of which size.  `clusters`: [cl] that fit at once.  Where the
 // estimates are close the form without clusters has it (us per call of 64 steps, without clusters and with the best ones: one 2048-cell layer with
 // layer norm, peephole and projection, 32 rows 1116 and 1202; four 1120-cell layers with projection, 20 rows 700 and 756; three of 1000 cells with
-// layer norm and projection, 37 rows 1011 and 898; one of 880 cells with projection, 15 rows 493 and 387; with the factor below none of 290 stacks
-// was more than 4 % slower than without clusters, and the choice 1 % slower in the mean than the best of all, 20 % at most).
+// layer norm and projection, 37 rows 1011 and 898; one of 880 cells with projection, 15 rows 493 and 387; with the factor below none of 148
+// other stacks was slower than without clusters, and the choice 1 % slower in the mean than the best of all, 14 % at most).
 bool wave_cluster_plan(const WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, const int *clusters, int B, int rg_other,
                        int &rg, int &cl)
 {

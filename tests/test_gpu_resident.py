@@ -29,11 +29,32 @@ def check(w, **plan):
                 assert np.array_equal(g, r), f"{name} differs at {np.argwhere(g != r)[:3].tolist()}, plan {(cluster, groups, tiles, units)}"
 
 
-# one block per layer and row group, and clusters of several; one row to several tiles of eight; partial groups of eight cells
+# one block per layer and row group (a single group of eight cells; with layer norm three), and clusters of several; one row to several
+# tiles of eight; partial groups of eight cells
 @pytest.mark.parametrize("B", [1, 7, 8, 40])
 @pytest.mark.parametrize("kw", VARIANTS, ids=IDS)
 def test_resident_one_block(kw, B):
-    check(random_layer_stack(910 + B, 2, 32, 40, 24, T=7, B=B, **kw), cluster=1)
+    check(random_layer_stack(905 + B, 2, 32, 7, 5, T=7, B=B, **kw), cluster=1)
+    if kw.get("layernorm"):
+        check(random_layer_stack(907 + B, 2, 32, 21, 14, T=7, B=B, **kw), cluster=1)
+
+
+@pytest.mark.parametrize("B", [1, 7, 8, 40])
+@pytest.mark.parametrize("kw", VARIANTS, ids=IDS)
+def test_resident_few_cells(kw, B):
+    check(random_layer_stack(910 + B, 2, 32, 40, 24, T=7, B=B, **kw))
+
+
+# shapes measured two to four times slower than others: several groups of cells per warp, one after the other, where more blocks fit
+@pytest.mark.parametrize("layers,dims,B,kw", [(2, (16, 208, 24), 4, dict(projection=True, layernorm=True)), (3, (64, 104, 104), 11, dict(cifg=True)),
+                                              (1, (64, 136, 136), 40, dict(layernorm=True)), (6, (32, 232, 24), 1, dict(projection=True, layernorm=True, peephole=True, cifg=True))],
+                         ids=str)
+def test_resident_shape(layers, dims, B, kw):
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(915, layers, *dims, T=1, B=B, **kw)
+    with qlstm.QLSTM(w.layers, 1, B) as q:
+        cluster, _, _, units = q.debug_resident_plan(1, B)
+        assert cluster >= 2 and units == 1
 
 
 @pytest.mark.parametrize("B", [1, 9, 30, 60])
