@@ -981,14 +981,17 @@ ResidentStack *resident_plan(const std::vector<const LayerParams *> &lp, const s
         L.dir = W.dir; L.y_off = W.y_off; L.tab_lay = W.tab_lay;
         layers.push_back(L);
     }
-    const void *f[3] = {rs_kernel(s->G, s->ln, s->peep, 1), rs_kernel(s->G, s->ln, s->peep, 2), rs_kernel(s->G, s->ln, s->peep, 4)};
-    for (const void *k : f)
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) != cudaSuccess ||
-            cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-            cudaGetLastError();
-            delete s;
-            return nullptr;
-        }
+    // (setting an attribute loads a kernel, some milliseconds the first time in a process: the forms of several groups of cells per warp only
+    // where a call takes them)
+    bool loaded[5] = {};
+    auto load = [&](int u) {
+        if (loaded[u]) return true;
+        const void *f = rs_kernel(s->G, s->ln, s->peep, u);
+        loaded[u] = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem) == cudaSuccess &&
+                    cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        if (!loaded[u]) cudaGetLastError();
+        return loaded[u];
+    };
     for (int cl = (int)std::max<size_t>(1, widest / max_smem); cl <= RS_MAX_CLUSTER; ++cl) {
         ResShape sh;
         sh.cl = cl;
@@ -999,6 +1002,7 @@ ResidentStack *resident_plan(const std::vector<const LayerParams *> &lp, const s
             fits = fits && rs_layout(L, cl, 1, 1, 1, s->ln, s->peep).total <= (size_t)max_smem;
         }
         if (!fits) continue;
+        if (!load(1)) break;
         sh.clusters = rs_max_clusters(s, cl, max_smem);
         if (sh.clusters < n) continue;
         s->shape.push_back(sh);
@@ -1006,16 +1010,19 @@ ResidentStack *resident_plan(const std::vector<const LayerParams *> &lp, const s
     s->by_rows.resize((size_t)max_B + 1);
     size_t groups = 0;
     bool any = false;
-    for (int B = 1; B <= max_B; ++B) {
-        double best = 0;
-        for (size_t i = 0; i < s->shape.size(); ++i) {
-            ResPlan p;
-            double us;
-            if (!rs_try_plan(s, s->shape[i], B, max_smem, p, us)) continue;
-            if (s->by_rows[B].shape >= 0 && us >= best) continue;
-            best = us;
-            p.shape = (int)i;
-            s->by_rows[B] = p;
+    for (int B = max_B; B >= 1; --B) {
+        // shapes that other calls of the handle take first: another one has to be 3 % ahead of them, for it has weight images of its own
+        double line = 1e9;
+        for (int fresh = 0; fresh < 2; ++fresh) {
+            if (fresh && s->by_rows[B].shape >= 0) line *= 0.97;
+            for (size_t i = 0; i < s->shape.size(); ++i) {
+                ResPlan p;
+                double us;
+                if (s->shape[i].used == (fresh == 1) || !rs_try_plan(s, s->shape[i], B, max_smem, p, us) || us >= line || !load(p.u)) continue;
+                line = us;
+                p.shape = (int)i;
+                s->by_rows[B] = p;
+            }
         }
         if (s->by_rows[B].shape < 0) continue;
         any = true;

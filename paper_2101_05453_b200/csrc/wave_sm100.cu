@@ -1126,9 +1126,12 @@ bool wave_describe(const WaveStack *s, const WavePlan &pl, int T, int B, bool ta
     return true;
 }
 
-// Clusters of cl blocks of the few-row kernel that fit on the device at once (a block per SM).
-int wave_max_clusters(const WaveStack *s, int cl)
+// Clusters of cl blocks of the few-row kernel that fit on the device at once (a block per SM).  Asked only for sizes that some call would take
+// (-1: not asked yet): the first question in a process loads the kernel, some milliseconds.
+int wave_max_clusters(const WaveStack *s, int cl, int (&known)[17])
 {
+    if (known[cl] >= 0) return known[cl];
+    const void *f = wave_small_kernel(s->G, s->ln, s->peep, true);
     cudaLaunchConfig_t c = {};
     c.gridDim = dim3(cl); c.blockDim = dim3(WV_THREADS); c.dynamicSmemBytes = (size_t)s->max_smem;
     cudaLaunchAttribute a[1];
@@ -1136,8 +1139,12 @@ int wave_max_clusters(const WaveStack *s, int cl)
     a[0].val.clusterDim.x = (unsigned)cl; a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
     c.attrs = a; c.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, wave_small_kernel(s->G, s->ln, s->peep, true), &c) != cudaSuccess) { cudaGetLastError(); return 0; }
-    return n;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) != cudaSuccess ||
+        cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, f, &c) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    return known[cl] = n;
 }
 
 // An estimate of a step of the few-row kernel in us: rg groups of `per` blocks, each a cluster or not.  Least squares over 2500 calls of 64
@@ -1165,25 +1172,33 @@ double wave_step_estimate(const WaveStack *s, const std::vector<const LayerParam
     return worst + (cluster ? 0.082 : 0.11) * std::max(0.0, 1e-6 * rg * s->weights - 60);
 }
 
-// Whether calls of B rows go to clusters, and to how many groups of clusters of which size.  `clusters`: [cl] that fit at once.  Where the
+// Whether calls of B rows go to clusters, and to how many groups of clusters of which size.  `known`: see wave_max_clusters.  Where the
 // estimates are close the form without clusters has it (us per call of 64 steps, without clusters and with the best ones: one 2048-cell layer with
 // layer norm, peephole and projection, 32 rows 1116 and 1202; four 1120-cell layers with projection, 20 rows 700 and 756; three of 1000 cells with
 // layer norm and projection, 37 rows 1011 and 898; one of 880 cells with projection, 15 rows 493 and 387; with the factor below none of 148
 // other stacks was slower than without clusters, and the choice 1 % slower in the mean than the best of all, 14 % at most).
-bool wave_cluster_plan(const WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, const int *clusters, int B, int rg_other,
+bool wave_cluster_plan(const WaveStack *s, const std::vector<const LayerParams *> &lp, const std::vector<WaveLayer> &base, int (&known)[17], int B, int rg_other,
                        int &rg, int &cl)
 {
     const int n = (int)lp.size();
     double best = 0.93 * wave_step_estimate(s, lp, base, rg_other, s->sm_count / (n * rg_other), false, B);
     cl = 0;
-    for (int size = 8; size <= 16; ++size)
-        for (int groups = 1; groups <= B && groups * n <= clusters[size]; groups *= 2) {
-            if ((B + groups - 1) / groups > WV_SMALL_ROWS) continue;
-            const double e = wave_step_estimate(s, lp, base, groups, size, true, B);
-            if (e >= best) continue;
-            best = e;
-            rg = groups; cl = size;
+    // sizes that other calls of the handle take first: another one has to be 3 % ahead of them, for it has weight images of its own
+    for (int fresh = 0; fresh < 2; ++fresh) {
+        double line = fresh && cl ? 0.97 * best : best;
+        for (int size = 8; size <= 16; ++size) {
+            bool taken = false;
+            for (const WavePlan &pl : s->plan) taken = taken || (pl.used && pl.cl == size);
+            if (taken == (fresh == 1)) continue;
+            for (int groups = 1; groups <= B && groups * n * size <= s->sm_count; groups *= 2) {
+                if ((B + groups - 1) / groups > WV_SMALL_ROWS) continue;
+                const double e = wave_step_estimate(s, lp, base, groups, size, true, B);
+                if (e >= line || groups * n > wave_max_clusters(s, size, known)) continue;
+                best = line = e;
+                rg = groups; cl = size;
+            }
         }
+    }
     return cl > 0;
 }
 
@@ -1307,16 +1322,9 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     WaveCall k;
     size_t smem, rows_alloc = 0, zero_words = 0, g_bytes = 0, c_bytes = 0;
     for (int B = 1; B <= s->max_B; ++B) s->fit_groups[B] = (uint16_t)wave_fit_groups(s, lp, B);
-    int clusters[17] = {};
-    if (s->tabs) {
-        const void *f = wave_small_kernel(s->G, s->ln, s->peep, true);
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, s->max_smem) == cudaSuccess &&
-            cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
-            for (int size = 8; size <= 16; ++size) clusters[size] = wave_max_clusters(s, size);
-        else
-            cudaGetLastError();
-    }
-    for (int B = 1; B <= s->max_B; ++B) {
+    int clusters[17];
+    for (int &v : clusters) v = -1;
+    for (int B = s->max_B; B >= 1 && s->tabs; --B) {
         int rg, cl;
         const int other = wave_row_groups(s, 1, lp, B);
         if (!wave_small_fits(s, lp, other, B, s->sm_count) || !wave_cluster_plan(s, lp, base, clusters, B, other, rg, cl)) continue;
@@ -1353,7 +1361,7 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
     // (only of the forms that some call takes: setting an attribute loads a kernel, some milliseconds the first time in a process)
     for (const WavePlan &pl : s->plan) {
         if (!pl.used) continue;
-        if (pl.cl) continue;                                   // (set above)
+        if (pl.cl) continue;                                   // (set by wave_max_clusters)
         const void *f[2] = {wave_small_kernel(s->G, s->ln, s->peep, false), nullptr};
         if (pl.mode == 0) { f[0] = wave_kernel_of<true>(s->G, s->ln, s->peep); f[1] = wave_kernel_of<false>(s->G, s->ln, s->peep); }
         for (const void *kernel : f)
@@ -1386,6 +1394,15 @@ int wave_create(const std::vector<const LayerParams *> &lp, int n_fwd, int max_T
                 if (!pl.used) continue;
                 WaveLayer &M = pl.layer[l];
                 M.in_img = L.in_img; M.out_img = L.out_img; M.m_img = L.m_img; M.tab = L.tab;
+                // (plans of one cluster size share their images: the blocks' shares are the same)
+                const WavePlan *same = nullptr;
+                for (const WavePlan *o = s->plan.data(); o < &pl && !same; ++o)
+                    if (pl.cl && o->used && o->cl == pl.cl) same = o;
+                if (same) {
+                    const WaveLayer &S = same->layer[l];
+                    M.img_w = S.img_w; M.img_r = S.img_r; M.img_p = S.img_p;
+                    continue;
+                }
                 int8_t *img[3];
                 for (int i = 0; i < 3; ++i) keep.take(img[i], M.w_size[i]);
                 M.img_w = img[0]; M.img_r = img[1]; M.img_p = img[2];

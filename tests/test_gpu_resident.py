@@ -23,6 +23,8 @@ def check(w, **plan):
             assert (cluster == 1) == (plan["cluster"] == 1), cluster
         if "tiles" in plan:
             assert tiles == plan["tiles"], tiles
+        if "units" in plan:
+            assert units >= plan["units"], units
         for _ in range(2):                                     # (a second call: what the first one left behind)
             got = run_gpu(w, handle=q)
             for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
@@ -76,6 +78,26 @@ def test_resident_odd_dimensions(kw, T):
 @pytest.mark.parametrize("kw", VARIANTS, ids=IDS)
 def test_resident_tiles_of_rows(kw, B, tiles):
     check(random_layer_stack(950 + B, 16, 32, 48, 32, T=3, B=B, **kw), tiles=tiles)
+
+
+# two to four groups of eight cells per warp, with one, two and four tiles of rows: deep stacks, whose layers get few blocks each
+@pytest.mark.parametrize("layers,dims,B", [(16, (32, 160, 80), 20), (8, (32, 256, 128), 60), (10, (32, 250, 125), 60), (8, (32, 64, 32), 200), (16, (32, 206, 101), 60)], ids=str)
+@pytest.mark.parametrize("kw", [dict(projection=True, cifg=True), dict(projection=True, layernorm=True), dict(projection=True, peephole=True, layernorm=True, cifg=True)], ids=IDS)
+def test_resident_groups_per_warp(kw, layers, dims, B):
+    check(random_layer_stack(955, layers, *dims, T=4, B=B, **kw), units=2)
+
+
+@pytest.mark.parametrize("layers,C,B", [(16, 160, 20), (8, 206, 60), (8, 160, 140), (10, 45, 140), (14, 112, 100)], ids=str)
+def test_resident_groups_per_warp_basic(layers, C, B):
+    check(random_layer_stack(956, layers, 32, C, C, T=4, B=B), units=2)
+
+
+# a handle's smaller calls share the weight images of a few cluster sizes
+def test_resident_calls_of_one_handle_share_shapes():
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(957, 2, 32, 256, 256, T=1, B=64)
+    with qlstm.QLSTM(w.layers, 4, 64) as q:
+        assert len({q.debug_resident_plan(4, B)[0] for B in range(1, 65)} - {0}) <= 4
 
 
 # gate sums so small that layer-norm quotients leave the fast range, or that whole rows are zero
