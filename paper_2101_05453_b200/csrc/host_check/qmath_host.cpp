@@ -3,22 +3,6 @@
 #include "../qmath.cuh"
 #include "../wave_math.cuh"
 
-namespace {
-using ql::floor_s32;
-// floor(n / d) for n < 2^57, d < 2^26 and a quotient below 2^31; x: reciprocal estimate of d (relative error 2^-21 at most)
-uint32_t wv_div(uint64_t n, uint32_t d, float x)
-{
-    uint32_t q = (uint32_t)((float)n * x);                     // within 2^11
-    int64_t r = (int64_t)(n - (uint64_t)q * d);
-    const int32_t c = floor_s32((float)r * x);                 // then within 1 (rounded towards zero, a negative one could be 2 off)
-    q += (uint32_t)c;
-    r -= (int64_t)c * d;
-    if (r < 0) { --q; r += d; }
-    if (r >= (int64_t)d) ++q;
-    return q;
-}
-}
-
 extern "C" {
 int32_t qmh_mbqm(int32_t x, int32_t mult, int32_t shift) { return ql::mbqm(x, ql::Scale{mult, shift}); }
 void qmh_mbqm_many(const int32_t *x, int n, int32_t mult, int32_t shift, int32_t *out)
@@ -74,7 +58,7 @@ void qmh_wave_quotients(const int32_t *q, int count, int32_t mean, uint32_t sigm
     ql::wv_limbs(sigma, hi, lo);
     for (int i = 0; i < count; ++i) out[i] = ql::wv_ln_quotient(q[i], hi, lo, mean);
 }
-uint32_t qmh_wave_div(uint64_t n, uint32_t d) { return wv_div(n, d, ql::rcp_est((float)d)); }
+void qmh_wave_limbs(uint32_t sigma, int32_t *out2) { ql::wv_limbs(sigma, out2[0], out2[1]); }
 void qmh_wave_skew(float v) { ql::wv_skew() = v; }
 int32_t qmh_line_value(int32_t e, int32_t x, int sh, int k) { return ql::act_line_value(e, x, sh, k); }
 }

@@ -311,16 +311,25 @@ def test_wave_statistics_with_estimates_as_wrong_as_the_hardwares(H, skew):
         H.qmh_wave_skew(0.0)
 
 
-def test_wave_division(H):
-    """wv_div over the range it is used for: n < 2^57, d < 2^26, quotient below 2^31."""
-    H.qmh_wave_div.restype = C.c_uint32
-    H.qmh_wave_div.argtypes = [C.c_uint64, C.c_uint32]
+@pytest.mark.parametrize("skew", [0.0, 2.0 ** -22, -2.0 ** -22])
+def test_wave_limbs(H, skew):
+    """wv_limbs over the sigmas it is used for, 2^20 to 2^25: the next multiple of 2^-73 above 1 / sigma, in two limbs of 31 bits, with the
+    reciprocal estimate exact and off by more than the instruction's documented error."""
+    H.qmh_wave_limbs.restype = None
+    H.qmh_wave_limbs.argtypes = [C.c_uint32, C.POINTER(C.c_int32)]
+    H.qmh_wave_skew.argtypes = [C.c_float]
     rng = np.random.default_rng(52)
-    for _ in range(20000):
-        d = int(rng.integers(1 << 12, 1 << 26))
-        for n in (1 << 42, int(rng.integers(0, min(d << 31, 1 << 57))), int(rng.integers(0, 1 << 30)) * d, max(int(rng.integers(1, 1 << 30)) * d - 1, 0)):
-            if n < min(d << 31, 1 << 57):
-                assert H.qmh_wave_div(n, d) == n // d, (n, d)
+    sigmas = [(1 << k) + d for k in range(20, 26) for d in (-1, 0, 1)] + [m << k for k in range(18, 22) for m in (3, 5, 7, 11)]
+    sigmas += [int(2.0 ** v) for v in rng.uniform(20, 25, 20000)]
+    out = (C.c_int32 * 2)()
+    H.qmh_wave_skew(skew)
+    try:
+        for s in sigmas:
+            if 1 << 20 <= s <= 1 << 25:
+                H.qmh_wave_limbs(s, out)
+                assert 0 <= out[1] < 1 << 31 and (out[0] << 31) + out[1] == (1 << 73) // s + 1, s
+    finally:
+        H.qmh_wave_skew(0.0)
 
 
 def test_wave_quotients_with_exact_ties(H):
