@@ -17,10 +17,11 @@ extern "C" {
 /* Kernel selection, for tests and measurements.  0 = automatic (default), 1 = simple kernels
  * (one thread per output, one launch per phase), 2 = fast kernels (tensor-core projection,
  * persistent recurrent kernel); 2 fails with QLSTM_ERR_DIM at run time if a shape is unsupported.
- * recurrent_impl 2 always runs layer after layer (projection launch + persistent kernel per layer), where 0 takes the wavefront kernels
- * for every call that they support (up to 256 rows, layers of one kind) but these: one step of one or two rows and a few other short
- * calls of up to four rows (whole-stack kernel), calls of few steps of many rows - T * 256 <= layers * (B - 32) - and single layers
- * of many rows (layer after layer).  Dimensions that are no multiples of 16 always take the wavefront kernels.
+ * recurrent_impl 2 always runs layer after layer (projection launch + persistent kernel per layer), where 0 takes the wavefront kernel with
+ * resident weights for every call that fits it (up to 256 rows, layers of one kind whose weights the shared memory of thread-block clusters
+ * holds), else the other wavefront kernels for every call that they support (up to 256 rows, layers of one kind) but these: one step of
+ * one or two rows and a few other short calls of up to four rows (whole-stack kernel), calls of few steps of many rows -
+ * T * 256 <= layers * (B - 32) - and single layers of many rows (layer after layer).  Dimensions that are no multiples of 16 always take the wavefront kernels.
  * 3 = like 2 but with the tensor-core matmuls even at batch <= 4, where 2 uses dp4a
  * mat-vecs; 4 = like 2 but with the dp4a mat-vecs up to batch 16 (the crossover is a measured default, not a limit);
  * 5 = the whole-stack kernel or QLSTM_ERR_DIM (batch > 16, or a dimension that is not a multiple of 16), with its
@@ -38,7 +39,8 @@ int qlstm_debug_barrier_timeout(qlstm_t *q, int missing_arrivals, unsigned long 
 
 /* The wavefront kernels' plan for a call of T steps and B rows on this handle: out4 (host) receives the kernel's form (1 few rows:
  * gate rows as the M side of the products; 0 many rows: batch rows as the M side; -1 none takes the call), the row groups that the
- * batch is split into, the units of at most 128 rows of a group, and whether an ordinary call of these sizes takes this path. */
+ * batch is split into, the units of at most 128 rows of a group, and whether an ordinary call of these sizes takes this path (not where the
+ * kernel with resident weights comes before it: qlstm_debug_resident). */
 int qlstm_debug_wave_plan(qlstm_t *q, int T, int B, int *out4);
 int qlstm_bidir_debug_wave_plan(qlstm_bidir_t *q, int T, int B, int *out4);
 

@@ -1519,7 +1519,7 @@ int wave_debug_plan(const WaveStack *s, int T, int B, bool tables, int *out4)
     out4[0] = pl ? pl->mode : -1;
     out4[1] = pl ? pl->rg : 0;
     out4[2] = units;
-    out4[3] = wave_preferred(s, T, B, tables) ? 1 : 0;
+    out4[3] = wave_preferred(s, T, B, tables) && !wave_resident_taken(s, T, B, tables) ? 1 : 0;
     return QLSTM_OK;
 }
 

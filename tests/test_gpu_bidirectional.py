@@ -16,7 +16,7 @@ def two_directions(seed, n_layers, I, C, O, T, B, **kw):
 
 
 @pytest.mark.parametrize("kw,B,T", [(dict(), 3, 9), (dict(projection=True, layernorm=True), 20, 6),
-                                    (dict(cifg=True, peephole=True), 130, 5), (dict(projection=True), 1, 12)],
+                                    (dict(cifg=True, peephole=True), 130, 5), (dict(projection=True), 1, 12), (dict(layernorm=True), 200, 1)],
                          ids=lambda v: "+".join(sorted(v)) or "basic" if isinstance(v, dict) else str(v))
 def test_bidirectional_matches_two_oracle_runs(kw, B, T):
     import torch
@@ -33,14 +33,18 @@ def test_bidirectional_matches_two_oracle_runs(kw, B, T):
         xd = torch.from_numpy(np.ascontiguousarray(x)).to(dev)
         st = [torch.from_numpy(a.copy()).to(dev) for a in (hf0, cf0, hb0, cb0)]
         y = torch.zeros((T, B, q.n_output), dtype=torch.int8, device=dev)
-        for _ in range(2):                                      # a second call on the same handle: workspaces are reused
+        assert q.debug_resident_plan(T, B)[0] >= 1
+        for resident in (0, 0, 1, 1):                           # 1: the kernels that larger stacks take; second calls: workspaces are reused
+            q.debug_resident(resident)
             for t_, a in zip(st, (hf0, cf0, hb0, cb0)):
                 t_.copy_(torch.from_numpy(a))
+            y.zero_()
             q.run(xd, T, B, st[0], st[1], st[2], st[3], y, stream=torch.cuda.current_stream().cuda_stream)
             q.last_status()
-            assert np.array_equal(y.cpu().numpy(), want)
+            assert np.array_equal(y.cpu().numpy(), want), resident
             for got, ref in zip(st, (hf, cf, hb, cb)):
-                assert np.array_equal(got.cpu().numpy(), ref)
+                assert np.array_equal(got.cpu().numpy(), ref), resident
+        assert q.debug_wave_plan(T, B)[3] == (T * 256 > 2 * (B - 32))      # (else one direction after the other)
 
 
 def test_bidirectional_argument_checks():

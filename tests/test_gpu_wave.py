@@ -91,7 +91,7 @@ def test_wave_many_rows_layernorm_of_small_deviations(shift, kw):
     check(w, MANY, 1)
 
 
-# both directions in one launch: few and many rows, one and two units
+# both directions in one launch: few and many rows, one and two units (and, where it fits, the kernel with resident weights)
 @pytest.mark.parametrize("B", [3, 70, 140])
 @pytest.mark.parametrize("kw", [dict(), dict(projection=True, layernorm=True)], ids=lambda k: "+".join(sorted(k)) or "basic")
 def test_wave_bidirectional(kw, B):
@@ -214,6 +214,7 @@ def test_wave_bidirectional_many_rows(B, units):
     yf, hf, cf, _ = R.run(f.layers, f.x, *f.initial_state())
     yb, hb, cb, _ = R.run(b.layers, f.x[::-1], *b.initial_state())
     with qlstm.BiQLSTM(f.layers, b.layers, T, B) as q:
+        q.debug_resident(1)
         plan = q.debug_wave_plan(T, B)
         assert plan[0] == MANY and plan[2:] == (units, 1), plan
         dev = torch.device("cuda:0")
@@ -226,8 +227,8 @@ def test_wave_bidirectional_many_rows(B, units):
             assert np.array_equal(got.cpu().numpy(), ref)
 
 
-# which path a call takes where the wavefront kernels were measured slower (lines in wave_preferred and wave_row_groups): few steps of one
-# row, wide single layers of many rows; and where the few-row form's groups would stream too much, the many-row form
+# which path a call takes, without the kernel with resident weights, where the wavefront kernels were measured slower (lines in
+# wave_preferred and wave_row_groups): few steps of one row, wide single layers of many rows; and where the few-row form's groups would stream too much, the many-row form
 @pytest.mark.parametrize("dims,layers,kw,T,B,taken,form", [
     ((64, 256, 256), 1, dict(), 2, 1, 0, 1), ((64, 256, 256), 1, dict(), 5, 1, 1, 1), ((64, 256, 128), 4, dict(projection=True), 8, 1, 0, 1),
     ((64, 256, 128), 4, dict(projection=True), 3, 1, 1, 1), ((64, 128, 128), 1, dict(), 1, 3, 0, 1), ((64, 256, 256), 2, dict(), 2, 2, 1, 1),
@@ -239,12 +240,16 @@ def test_wave_selection(dims, layers, kw, T, B, taken, form):
     h0, c0 = w.initial_state()
     want = R.run(w.layers, w.x, h0, c0)
     with qlstm.QLSTM(w.layers, T, B) as q:
+        q.debug_resident(1)
         plan = q.debug_wave_plan(T, B)
         assert (plan[3], plan[0]) == (taken, form), plan
-        for impl in ((0, 0), (0, WAVE)):
+        for resident, impl in ((1, (0, 0)), (1, (0, WAVE)), (0, (0, 0))):
+            q.debug_resident(resident)
             got = run_gpu(w, handle=q, impl=impl)
             for name, g, r in zip(("y", "h", "c"), got[:3], want[:3]):
-                assert np.array_equal(g, r), (name, impl)
+                assert np.array_equal(g, r), (name, resident, impl)
+        # (with automatic selection the kernel with resident weights comes first)
+        assert q.debug_wave_plan(T, B)[3] == (0 if q.debug_resident_plan(T, B)[0] else taken)
 
 
 def test_wave_timeout_is_reported_and_the_handle_recovers():
