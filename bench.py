@@ -469,7 +469,7 @@ def main():
                        projection_frac_of_2x_bf16_burst=tops / int8_burst,
                        recurrent_us_per_layer_step=1e3 * pr["recurrent_ms"] / (n * nl * wl.T))
         else:
-            ent.update(path="one launch for all layers and steps (wavefront kernels; whole-stack kernel for one step of one or two rows)",
+            ent.update(path="one launch for all layers and steps (wavefront kernels, with resident weights where they fit; whole-stack kernel for one step of one or two rows)",
                        us_per_layer_step=1e3 * ms / (nl * wl.T))
         if wl.B <= 4:
             ent["streaming_us_per_call_T1"] = streaming_us(qh, wl)
