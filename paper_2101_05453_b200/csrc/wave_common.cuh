@@ -1,4 +1,4 @@
-// What the two wavefront kernels share: the description of a call, bounded waits, the exchanges between the blocks of a
+// What the wavefront kernels share: the description of a call, bounded waits, the exchanges between the blocks of a
 // group, and the fixed-point pieces of a step.  wave_sm100.cu has the overview.
 #pragma once
 

@@ -13,7 +13,7 @@
 // m, h - goes from shared memory into the shared memory of the peers (16 or 8 bytes at a time, counted on an mbarrier there) instead of
 // through L2 with a counter to poll and a copy back; only what the layer above reads is still written and published there, off the chain,
 // each block in a word of its own (wv_wait_blocks).
-// Without, groups may have any number of blocks.  The plan takes the cheaper one (wave_cluster_plan).
+// Without, groups may have any number of blocks.  A model fitted to measurements of both chooses (wave_cluster_plan).
 #include <cstring>
 
 #include "wave_common.cuh"
