@@ -753,20 +753,21 @@ __global__ void __launch_bounds__(WV_THREADS, 1) k_wave_small_sm100(const __grid
 
     // ---------------- teardown ----------------
     ptx::cta_sync();
-    if (*abort_flag) {
+    const bool aborted = *abort_flag != 0;
+    if (aborted) {
         // a wait ran out: copies and MMAs in flight end, then report
         ws_drain(ctl, k.nb, warp);
-        if (threadIdx.x == 0) {
-            atomicExch(k.abort_word, 1u); atomicExch(k.status, 2);
-            if (CL) {
-                // what peers sent before they left arrives within microseconds; this block does not end before
-                const unsigned long long t0 = wv_timer();
-                while (wv_timer() - t0 < 50000ull) {}
-            }
-        }
+        if (threadIdx.x == 0) { atomicExch(k.abort_word, 1u); atomicExch(k.status, 2); }
     }
     ptx::cta_sync();
-    if (CL) wv_cluster_sync();                                 // no block ends while a peer may still store into it
+    if (CL) {
+        wv_cluster_sync();                                     // no block ends while a peer may still store into it:
+        if (aborted && threadIdx.x == 0) {
+            // what peers sent before they came here arrives within microseconds (a block that has not given up has waited for all of it)
+            const unsigned long long t0 = wv_timer();
+            while (wv_timer() - t0 < 50000ull) {}
+        }
+    }
     if (warp == 2) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem_base, 512);

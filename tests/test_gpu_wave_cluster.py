@@ -53,3 +53,33 @@ def test_wave_cluster_is_left_alone_where_it_is_slower(layers, dims, B, kw):
     w = random_layer_stack(990 + B, layers, *dims, T=2, B=B, **kw)
     with qlstm.QLSTM(w.layers, 2, B) as q:
         assert q.debug_wave_cluster(2, B) == 0 and q.debug_wave_plan(2, B)[0] == 1
+
+
+# a wait that runs out: reported, the caller's state untouched, nothing in flight for the calls that follow
+@pytest.mark.parametrize("T", [3, 12])
+@pytest.mark.parametrize("kw", VARIANTS, ids=lambda k: "+".join(sorted(k)) or "basic")
+def test_wave_cluster_abort_leaves_state_and_handle_as_they_were(kw, T):
+    import torch
+    import paper_2101_05453_b200 as qlstm
+    w = random_layer_stack(995, 3, 48, 272, 112, T=T, B=11, **kw)
+    want = R.run(w.layers, w.x, *w.initial_state())
+    dev = torch.device("cuda:0")
+    with qlstm.QLSTM(w.layers, T, 11) as q:
+        assert q.debug_wave_cluster(T, 11) >= 8
+        x = torch.from_numpy(w.x).to(dev)
+        y = torch.zeros((T, 11, w.layers[-1].n_output), dtype=torch.int8, device=dev)
+        rng = np.random.default_rng(T)
+        h0, c0 = (rng.integers(-100, 100, a.shape).astype(a.dtype) for a in w.initial_state())
+        for limit in (300_000, 3_000_000):
+            h, c = torch.from_numpy(h0).to(dev), torch.from_numpy(c0).to(dev)
+            q.debug_barrier_timeout(1, limit)
+            q.set_impl(0, WAVE)
+            q.run(x, T, 11, h, c, y, stream=torch.cuda.current_stream().cuda_stream)
+            with pytest.raises(qlstm.QlstmError) as e:
+                q.last_status()
+            assert e.value.code == qlstm.binding.ERR_TIMEOUT
+            assert np.array_equal(h.cpu().numpy(), h0) and np.array_equal(c.cpu().numpy(), c0)
+            q.debug_barrier_timeout(0)
+            for _ in range(2):
+                for name, g, r in zip(("y", "h", "c"), run_gpu(w, handle=q, impl=(0, WAVE))[:3], want[:3]):
+                    assert np.array_equal(g, r), name
